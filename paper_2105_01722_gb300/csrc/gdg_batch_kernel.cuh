@@ -134,7 +134,7 @@ template <int N1, int STAGE, int VARIANT>
 __global__ void __launch_bounds__(nthreads_for(N1 * N1), batch_min_blocks(N1, VARIANT))
 k_batch_all(const BatchProb *__restrict__ probs, int n_probs, const int2 *__restrict__ items, int n_items,
             int chunk) {
-    extern __shared__ double smem[];
+    extern __shared__ __align__(16) double smem[];
     __shared__ VarParams s_vp;
     __shared__ VarBufs s_b;
     __shared__ double s_c[2];

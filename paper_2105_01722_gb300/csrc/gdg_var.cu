@@ -47,14 +47,15 @@ size_t geom_smem(int N1, int Q) {
 }
 size_t traces_smem(int N1, int Q) { return sizeof(double) * ((size_t)tab_len(Q, N1) + 2 * N1 * N1 + 12 * N1); }
 
-template <int N1>
-size_t stage_smem(int Q, bool mixed, bool no_matrix) { return StageSmem<N1>::bytes(Q, mixed, no_matrix); }
 size_t invert_smem(int N1) { return sizeof(double) * (2 * (size_t)N1 * N1 * N1 * N1 + (size_t)N1 * N1); }
-size_t fold_smem(int N1) { return sizeof(double) * ((size_t)fold_rlen(N1) + 12 * (size_t)N1 + 2 * (size_t)N1 * N1); }
 
-// The dynamic shared-memory limit is a property of the kernel function, shared
-// by every context: always raise it to the device's opt-in maximum so that a
-// context with smaller needs cannot lower it under another one.
+const VarOps &ops_of(int n1) {
+    static const VarOps *const all[] = {&var_ops_2, &var_ops_3, &var_ops_4, &var_ops_5, &var_ops_6,
+                                        &var_ops_7, &var_ops_8, &var_ops_9, &var_ops_10};
+    return *all[n1 - 2];
+}
+
+// see VarLaunch::attrs
 template <int N1>
 void set_attrs() {
     int dev = 0, lim = 0;
@@ -62,34 +63,13 @@ void set_attrs() {
     cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaFuncSetAttribute(k_var_geom<N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_var_traces<N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_var_stage<N1, M_RHS>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_var_stage<N1, M_S1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_var_stage<N1, M_S23>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_var_stage<N1, M_S4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_var_pcg<N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_var_invert<N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_var_fold<N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-}
-
-template <int N1>
-void launch_stage_n(const VarData &D, int mode, const VarBufs &b, double cA, double cY, cudaStream_t s) {
-    const dim3 grid(D.vp.ne), block(nthreads_for(N1 * N1));
-    const size_t sm = D.smem_stage;
-    switch (mode) {
-    case M_RHS: k_var_stage<N1, M_RHS><<<grid, block, sm, s>>>(D.vp, b, cA, cY); break;
-    case M_S1: k_var_stage<N1, M_S1><<<grid, block, sm, s>>>(D.vp, b, cA, cY); break;
-    case M_S23: k_var_stage<N1, M_S23><<<grid, block, sm, s>>>(D.vp, b, cA, cY); break;
-    default: k_var_stage<N1, M_S4><<<grid, block, sm, s>>>(D.vp, b, cA, cY); break;
-    }
+    ops_of(N1).attrs(lim);
 }
 
 void launch_stage_raw(gdg_ctx *ctx, int mode, const VarBufs &b, double cA, double cY, cudaStream_t s) {
     const VarData &D = *ctx->var;
-    switch (ctx->n1) {
-#define X(n) case n: launch_stage_n<n>(D, mode, b, cA, cY, s); break;
-        GDG_VAR_CASES(X)
-#undef X
-    }
+    ops_of(ctx->n1).stage(D.vp, D.smem_stage, mode, b, cA, cY, s);
 }
 
 // One RK stage.  With an attached network the stage is split in three
@@ -126,12 +106,7 @@ void launch_traces(gdg_ctx *ctx, const double *u, const double *v, double *tr, c
 
 void launch_pcg_raw(gdg_ctx *ctx, int which, const double *b, double *x, cudaStream_t s) {
     const VarData &D = *ctx->var;
-    const dim3 grid(ctx->ne), block(nthreads_for(ctx->n1 * ctx->n1));
-    switch (ctx->n1) {
-#define X(n) case n: k_var_pcg<n><<<grid, block, D.smem_pcg, s>>>(D.vp, which == GDG_OP_S, b, x, D.d_iters, D.d_rel, D.d_sweeps); break;
-        GDG_VAR_CASES(X)
-#undef X
-    }
+    ops_of(ctx->n1).pcg(D.vp, D.smem_pcg, which == GDG_OP_S, b, x, D.d_iters, D.d_rel, D.d_sweeps, s);
 }
 
 double *vbuf(gdg_ctx *ctx, int i) { return ctx->var->d_state + (size_t)i * ctx->ndof; }
@@ -195,36 +170,29 @@ int gdg_var_setup(gdg_ctx *ctx) {
         }
     for (int i = 0; i < n1; ++i) { dL[i] = ctx->dphiL[i]; dR[i] = ctx->dphiR[i]; lam[i] = ctx->lamh[i]; }
     for (int i = 0; i < NA; ++i) Ps[i] = ctx->Psih[i];
-    // modes in parity order (the even ones first, each class in the original
-    // ascending-lambda order, so the constant mode stays first) where the
-    // basis has the r -> 1-r symmetry: the FP64 preconditioner then works by
-    // node pairs (precondition_parity)
-    bool parity = true;
+    // Psi as integers for the preconditioner: rows and columns sum to at most 1 in units of 2^ps_exp
+    std::vector<int2> psx(NA);
+    int ps_exp = 0;
     {
         double big = 0.0;
-        for (int i = 0; i < NA; ++i) big = std::max(big, std::fabs(Ps[i]));
-        std::vector<int> ev, od;
-        for (int k = 0; k < n1 && parity; ++k) {
-            bool even = true, odd = true;
-            for (int i = 0; i < n1; ++i) {
-                const double a = Ps[i * n1 + k], m = Ps[(n1 - 1 - i) * n1 + k];
-                if (std::fabs(m - a) > 1e-9 * big) even = false;
-                if (std::fabs(m + a) > 1e-9 * big) odd = false;
-            }
-            if (even) ev.push_back(k);
-            else if (odd) od.push_back(k);
-            else parity = false;
+        for (int a = 0; a < n1; ++a) {
+            double row = 0.0, col = 0.0;
+            for (int k = 0; k < n1; ++k) { row += std::fabs(Ps[a * n1 + k]); col += std::fabs(Ps[k * n1 + a]); }
+            big = std::max(big, std::max(row, col));
         }
-        parity = parity && (int)ev.size() == (n1 + 1) / 2 && ev[0] == 0;
-        if (parity) {
-            std::vector<int> order(ev);
-            order.insert(order.end(), od.begin(), od.end());
-            const std::vector<double> P0(Ps, Ps + NA), L0(lam, lam + n1);
-            for (int k = 0; k < n1; ++k) {
-                lam[k] = L0[order[k]];
-                for (int i = 0; i < n1; ++i) Ps[i * n1 + k] = P0[i * n1 + order[k]];
-            }
+        std::frexp(big * (1.0 + 1e-14), &ps_exp);
+        for (int i = 0; i < NA; ++i) {
+            const long long v = std::llrint(std::ldexp(Ps[i], FX_ONE - ps_exp));
+            const long long half = 1ll << (FX_LIMB - 1), lo = ((v + half) & ((1ll << FX_LIMB) - 1)) - half;
+            psx[i] = make_int2((int)((v - lo) >> FX_LIMB), (int)lo);
         }
+    }
+    // the slopes across a face against the values behind them (lift_lines)
+    int slope_exp = 0;
+    {
+        double sl = 0.0, sr = 0.0;
+        for (int i = 0; i < n1; ++i) { sl += std::fabs(dL[i]); sr += std::fabs(dR[i]); }
+        std::frexp(std::max(sl, sr), &slope_exp);
     }
 
     const size_t nd = (size_t)ctx->ndof;
@@ -275,7 +243,6 @@ int gdg_var_setup(gdg_ctx *ctx) {
     VarParams &P = D->vp;
     P.nx = ctx->nx; P.ny = ctx->ny; P.ne = ctx->ne; P.Q = Q;
     P.affine = D->d_affine;
-    P.parity = parity;
     P.per_x = ctx->pb.bc[0] == GDG_BC_PERIODIC;
     P.per_y = ctx->pb.bc[1] == GDG_BC_PERIODIC;
     P.upwind = ctx->pb.flux == GDG_FLUX_UPWIND;
@@ -294,15 +261,14 @@ int gdg_var_setup(gdg_ctx *ctx) {
     switch (n1) {
 #define X(n)                                                                                   \
     case n:                                                                                    \
-        D->smem_stage = stage_smem<n>(Q, ctx->pb.precision == GDG_MIXED, ctx->pb.solver == GDG_SOLVE_INVERSE); \
-        D->smem_pcg = stage_smem<n>(Q, ctx->pb.precision == GDG_MIXED, false);                  \
+        D->smem_stage = D->smem_pcg = StageSmem<n>::bytes();                                     \
         set_attrs<n>();                                                                        \
         break;
         GDG_VAR_CASES(X)
 #undef X
     }
     if (D->smem_pcg > 220 * 1024 || D->smem_geom > 220 * 1024 ||
-        (ctx->pb.solver == GDG_SOLVE_INVERSE && (invert_smem(n1) > 220 * 1024 || fold_smem(n1) > 220 * 1024)))
+        (ctx->pb.solver == GDG_SOLVE_INVERSE && invert_smem(n1) > 220 * 1024))
         return gdg_set_err(ctx, GDG_EUNSUPPORTED, "element too large for shared memory (reduce nquad)");
     const double *Xd = D->d_nodes, *Yd = D->d_nodes + nd, *Cd = D->d_nodes + 2 * nd;
     switch (n1) {
@@ -318,7 +284,20 @@ int gdg_var_setup(gdg_ctx *ctx) {
         GDG_VAR_CASES(X)
 #undef X
     }
-    P.FM = D->d_FM;
+    if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_FMq, (size_t)ctx->ne * 12 * n1 * sizeof(short2)), "alloc FMq")) ||
+        (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_Psx, psx.size() * sizeof(int2)), "alloc Psi")) ||
+        (st = gdg_cuda_check(ctx, cudaMemcpy(D->d_Psx, psx.data(), psx.size() * sizeof(int2), cudaMemcpyHostToDevice), "upload Psi")))
+        return st;
+    switch (n1) {
+#define X(n) case n: k_fm_pack<n><<<ctx->ne, nthreads_for(n * n)>>>(D->d_FM, slope_exp, D->d_FMq); break;
+        GDG_VAR_CASES(X)
+#undef X
+    }
+    P.FM = reinterpret_cast<const int2 *>(D->d_FM);
+    P.FMq = D->d_FMq;
+    P.slope_exp = slope_exp;
+    P.Psx = D->d_Psx;
+    P.Ps_exp = ps_exp;
     P.src_e = -1;   // no point source until gdg_set_point_source
     if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_time, sizeof(double)), "alloc time")) ||
         (st = gdg_cuda_check(ctx, cudaMemset(D->d_time, 0, sizeof(double)), "time")))
@@ -344,42 +323,40 @@ int gdg_var_setup(gdg_ctx *ctx) {
     }
     P.dS = D->d_dS;
     P.inverse = ctx->pb.solver == GDG_SOLVE_INVERSE;
-    if (P.inverse) {   // element inverses (S_c2 + w w^T)^-1 and M_J^-1, folded with the lifts
+    const size_t fxm = (size_t)ctx->ne * fx_tri_len(NA);   // one set of packed integer matrices
+    const int sets = P.inverse ? 4 : 2;
+    if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_fx, sets * fxm * sizeof(int2)), "alloc integer matrices")) ||
+        (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_fxd, sets * nd), "alloc exponents")))
+        return st;
+    if (P.inverse) {   // element inverses (S_c2 + w w^T)^-1 and M_J^-1
         const size_t nm = nd * NA;
         if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_Ainv, nm * sizeof(double)), "alloc Ainv")) ||
-            (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_Minv, nm * sizeof(double)), "alloc Minv")) ||
-            (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_G, nd * fold_cols(n1) * sizeof(double)), "alloc G")))
+            (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_Minv, nm * sizeof(double)), "alloc Minv")))
             return st;
-        const size_t ism = invert_smem(n1), fsm = fold_smem(n1);
+        const size_t ism = invert_smem(n1);
         switch (n1) {
 #define X(n)                                                                                         \
     case n:                                                                                          \
         k_var_invert<n><<<ctx->ne, nthreads_for(n * n), ism>>>(D->d_S, D->d_w, D->d_Ainv);           \
         k_var_invert<n><<<ctx->ne, nthreads_for(n * n), ism>>>(D->d_M, nullptr, D->d_Minv);          \
-        k_var_fold<n><<<ctx->ne, nthreads_for(n * n), fsm>>>(D->d_S, D->d_Ainv, D->d_Minv, D->d_tab, Q, D->d_G); \
         break;
             GDG_VAR_CASES(X)
 #undef X
         }
-        P.G = D->d_G;
     }
-    if (P.mixed) {   // FP32 copies of the element matrices (packed lower triangles) for the inner solves
-        const size_t nm = (size_t)ctx->ne * tri_len(NA);
-        if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_S32, nm * sizeof(float)), "alloc S32")) ||
-            (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_M32, nm * sizeof(float)), "alloc M32")))
-            return st;
+    FxMatrix *const fxs[4] = {&P.Sx, &P.Mx, &P.Ax, &P.Vx};
+    const double *const from[4] = {D->d_S, D->d_M, D->d_Ainv, D->d_Minv};
+    for (int k = 0; k < sets; ++k) {
+        int2 *A = D->d_fx + k * fxm;
+        signed char *d = D->d_fxd + k * nd;
         const int grid = (int)std::min<long long>(ctx->ne, 65535);
         switch (n1) {
-#define X(n)                                                                  \
-    case n:                                                                   \
-        k_to_f32_lower<n><<<grid, 128>>>(ctx->ne, D->d_S, D->d_S32);          \
-        k_to_f32_lower<n><<<grid, 128>>>(ctx->ne, D->d_M, D->d_M32);          \
-        break;
+#define X(n) case n: k_fx_pack<n><<<grid, 128>>>(ctx->ne, from[k], A, d); break;
             GDG_VAR_CASES(X)
 #undef X
         }
-        P.S32 = D->d_S32;
-        P.M32 = D->d_M32;
+        fxs[k]->A = A;
+        fxs[k]->d = d;
     }
     st = gdg_cuda_check(ctx, cudaDeviceSynchronize(), "assembly");
     cudaFree(D->d_nodes);
@@ -399,7 +376,7 @@ int gdg_var_setup(gdg_ctx *ctx) {
 void gdg_var_free(gdg_ctx *ctx) {
     VarData *D = ctx->var;
     if (!D) return;
-    cudaFree(D->d_S); cudaFree(D->d_M); cudaFree(D->d_S32); cudaFree(D->d_M32); cudaFree(D->d_dS); cudaFree(D->d_Ainv); cudaFree(D->d_Minv); cudaFree(D->d_G); cudaFree(D->d_FM); cudaFree(D->d_time); cudaFree(D->d_src); cudaFree(D->d_w); cudaFree(D->d_pre); cudaFree(D->d_face); cudaFree(D->d_affine);
+    cudaFree(D->d_S); cudaFree(D->d_M); cudaFree(D->d_dS); cudaFree(D->d_Ainv); cudaFree(D->d_Minv); cudaFree(D->d_fx); cudaFree(D->d_fxd); cudaFree(D->d_FMq); cudaFree(D->d_Psx); cudaFree(D->d_FM); cudaFree(D->d_time); cudaFree(D->d_src); cudaFree(D->d_w); cudaFree(D->d_pre); cudaFree(D->d_face); cudaFree(D->d_affine);
     cudaFree(D->d_tab); cudaFree(D->d_nodes); cudaFree(D->d_state); cudaFree(D->d_tr);
     cudaFree(D->d_c2feat); cudaFree(D->d_wbf16); cudaFree(D->d_mlp);
     cudaFree(D->d_ru); cudaFree(D->d_rv); cudaFree(D->d_x0u);
@@ -653,41 +630,12 @@ extern "C" int gdg_set_point_source(gdg_ctx *ctx, int element, double r, double 
         return GDG_OK;
     }
     const int n1 = ctx->n1, NA = n1 * n1;
-    std::vector<double> pr(n1), dpr(n1), ps(n1), dps(n1), w(2 * (size_t)NA, 0.0);
+    std::vector<double> pr(n1), dpr(n1), ps(n1), dps(n1), w((size_t)NA, 0.0);
     gdg_eval_basis(ctx->p, ctx->N, r, -1, pr.data(), dpr.data());
     gdg_eval_basis(ctx->p, ctx->N, s, -1, ps.data(), dps.data());
     for (int j = 0; j < n1; ++j)
         for (int i = 0; i < n1; ++i) w[(size_t)j * n1 + i] = ps[j] * pr[i];
-    if (D.vp.inverse) {   // the inverse route adds M_J^-1 w: Gaussian elimination with partial pivoting
-        std::vector<double> M((size_t)NA * NA), x(w.begin(), w.begin() + NA);
-        if ((st = gdg_cuda_check(ctx, cudaMemcpy(M.data(), D.d_M + (size_t)element * NA * NA, M.size() * sizeof(double),
-                                                 cudaMemcpyDeviceToHost), "point source: mass matrix")))
-            return st;
-        for (int k = 0; k < NA; ++k) {
-            int piv = k;
-            for (int i = k + 1; i < NA; ++i)
-                if (std::fabs(M[(size_t)i * NA + k]) > std::fabs(M[(size_t)piv * NA + k])) piv = i;
-            if (piv != k) {
-                for (int c = 0; c < NA; ++c) std::swap(M[(size_t)k * NA + c], M[(size_t)piv * NA + c]);
-                std::swap(x[k], x[piv]);
-            }
-            const double d = M[(size_t)k * NA + k];
-            if (!(std::fabs(d) > 0.0)) return gdg_set_err(ctx, GDG_EINVAL, "point source: singular mass matrix");
-            for (int i = k + 1; i < NA; ++i) {
-                const double m = M[(size_t)i * NA + k] / d;
-                if (m == 0.0) continue;
-                for (int c = k; c < NA; ++c) M[(size_t)i * NA + c] -= m * M[(size_t)k * NA + c];
-                x[i] -= m * x[k];
-            }
-        }
-        for (int k = NA - 1; k >= 0; --k) {
-            double acc = x[k];
-            for (int c = k + 1; c < NA; ++c) acc -= M[(size_t)k * NA + c] * x[c];
-            x[k] = acc / M[(size_t)k * NA + k];
-        }
-        for (int a = 0; a < NA; ++a) w[(size_t)NA + a] = x[a];
-    }
-    if (!D.d_src && (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D.d_src, 2 * (size_t)NA * sizeof(double)), "alloc source")))
+    if (!D.d_src && (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D.d_src, (size_t)NA * sizeof(double)), "alloc source")))
         return st;
     if ((st = gdg_cuda_check(ctx, cudaMemcpy(D.d_src, w.data(), w.size() * sizeof(double), cudaMemcpyHostToDevice),
                              "point source: upload")))
@@ -699,5 +647,19 @@ extern "C" int gdg_set_point_source(gdg_ctx *ctx, int element, double r, double 
     return GDG_OK;
 }
 
-// this translation unit's check slot (gdg_checks.cuh)
-GDG_CHECKS_READER(gdg_checks_read_var)
+// the check slots of this translation unit and of the element kernels' (gdg_checks.cuh)
+static GDG_CHECKS_READER(var_checks_read)
+int gdg_checks_read_var(GdgCheckSlot *out, int reset) {
+    GdgCheckSlot acc{};
+    if (var_checks_read(&acc, reset)) return -1;
+    for (int n1 = 2; n1 <= GDG_VAR_MAXN1; ++n1) {
+        GdgCheckSlot s{};
+        // one slot a unit: N+1 = 2..5 share theirs
+        if (n1 >= 3 && n1 <= 5) continue;
+        if (ops_of(n1).checks(&s, reset)) return -1;
+        if (s.count && !acc.count) acc = s;
+        else acc.count += s.count;
+    }
+    *out = acc;
+    return 0;
+}

@@ -5,9 +5,16 @@
 #include "gdg_checks.cuh"
 #include <cmath>
 
+#include "gdg_fx.cuh"
 #include "gdg_internal.h"
 
 #define GDG_VAR_MAXN1 10
+
+// element matrices as integers (k_fx_pack)
+struct FxMatrix {
+    const int2 *A;
+    const signed char *d;
+};
 
 struct VarParams {
     int nx, ny, ne, Q;
@@ -18,37 +25,71 @@ struct VarParams {
     int maxit, precond;   // GDG_PC_*
     const double *tab;    // B[Q][N1], D[Q][N1], wq[Q], dphiL[N1], dphiR[N1], Psi[N1][N1], lam[N1]
     const double *S, *M, *w, *pre, *face;
-    const float *S32, *M32;      // FP32 copies of S and M (mixed precision only)
     const double *dS;            // [ne][N1*N1] frozen-coefficient preconditioner diagonal (S system)
-    const double *FM;            // [ne][4 faces][6 N1 columns][3 N1 rows] face operators (k_var_facemat)
+    // the operators of the stage as integers (gdg_fx.cuh).  Element matrices: packed lower triangles
+    // (fx_tri_len entries an element) and the exponents d of their rows [ne][N1*N1]
+    FxMatrix Sx, Mx;             // S_c2, M_J
+    FxMatrix Ax, Vx;             // (S_c2 + w w^T)^-1 - 1 1^T (k_var_invert), M_J^-1 (GDG_SOLVE_INVERSE)
+    const int2 *FM;              // [ne][4 faces][6 N1 columns][3 N1 rows] face operators (k_var_facemat)
+    const short2 *FMq;           // [ne][4 faces][3 N1] exponents of a row's v columns and u columns
+    int slope_exp;               // the u slopes along a face normal count as 2^-slope_exp of the u values
+    const int2 *Psx;             // Psi in units of 2^(Ps_exp - 57), rows and columns summing to at most 2^57
+    int Ps_exp;
     // point source f = src_amp sin(src_omega t) delta(x - x_s) (gdg_set_point_source)
     int src_e;                   // element holding x_s (-1: no source)
     double src_amp, src_omega;
-    const double *src_w;         // [2][NA]: phi_a(x_s), and M_J^-1 of it (inverse route)
+    const double *src_w;         // [NA]: phi_a(x_s)
     double *time;                // source time at the start of the current RK step
-    int inverse;                 // GDG_SOLVE_INVERSE: element inverses folded into G instead of PCG
-    const double *G;             // [ne][12 N1 + NA][NA] folded operators, column-major (fold_cols)
+    int inverse;                 // GDG_SOLVE_INVERSE: element inverses instead of PCG
     unsigned long long *stats;   // [0] sum it_u, [1] sum it_v, [2] max it_u, [3] max it_v,
                                  // [4] unconverged u, [5] unconverged v, [6] element solves,
                                  // [7] sum sweeps u, [8] sum sweeps v, [9] max sweeps u, [10] max sweeps v
     int mixed;                   // FP32 inner PCG + FP64 refinement
     const unsigned char *affine; // [ne] 1: the element is a parallelogram (J constant), so the
                                  // frozen-coefficient mass preconditioner is M_J^-1 exactly
-    int parity;                  // the table's modes are in parity order (even modes first,
-                                 // Psi[N1-1-i][m] = +-Psi[i][m]): FP64 preconditioner by pairs
     int refine_max;              // FP64 refinement sweeps per solve
     float refine_rtol;           // inner FP32 PCG relative tolerance
 };
 
+struct VarBufs {
+    const double *yU, *yV;   // stage input (nodal)
+    double *nU, *nV, *aU, *aV, *oU, *oV;
+    const double *trin;
+    double *trout;
+    // split stage for the learned initial guess: part 0 = whole stage;
+    // part 1 = write the residuals r_u, r_v and stop; part 2 = take r_u, r_v
+    // and the u_t guess x0u from memory and solve (falling back to x0 = 0 when
+    // the guess's residual is not smaller than ||r_u||)
+    int part;
+    double *ru, *rv;
+    const double *x0u;
+    double tstage;           // this stage's time offset in the RK step (0, dt/2, dt/2, dt)
+};
+
+struct VarData;
+
+// The element kernels of one N1: their own translation unit each (gdg_var_n*.cu),
+// so that they compile in parallel.
+struct VarOps {
+    void (*attrs)(int smem_limit);
+    void (*stage)(const VarParams &P, size_t smem, int mode, const VarBufs &b, double cA, double cY, cudaStream_t s);
+    void (*pcg)(const VarParams &P, size_t smem, int which, const double *b, double *x, int *iters, double *rel,
+                int *sweeps, cudaStream_t s);
+    int (*checks)(GdgCheckSlot *out, int reset);   // the unit's check slot (gdg_checks.cuh)
+};
+extern const VarOps var_ops_2, var_ops_3, var_ops_4, var_ops_5, var_ops_6, var_ops_7, var_ops_8, var_ops_9, var_ops_10;
+
 struct VarData {
     int nq = 0, Q = 0, NA = 0;
     double *d_S = nullptr, *d_M = nullptr, *d_w = nullptr, *d_pre = nullptr, *d_face = nullptr;
-    float *d_S32 = nullptr, *d_M32 = nullptr;
     double *d_dS = nullptr;
-    double *d_G = nullptr;                       // folded operators (GDG_SOLVE_INVERSE)
-    double *d_FM = nullptr;                      // face operators
-    double *d_time = nullptr, *d_src = nullptr;  // point source: time, weights [2][NA]
-    double *d_Ainv = nullptr, *d_Minv = nullptr; // setup temporaries of the fold, freed after it
+    int2 *d_fx = nullptr;                        // packed integer matrices: S, M (, A^-1, M^-1)
+    signed char *d_fxd = nullptr;                // their row exponents
+    double *d_FM = nullptr;                      // face operators (integers after k_fm_pack)
+    short2 *d_FMq = nullptr;
+    int2 *d_Psx = nullptr;
+    double *d_time = nullptr, *d_src = nullptr;  // point source: time, weights [NA]
+    double *d_Ainv = nullptr, *d_Minv = nullptr; // setup temporaries of the inverses, freed after it
     double *d_tab = nullptr, *d_nodes = nullptr;
     unsigned char *d_affine = nullptr;           // per element: a parallelogram
     double *d_state = nullptr, *d_tr = nullptr;
@@ -93,23 +134,6 @@ __device__ __forceinline__ Tabs tabs_at(const double *base, int Q, int N1) {
     return t;
 }
 __host__ __device__ constexpr int tab_len(int Q, int N1) { return 2 * Q * N1 + Q + 2 * N1 + N1 * N1 + N1; }
-// the tables after B and D (wq, dphiL, dphiR, Psi, lam)
-__host__ __device__ constexpr int tab_tail_len(int Q, int N1) { return Q + 2 * N1 + N1 * N1 + N1; }
-
-// B and D read from global memory (L1-cached), the rest from a shared copy of
-// the tail: keeps the stage kernels' shared memory independent of 2 Q N1
-__device__ __forceinline__ Tabs tabs_split(const double *gtab, const double *tail, int Q, int N1) {
-    Tabs t;
-    t.B = gtab;
-    t.D = gtab + Q * N1;
-    t.wq = tail;
-    t.dphiL = t.wq + Q;
-    t.dphiR = t.dphiL + N1;
-    t.Ps = t.dphiR + N1;
-    t.lam = t.Ps + N1 * N1;
-    return t;
-}
-
 // copy the 1-D tables into shared memory
 __device__ void load_tabs(double *dst, const double *src, int n) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
@@ -162,437 +186,451 @@ __device__ __forceinline__ T block_sum(T v, double *red) {
     return s;
 }
 
-template <int NA, typename T>
-__device__ __forceinline__ T block_dot(const T *a, const T *b, double *red) {
-    const int t = threadIdx.x;
-    return block_sum<T>(t < NA ? a[t] * b[t] : (T)0, red);
+// ---------------------------------------------------- element solves -----
+//
+// One block works on one element, thread t owns entry t of every vector (in a
+// register).  Products with the element matrices and the preconditioner run on
+// integers (gdg_fx.cuh), and the FP64 work left is kept to what one thread per
+// entry, or warp 0 alone, can do: an FP64 warp instruction takes 16 cycles of
+// the SM's pipe whatever its active lanes.  (One warp per element with three
+// rows a lane issues a third fewer instructions but leaves 7 warps an SM, too
+// few to hide the integer pipe's latency: 12.2 against 9.5 ms a PCG step of 128 x 128 elements at p = 5.)
+
+// one element's matrix and the block's scratch
+struct FxSystem {
+    const int2 *A;   // packed integers (shared)
+    int d;           // exponent of the thread's row
+    int2 *X, *X2;    // limb vectors (shared, 16-byte aligned)
+    int *slot;       // shared: two sets of 8 ints, used in turn
+};
+
+constexpr int FX_NAN = 1 << 20;   // block exponent of a vector with an Inf or NaN
+
+// exponent of v 2^shift for the maximum of a vector (zero and subnormals: below every other)
+__device__ __forceinline__ int fx_key(double v, int shift = 0) {
+    const int e = fx_expo(v);
+    return e == 0 ? -FX_NAN : e == 0x7ff ? FX_NAN : e + shift;
 }
 
-// Lower triangle of a symmetric NA x NA matrix, row by row: entry (i, k),
-// k <= i, at i (i + 1) / 2 + k.  The FP32 element matrices of the mixed
-// solves are kept this way (half the shared memory of the full matrix).
-__host__ __device__ constexpr int tri_len(int na) { return na * (na + 1) / 2; }
+// largest k of the block (at most 4 warps).  One barrier: consecutive calls use
+// the two slot sets in turn (`set` 0 or 1), so a set is rewritten only after
+// the barrier that follows its last read.
+__device__ __forceinline__ int fx_block_max(int k, int *slot, int set) {
+    k = __reduce_max_sync(0xffffffffu, k);
+    int *sl = slot + 8 * set;
+    if ((threadIdx.x & 31) == 0) sl[threadIdx.x >> 5] = k;
+    __syncthreads();
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) k = max(k, sl[w]);
+    return k;
+}
 
-// y = A x for a symmetric A held as its packed lower triangle: row t reads
-// (t, 0..t) from row t and (k, t) for k > t from the rows below, so every
-// product and the order of the sum are those of the full row-major matvec.
-template <int NA, typename T>
-__device__ __forceinline__ void matvec_packed(const T *L, const T *x, T *y) {
-    const int t = threadIdx.x;
-    if (t < NA) {
-        T s = 0;
-        const int row = t * (t + 1) / 2;
-        int col = t;                    // k (k + 1) / 2 + t at k = 0
-#pragma unroll 9
-        for (int k = 0; k < NA; ++k) {
-            s = fma(k <= t ? L[row + k] : L[col], x[k], s);
-            col += k + 1;
-        }
-        y[t] = s;
+// T 2^q, or NaN where the vector behind T had an Inf or NaN
+__device__ __forceinline__ double fx_value(long long T, int q, int emax) {
+    return emax >= FX_NAN / 2 ? __longlong_as_double(0x7ff8000000000000ll) : fx_scale(T, q);
+}
+
+// mad(entry (t, k), k) over row t of the packed matrix: the columns of earlier
+// warps' rows lie in row t, those of later warps' rows in the rows below (both
+// at fixed strides), and only those of the own warp's rows need a choice
+template <int NA, typename MAD>
+__device__ __forceinline__ void fx_row(const int2 *A, MAD mad) {
+    const int t = threadIdx.x, k0 = t & ~31, k1 = min(k0 + 32, NA);
+    const int2 *row = A + t * (t + 1) / 2;             // entry (t, k), k <= t
+#pragma unroll 8
+    for (int k = 0; k < k0; ++k) mad(row[k], k);
+    const int2 *col = A + k0 * (k0 + 1) / 2 + t;       // entry (k, t), moving with k
+#pragma unroll 8
+    for (int k = k0; k < k1; ++k) {
+        mad(*(k <= t ? row + k : col), k);
+        col += k + 1;
     }
-    __syncthreads();
-}
-
-// y = A x for a symmetric NA x NA matrix in global memory, read by columns
-// (thread t reads column t: coalesced), summed in row order
-template <int NA>
-__device__ __forceinline__ void matvec_g(const double *__restrict__ A, const double *x, double *y) {
-    const int t = threadIdx.x;
-    if (t < NA) {
-        double s = 0.0;
-        const double *col = A + t;
-#pragma unroll 9
-        for (int k = 0; k < NA; ++k) s += __ldg(col + (size_t)k * NA) * x[k];
-        y[t] = s;
+#pragma unroll 8
+    for (int k = k1; k < NA; ++k) {
+        mad(*col, k);
+        col += k + 1;
     }
-    __syncthreads();
 }
 
-// FP64 dot products of NA-vectors in shared memory summed by warp 0 alone:
-// lane i accumulates entries i, i+32, i+64, ... (FMA chain), then a butterfly.
-// The FP64 pipe issues a warp instruction at full cost whatever its active
-// lanes (measured on GB300: one active lane per warp takes as long as 32), so
-// one warp doing the whole sum costs 3 + 5 FP64 warp instructions where every
-// warp adding its partial cost 27 for a 96-thread block.  The other warps wait
-// at the barrier.  Fixed order: deterministic.  Leading barrier: the inputs
-// are written (and the previous result has been read) before warp 0 starts.
+// The thread's entry of A x for its entry of x.  Two barriers; `set` as in
+// fx_block_max.
 template <int NA>
-__device__ __forceinline__ double warp0_dot(const double *a, const double *b, double *red) {
+__device__ __forceinline__ double fx_matvec(const FxSystem &f, double x, int set) {
+    const int t = threadIdx.x;
+    const int emax = fx_block_max(t < NA ? fx_key(x, f.d) : -FX_NAN, f.slot, set);
+    if (t < NA) f.X[t] = fx_split(fx_int(x, emax, f.d));
     __syncthreads();
-    if (threadIdx.x < 32) {
-        double s = 0.0;
+    FxSum s;
+    const int2 *X = f.X;
+    if (t < NA) fx_row<NA>(f.A, [&](int2 a, int k) { s.mad(a, X[k]); });
+    return fx_value(s.top(), fx_top_exp(emax) + f.d, emax);
+}
+
+// Psi of the frozen-coefficient preconditioner as integers (shared), and the
+// thread's entry of the diagonal; or none
+struct FxPrecond {
+    const int2 *Ps;
+    int pexp;
+    double d;
+    bool none;
+};
+
+// z = Psi2 diag(d) Psi2^T r, Psi2 = Psi (x) Psi (index j*N1+i), on integers:
+// four contractions of N1 terms, the vector rescaled to its largest entry
+// before the first and, after the diagonal, before the third (two in a row
+// keep at least 52 bits: Psi's rows and columns sum to at most 1 in units of
+// 2^pexp).  Four FP64 operations a node where the contractions by node pairs
+// took 27.  Uses both slot sets; ends without a barrier.
+template <int N1>
+__device__ __forceinline__ double fx_precondition(const FxSystem &f, const FxPrecond &p, double r) {
+    constexpr int NA = N1 * N1;
+    const int t = threadIdx.x;
+    if (p.none) return r;
+    const bool on = t < NA;
+    const int a = on ? t / N1 : 0, c = on ? t - a * N1 : 0;
+    const int e1 = fx_block_max(on ? fx_key(r) : -FX_NAN, f.slot, 0);
+    if (on) f.X[t] = fx_split(fx_int(r, e1));
+    __syncthreads();
+    if (on) {   // x modes: sum_i r[j][i] Psi[i][k]
+        FxSum s;
 #pragma unroll
-        for (int k = threadIdx.x; k < NA; k += 32) s = fma(a[k], b[k], s);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) red[0] = s;
+        for (int q = 0; q < N1; ++q) s.mad(p.Ps[q * N1 + c], f.X[a * N1 + q]);
+        f.X2[t] = s.next();
     }
     __syncthreads();
-    return red[0];
+    double v = 0.0;
+    if (on) {   // y modes and the diagonal: d[l][k] sum_j Psi[j][l] t[j][k]
+        FxSum s;
+#pragma unroll
+        for (int q = 0; q < N1; ++q) s.mad(p.Ps[q * N1 + a], f.X2[q * N1 + c]);
+        v = (double)s.top() * p.d;
+    }
+    const int e2 = fx_block_max(on ? fx_key(v) : -FX_NAN, f.slot, 1);
+    if (on) f.X[t] = fx_split(fx_int(v, e2));
+    __syncthreads();
+    if (on) {   // back in x: sum_k t[l][k] Psi[i][k]
+        FxSum s;
+#pragma unroll
+        for (int q = 0; q < N1; ++q) s.mad(p.Ps[c * N1 + q], f.X[a * N1 + q]);
+        f.X2[t] = s.next();
+    }
+    __syncthreads();
+    FxSum s;   // back in y: sum_l Psi[j][l] t[l][i]
+    if (on) {
+#pragma unroll
+        for (int q = 0; q < N1; ++q) s.mad(p.Ps[a * N1 + q], f.X2[q * N1 + c]);
+    }
+    return fx_value(s.top(), 4 * p.pexp + e1 + e2 + 2 * fx_top_exp(0), max(e1, e2));
 }
 
-// two such dot products with one pair of barriers: a.b and c.d.  The first
-// butterfly level splits the two sums between the half-warps (lanes 0-15
-// keep a.b, lanes 16-31 c.d, each adding its partner's partial of its own
-// sum), so the five levels cost five FP64 additions, not ten.
+// warp 0: the sums of a[k] b[k] and of c[k] d[k] over the NA entries in shared
+// memory, each in every lane.  A lane adds its entries in order, then a
+// butterfly whose first level leaves one sum to each half-warp, so the five
+// levels cost five FP64 additions, not ten.
 template <int NA>
-__device__ __forceinline__ void warp0_dot2(const double *a, const double *b, const double *c, const double *d,
+__device__ __forceinline__ void lane_dot2(const double *a, const double *b, const double *c, const double *d,
+                                          double &ab, double &cd) {
+    double s = 0.0, q = 0.0;
+#pragma unroll
+    for (int k = threadIdx.x; k < NA; k += 32) {
+        s = fma(a[k], b[k], s);
+        q = fma(c[k], d[k], q);
+    }
+    const bool lo = threadIdx.x < 16;
+    double v = (lo ? s : q) + __shfl_xor_sync(0xffffffffu, lo ? q : s, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    ab = __shfl_sync(0xffffffffu, v, 0);
+    cd = __shfl_sync(0xffffffffu, v, 16);
+}
+
+// the same for the whole block (leading barrier: the vectors are written)
+template <int NA>
+__device__ __forceinline__ void block_dot2(const double *a, const double *b, const double *c, const double *d,
                                            double *red, double &ab, double &cd) {
     __syncthreads();
     if (threadIdx.x < 32) {
-        double s = 0.0, q = 0.0;
-#pragma unroll
-        for (int k = threadIdx.x; k < NA; k += 32) {
-            s = fma(a[k], b[k], s);
-            q = fma(c[k], d[k], q);
-        }
-        const bool lo = threadIdx.x < 16;
-        double v = (lo ? s : q) + __shfl_xor_sync(0xffffffffu, lo ? q : s, 16);
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0) red[0] = v;
-        if (threadIdx.x == 16) red[1] = v;
+        lane_dot2<NA>(a, b, c, d, ab, cd);
+        if (threadIdx.x == 0) { red[0] = ab; red[1] = cd; }
     }
     __syncthreads();
     ab = red[0];
     cd = red[1];
 }
 
-// two block sums with one pair of barriers (same order as block_sum)
-template <typename T>
-__device__ __forceinline__ void block_sum2(T &a, T &b, double *red) {
+// sqrt(rr) <= thr, the square root taken only where the squares are too close
+// to decide (or out of range)
+__device__ __forceinline__ bool norm_below(double rr, double thr) {
+    const double t2 = thr * thr;
+    if (t2 > 1e-280 && t2 < 1e280) {
+        if (rr > t2 * (1.0 + 1e-14)) return false;
+        if (rr < t2 * (1.0 - 1e-14)) return true;
+    }
+    return sqrt(rr) <= thr;
+}
+
+// the block's vectors of a solve (shared, NA doubles each) and its scalars
+struct SolveBufs {
+    double *r, *z, *p, *Ap, *red;   // red: 8 doubles
+    const double *w;
+};
+
+// x0 and r0 = b - A x0 (- w (w.x0)) of a solve: x0 = 0, or the guess in x,
+// dropped (*fell = 1) when `fallback` and its true residual is no smaller than b
+template <int NA>
+__device__ __forceinline__ double first_residual(const FxSystem &f, const SolveBufs &v, bool W, double w, double b,
+                                                 double &x, bool x0_zero, bool fallback, int *fell) {
+    const int t = threadIdx.x;
+    if (x0_zero) {
+        x = 0.0;
+        return b;
+    }
+    double r = b - fx_matvec<NA>(f, x, 0);
+    if (t < NA) v.z[t] = x;
+    if (W) {
+        double wx, same;
+        block_dot2<NA>(v.w, v.z, v.w, v.z, v.red, wx, same);
+        r -= w * wx;
+    }
+    if (fallback) {
+        double rr, bb;
+        if (t < NA) { v.r[t] = r; v.p[t] = b; }
+        block_dot2<NA>(v.r, v.r, v.p, v.p, v.red, rr, bb);
+        if (rr >= bb) {
+            x = 0.0;
+            r = b;
+            *fell = 1;
+        }
+        __syncthreads();
+    }
+    return r;
+}
+
+// Preconditioned CG on A (+ w w^T when W) with x0 = x (x0_zero: x0 = 0).
+// Stops when ||r|| <= rtol ||b|| (tested before each iteration), after
+// maxit iterations, or when r.z = 0.  Returns the iteration count; *relres is
+// formed when asked for or when the cap was reached.  b, x, w: the thread's
+// entries.
+template <int N1>
+__device__ __forceinline__ int pcg(const FxSystem &f, const FxPrecond &pre, const SolveBufs &v, bool W, double w,
+                                   double b, double &x, double rtol, int maxit, bool x0_zero, double *relres,
+                                   bool fallback, int *fell, bool want_rel) {
+    constexpr int NA = N1 * N1;
+    const int t = threadIdx.x;
+    const bool on = t < NA, warp0 = t < 32;
+    double r = first_residual<NA>(f, v, W, w, b, x, x0_zero, fallback, fell);
+    if (on) { v.r[t] = r; v.p[t] = b; }
+    double b2 = 0.0, thr = 0.0;   // warp 0's
+    double p = 0.0, rz = 0.0, rr = 0.0;
+    int it = -1;   // the first pass only forms z and p
+    while (true) {
+        const double z = fx_precondition<N1>(f, pre, r);
+        if (on) v.z[t] = z;
+        __syncthreads();
+        ++it;
+        if (warp0) {
+            double rzn, rrn, beta = 0.0;
+            lane_dot2<NA>(v.r, v.z, v.r, v.r, rzn, rrn);
+            if (it == 0) {
+                double same;
+                lane_dot2<NA>(v.p, v.p, v.p, v.p, b2, same);
+                thr = rtol * sqrt(b2);
+            }
+            const bool done = it >= maxit || norm_below(rrn, thr) || rzn == 0.0;
+            if (it && !done) beta = rzn / rz;
+            if (t == 0) { v.red[0] = beta; v.red[1] = done ? 1.0 : 0.0; v.red[2] = rrn; }
+            rz = rzn;
+        }
+        __syncthreads();
+        if (v.red[1] != 0.0) break;
+        p = it ? z + v.red[0] * p : z;
+        if (on) v.p[t] = p;
+        const double Ap = fx_matvec<NA>(f, p, 0);
+        if (on) v.Ap[t] = Ap;
+        __syncthreads();
+        if (warp0) {   // p.(A + w w^T)p = p.Ap + (w.p)^2
+            double pAp, wp;
+            lane_dot2<NA>(v.p, v.Ap, W ? v.w : v.p, W ? v.p : v.Ap, pAp, wp);
+            if (W) pAp += wp * wp;
+            const double alpha = rz / pAp;
+            if (t == 0) { v.red[4] = alpha; v.red[5] = wp; }
+        }
+        __syncthreads();
+        const double alpha = v.red[4];
+        x += alpha * p;
+        r -= alpha * (W ? Ap + w * v.red[5] : Ap);
+        if (on) v.r[t] = r;
+    }
+    rr = v.red[2];
+    if (want_rel || it >= maxit) {   // the cap, or the caller's statistics
+        __syncthreads();
+        if (t == 0) v.red[3] = b2 > 0.0 ? sqrt(rr) / sqrt(b2) : 0.0;
+        __syncthreads();
+        *relres = v.red[3];
+    } else {
+        *relres = 0.0;
+    }
+    __syncthreads();
+    return it;
+}
+
+// ---- the FP32 inner solves of the mixed form
+
+// the inner system: the thread's row scale 2^d, preconditioner diagonal and w
+struct Inner32 {
+    float sc, d, w;
+    const float *Ps;       // shared
+    float *t1, *t2, *red;  // shared scratch: NA floats each; two sets of 8 partial sums
+    float rtol;
+    int maxit;
+    bool none;
+};
+
+// The thread's entry of A x in 32 bits: the upper limbs of A (29 bits against
+// the largest of the scaled matrix, where a float has 24) and x as an integer
+// of 28 bits against its largest entry, summed exactly.
+template <int NA>
+__device__ __forceinline__ float fx_matvec32(const FxSystem &f, float sc, float x) {
+    const int t = threadIdx.x;
+    const float v = x * sc;
+    const int e = fx_block_max(t < NA ? (__float_as_int(v) >> 23) & 0xff : 0, f.slot, 0);   // |v| < 2^(e - 126)
+    int *X = reinterpret_cast<int *>(f.X);
+    if (t < NA) X[t] = __float2int_rn(v * __int_as_float(max(1, min(254, 281 - e)) << 23));   // v 2^(154 - e)
+    __syncthreads();
+    long long s = 0;
+    if (t < NA) fx_row<NA>(f.A, [&](int2 a, int k) { s += (long long)a.x * X[k]; });
+    // a.x in units of 2^-28: the sum times 2^(e - 182)
+    const float down = e == 255 ? __int_as_float(0x7fc00000) : __int_as_float(max(1, min(254, e - 23)) << 23);
+    return ((float)(int)(s >> 32) + (float)(unsigned)s * 2.3283064365386963e-10f) * down * sc;
+}
+
+// the thread's entry of z = Psi2 diag(d) Psi2^T r in FP32; ends without a barrier
+template <int N1>
+__device__ __forceinline__ float precondition32(const Inner32 &in, float r) {
+    constexpr int NA = N1 * N1;
+    const int t = threadIdx.x;
+    if (in.none) return r;
+    const bool on = t < NA;
+    const int a = on ? t / N1 : 0, c = on ? t - a * N1 : 0;
+    if (on) in.t1[t] = r;
+    __syncthreads();
+    float s = 0.f;
+#pragma unroll
+    for (int q = 0; q < N1; ++q) s = fmaf(in.t1[a * N1 + q], in.Ps[q * N1 + c], s);
+    if (on) in.t2[t] = s;
+    __syncthreads();
+    s = 0.f;
+#pragma unroll
+    for (int q = 0; q < N1; ++q) s = fmaf(in.Ps[q * N1 + a], in.t2[q * N1 + c], s);
+    if (on) in.t1[t] = in.d * s;
+    __syncthreads();
+    s = 0.f;
+#pragma unroll
+    for (int q = 0; q < N1; ++q) s = fmaf(in.t1[a * N1 + q], in.Ps[c * N1 + q], s);
+    if (on) in.t2[t] = s;
+    __syncthreads();
+    s = 0.f;
+#pragma unroll
+    for (int q = 0; q < N1; ++q) s = fmaf(in.Ps[a * N1 + q], in.t2[q * N1 + c], s);
+    return s;
+}
+
+// two block sums with one barrier (the two sets of partial sums in turn)
+__device__ __forceinline__ void block_sum2(float &a, float &b, float *red, int set) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         a += __shfl_xor_sync(0xffffffffu, a, o);
         b += __shfl_xor_sync(0xffffffffu, b, o);
     }
-    const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    T *part = reinterpret_cast<T *>(red);
+    float *part = red + 8 * set;
+    const int w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) { part[w] = a; part[4 + w] = b; }
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) { part[w] = a; part[16 + w] = b; }
-    __syncthreads();
-    T sa = 0, sb = 0;
-    for (int i = 0; i < nw; ++i) { sa += part[i]; sb += part[16 + i]; }
-    a = sa;
-    b = sb;
+    a = b = 0.f;
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) { a += part[i]; b += part[4 + i]; }
 }
 
-// z = Psi2 diag(d) Psi2^T r, Psi2 = Psi (x) Psi (index j*N1+i), or z = r
-template <int N1, typename T>
-__device__ void precondition(const T *r, T *z, const T *Ps, const T *d, T *t1, T *t2, bool none) {
-    constexpr int NA = N1 * N1;
-    const int t = threadIdx.x;
-    if (none) {
-        if (t < NA) z[t] = r[t];
-        __syncthreads();
-        return;
-    }
-    const int a = t / N1, c = t - (t / N1) * N1;
-    if (t < NA) {   // t1[j][k] = sum_i r[j][i] Psi[i][k]
-        T s = 0;
-#pragma unroll
-        for (int i = 0; i < N1; ++i) s += r[a * N1 + i] * Ps[i * N1 + c];
-        t1[t] = s;
-    }
-    __syncthreads();
-    if (t < NA) {   // t2[l][k] = d[l][k] sum_j Psi[j][l] t1[j][k]
-        T s = 0;
-#pragma unroll
-        for (int j = 0; j < N1; ++j) s += Ps[j * N1 + a] * t1[j * N1 + c];
-        t2[t] = d[t] * s;
-    }
-    __syncthreads();
-    if (t < NA) {   // t1[l][i] = sum_k t2[l][k] Psi[i][k]
-        T s = 0;
-#pragma unroll
-        for (int k = 0; k < N1; ++k) s += t2[a * N1 + k] * Ps[c * N1 + k];
-        t1[t] = s;
-    }
-    __syncthreads();
-    if (t < NA) {   // z[j][i] = sum_l Psi[j][l] t1[l][i]
-        T s = 0;
-#pragma unroll
-        for (int l = 0; l < N1; ++l) s += Ps[a * N1 + l] * t1[l * N1 + c];
-        z[t] = s;
-    }
-    __syncthreads();
-}
-
-// The same z = Psi2 diag(d) Psi2^T r (FP64) with the modes in parity order:
-// the NE = ceil(N1/2) even modes first, Psi[N1-1-i][m] = Psi[i][m] for them
-// and -Psi[i][m] for the odd ones.  Each 1-D contraction then splits into an
-// even part over the NE node-pair sums (the middle node alone when N1 is odd)
-// and an odd part over the N1 - NE node-pair differences, so every output is
-// a dot of at most NE terms instead of N1: the four contractions cost about
-// half the multiplies, for a combination pass at each end.  Work arrays in
-// class layout: index q < NE is the even class with pair q, q >= NE the odd
-// class with pair q - NE (pair p: nodes p and N1-1-p).
+// FP32 PCG from x0 = 0 on A + w w^T (w = 0 for the mass system) for a
+// right-hand side of unit norm, r its entry: stops when ||r|| <= rtol, after
+// maxit iterations or at r.z = 0.  x: the thread's entry of the result.
 template <int N1>
-__device__ void precondition_parity(const double *r, double *z, const double *Ps, const double *d, double *t1,
-                                    double *t2) {
-    constexpr int NA = N1 * N1, NE = (N1 + 1) / 2;
-    const int t = threadIdx.x;
-    const int a = t / N1, b = t - (t / N1) * N1;
-    // pairs and signs of the nodes of this thread (used by the first and last pass)
-    if (t < NA) {   // combine r over node pairs, both directions -> t1[a][b] (class layout)
-        const bool oy = a >= NE, ox = b >= NE;
-        const int ry = oy ? a - NE : a, rx = ox ? b - NE : b;
-        const int my = N1 - 1 - ry, mx = N1 - 1 - rx;
-        double c0 = r[ry * N1 + rx], c1 = 0.0;
-        if (mx != rx) c0 = ox ? c0 - r[ry * N1 + mx] : c0 + r[ry * N1 + mx];
-        if (my != ry) {
-            c1 = r[my * N1 + rx];
-            if (mx != rx) c1 = ox ? c1 - r[my * N1 + mx] : c1 + r[my * N1 + mx];
-            c0 = oy ? c0 - c1 : c0 + c1;
-        }
-        t1[t] = c0;
-    }
-    __syncthreads();
-    if (t < NA) {   // x modes: t2[a][k] = sum over the class of k of t1[a][q] Psi[q][k]
-        const int q0 = b >= NE ? NE : 0, nq = b >= NE ? N1 - NE : NE;
-        double s = 0.0;
-#pragma unroll
-        for (int q = 0; q < NE; ++q)
-            if (q < nq) s = fma(t1[a * N1 + q0 + q], Ps[q * N1 + b], s);
-        t2[t] = s;
-    }
-    __syncthreads();
-    if (t < NA) {   // y modes and the diagonal: t1[l][k] = d[l][k] sum over the class of l
-        const int q0 = a >= NE ? NE : 0, nq = a >= NE ? N1 - NE : NE;
-        double s = 0.0;
-#pragma unroll
-        for (int q = 0; q < NE; ++q)
-            if (q < nq) s = fma(t2[(q0 + q) * N1 + b], Ps[q * N1 + a], s);
-        t1[t] = d[t] * s;
-    }
-    __syncthreads();
-    if (t < NA) {   // back to y pairs: t2[a][k] = sum over the modes l of the class of a
-        const int l0 = a >= NE ? NE : 0, nl = a >= NE ? N1 - NE : NE, p = a >= NE ? a - NE : a;
-        double s = 0.0;
-#pragma unroll
-        for (int q = 0; q < NE; ++q)
-            if (q < nl) s = fma(Ps[p * N1 + l0 + q], t1[(l0 + q) * N1 + b], s);
-        t2[t] = s;
-    }
-    __syncthreads();
-    if (t < NA) {   // back to x pairs: t1[a][b] = sum over the modes k of the class of b
-        const int k0 = b >= NE ? NE : 0, nk = b >= NE ? N1 - NE : NE, p = b >= NE ? b - NE : b;
-        double s = 0.0;
-#pragma unroll
-        for (int q = 0; q < NE; ++q)
-            if (q < nk) s = fma(Ps[p * N1 + k0 + q], t2[a * N1 + k0 + q], s);
-        t1[t] = s;
-    }
-    __syncthreads();
-    if (t < NA) {   // nodes: z[j][i] = (even + sx odd in x) (even + sy odd in y)
-        const int j = a, i = b;
-        const int pj = j < N1 - 1 - j ? j : N1 - 1 - j, pi = i < N1 - 1 - i ? i : N1 - 1 - i;
-        const bool midj = pj == N1 - 1 - pj, midi = pi == N1 - 1 - pi;
-        const double sy = j == pj ? 1.0 : -1.0, sx = i == pi ? 1.0 : -1.0;
-        double v = t1[pj * N1 + pi];
-        if (!midi) v = fma(sx, t1[pj * N1 + NE + pi], v);
-        if (!midj) {
-            double o = t1[(NE + pj) * N1 + pi];
-            if (!midi) o = fma(sx, t1[(NE + pj) * N1 + NE + pi], o);
-            v = fma(sy, o, v);
-        }
-        z[t] = v;
-    }
-    __syncthreads();
-}
-
-// Preconditioned CG on A (packed lower triangle; + w w^T when W) with x0 = x
-// (x0_zero: x0 = 0).
-// Stops when ||r|| <= rtol ||b|| (tested before each iteration), after
-// maxit iterations, or when r.z = 0.  Returns the iteration count.
-template <int N1, bool W>
-__device__ int pcg(const double *A, const double *w, const double *b, double *x, double *r, double *z,
-                   double *p, double *Ap, const double *Ps, const double *d, double *t1, double *t2,
-                   double *red, double rtol, int maxit, bool none, bool x0_zero, double *relres,
-                   bool fallback = false, int *fell = nullptr, bool parity = false) {
+__device__ __forceinline__ int pcg32(const FxSystem &f, const Inner32 &in, float r, float &x) {
     constexpr int NA = N1 * N1;
-    const int t = threadIdx.x;
-    if (x0_zero) {
-        if (t < NA) { x[t] = 0.0; r[t] = b[t]; }
-        __syncthreads();
-    } else {
-        matvec_packed<NA, double>(A, x, Ap);
-        double wx = W ? warp0_dot<NA>(w, x, red) : 0.0;
-        if (t < NA) r[t] = b[t] - Ap[t] - (W ? w[t] * wx : 0.0);
-        __syncthreads();
-        // a guess that does not beat x0 = 0 (true FP64 residual) is dropped
-        double rr0, bb0;
-        if (fallback) warp0_dot2<NA>(r, r, b, b, red, rr0, bb0);
-        if (fallback && rr0 >= bb0) {
-            if (t < NA) { x[t] = 0.0; r[t] = b[t]; }
-            __syncthreads();
-            if (fell) *fell = 1;
-        }
-    }
-    const double bnorm = sqrt(warp0_dot<NA>(b, b, red));
-    if (parity && !none) precondition_parity<N1>(r, z, Ps, d, t1, t2);
-    else precondition<N1>(r, z, Ps, d, t1, t2, none);
-    if (t < NA) p[t] = z[t];
-    // r.z and r.r in one reduction, before the loop and after every update
-    double rz, rr;
-    warp0_dot2<NA>(r, z, r, r, red, rz, rr);
-    int it = 0;
-    while (it < maxit) {
-        if (sqrt(rr) <= rtol * bnorm || rz == 0.0) break;
-        matvec_packed<NA, double>(A, p, Ap);
-        // p.(A + w w^T)p = p.Ap + (w.p)^2: one reduction for both
-        double pAp, wp = 0.0;
-        if (W) {
-            warp0_dot2<NA>(p, Ap, w, p, red, pAp, wp);
-            pAp += wp * wp;
-        } else {
-            pAp = warp0_dot<NA>(p, Ap, red);
-        }
-        const double alpha = rz / pAp;
-        if (t < NA) {
-            x[t] += alpha * p[t];
-            r[t] -= alpha * (W ? Ap[t] + w[t] * wp : Ap[t]);
-        }
-        __syncthreads();
-        if (parity && !none) precondition_parity<N1>(r, z, Ps, d, t1, t2);
-        else precondition<N1>(r, z, Ps, d, t1, t2, none);
-        double rzn;
-        warp0_dot2<NA>(r, z, r, r, red, rzn, rr);
-        const double beta = rzn / rz;
-        if (t < NA) p[t] = z[t] + beta * p[t];
-        __syncthreads();
-        rz = rzn;
+    const bool on = threadIdx.x < NA;
+    float p = 0.f, rz = 0.f;
+    x = 0.f;
+    int it = -1;
+    while (true) {
+        const float z = precondition32<N1>(in, r);
+        float rzn = on ? r * z : 0.f, rr = on ? r * r : 0.f;
+        block_sum2(rzn, rr, in.red, 0);
         ++it;
-    }
-    *relres = bnorm > 0.0 ? sqrt(rr) / bnorm : 0.0;
-    return it;
-}
-
-// FP32 PCG from x0 = 0 on A32 (packed lower triangle; + w32 w32^T when W)
-// for a right-hand side of unit norm: stops when ||r|| <= irtol, after imaxit iterations or at r.z = 0.
-template <int N1, bool W>
-__device__ int pcg32(const float *A, const float *w, const float *b, float *x, float *r, float *z, float *p,
-                     float *Ap, const float *Ps, const float *d, float *t1, float *t2, double *red, float irtol,
-                     int imaxit, bool none) {
-    constexpr int NA = N1 * N1;
-    const int t = threadIdx.x;
-    if (t < NA) { x[t] = 0.f; r[t] = b[t]; }
-    __syncthreads();
-    precondition<N1, float>(r, z, Ps, d, t1, t2, none);
-    if (t < NA) p[t] = z[t];
-    float rz = t < NA ? r[t] * z[t] : 0.f, rr = t < NA ? r[t] * r[t] : 0.f;
-    block_sum2<float>(rz, rr, red);
-    int it = 0;
-    while (it < imaxit) {
-        if (sqrtf(rr) <= irtol || rz == 0.f) break;
-        matvec_packed<NA, float>(A, p, Ap);
-        // p.(A + w w^T)p = p.Ap + (w.p)^2: one reduction for both
-        float pAp = t < NA ? p[t] * Ap[t] : 0.f, wp = (W && t < NA) ? w[t] * p[t] : 0.f;
-        block_sum2<float>(pAp, wp, red);
-        if (W) pAp += wp * wp;
-        const float alpha = rz / pAp;
-        if (t < NA) {
-            x[t] += alpha * p[t];
-            r[t] -= alpha * (Ap[t] + (W ? w[t] * wp : 0.f));
-        }
-        __syncthreads();
-        precondition<N1, float>(r, z, Ps, d, t1, t2, none);
-        float rzn = t < NA ? r[t] * z[t] : 0.f;
-        rr = t < NA ? r[t] * r[t] : 0.f;
-        block_sum2<float>(rzn, rr, red);
-        const float beta = rzn / rz;
-        if (t < NA) p[t] = z[t] + beta * p[t];
-        __syncthreads();
+        if (it >= in.maxit || sqrtf(rr) <= in.rtol || rzn == 0.f) break;
+        p = it ? z + (rzn / rz) * p : z;
         rz = rzn;
-        ++it;
+        const float Ap = fx_matvec32<NA>(f, in.sc, p);
+        float pAp = on ? p * Ap : 0.f, wp = on ? in.w * p : 0.f;
+        block_sum2(pAp, wp, in.red, 1);
+        const float alpha = rz / (pAp + wp * wp);   // p.(A + w w^T)p = p.Ap + (w.p)^2
+        x += alpha * p;
+        r -= alpha * (Ap + in.w * wp);
     }
     return it;
 }
 
 // Mixed-precision solve of A x = b (+ w w^T when W): iterative refinement with
-// the FP64 matrix (symmetric, in global memory) for every residual and FP32
-// PCG for every correction.
+// FP64-accurate products with A for every residual and FP32 PCG for every
+// correction.
 //   r = b - A x (FP64);  while ||r|| > rtol ||b||:  A c ~= r/||r|| (FP32 PCG),
 //   x += ||r|| c (FP64);  r = b - A x (FP64)
 // The stopping test is the FP64 PCG's (true FP64 residual), so the accuracy
 // is that of the FP64 solver at the same rtol.  Returns the sweeps (FP64
 // residual evaluations after the first); *inner = FP32 iterations.
-struct SolveScratch32 {
-    float *A32, *Ps32, *d32, *w32;          // matrix, preconditioner basis and diagonal, w
-    float *rhs, *x, *res, *z, *p, *Ap, *t1, *t2;
-};
-
-// FP64 step: when `step64` is given (z, t1, t2, Ps, d of the FP64
-// preconditioner) and x0 = 0, the solve first takes the FP64 preconditioned
-// steepest-descent step x = alpha P^-1 b (the first FP64 PCG iterate); where
-// the frozen-coefficient preconditioner is exact (the mass matrix of an affine
-// element) that step already meets the tolerance and no FP32 sweep runs.
-struct Step64 {
-    double *z, *t1, *t2;
-    const double *Ps, *d;
-    bool parity;   // modes in parity order (precondition_parity)
-};
-
-template <int N1, bool W>
-__device__ int refine(const double *__restrict__ A, const double *w, const double *b, double *x, double *r, double *Ap,
-                      const SolveScratch32 &f, double *red, double rtol, int maxsweep, float irtol,
-                      int imaxit, bool none, bool x0_zero, int *inner, double *relres,
-                      bool fallback = false, int *fell = nullptr, const Step64 *step64 = nullptr) {
+// FP64 step: when `step64` is set and x0 = 0, the solve (of the mass system)
+// first takes the FP64 preconditioned steepest-descent step x = alpha P^-1 b
+// (the first FP64 PCG iterate); where the frozen-coefficient preconditioner is
+// exact (the mass matrix of an affine element) that step already meets the
+// tolerance and no FP32 sweep runs.
+template <int N1>
+__device__ __forceinline__ int refine(const FxSystem &f, const FxPrecond &pre, const Inner32 &in, const SolveBufs &v,
+                                      bool W, double w, double b, double &x, double rtol, int maxsweep, bool x0_zero,
+                                      int *inner, double *relres, bool fallback, int *fell, bool step64) {
     constexpr int NA = N1 * N1;
     const int t = threadIdx.x;
+    const bool on = t < NA;
+    double r;
     if (x0_zero && step64) {
-        if (step64->parity && !none)
-            precondition_parity<N1>(b, step64->z, step64->Ps, step64->d, step64->t1, step64->t2);
-        else
-            precondition<N1>(b, step64->z, step64->Ps, step64->d, step64->t1, step64->t2, none);
-        matvec_g<NA>(A, step64->z, Ap);
-        if (W) {
-            const double wz = warp0_dot<NA>(w, step64->z, red);
-            if (t < NA) Ap[t] += w[t] * wz;
-            __syncthreads();
-        }
+        const double z = fx_precondition<N1>(f, pre, b), Az = fx_matvec<NA>(f, z, 0);
+        if (on) { v.z[t] = z; v.r[t] = Az; v.p[t] = b; }   // (v.Ap holds the inner solves' Psi)
         double bz, zAz;
-        warp0_dot2<NA>(b, step64->z, step64->z, Ap, red, bz, zAz);
+        block_dot2<NA>(v.p, v.z, v.z, v.r, v.red, bz, zAz);
         const double alpha = zAz > 0.0 ? bz / zAz : 0.0;
-        if (t < NA) {
-            x[t] = alpha * step64->z[t];
-            r[t] = b[t] - alpha * Ap[t];
-        }
-        __syncthreads();
-    } else if (x0_zero) {
-        if (t < NA) { x[t] = 0.0; r[t] = b[t]; }
-        __syncthreads();
+        x = alpha * z;
+        r = b - alpha * Az;
     } else {
-        matvec_g<NA>(A, x, Ap);
-        const double wx = W ? warp0_dot<NA>(w, x, red) : 0.0;
-        if (t < NA) r[t] = b[t] - Ap[t] - (W ? w[t] * wx : 0.0);
-        __syncthreads();
-        double rr0, bb0;
-        if (fallback) warp0_dot2<NA>(r, r, b, b, red, rr0, bb0);
-        if (fallback && rr0 >= bb0) {
-            if (t < NA) { x[t] = 0.0; r[t] = b[t]; }
-            __syncthreads();
-            if (fell) *fell = 1;
-        }
+        r = first_residual<NA>(f, v, W, w, b, x, x0_zero, fallback, fell);
     }
+    if (on) { v.r[t] = r; v.p[t] = b; }
     double bb, rr;
-    warp0_dot2<NA>(b, b, r, r, red, bb, rr);
+    block_dot2<NA>(v.p, v.p, v.r, v.r, v.red, bb, rr);
     const double bnorm = sqrt(bb);
-    int sweeps = 0, its = 0;
     double rn = sqrt(rr);
+    int sweeps = 0, its = 0;
     while (sweeps < maxsweep && rn > rtol * bnorm && rn > 0.0) {
         const double inv = 1.0 / rn;
-        if (t < NA) f.rhs[t] = (float)(r[t] * inv);
-        __syncthreads();
-        its += pcg32<N1, W>(f.A32, f.w32, f.rhs, f.x, f.res, f.z, f.p, f.Ap, f.Ps32, f.d32, f.t1, f.t2, red,
-                            irtol, imaxit, none);
-        if (t < NA) x[t] += rn * (double)f.x[t];
-        __syncthreads();
-        matvec_g<NA>(A, x, Ap);
-        const double wx = W ? warp0_dot<NA>(w, x, red) : 0.0;
-        if (t < NA) r[t] = b[t] - Ap[t] - (W ? w[t] * wx : 0.0);
-        __syncthreads();
-        rn = sqrt(warp0_dot<NA>(r, r, red));
+        float c;
+        its += pcg32<N1>(f, in, on ? (float)(r * inv) : 0.f, c);
+        x += rn * (double)c;
+        r = b - fx_matvec<NA>(f, on ? x : 0.0, 0);
+        if (W) {
+            if (on) v.z[t] = x;
+            double wx, same;
+            block_dot2<NA>(v.w, v.z, v.w, v.z, v.red, wx, same);
+            r -= w * wx;
+        }
+        if (on) v.r[t] = r;
+        double same;
+        block_dot2<NA>(v.r, v.r, v.r, v.r, v.red, rr, same);
+        rn = sqrt(rr);
         ++sweeps;
     }
     *inner = its;
@@ -602,31 +640,11 @@ __device__ int refine(const double *__restrict__ A, const double *w, const doubl
 
 // asynchronous global -> shared copies (cp.async): every copy of a matrix is
 // in flight at once instead of a register round trip per element
-__device__ __forceinline__ void cp_async_8(void *dst, const void *src) {
+__device__ __forceinline__ void cp_async_16(void *dst, const void *src) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_4(void *dst, const void *src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-// FP32 element matrix (the packed lower triangle made at setup) and FP32
-// copies of the preconditioner data
-template <int N1>
-__device__ void to_fp32(const float *A32g, float *A32, const double *Ps, float *Ps32, const double *d, float *d32,
-                        const double *w, float *w32) {
-    constexpr int NA = N1 * N1;
-    for (int i = threadIdx.x; i < tri_len(NA); i += blockDim.x) cp_async_4(A32 + i, A32g + i);
-    for (int i = threadIdx.x; i < N1 * N1; i += blockDim.x) Ps32[i] = (float)Ps[i];
-    for (int i = threadIdx.x; i < NA; i += blockDim.x) {
-        d32[i] = (float)d[i];
-        if (w) w32[i] = (float)w[i];
-    }
-    cp_async_wait_all();
-    __syncthreads();
-}
 
 // diagonal of the frozen-coefficient preconditioner in the modified basis,
 // made once at setup: dS[e][l*N1+k] = 1 / (Gss lam_l + Grr lam_k) (1 on the
@@ -644,16 +662,6 @@ k_fdm_diag(const double *__restrict__ lam, double *pre, double *dS) {
     if (t == 0) pre[(size_t)e * 4 + 3] = 1.0 / Jb;
 }
 
-template <int N1>
-__device__ void fdm_diagonals(const VarParams &P, int e, double *dS, double *dM) {
-    constexpr int NA = N1 * N1;
-    const int t = threadIdx.x;
-    if (t < NA) {
-        dS[t] = P.dS[(size_t)e * NA + t];
-        dM[t] = P.pre[(size_t)e * 4 + 3];
-    }
-}
-
 // --------------------------------------------------------- assembly -------
 
 template <int N1>
@@ -661,7 +669,7 @@ __global__ void __launch_bounds__(GEOM_THREADS)
 k_var_geom(VarParams P, const double *X, const double *Y, const double *C2, double *Sout, double *Mout,
            double *wout, double *pre, double *face) {
     constexpr int NA = N1 * N1;
-    extern __shared__ double sm[];
+    extern __shared__ __align__(16) double sm[];
     const int Q = P.Q, e = blockIdx.x, t = threadIdx.x;
     double *tb = sm;
     double *nx_ = tb + tab_len(Q, N1);
@@ -827,32 +835,28 @@ k_var_geom(VarParams P, const double *X, const double *Y, const double *C2, doub
 
 // line data of the 4 faces from nodal U, V in shared memory:
 // L[(f*3 + m)*N1 + j]: m = 0 value line of v, 1 the r-derivative data, 2 the s-derivative data
+// by the `nt` threads t = 0.. of a warp or block
 template <int N1>
-__device__ void face_lines(const double *U, const double *V, const Tabs &T, double *L) {
-    for (int task = threadIdx.x; task < 12 * N1; task += blockDim.x) {
+__device__ __forceinline__ void face_lines(const double *U, const double *V, const Tabs &T, double *L, int t, int nt) {
+    for (int task = t; task < 12 * N1; task += nt) {
         const int f = task / (3 * N1), m = (task / N1) % 3, j = task % N1;
         const double *dphi = (f == 0 || f == 2) ? T.dphiL : T.dphiR;
         const int edge = (f == 0 || f == 2) ? 0 : N1 - 1;
+        // one slope (m = 1 on x faces, 2 on y faces) and two values a line
+        const bool slope = f < 2 ? m == 1 : m == 2;
+        const double *line = f < 2 ? U + j * N1 : U + j;
+        const int step = f < 2 ? 1 : N1;
         double s = 0.0;
-        if (f < 2) {   // x faces, line index j (rows)
-            if (m == 0) s = V[j * N1 + edge];
-            else if (m == 1) { for (int i = 0; i < N1; ++i) s += U[j * N1 + i] * dphi[i]; }
-            else s = U[j * N1 + edge];
-        } else {       // y faces, line index i (columns)
-            const int i = j;
-            if (m == 0) s = V[edge * N1 + i];
-            else if (m == 1) s = U[edge * N1 + i];
-            else { for (int jj = 0; jj < N1; ++jj) s += U[jj * N1 + i] * dphi[jj]; }
-        }
+        if (slope) { for (int i = 0; i < N1; ++i) s += line[i * step] * dphi[i]; }
+        else s = (m == 0 ? (f < 2 ? V + j * N1 : V + j) : line)[edge * step];
         L[task] = s;
     }
-    __syncthreads();
 }
 
 template <int N1>
 __global__ void k_var_traces(VarParams P, const double *u, const double *v, double *trout) {
     constexpr int NA = N1 * N1;
-    extern __shared__ double sm[];
+    extern __shared__ __align__(16) double sm[];
     const int Q = P.Q, e = blockIdx.x;
     double *tb = sm, *U = tb + tab_len(Q, N1), *V = U + NA;
     load_tabs(tb, P.tab, tab_len(Q, N1));
@@ -862,26 +866,12 @@ __global__ void k_var_traces(VarParams P, const double *u, const double *v, doub
     }
     __syncthreads();
     const Tabs T = tabs_at(tb, Q, N1);
-    face_lines<N1>(U, V, T, trout + lix<N1>(e, 0));
+    face_lines<N1>(U, V, T, trout + lix<N1>(e, 0), threadIdx.x, blockDim.x);
 }
 
 // ------------------------------------------------------------ stage ------
 
 
-struct VarBufs {
-    const double *yU, *yV;   // stage input (nodal)
-    double *nU, *nV, *aU, *aV, *oU, *oV;
-    const double *trin;
-    double *trout;
-    // split stage for the learned initial guess: part 0 = whole stage;
-    // part 1 = write the residuals r_u, r_v and stop; part 2 = take r_u, r_v
-    // and the u_t guess x0u from memory and solve (falling back to x0 = 0 when
-    // the guess's residual is not smaller than ||r_u||)
-    int part;
-    double *ru, *rv;
-    const double *x0u;
-    double tstage;           // this stage's time offset in the RK step (0, dt/2, dt/2, dt)
-};
 
 // load of the point source on r_v at this stage: int phi_a f = phi_a(x_s) s(t)
 __device__ __forceinline__ double source_amplitude(const VarParams &P, const VarBufs &b) {
@@ -890,73 +880,61 @@ __device__ __forceinline__ double source_amplitude(const VarParams &P, const Var
 
 __global__ void k_set_time(double *time, double t0) { *time = t0; }
 
+// Shared memory of one element's block, in doubles: the packed matrix, Psi, w
+// and one scratch region for the phases of a stage in turn: the lifts (limbs of
+// the face lines, line integrals), the solves (vectors and limb vectors; the
+// FP32 vectors in the place of p and Ap), the new state whose face lines go out.
 template <int N1>
 struct StageSmem {
     static constexpr int NA = N1 * N1;
-    static constexpr int RED = 20;   // reduction scratch: 2 x 16 warp partials at most, in doubles
-    // A: the FP64 element matrix, packed lower triangle (FP64 solves only; the
-    // mixed solves read the full matrix from global memory for their few FP64
-    // residuals)
-    double *A, *tb, *Yu, *Yv, *ru, *rv, *x, *r, *z, *p, *Ap, *w, *dS, *dM, *t1, *t2, *fw, *L, *red;
-    // FP32 area (mixed precision only): matrix, preconditioner and PCG vectors
-    float *A32, *Ps32, *dS32, *dM32, *w32, *r32, *z32, *p32, *Ap32, *c32, *u32, *v32, *t132, *t232;
-    // Mixed: no FP64 PCG runs, so p is not allocated, and one scratch region
-    // of FP32 PCG vectors serves three phases of the stage in turn: the face
-    // lines and line integrals of the lifts (fw, L: 36 N1 doubles), then the
-    // FP64 preconditioned step's z, t1, t2 (3 NA doubles; parallelograms
-    // only), then the FP32 PCG vectors of the refinement sweeps.  The tail of
-    // the 1-D tables (wq, dphi, Psi, lam) is read from global memory through
-    // L1 (Psi serves in FP64 once per solve).  24.1 KB a block at N1 = 9:
-    // 9 elements per SM, in the batched launch too (with its parameter
-    // slots).
-    static constexpr int SCR32 = 8 * NA > 72 * N1 ? 8 * NA : 72 * N1;   // scratch floats (>= 6 NA)
-    static constexpr int SCR64 = 4 * NA > 36 * N1 ? 4 * NA : 36 * N1;   // FP64 path: z, p, t1, t2 / fw, L
-    __device__ StageSmem(double *base, int Q, bool mixed, bool no_matrix = false) {
-        tb = mixed ? nullptr : base;   // tail of the 1-D tables (tab_tail_len)
-        Yu = base + (mixed ? 0 : tab_tail_len(Q, N1));
-        Yv = Yu + NA; ru = Yv + NA; rv = ru + NA; x = rv + NA; r = x + NA;
-        if (mixed) {
-            Ap = r + NA; w = Ap + NA; dS = w + NA; dM = dS + NA;
-            red = dM + NA;
-            A = nullptr;
-            p = nullptr;
-            double *scr = red + RED;                       // 8-byte aligned
-            fw = scr; L = fw + 24 * N1;                    // lifts
-            z = scr; t1 = z + NA; t2 = t1 + NA;            // FP64 step (after the lifts)
-            r32 = reinterpret_cast<float *>(scr);          // refinement sweeps (after both)
-            z32 = r32 + NA; p32 = z32 + NA; Ap32 = p32 + NA; c32 = Ap32 + NA;
-            u32 = c32 + NA; t132 = u32 + NA; t232 = t132 + NA;
-            v32 = nullptr;
-            A32 = r32 + SCR32;
-            Ps32 = A32 + tri_len(NA); dS32 = Ps32 + N1 * N1; dM32 = dS32 + NA; w32 = dM32 + NA;
-        } else {
-            // FP64 PCG / inverses: the lifts' face lines and line integrals
-            // (fw, L) share one region with the PCG vectors z, p, t1, t2,
-            // which run after the lifts (the inverse route uses no PCG)
-            double *scr = r + NA;
-            z = scr; p = z + NA; t1 = p + NA; t2 = t1 + NA;
-            fw = scr; L = fw + 24 * N1;
-            Ap = scr + SCR64; w = Ap + NA; dS = w + NA; dM = dS + NA;
-            red = dM + NA;
-            A = no_matrix ? nullptr : red + RED;
-            A32 = Ps32 = dS32 = dM32 = w32 = r32 = z32 = p32 = Ap32 = c32 = u32 = v32 = t132 = t232 = nullptr;
-        }
+    static constexpr int NP = (NA + 1) & ~1;   // limb vectors start on 16 bytes
+    static constexpr int SCR = 36 * N1 > 6 * NP ? (36 * N1 + 1) & ~1 : 6 * NP;
+    static constexpr int LEN = fx_tri_len(NA) + 2 * NP + SCR + 24;   // 31.4 KB at N1 = 9: 7 blocks an SM
+    int2 *A, *Ps, *lines, *X, *X2;
+    int *slot;
+    double *L, *U, *V, *w, *r, *z, *p, *Ap, *red;
+    float *Ps32, *t1, *t2, *red32;
+    __device__ StageSmem(double *base) {
+        A = reinterpret_cast<int2 *>(base);
+        Ps = A + fx_tri_len(NA);
+        w = base + fx_tri_len(NA) + NP;
+        double *scr = w + NP;
+        lines = reinterpret_cast<int2 *>(scr);
+        L = scr + 24 * N1;
+        X = lines;
+        X2 = X + NP;
+        r = scr + 2 * NP;
+        z = r + NP;
+        p = z + NP;
+        Ap = p + NP;
+        t1 = reinterpret_cast<float *>(p);
+        t2 = t1 + NP;
+        Ps32 = reinterpret_cast<float *>(Ap);
+        U = scr;
+        V = scr + NP;
+        red = scr + SCR;                                  // 8 doubles
+        slot = reinterpret_cast<int *>(red + 8);          // 16 ints
+        red32 = reinterpret_cast<float *>(red + 16);      // 16 floats
     }
-    static size_t bytes(int Q, bool mixed, bool no_matrix = false) {
-        if (mixed)
-            return sizeof(double) * ((size_t)10 * NA + RED) +
-                   sizeof(float) * ((size_t)SCR32 + tri_len(NA) + N1 * N1 + 3 * NA);
-        size_t d = sizeof(double) * ((size_t)tab_tail_len(Q, N1) + 10 * NA + SCR64 + RED);
-        if (!no_matrix) d += sizeof(double) * (size_t)tri_len(NA);
-        return d;
+    static constexpr size_t bytes() { return sizeof(double) * (size_t)LEN; }
+    __device__ __forceinline__ FxSystem system(const FxMatrix &m, int e) const {
+        return FxSystem{A, threadIdx.x < NA ? m.d[(size_t)e * NA + threadIdx.x] : 0, X, X2, slot};
     }
-    __device__ SolveScratch32 scratch32(bool s_system) const {
-        SolveScratch32 f;
-        f.A32 = A32; f.Ps32 = Ps32; f.d32 = s_system ? dS32 : dM32; f.w32 = w32;
-        f.rhs = r32; f.x = c32; f.res = u32; f.z = z32; f.p = p32; f.Ap = Ap32; f.t1 = t132; f.t2 = t232;
-        return f;
-    }
+    __device__ __forceinline__ SolveBufs bufs() const { return SolveBufs{r, z, p, Ap, red, w}; }
 };
+
+// start the copy of an element's packed matrix into shared memory
+template <int N1>
+__device__ __forceinline__ void load_fx(int2 *A, const FxMatrix &m, int e) {
+    constexpr int LEN = fx_tri_len(N1 * N1);
+    const int2 *src = m.A + (size_t)e * LEN;
+    for (int i = 2 * threadIdx.x; i < LEN; i += 2 * blockDim.x) cp_async_16(A + i, src + i);
+}
+// wait for it (the whole block)
+__device__ __forceinline__ void fx_arrived() {
+    cp_async_wait_all();
+    __syncthreads();
+}
 
 // Face terms.  Per face f of an element the fluxes of Section 2.2.1 at the Q
 // face quadrature points, weighted and integrated against the face basis
@@ -1012,7 +990,7 @@ template <int N1>
 __global__ void __launch_bounds__(nthreads_for(N1 * N1))
 k_var_facemat(VarParams P, double *__restrict__ FM) {
     constexpr int NL = 3 * N1;
-    extern __shared__ double fw[];
+    extern __shared__ __align__(16) double fw[];
     const int Q = P.Q, e = blockIdx.x, t = threadIdx.x;
     const Tabs T = tabs_at(P.tab, Q, N1);
     for (int f = 0; f < 4; ++f) {
@@ -1048,313 +1026,317 @@ k_var_facemat(VarParams P, double *__restrict__ FM) {
     }
 }
 
-// line integrals L[f][m][j] of the element's four faces from its own face
-// lines and its neighbours' (lines: 24 N1 doubles of shared scratch)
+// The face operators as integers, in place (one thread per row r of a face,
+// which alone reads and writes that row).  A row's columns fall in two groups,
+// each in units of 2^(q - 57): the v lines and the u lines, whose vectors get
+// a block exponent each (u and v may differ by any factor).  The u group holds
+// values along the face and slopes across it; the slopes count as
+// 2^-slope_exp of themselves, 2^slope_exp >= sum |phi'|, so that they are no
+// larger than the values behind them.
 template <int N1>
-__device__ void lift_lines(const VarParams &P, int e, const double *trin, double *lines, double *L) {
+__device__ __forceinline__ bool slope_line(int f, int m) { return f < 2 ? m == 1 : m == 2; }
+
+template <int N1>
+__global__ void __launch_bounds__(nthreads_for(N1 * N1))
+k_fm_pack(double *FM, int slope_exp, short2 *FMq) {
     constexpr int NL = 3 * N1;
-    for (int i = threadIdx.x; i < 4 * NL; i += blockDim.x) {
-        const int f = i / NL, c = i - (i / NL) * NL;
-        int fo;
-        const int nb = neighbour(P, e, f, fo);
-        lines[i] = trin[lix<N1>(e, 0) + i];
-        lines[4 * NL + i] = nb >= 0 ? trin[lix<N1>(nb, fo) + c] : 0.0;
-    }
-    __syncthreads();
+    const int e = blockIdx.x;
     for (int task = threadIdx.x; task < 4 * NL; task += blockDim.x) {
         const int f = task / NL, r = task - (task / NL) * NL;
-        int fo;
-        const int nb = neighbour(P, e, f, fo);
-        const double *col = P.FM + ((size_t)e * 4 + f) * 2 * NL * NL + r;
-        const double *own = lines + f * NL, *nbl = lines + 4 * NL + f * NL;
-        double sum = 0.0;
-#pragma unroll 9
-        for (int c = 0; c < NL; ++c) sum += __ldg(col + (size_t)c * NL) * own[c];
-        if (nb >= 0) {
-#pragma unroll 9
-            for (int c = 0; c < NL; ++c) sum += __ldg(col + (size_t)(NL + c) * NL) * nbl[c];
+        double *col = FM + ((size_t)e * 4 + f) * 2 * NL * NL + r;
+        int qv = -FX_NAN, qu = -FX_NAN;
+        for (int c = 0; c < 2 * NL; ++c) {
+            const int m = (c % NL) / N1;
+            const int k = fx_key(col[(size_t)c * NL], slope_line<N1>(f, m) ? slope_exp : 0) - 1022;   // |v| < 2^k
+            if (m == 0) qv = max(qv, k); else qu = max(qu, k);
         }
-        L[task] = sum;
+        qv = max(-16000, min(qv, 16000));
+        qu = max(-16000, min(qu, 16000));
+        FMq[((size_t)e * 4 + f) * NL + r] = make_short2((short)qv, (short)qu);
+        for (int c = 0; c < 2 * NL; ++c) {
+            const int m = (c % NL) / N1;
+            double *v = col + (size_t)c * NL;
+            const int2 a = fx_split(fx_int(*v, (m == 0 ? qv : qu) + 1022, slope_line<N1>(f, m) ? slope_exp : 0));
+            *reinterpret_cast<int2 *>(v) = a;
+        }
+    }
+}
+
+// line integrals L[f][m][j] of the element's four faces from its own face
+// lines and its neighbours' (lines: 24 N1 limb pairs of shared scratch).
+// A row's 6 N1 coefficients go to two threads, one for the own and one for the
+// neighbour's lines, whose exact sums are then added.  Bound by the 46.7 KB of
+// face operators an element reads (N1 = 9).
+template <int N1>
+__device__ __forceinline__ void lift_lines(const VarParams &P, int e, const double *trin, int2 *lines, int *slot,
+                                           double *L) {
+    constexpr int NL = 3 * N1, BD = nthreads_for(N1 * N1), PER = (4 * NL + BD - 1) / BD;
+    const int t = threadIdx.x;
+    double own[PER], nbl[PER];
+    int kv = -FX_NAN, ku = -FX_NAN;
+#pragma unroll
+    for (int s = 0; s < PER; ++s) {
+        const int i = t + BD * s;
+        own[s] = nbl[s] = 0.0;
+        if (i < 4 * NL) {
+            const int f = i / NL, c = i - f * NL, m = c / N1;
+            int fo;
+            const int nb = neighbour(P, e, f, fo);
+            own[s] = trin[lix<N1>(e, 0) + i];
+            if (nb >= 0) nbl[s] = trin[lix<N1>(nb, fo) + c];
+            const int sh = slope_line<N1>(f, m) ? -P.slope_exp : 0;
+            const int k = max(fx_key(own[s], sh), fx_key(nbl[s], sh));
+            if (m == 0) kv = max(kv, k); else ku = max(ku, k);
+        }
+    }
+    kv = __reduce_max_sync(0xffffffffu, kv);
+    ku = __reduce_max_sync(0xffffffffu, ku);
+    if ((t & 31) == 0) { slot[8 + (t >> 5)] = kv; slot[12 + (t >> 5)] = ku; }   // set 1
+    __syncthreads();
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { kv = max(kv, slot[8 + w]); ku = max(ku, slot[12 + w]); }
+#pragma unroll
+    for (int s = 0; s < PER; ++s) {
+        const int i = t + BD * s;
+        if (i < 4 * NL) {
+            const int f = i / NL, m = (i - f * NL) / N1;
+            const int sh = slope_line<N1>(f, m) ? -P.slope_exp : 0, k = m == 0 ? kv : ku;
+            lines[i] = fx_split(fx_int(own[s], k, sh));
+            lines[4 * NL + i] = fx_split(fx_int(nbl[s], k, sh));   // zero on a Dirichlet side
+        }
+    }
+    __syncthreads();
+    constexpr int PAIRS = BD / 2;
+#pragma unroll 1
+    for (int task0 = 0; task0 < 4 * NL; task0 += PAIRS) {
+        const int task = min(task0 + (t >> 1), 4 * NL - 1), side = t & 1, f = task / NL;
+        const int2 *a = P.FM + (((size_t)e * 4 + f) * 2 + side) * NL * NL + (task - f * NL);
+        const int2 *x = lines + side * 4 * NL + f * NL;
+        FxSum sv, su;
+#pragma unroll
+        for (int c = 0; c < N1; ++c) sv.mad(__ldg(a + (size_t)c * NL), x[c]);
+#pragma unroll
+        for (int c = N1; c < NL; ++c) su.mad(__ldg(a + (size_t)c * NL), x[c]);
+        long long T = sv.top(), S = su.top();
+        T += __shfl_xor_sync(0xffffffffu, T, 1);
+        S += __shfl_xor_sync(0xffffffffu, S, 1);
+        const short2 q = P.FMq[(size_t)e * 4 * NL + task];
+        // one conversion a thread: the even one takes the v sum, the odd one the u sum
+        double y = side ? fx_value(S, fx_top_exp(ku) + q.y, ku) : fx_value(T, fx_top_exp(kv) + q.x, kv);
+        y += __shfl_xor_sync(0xffffffffu, y, 1);
+        if (side == 0 && task0 + (t >> 1) < 4 * NL) L[task] = y;
     }
     __syncthreads();
 }
 
-// r_u, r_v (r_v without the stiffness term) from the face line integrals
+// r_u, r_v (r_v without the stiffness term) at node t from the face line integrals
 template <int N1>
-__device__ __forceinline__ void lift_assemble(const double *L, const Tabs &T, double *ru, double *rv) {
+__device__ __forceinline__ void lift_assemble(const double *L, const Tabs &T, int t, double &ru, double &rv) {
+    const int j = t / N1, i = t - (t / N1) * N1;
+    const double *Lx0 = L, *Lx1 = L + 3 * N1, *Ly0 = L + 6 * N1, *Ly1 = L + 9 * N1;
+    double u_ = T.dphiL[i] * Lx0[j] + T.dphiR[i] * Lx1[j] + T.dphiL[j] * Ly0[N1 + i] + T.dphiR[j] * Ly1[N1 + i];
+    double v_ = 0.0;
+    if (i == 0) { u_ += Lx0[N1 + j]; v_ += Lx0[2 * N1 + j]; }
+    if (i == N1 - 1) { u_ += Lx1[N1 + j]; v_ += Lx1[2 * N1 + j]; }
+    if (j == 0) { u_ += Ly0[i]; v_ += Ly0[2 * N1 + i]; }
+    if (j == N1 - 1) { u_ += Ly1[i]; v_ += Ly1[2 * N1 + i]; }
+    ru = u_;
+    rv = v_;
+}
+
+// Psi into shared memory, as integers or, for the inner solves, in FP32
+template <int N1>
+__device__ __forceinline__ void load_psi(const VarParams &P, const StageSmem<N1> &s) {
+    if (threadIdx.x < N1 * N1) s.Ps[threadIdx.x] = P.Psx[threadIdx.x];
+}
+
+// solve one of the element's systems (W: the u_t system, + w w^T) from the
+// right-hand side b; x: the guess (unless zero) and the result
+template <int N1>
+__device__ __forceinline__ void solve(const VarParams &P, const StageSmem<N1> &s, const Tabs &T, int e, bool W, double w,
+                                      double b, double &x, bool zero, bool guess, int *iters, int *sweeps, int *fell,
+                                      double *rel, bool want_rel) {
     constexpr int NA = N1 * N1;
     const int t = threadIdx.x;
-    if (t < NA) {
-        const int j = t / N1, i = t - (t / N1) * N1;
-        const double *Lx0 = L, *Lx1 = L + 3 * N1, *Ly0 = L + 6 * N1, *Ly1 = L + 9 * N1;
-        double u_ = T.dphiL[i] * Lx0[j] + T.dphiR[i] * Lx1[j] + T.dphiL[j] * Ly0[N1 + i] + T.dphiR[j] * Ly1[N1 + i];
-        double v_ = 0.0;
-        if (i == 0) { u_ += Lx0[N1 + j]; v_ += Lx0[2 * N1 + j]; }
-        if (i == N1 - 1) { u_ += Lx1[N1 + j]; v_ += Lx1[2 * N1 + j]; }
-        if (j == 0) { u_ += Ly0[i]; v_ += Ly0[2 * N1 + i]; }
-        if (j == N1 - 1) { u_ += Ly1[i]; v_ += Ly1[2 * N1 + i]; }
-        ru[t] = u_;
-        rv[t] = v_;
+    const bool on = t < NA;
+    const FxSystem f = s.system(W ? P.Sx : P.Mx, e);
+    const FxPrecond pre{s.Ps, P.Ps_exp, W ? (on ? P.dS[(size_t)e * NA + t] : 0.0) : P.pre[(size_t)e * 4 + 3],
+                        P.precond == GDG_PC_NONE};
+    if (P.mixed) {
+        Inner32 in;
+        in.sc = __int_as_float(max(1, min(254, 127 + f.d)) << 23);
+        in.d = (float)pre.d;
+        in.w = W ? (float)w : 0.f;
+        in.Ps = s.Ps32;
+        in.t1 = s.t1;
+        in.t2 = s.t2;
+        in.red = s.red32;
+        in.rtol = P.refine_rtol;
+        in.maxit = P.maxit;
+        in.none = pre.none;
+        // in the mass system the FP64 preconditioned step first, only where it
+        // solves it outright (a parallelogram); elsewhere it would cost an FP64
+        // product and still leave two FP32 sweeps
+        *sweeps = refine<N1>(f, pre, in, s.bufs(), W, w, b, x, P.rtol, P.refine_max, zero, iters, rel, guess, fell,
+                             !W && P.affine[e]);
+    } else {
+        *sweeps = 0;
+        *iters = pcg<N1>(f, pre, s.bufs(), W, w, b, x, P.rtol, P.maxit, zero, rel, guess, fell, want_rel);
     }
-    __syncthreads();
 }
 
-// face fluxes and lifts: r_u, r_v (r_v without the stiffness term)
-template <int N1>
-__device__ void lifts(const VarParams &P, int e, const double *trin, const Tabs &T, double *lines, double *L,
-                      double *ru, double *rv) {
-    lift_lines<N1>(P, e, trin, lines, L);
-    lift_assemble<N1>(L, T, ru, rv);
-}
-
-// Columns of the folded operators of the precomputed-inverse route, per
-// element (each column NA doubles, thread t reads entry t: coalesced):
-//   0 .. 8 N1 - 1         G_u = (S_c2 + w w^T)^-1 R_u, R_u the lift of the
-//                         m = 0, 1 line integrals into r_u (column f*2N1 + m*N1 + j)
-//   8 N1 .. 12 N1 - 1     G_v = M_J^-1 R_v, R_v the lift of the m = 2 line
-//                         integrals into r_v (column 8N1 + f*N1 + j)
-//   12 N1 .. 12 N1 + NA-1 K = M_J^-1 S_c2
-// so that dU/dt = V + G_u L_u and dV/dt = G_v L_v - K U.
-__host__ __device__ constexpr int fold_cols(int N1) { return 12 * N1 + N1 * N1; }
-// shared staging of the fold's right-hand factors: R_u (NA x 8 N1), R_v
-// (NA x 4 N1) and S_c2 (NA x NA) in turn; 8 N1 > NA for N1 < 8
-__host__ __device__ constexpr int fold_rlen(int N1) { return N1 * N1 * (8 * N1 > N1 * N1 ? 8 * N1 : N1 * N1); }
-
-// dU/dt = V + G_u L_u and dV/dt = G_v L_v - K U from the folded operators Ge
-// of one element (columns as in fold_cols); L the face line integrals
-template <int N1>
-__device__ __forceinline__ void fold_apply(const double *__restrict__ Ge, const double *L, const double *Yu,
-                                           const double *Yv, double *du, double *dv) {
-    constexpr int NA = N1 * N1;
-    const int t = threadIdx.x;
-    if (t < NA) {
-        const double *g = Ge + t;
-        double su = 0.0, sv = 0.0, sk = 0.0;
-#pragma unroll
-        for (int f = 0; f < 4; ++f) {
-#pragma unroll
-            for (int c = 0; c < 2 * N1; ++c)
-                su = fma(__ldg(g + (size_t)(f * 2 * N1 + c) * NA), L[f * 3 * N1 + c], su);
-        }
-#pragma unroll
-        for (int f = 0; f < 4; ++f) {
-#pragma unroll
-            for (int j = 0; j < N1; ++j)
-                sv = fma(__ldg(g + (size_t)(8 * N1 + f * N1 + j) * NA), L[f * 3 * N1 + 2 * N1 + j], sv);
-        }
-#pragma unroll 9
-        for (int c = 0; c < NA; ++c) sk = fma(__ldg(g + (size_t)(12 * N1 + c) * NA), Yu[c], sk);
-        du[t] = Yv[t] + su;
-        dv[t] = sv - sk;
-    }
-    __syncthreads();
-}
-
-// the lower triangle of a symmetric element matrix into shared memory,
-// packed (tri_len doubles: half the full matrix)
-template <int N1>
-__device__ void load_matrix(double *A, const double *src) {
-    constexpr int NA = N1 * N1;
-    // element matrices start at e*NA*NA doubles: only 8-byte alignment is guaranteed
-    for (int q = threadIdx.x; q < NA * NA; q += blockDim.x) {
-        const int i = q / NA, k = q - (q / NA) * NA;
-        if (k <= i) cp_async_8(A + i * (i + 1) / 2 + k, src + q);
-    }
-    cp_async_wait_all();
-    __syncthreads();
-}
-
-// One element's RK stage (one CTA of nthreads_for(N1*N1) threads).
+// One element's RK stage (one block of nthreads_for(N1*N1) threads).
 template <int N1, int MODE>
 __device__ __forceinline__ void var_stage_body(const VarParams &P, const VarBufs &b, double cA, double cY, int e,
                                                double *smraw) {
     constexpr int NA = N1 * N1;
-    StageSmem<N1> s(smraw, P.Q, P.mixed, P.inverse);
+    const StageSmem<N1> s(smraw);
     const int t = threadIdx.x;
-    const size_t off = (size_t)e * NA;
-    const double *Sg = P.S + (size_t)e * NA * NA, *Mg = P.M + (size_t)e * NA * NA;
-    if (s.tb) load_tabs(s.tb, P.tab + 2 * P.Q * N1, tab_tail_len(P.Q, N1));
-    if (t < NA) {
-        s.Yu[t] = b.yU[off + t];
-        s.Yv[t] = b.yV[off + t];
-        s.w[t] = P.w[off + t];
-    }
-    __syncthreads();
-    const Tabs T = tabs_split(P.tab, s.tb ? s.tb : P.tab + 2 * P.Q * N1, P.Q, N1);
-    fdm_diagonals<N1>(P, e, s.dS, s.dM);
+    const bool on = t < NA;
+    const size_t at = (size_t)e * NA + (on ? t : 0);
+    load_fx<N1>(s.A, P.Sx, e);
+    const Tabs T = tabs_at(P.tab, P.Q, N1);
+    const double Yu = on ? b.yU[at] : 0.0, Yv = on ? b.yV[at] : 0.0, w = on ? P.w[at] : 0.0;
+    double ru = 0.0, rv = 0.0, x = 0.0;
+    if (on) s.w[t] = w;
+    if (!P.inverse) load_psi<N1>(P, s);
     const bool guess = b.part == 2;
-    if (P.inverse) {
-        lift_lines<N1>(P, e, b.trin, s.fw, s.L);
-        fold_apply<N1>(P.G + (size_t)e * fold_cols(N1) * NA, s.L, s.Yu, s.Yv, s.ru, s.x);
-        if (e == P.src_e) {   // dV/dt += M_J^-1 phi(x_s) s(t)
-            const double amp = source_amplitude(P, b);
-            if (t < NA) s.x[t] += amp * P.src_w[NA + t];
-            __syncthreads();
-        }
-    } else if (!guess) {
-        lifts<N1>(P, e, b.trin, T, s.fw, s.L, s.ru, s.rv);
-        // stiffness: r_v -= S U
-        if (P.mixed || P.inverse) {
-            matvec_g<NA>(Sg, s.Yu, s.Ap);
-        } else {
-            load_matrix<N1>(s.A, Sg);
-            matvec_packed<NA, double>(s.A, s.Yu, s.Ap);
-        }
-        if (t < NA) s.rv[t] -= s.Ap[t];
+    fx_arrived();
+    if (!guess) {
+        const double SU = fx_matvec<NA>(s.system(P.Sx, e), Yu, 0);
         __syncthreads();
-        if (e == P.src_e) {   // block-uniform
-            const double amp = source_amplitude(P, b);
-            if (t < NA) s.rv[t] += amp * P.src_w[t];
-            __syncthreads();
+        if (P.inverse && b.part != 1) load_fx<N1>(s.A, P.Ax, e);   // on its way during the lifts
+        lift_lines<N1>(P, e, b.trin, s.lines, s.slot, s.L);
+        if (on) {
+            lift_assemble<N1>(s.L, T, t, ru, rv);
+            rv -= SU;
+            if (e == P.src_e) rv += source_amplitude(P, b) * P.src_w[t];
         }
         if (b.part == 1) {
-            if (t < NA) { b.ru[off + t] = s.ru[t]; b.rv[off + t] = s.rv[t]; }
+            if (on) { b.ru[at] = ru; b.rv[at] = rv; }
             return;
         }
+        __syncthreads();   // L is read
+    } else if (on) {
+        ru = b.ru[at];
+        rv = b.rv[at];
+        x = b.x0u[at];
+    }
+    if (P.inverse) {   // dU/dt = V + (S_c2 + w w^T)^-1 r_u (k_var_invert), dV/dt = M_J^-1 r_v
+#pragma unroll 1
+        for (int sys = 0; sys < 2; ++sys) {
+            fx_arrived();
+            const double y = fx_matvec<NA>(s.system(sys ? P.Vx : P.Ax, e), ru, 0);
+            __syncthreads();
+            if (sys == 0) {
+                load_fx<N1>(s.A, P.Vx, e);
+                ru = rv;
+                rv = Yv + y;   // dU/dt
+            }
+            x = y;             // dV/dt after the second pass
+        }
+        if (t == 0 && P.stats) atomicAdd(&P.stats[6], 1ull);
     } else {
-        if (t < NA) { s.ru[t] = b.ru[off + t]; s.rv[t] = b.rv[off + t]; s.x[t] = b.x0u[off + t]; }
-        if (!P.mixed) load_matrix<N1>(s.A, Sg);
+        int it[2], sw[2], fell = 0;
+        bool bad[2];
+#pragma unroll 1
+        for (int sys = 0; sys < 2; ++sys) {   // the u_t system from r_u, then the v_t system from r_v
+            double rel = 0.0;
+            if (P.mixed && on) s.Ps32[t] = (float)T.Ps[t];
+            if (sys) fx_arrived();
+            solve<N1>(P, s, T, e, sys == 0, w, ru, x, sys || !guess, guess && !sys, &it[sys], &sw[sys], &fell, &rel, false);
+            bad[sys] = (P.mixed ? sw[sys] >= P.refine_max : it[sys] >= P.maxit) && rel > P.rtol;
+            __syncthreads();
+            if (sys == 0) {
+                load_fx<N1>(s.A, P.Mx, e);
+                ru = rv;
+                rv = Yv + x;   // dU/dt
+            }
+        }
+        if (t == 0 && P.stats) {
+            atomicAdd(&P.stats[0], (unsigned long long)it[0]);
+            atomicAdd(&P.stats[1], (unsigned long long)it[1]);
+            atomicMax(&P.stats[2], (unsigned long long)it[0]);
+            atomicMax(&P.stats[3], (unsigned long long)it[1]);
+            if (bad[0]) atomicAdd(&P.stats[4], 1ull);
+            if (bad[1]) atomicAdd(&P.stats[5], 1ull);
+            atomicAdd(&P.stats[6], 1ull);
+            atomicAdd(&P.stats[7], (unsigned long long)sw[0]);
+            atomicAdd(&P.stats[8], (unsigned long long)sw[1]);
+            atomicMax(&P.stats[9], (unsigned long long)sw[0]);
+            atomicMax(&P.stats[10], (unsigned long long)sw[1]);
+            if (guess) atomicAdd(&P.stats[11], 1ull);          // solves started from a guess
+            if (fell) atomicAdd(&P.stats[12], 1ull);           // ... of which fell back to x0 = 0
+        }
     }
-    const bool none = P.precond == GDG_PC_NONE;
-    double rel_u = 0.0, rel_v = 0.0;
-    int it_u = 0, it_v = 0, sw_u = 0, sw_v = 0, fell = 0;
-    bool bad_u = false, bad_v = false;
-    if (P.inverse) {
-        // dU/dt, dV/dt already in ru, x (fold_apply)
-    } else {
-    if (P.mixed) {
-        to_fp32<N1>(P.S32 + (size_t)e * tri_len(NA), s.A32, T.Ps, s.Ps32, s.dS, s.dS32, s.w, s.w32);
-        sw_u = refine<N1, true>(Sg, s.w, s.ru, s.x, s.r, s.Ap, s.scratch32(true), s.red, P.rtol, P.refine_max,
-                                P.refine_rtol, P.maxit, none, !guess, &it_u, &rel_u, guess, &fell);
-        bad_u = sw_u >= P.refine_max && rel_u > P.rtol;
-    } else {
-        it_u = pcg<N1, true>(s.A, s.w, s.ru, s.x, s.r, s.z, s.p, s.Ap, T.Ps, s.dS, s.t1, s.t2, s.red, P.rtol,
-                             P.maxit, none, !guess, &rel_u, guess, &fell, P.parity != 0);
-        bad_u = it_u >= P.maxit && rel_u > P.rtol;
-    }
-    if (t < NA) s.ru[t] = s.Yv[t] + s.x[t];   // dU/dt
-    __syncthreads();
-    if (!P.mixed) load_matrix<N1>(s.A, Mg);
-    if (P.mixed) {
-        to_fp32<N1>(P.M32 + (size_t)e * tri_len(NA), s.A32, T.Ps, s.Ps32, s.dM, s.dM32, nullptr, nullptr);
-        // the FP64 preconditioned step first only where it solves the mass
-        // system outright (a parallelogram); elsewhere it would cost an FP64
-        // product and still leave two FP32 sweeps
-        const Step64 st64{s.z, s.t1, s.t2, T.Ps, s.dM, P.parity != 0};
-        sw_v = refine<N1, false>(Mg, s.w, s.rv, s.x, s.r, s.Ap, s.scratch32(false), s.red, P.rtol,
-                                 P.refine_max, P.refine_rtol, P.maxit, none, true, &it_v, &rel_v, false, nullptr,
-                                 P.affine[e] ? &st64 : nullptr);
-        bad_v = sw_v >= P.refine_max && rel_v > P.rtol;
-    } else {
-        it_v = pcg<N1, false>(s.A, s.w, s.rv, s.x, s.r, s.z, s.p, s.Ap, T.Ps, s.dM, s.t1, s.t2, s.red, P.rtol,
-                              P.maxit, none, true, &rel_v, false, nullptr, P.parity != 0);
-        bad_v = it_v >= P.maxit && rel_v > P.rtol;
-    }
-    }
-    if (t == 0 && P.stats) {
-        atomicAdd(&P.stats[0], (unsigned long long)it_u);
-        atomicAdd(&P.stats[1], (unsigned long long)it_v);
-        atomicMax(&P.stats[2], (unsigned long long)it_u);
-        atomicMax(&P.stats[3], (unsigned long long)it_v);
-        if (bad_u) atomicAdd(&P.stats[4], 1ull);
-        if (bad_v) atomicAdd(&P.stats[5], 1ull);
-        atomicAdd(&P.stats[6], 1ull);
-        atomicAdd(&P.stats[7], (unsigned long long)sw_u);
-        atomicAdd(&P.stats[8], (unsigned long long)sw_v);
-        atomicMax(&P.stats[9], (unsigned long long)sw_u);
-        atomicMax(&P.stats[10], (unsigned long long)sw_v);
-        if (guess) atomicAdd(&P.stats[11], 1ull);          // solves started from a guess
-        if (fell) atomicAdd(&P.stats[12], 1ull);           // ... of which fell back to x0 = 0
-    }
-    // k = (ru, x); RK combine into Yu / Yv (next stage input) in shared memory
-    if (t < NA) {
-        const double ku = s.ru[t], kv = s.x[t];
+    // k = (rv, x); RK combine into the next stage input
+    if (on) {
+        const double ku = rv, kv = x;
+        double nu = 0.0, nv = 0.0;
         if (MODE == M_RHS) {
-            b.oU[off + t] = ku;
-            b.oV[off + t] = kv;
+            b.oU[at] = ku;
+            b.oV[at] = kv;
         } else if (MODE == M_S1) {
-            b.aU[off + t] = cA * ku;
-            b.aV[off + t] = cA * kv;
-            s.Yu[t] = s.Yu[t] + cY * ku;
-            s.Yv[t] = s.Yv[t] + cY * kv;
+            b.aU[at] = cA * ku;
+            b.aV[at] = cA * kv;
+            nu = Yu + cY * ku;
+            nv = Yv + cY * kv;
         } else if (MODE == M_S23) {
-            b.aU[off + t] += cA * ku;
-            b.aV[off + t] += cA * kv;
-            s.Yu[t] = b.nU[off + t] + cY * ku;
-            s.Yv[t] = b.nV[off + t] + cY * kv;
+            b.aU[at] += cA * ku;
+            b.aV[at] += cA * kv;
+            nu = b.nU[at] + cY * ku;
+            nv = b.nV[at] + cY * kv;
         } else {
-            s.Yu[t] = b.nU[off + t] + b.aU[off + t] + cA * ku;
-            s.Yv[t] = b.nV[off + t] + b.aV[off + t] + cA * kv;
+            nu = b.nU[at] + b.aU[at] + cA * ku;
+            nv = b.nV[at] + b.aV[at] + cA * kv;
         }
         if (MODE != M_RHS) {
-            double *dU = MODE == M_S4 ? b.nU : b.oU;
-            double *dV = MODE == M_S4 ? b.nV : b.oV;
-            dU[off + t] = s.Yu[t];
-            dV[off + t] = s.Yv[t];
+            (MODE == M_S4 ? b.nU : b.oU)[at] = nu;
+            (MODE == M_S4 ? b.nV : b.oV)[at] = nv;
+            s.U[t] = nu;
+            s.V[t] = nv;
         }
     }
     // the source block (the only reader of the source time) starts the next step
     if (MODE == M_S4 && e == P.src_e && t == 0) *P.time += b.tstage;
     if (MODE == M_RHS) return;
     __syncthreads();
-    face_lines<N1>(s.Yu, s.Yv, T, b.trout + lix<N1>(e, 0));
+    face_lines<N1>(s.U, s.V, T, b.trout + lix<N1>(e, 0), t, blockDim.x);
 }
 
-// Resident blocks promised to ptxas for the stage kernel: 10 where a block is
-// at most 3 warps (the element-inverse route streams its operators and wants
-// every warp it can get; the PCG bodies fit the resulting 64 registers
-// without spilling), kVarMinBlocks for larger elements.
-__host__ __device__ constexpr int var_stage_min_blocks(int n1) {
-    return nthreads_for(n1 * n1) <= 96 ? 10 : kVarMinBlocks;
-}
+// Resident blocks promised to ptxas for the stage kernel: the 7 that the shared
+// memory of a block of at most 3 warps allows, 4 for larger elements.
+__host__ __device__ constexpr int var_stage_min_blocks(int n1) { return nthreads_for(n1 * n1) <= 96 ? 7 : 4; }
 
 template <int N1, int MODE>
 __global__ void __launch_bounds__(nthreads_for(N1 * N1), var_stage_min_blocks(N1))
 k_var_stage(VarParams P, VarBufs b, double cA, double cY) {
-    extern __shared__ double smraw[];
+    extern __shared__ __align__(16) double smraw[];
     var_stage_body<N1, MODE>(P, b, cA, cY, blockIdx.x, smraw);
 }
 
 // standalone element PCG (gdg_pcg): which = 0 M, 1 S (+ w w^T)
 template <int N1>
-__global__ void __launch_bounds__(nthreads_for(N1 * N1), kVarMinBlocks)
+__global__ void __launch_bounds__(nthreads_for(N1 * N1), var_stage_min_blocks(N1))
 k_var_pcg(VarParams P, int which, const double *bvec, double *xvec, int *iters, double *rel, int *sweeps) {
     constexpr int NA = N1 * N1;
-    extern __shared__ double smraw[];
-    StageSmem<N1> s(smraw, P.Q, P.mixed, false);
+    extern __shared__ __align__(16) double smraw[];
+    const StageSmem<N1> s(smraw);
     const int e = blockIdx.x, t = threadIdx.x;
-    const size_t off = (size_t)e * NA;
-    if (s.tb) load_tabs(s.tb, P.tab + 2 * P.Q * N1, tab_tail_len(P.Q, N1));
-    if (t < NA) {
-        s.ru[t] = bvec[off + t];
-        s.x[t] = xvec[off + t];
-        s.w[t] = P.w[off + t];
+    const bool on = t < NA;
+    const size_t at = (size_t)e * NA + (on ? t : 0);
+    load_fx<N1>(s.A, which ? P.Sx : P.Mx, e);
+    const Tabs T = tabs_at(P.tab, P.Q, N1);
+    const double b = on ? bvec[at] : 0.0, w = on ? P.w[at] : 0.0;
+    double x = on ? xvec[at] : 0.0, rr;
+    int it, sw = 0, fell = 0;
+    if (on) {
+        s.w[t] = w;
+        if (P.mixed) s.Ps32[t] = (float)T.Ps[t];
     }
-    __syncthreads();
-    const Tabs T = tabs_split(P.tab, s.tb ? s.tb : P.tab + 2 * P.Q * N1, P.Q, N1);
-    fdm_diagonals<N1>(P, e, s.dS, s.dM);
-    const double *Ag = (which ? P.S : P.M) + (size_t)e * NA * NA;
-    if (!P.mixed) load_matrix<N1>(s.A, Ag);
-    const bool none = P.precond == GDG_PC_NONE;
-    double rr;
-    int it, sw = 0;
-    if (P.mixed) {
-        to_fp32<N1>((which ? P.S32 : P.M32) + (size_t)e * tri_len(NA), s.A32, T.Ps, s.Ps32, which ? s.dS : s.dM,
-                    which ? s.dS32 : s.dM32, which ? s.w : nullptr, s.w32);
-        if (which)
-            sw = refine<N1, true>(Ag, s.w, s.ru, s.x, s.r, s.Ap, s.scratch32(true), s.red, P.rtol, P.refine_max,
-                                  P.refine_rtol, P.maxit, none, false, &it, &rr);
-        else
-            sw = refine<N1, false>(Ag, s.w, s.ru, s.x, s.r, s.Ap, s.scratch32(false), s.red, P.rtol,
-                                   P.refine_max, P.refine_rtol, P.maxit, none, false, &it, &rr);
-    } else if (which) {
-        it = pcg<N1, true>(s.A, s.w, s.ru, s.x, s.r, s.z, s.p, s.Ap, T.Ps, s.dS, s.t1, s.t2, s.red, P.rtol,
-                           P.maxit, none, false, &rr, false, nullptr, P.parity != 0);
-    } else {
-        it = pcg<N1, false>(s.A, s.w, s.ru, s.x, s.r, s.z, s.p, s.Ap, T.Ps, s.dM, s.t1, s.t2, s.red, P.rtol,
-                            P.maxit, none, false, &rr, false, nullptr, P.parity != 0);
-    }
-    if (t < NA) xvec[off + t] = s.x[t];
+    load_psi<N1>(P, s);
+    fx_arrived();
+    solve<N1>(P, s, T, e, which != 0, w, b, x, false, false, &it, &sw, &fell, &rr, true);
+    if (on) xvec[at] = x;
     if (t == 0) {
         iters[e] = it;
         rel[e] = rr;
@@ -1364,15 +1346,20 @@ k_var_pcg(VarParams P, int which, const double *bvec, double *xvec, int *iters, 
 
 // Element inverse at setup (GDG_SOLVE_INVERSE; the precomputed-inverse route
 // of Section 3.1 applied to the element systems of Section 7.1):
-// Dst[e] = (Src[e] + w_e w_e^T)^-1 (w != nullptr) or Src[e]^-1, by Cholesky
+// Dst[e] = (Src[e] + w_e w_e^T)^-1 - 1 1^T (w != nullptr) or Src[e]^-1.
+// The u_t system's right-hand sides have 1^T r_u = 0 (the constant test
+// function has no gradient), and w^T y = 1^T r_u for its solution y, since
+// (S + w w^T) 1 = w; subtracting 1 1^T takes the rounding of 1^T r_u out of
+// w^T y = 0 and changes nothing else (still symmetric, and positive
+// semidefinite).  By Cholesky
 // A = L L^T in shared memory and one forward + back substitution per column
 // of the identity (thread j solves column j); the result is made exactly
-// symmetric (lower := upper) so that it can be applied by columns.
+// symmetric (lower := upper) for the packed form.
 template <int N1>
 __global__ void __launch_bounds__(nthreads_for(N1 * N1))
 k_var_invert(const double *__restrict__ Src, const double *__restrict__ w, double *__restrict__ Dst) {
     constexpr int NA = N1 * N1;
-    extern __shared__ double sm[];
+    extern __shared__ __align__(16) double sm[];
     double *A = sm, *B = A + NA * NA, *dinv = B + NA * NA;
     const int e = blockIdx.x, t = threadIdx.x, nt = blockDim.x;
     const double *src = Src + (size_t)e * NA * NA;
@@ -1429,90 +1416,35 @@ k_var_invert(const double *__restrict__ Src, const double *__restrict__ w, doubl
     double *dst = Dst + (size_t)e * NA * NA;
     for (int i = t; i < NA * NA; i += nt) {
         const int r = i / NA, c = i - (i / NA) * NA;
-        dst[i] = r > c ? B[c * NA + r] : B[i];
+        dst[i] = (r > c ? B[c * NA + r] : B[i]) - (we ? 1.0 : 0.0);
     }
 }
 
-// out[c][r] = sum_k A[r][k] R[k][c] for one element, row r per thread: A
-// exactly symmetric (row r read as column r, coalesced), R [NA][NCOL] in
-// shared memory, out column-major with column stride NA
-template <int N1, int NCOL>
-__device__ __forceinline__ void fold_product(const double *__restrict__ A, const double *R, double *out) {
-    constexpr int NA = N1 * N1, CB = 12;
-    const int r = threadIdx.x;
-    if (r < NA) {
-        for (int c0 = 0; c0 < NCOL; c0 += CB) {
-            double acc[CB];
-#pragma unroll
-            for (int i = 0; i < CB; ++i) acc[i] = 0.0;
-            for (int k = 0; k < NA; ++k) {
-                const double a = __ldg(A + (size_t)k * NA + r);
-                const double *rk = R + k * NCOL + c0;
-#pragma unroll
-                for (int i = 0; i < CB; ++i)
-                    if (c0 + i < NCOL) acc[i] = fma(a, rk[i], acc[i]);
-            }
-#pragma unroll
-            for (int i = 0; i < CB; ++i)
-                if (c0 + i < NCOL) out[(size_t)(c0 + i) * NA + r] = acc[i];
-        }
-    }
-    __syncthreads();
-}
-
-// Folded operators of the precomputed-inverse route (fold_cols), one CTA per
-// element. The lift matrices R_u, R_v are built a column at a time by lifting
-// a unit line integral with lift_assemble (the stage's own lift), then
-// multiplied by the element inverses; K = M_J^-1 S_c2.
+// Integer form of ne exactly symmetric NA x NA element matrices (gdg_fx.cuh):
+// packed lower triangles and row exponents, one block per element
 template <int N1>
-__global__ void __launch_bounds__(nthreads_for(N1 * N1))
-k_var_fold(const double *__restrict__ S, const double *__restrict__ Ainv, const double *__restrict__ Minv,
-           const double *__restrict__ tab, int Q, double *__restrict__ G) {
+__global__ void k_fx_pack(int ne, const double *__restrict__ src, int2 *__restrict__ dst,
+                          signed char *__restrict__ dexp) {
     constexpr int NA = N1 * N1;
-    extern __shared__ double sm[];
-    double *R = sm, *L = R + fold_rlen(N1), *tu = L + 12 * N1, *tv = tu + NA;
-    const int e = blockIdx.x, t = threadIdx.x, nt = blockDim.x;
-    const Tabs T = tabs_at(tab, Q, N1);
-    const size_t m2 = (size_t)e * NA * NA;
-    double *Ge = G + (size_t)e * fold_cols(N1) * NA;
-    for (int c = 0; c < 8 * N1; ++c) {   // R_u: line integrals (f, m < 2, j)
-        const int f = c / (2 * N1), mj = c - f * 2 * N1;
-        for (int k = t; k < 12 * N1; k += nt) L[k] = k == f * 3 * N1 + mj ? 1.0 : 0.0;
-        __syncthreads();
-        lift_assemble<N1>(L, T, tu, tv);   // ends with a barrier: L free again
-        if (t < NA) R[t * 8 * N1 + c] = tu[t];
-    }
-    __syncthreads();
-    fold_product<N1, 8 * N1>(Ainv + m2, R, Ge);
-    for (int c = 0; c < 4 * N1; ++c) {   // R_v: line integrals (f, m = 2, j)
-        const int f = c / N1, j = c - f * N1;
-        for (int k = t; k < 12 * N1; k += nt) L[k] = k == f * 3 * N1 + 2 * N1 + j ? 1.0 : 0.0;
-        __syncthreads();
-        lift_assemble<N1>(L, T, tu, tv);
-        if (t < NA) R[t * 4 * N1 + c] = tv[t];
-    }
-    __syncthreads();
-    fold_product<N1, 4 * N1>(Minv + m2, R, Ge + (size_t)8 * N1 * NA);
-    for (int i = t; i < NA * NA; i += nt) R[i] = S[m2 + i];
-    __syncthreads();
-    fold_product<N1, NA>(Minv + m2, R, Ge + (size_t)12 * N1 * NA);
-}
-
-// FP32 copy (round to nearest) of the lower triangles of ne symmetric
-// NA x NA element matrices, packed (tri_len); one block per element
-template <int N1>
-__global__ void k_to_f32_lower(int ne, const double *__restrict__ src, float *__restrict__ dst) {
-    constexpr int NA = N1 * N1;
+    __shared__ int d[NA];
     for (int e = blockIdx.x; e < ne; e += gridDim.x) {
         const double *A = src + (size_t)e * NA * NA;
-        float *L = dst + (size_t)e * tri_len(NA);
+        for (int i = threadIdx.x; i < NA; i += blockDim.x) {
+            // A_ii < 2^k: half of it, rounded up
+            const int k = fx_expo(A[(size_t)i * NA + i]) - 1022;
+            d[i] = max(-120, min((k + 1) >> 1, 120));
+            dexp[(size_t)e * NA + i] = (signed char)d[i];
+        }
+        __syncthreads();
+        int2 *L = dst + (size_t)e * fx_tri_len(NA);
         for (int q = threadIdx.x; q < NA * NA; q += blockDim.x) {
             const int i = q / NA, k = q - (q / NA) * NA;
-            if (k <= i) L[i * (i + 1) / 2 + k] = (float)A[q];
+            if (k <= i) L[i * (i + 1) / 2 + k] = fx_split(__double2ll_rn(scalbn(A[q], FX_ONE - d[i] - d[k])));
         }
+        if (NA * (NA + 1) / 2 < fx_tri_len(NA) && threadIdx.x == 0) L[NA * (NA + 1) / 2] = make_int2(0, 0);
+        __syncthreads();
     }
 }
-
 // per-element V^T M V + U^T S U
 template <int N1>
 __global__ void __launch_bounds__(nthreads_for(N1 * N1), kVarMinBlocks)

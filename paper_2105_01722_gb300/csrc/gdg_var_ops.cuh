@@ -1,0 +1,41 @@
+// Host entry points of the element kernels of one N1 (VarOps): what each
+// gdg_var_n*.cu instantiates.
+#pragma once
+
+#include "gdg_var_kernels.cuh"
+
+namespace {
+
+template <int N1>
+struct VarLaunch {
+    // The dynamic shared-memory limit is a property of the kernel function, shared
+    // by every context: always raised to the device's opt-in maximum so that a
+    // context with smaller needs cannot lower it under another one.
+    static void attrs(int lim) {
+        cudaFuncSetAttribute(k_var_stage<N1, M_RHS>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_var_stage<N1, M_S1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_var_stage<N1, M_S23>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_var_stage<N1, M_S4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_var_pcg<N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    }
+    static void stage(const VarParams &P, size_t sm, int mode, const VarBufs &b, double cA, double cY, cudaStream_t s) {
+        const dim3 grid(P.ne), block(nthreads_for(N1 * N1));   // one block per element
+        switch (mode) {
+        case M_RHS: k_var_stage<N1, M_RHS><<<grid, block, sm, s>>>(P, b, cA, cY); break;
+        case M_S1: k_var_stage<N1, M_S1><<<grid, block, sm, s>>>(P, b, cA, cY); break;
+        case M_S23: k_var_stage<N1, M_S23><<<grid, block, sm, s>>>(P, b, cA, cY); break;
+        default: k_var_stage<N1, M_S4><<<grid, block, sm, s>>>(P, b, cA, cY); break;
+        }
+    }
+    static void pcg(const VarParams &P, size_t sm, int which, const double *b, double *x, int *iters, double *rel,
+                    int *sweeps, cudaStream_t s) {
+        k_var_pcg<N1><<<P.ne, nthreads_for(N1 * N1), sm, s>>>(P, which, b, x, iters, rel, sweeps);
+    }
+};
+
+GDG_CHECKS_READER(var_unit_checks)
+
+}  // namespace
+
+#define GDG_VAR_OPS(n) \
+    extern const VarOps var_ops_##n = {VarLaunch<n>::attrs, VarLaunch<n>::stage, VarLaunch<n>::pcg, var_unit_checks};
