@@ -10,10 +10,10 @@
 // r_u / ||r_u||; output: a guess of y / ||r_u|| for (S_c2 + w w^T) y = r_u.
 //
 // Kernels
-//   k_mlp_forward   Y = net(X) for B samples (32 per CTA, weights in smem)
-//   k_mlp_backward  per-CTA partial loss and gradients of the mean squared
-//                   error, for the samples idx[0..B) of a dataset
-//   k_mlp_reduce    fixed-order sum of the CTA partials (deterministic)
+//   k_mlp_forward   Y = net(X) for B samples
+//   k_mlp_samples   forward and backward pass of every sample of a minibatch:
+//                   its activations, the errors at its layers, its loss
+//   k_mlp_grad      gradients and loss from those, summed in a fixed order
 //   k_mlp_adam      Adam update of the master copy, refresh of the BF16 copy
 #include <cuda_bf16.h>
 
@@ -31,177 +31,275 @@ constexpr int WB_W1 = 0, WB_W2 = HID * IN, WB_W3 = WB_W2 + HID * HID, NWEIGHT = 
 static_assert(NPARAM == GDG_MLP_NPARAM, "parameter count");
 static_assert(NWEIGHT == GDG_MLP_NWEIGHT, "weight count");
 
-constexpr int SPB = 32;        // samples per CTA
-constexpr int THREADS = 256;
+// Weights in shared memory: BF16 rows padded to 16 bytes more than a multiple
+// of 128, so that the 16-byte reads of the 8 lanes of a phase (one row each)
+// fall on different banks; rows of W1 are padded with zeros to 168 inputs.
+constexpr int KP = 168, S1 = KP, S2 = 72, S3 = 72;
+constexpr int SW1 = 0, SW2 = SW1 + HID * S1, SW3 = SW2 + HID * S2, SWEND = SW3 + OUT * S3;
+static_assert((S1 * 2) % 16 == 0 && (S2 * 2) % 16 == 0, "16-byte rows");
+constexpr int MAXOUT = 88;   // OUT rounded up to a multiple of 8
 
+// shared memory of a block with S samples
+template <int S>
 struct MlpSmem {
-    float *W1, *W2, *W3, *b1, *b2, *b3, *x, *h1, *h2, *y;
+    __nv_bfloat16 *w;
+    float *b1, *b2, *b3, *x, *h1, *h2, *y;
     __device__ MlpSmem(float *base) {
-        W1 = base; W2 = W1 + HID * IN; W3 = W2 + HID * HID;
-        b1 = W3 + OUT * HID; b2 = b1 + HID; b3 = b2 + HID;
-        x = b3 + OUT; h1 = x + SPB * IN; h2 = h1 + SPB * HID; y = h2 + SPB * HID;
+        w = reinterpret_cast<__nv_bfloat16 *>(base);
+        b1 = base + SWEND / 2;
+        b2 = b1 + HID;
+        b3 = b2 + HID;
+        x = b3 + MAXOUT;
+        h1 = x + S * KP;
+        h2 = h1 + S * HID;
+        y = h2 + S * HID;
     }
-    __host__ __device__ static constexpr size_t floats() { return NWEIGHT + 2 * HID + OUT + SPB * (IN + 2 * HID + OUT); }
+    __host__ __device__ static constexpr size_t floats() { return SWEND / 2 + 2 * HID + MAXOUT + S * (KP + 2 * HID + MAXOUT); }
 };
+static_assert(SWEND % 8 == 0, "16-byte aligned floats behind the weights");
 
-// weights BF16 -> FP32 into shared memory, biases from the master block
-__device__ void load_net(const __nv_bfloat16 *wb, const float *params, MlpSmem &s) {
-    for (int i = threadIdx.x; i < NWEIGHT; i += blockDim.x) s.W1[i] = __bfloat162float(wb[i]);
+// weights and biases into shared memory (rows of 2-byte pairs: IN, HID are even)
+__device__ __forceinline__ void load_net(const __nv_bfloat16 *wb, const float *params, __nv_bfloat16 *w, float *b1,
+                                         float *b2, float *b3) {
+    if (reinterpret_cast<uintptr_t>(wb) & 3) {   // BF16s that do not start on a word: one at a time
+        for (int i = threadIdx.x; i < HID * KP; i += blockDim.x)
+            w[i] = i % KP < IN ? wb[i / KP * IN + i % KP] : __float2bfloat16(0.f);
+        for (int i = threadIdx.x; i < (HID + OUT) * HID; i += blockDim.x) w[SW2 + i / HID * S2 + i % HID] = wb[WB_W2 + i];
+    }
+    const unsigned *src = reinterpret_cast<const unsigned *>(wb);
+    unsigned *dst = reinterpret_cast<unsigned *>(w);
+    const bool words = !(reinterpret_cast<uintptr_t>(wb) & 3);
+    for (int i = threadIdx.x; words && i < HID * KP / 2; i += blockDim.x) {
+        const int j = i / (KP / 2), k = i - j * (KP / 2);
+        dst[i] = k < IN / 2 ? src[j * (IN / 2) + k] : 0u;
+    }
+    for (int i = threadIdx.x; words && i < (HID + OUT) * (HID / 2); i += blockDim.x) {   // W2 and W3: rows of HID
+        const int j = i / (HID / 2), k = i - j * (HID / 2);
+        dst[SW2 / 2 + j * (S2 / 2) + k] = src[WB_W2 / 2 + i];
+    }
     for (int i = threadIdx.x; i < HID; i += blockDim.x) {
-        s.b1[i] = params[OFF_B1 + i];
-        s.b2[i] = params[OFF_B2 + i];
+        b1[i] = params[OFF_B1 + i];
+        b2[i] = params[OFF_B2 + i];
     }
-    for (int i = threadIdx.x; i < OUT; i += blockDim.x) s.b3[i] = params[OFF_B3 + i];
+    for (int i = threadIdx.x; i < OUT; i += blockDim.x) b3[i] = params[OFF_B3 + i];
 }
 
-// forward pass of the SPB samples in s.x (ns valid): h1, h2, y in shared memory
-__device__ void forward_tile(MlpSmem &s, int ns) {
-    for (int o = threadIdx.x; o < SPB * HID; o += blockDim.x) {
-        const int n = o / HID, j = o - (o / HID) * HID;
-        float a = s.b1[j];
-        if (n < ns) {
-            const float *w = s.W1 + j * IN, *x = s.x + n * IN;
-#pragma unroll 6
-            for (int k = 0; k < IN; ++k) a = fmaf(w[k], x[k], a);
+// acc[n] += sum_k W[k] in[n][k] for the NS samples of a thread: 8 weights a
+// read, two partial sums a sample
+template <int K, int NS>
+__device__ __forceinline__ void dot_rows(const __nv_bfloat16 *W, const float *in, int stride, float (&acc)[NS]) {
+    float odd[NS];
+#pragma unroll
+    for (int n = 0; n < NS; ++n) odd[n] = 0.f;
+#pragma unroll 3
+    for (int k = 0; k < K; k += 8) {
+        const uint4 w4 = *reinterpret_cast<const uint4 *>(W + k);
+        const unsigned u[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+        for (int n = 0; n < NS; ++n) {
+            const float4 p = *reinterpret_cast<const float4 *>(in + n * stride + k);
+            const float4 q = *reinterpret_cast<const float4 *>(in + n * stride + k + 4);
+            const float v[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {   // a BF16 is the upper half of a float
+                acc[n] = fmaf(__uint_as_float(u[i] << 16), v[2 * i], acc[n]);
+                odd[n] = fmaf(__uint_as_float(u[i] & 0xffff0000u), v[2 * i + 1], odd[n]);
+            }
         }
-        s.h1[o] = tanhf(a);
     }
+#pragma unroll
+    for (int n = 0; n < NS; ++n) acc[n] += odd[n];
+}
+
+// forward pass of the block's S samples in s.x: h1, h2, y.  Thread t: neuron
+// t % 64 (and the 17 outputs above 64 in a second turn) of the NS samples of
+// group t / 64.
+template <int S, int NS>
+__device__ __forceinline__ void forward_tile(const MlpSmem<S> &s) {
+    const int j = threadIdx.x & 63, n0 = (threadIdx.x >> 6) * NS;
+    float a[NS];
+#pragma unroll
+    for (int n = 0; n < NS; ++n) a[n] = s.b1[j];
+    dot_rows<KP, NS>(s.w + SW1 + j * S1, s.x + n0 * KP, KP, a);
+#pragma unroll
+    for (int n = 0; n < NS; ++n) { s.h1[(n0 + n) * HID + j] = tanhf(a[n]); a[n] = s.b2[j]; }
     __syncthreads();
-    for (int o = threadIdx.x; o < SPB * HID; o += blockDim.x) {
-        const int n = o / HID, j = o - (o / HID) * HID;
-        float a = s.b2[j];
-        const float *w = s.W2 + j * HID, *h = s.h1 + n * HID;
-#pragma unroll 8
-        for (int k = 0; k < HID; ++k) a = fmaf(w[k], h[k], a);
-        s.h2[o] = tanhf(a);
-    }
+    dot_rows<HID, NS>(s.w + SW2 + j * S2, s.h1 + n0 * HID, HID, a);
+#pragma unroll
+    for (int n = 0; n < NS; ++n) s.h2[(n0 + n) * HID + j] = tanhf(a[n]);
     __syncthreads();
-    for (int o = threadIdx.x; o < SPB * OUT; o += blockDim.x) {
-        const int n = o / OUT, j = o - (o / OUT) * OUT;
-        float a = s.b3[j];
-        const float *w = s.W3 + j * HID, *h = s.h2 + n * HID;
-#pragma unroll 8
-        for (int k = 0; k < HID; ++k) a = fmaf(w[k], h[k], a);
-        s.y[o] = a;
+    for (int o = j; o < OUT; o += 64) {
+#pragma unroll
+        for (int n = 0; n < NS; ++n) a[n] = s.b3[o];
+        dot_rows<HID, NS>(s.w + SW3 + o * S3, s.h2 + n0 * HID, HID, a);
+#pragma unroll
+        for (int n = 0; n < NS; ++n) s.y[(n0 + n) * MAXOUT + o] = a[n];
     }
     __syncthreads();
 }
+
+// inference: 16 samples a block, 4 a thread, so that a weight read serves 4
+constexpr int SPB = 16, THREADS = 256;
 
 __global__ void __launch_bounds__(THREADS)
 k_mlp_forward(const __nv_bfloat16 *wb, const float *params, const float *X, int B, float *Y) {
-    extern __shared__ float smf[];
-    MlpSmem s(smf);
-    load_net(wb, params, s);
+    extern __shared__ __align__(16) float smf[];
+    const MlpSmem<SPB> s(smf);
+    load_net(wb, params, s.w, s.b1, s.b2, s.b3);
     const int n0 = blockIdx.x * SPB, ns = min(SPB, B - n0);
-    for (int i = threadIdx.x; i < SPB * IN; i += blockDim.x)
-        s.x[i] = (i / IN) < ns ? X[(size_t)n0 * IN + i] : 0.f;
+    for (int i = threadIdx.x; i < SPB * KP; i += blockDim.x) {
+        const int n = i / KP, k = i - n * KP;
+        s.x[i] = n < ns && k < IN ? X[(size_t)(n0 + n) * IN + k] : 0.f;
+    }
     __syncthreads();
-    forward_tile(s, ns);
-    for (int i = threadIdx.x; i < ns * OUT; i += blockDim.x) Y[(size_t)n0 * OUT + i] = s.y[i];
+    forward_tile<SPB, 4>(s);
+    for (int i = threadIdx.x; i < ns * OUT; i += blockDim.x) Y[(size_t)n0 * OUT + i] = s.y[i / OUT * MAXOUT + i % OUT];
 }
 
-// Per-CTA partials of loss = (1/B) sum ||yhat - t||^2 and of its gradient for
-// the samples idx[blockIdx.x*SPB ...] (idx may be null: samples in order).
-// partial: [gridDim.x][NPARAM + 1] (the last entry is the loss share).
-__global__ void __launch_bounds__(THREADS)
-k_mlp_backward(const __nv_bfloat16 *wb, const float *params, const float *X, const float *T, const int *idx,
-               int B, float *partial) {
-    extern __shared__ float smf[];
-    MlpSmem s(smf);
-    float *g3 = s.y;                    // reuses y after the loss
-    float *g2 = s.y + SPB * OUT;        // SPB*HID
-    float *g1 = g2 + SPB * HID;         // SPB*HID
-    float *red = g1 + SPB * HID;        // THREADS
-    load_net(wb, params, s);
-    const int n0 = blockIdx.x * SPB, ns = min(SPB, B - n0);
-    for (int i = threadIdx.x; i < SPB * IN; i += blockDim.x) {
-        const int n = i / IN;
-        s.x[i] = n < ns ? X[(size_t)(idx ? idx[n0 + n] : n0 + n) * IN + (i - n * IN)] : 0.f;
+// One minibatch: two kernels.  (One block of 32 samples computing its share of
+// every gradient left 144 of 152 SMs idle at 256 samples, and its weight reads,
+// 64 floats apart, hit one bank: 103 us; now 10 us for both.)
+//
+// k_mlp_samples: 2 samples a block, so that 256 samples use 128 SMs.  Record of
+// a sample in `rec`: h1, h2, g1, g2, g3 (the errors before the layers'
+// activations), loss.
+constexpr int SPT = 2, TTHREADS = 128;
+constexpr int R_H1 = 0, R_H2 = HID, R_G1 = 2 * HID, R_G2 = 3 * HID, R_G3 = 4 * HID, R_LOSS = R_G3 + OUT, REC = R_LOSS + 1;
+constexpr int PART = 32;     // samples a unit of the caller's buffer is counted in (gdg_mlp_partial_len)
+static_assert(PART * REC <= NPARAM + 1, "records fit the caller's buffer");
+
+__global__ void __launch_bounds__(TTHREADS)
+k_mlp_samples(const __nv_bfloat16 *wb, const float *params, const float *X, const float *T, const int *idx, int B,
+              float *rec) {
+    extern __shared__ __align__(16) float smf[];
+    const MlpSmem<SPT> s(smf);
+    float *g3 = smf + MlpSmem<SPT>::floats(), *g2 = g3 + SPT * MAXOUT;
+    load_net(wb, params, s.w, s.b1, s.b2, s.b3);
+    const int n0 = blockIdx.x * SPT;
+    for (int i = threadIdx.x; i < SPT * KP; i += blockDim.x) {
+        const int n = i / KP, k = i - n * KP;
+        s.x[i] = n0 + n < B && k < IN ? X[(size_t)(idx ? idx[n0 + n] : n0 + n) * IN + k] : 0.f;
     }
     __syncthreads();
-    forward_tile(s, ns);
-    // g3 = 2 (yhat - t) / B, loss share
-    float lsum = 0.f;
-    for (int o = threadIdx.x; o < SPB * OUT; o += blockDim.x) {
-        const int n = o / OUT;
-        float g = 0.f;
-        if (n < ns) {
-            const float d = s.y[o] - T[(size_t)(idx ? idx[n0 + n] : n0 + n) * OUT + (o - n * OUT)];
-            lsum += d * d;
-            g = 2.f * d / (float)B;
-        }
-        g3[o] = g;
+    forward_tile<SPT, 1>(s);
+    const int n = threadIdx.x >> 6, j = threadIdx.x & 63;
+    const bool valid = n0 + n < B;
+    float *out = rec + (size_t)(n0 + n) * REC;
+    // g3 = 2 (yhat - t) / B, and the sample's share of the loss
+    for (int o = j; o < OUT; o += 64) {
+        const float d = valid ? s.y[n * MAXOUT + o] - T[(size_t)(idx ? idx[n0 + n] : n0 + n) * OUT + o] : 0.f;
+        s.y[n * MAXOUT + o] = d * d;
+        const float g = 2.f * d / (float)B;
+        g3[n * MAXOUT + o] = g;
+        if (valid) out[R_G3 + o] = g;
     }
-    red[threadIdx.x] = lsum;
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+    // g2 = (g3 W3) (1 - h2^2)
+    const __nv_bfloat16 *w3 = s.w + SW3 + j;
+    float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+#pragma unroll 3
+    for (int o = 0; o < OUT; o += 3) {
+        a0 = fmaf(g3[n * MAXOUT + o], __bfloat162float(w3[o * S3]), a0);
+        a1 = fmaf(g3[n * MAXOUT + o + 1], __bfloat162float(w3[(o + 1) * S3]), a1);
+        a2 = fmaf(g3[n * MAXOUT + o + 2], __bfloat162float(w3[(o + 2) * S3]), a2);
+    }
+    const float h2 = s.h2[n * HID + j], h1 = s.h1[n * HID + j];
+    const float e2 = (a0 + a1 + a2) * (1.f - h2 * h2);
+    g2[n * HID + j] = e2;
+    __syncthreads();
+    // g1 = (g2 W2) (1 - h1^2)
+    const __nv_bfloat16 *w2 = s.w + SW2 + j;
+    a0 = a1 = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < HID; k += 2) {
+        a0 = fmaf(g2[n * HID + k], __bfloat162float(w2[k * S2]), a0);
+        a1 = fmaf(g2[n * HID + k + 1], __bfloat162float(w2[(k + 1) * S2]), a1);
+    }
+    if (valid) {
+        out[R_H1 + j] = h1;
+        out[R_H2 + j] = h2;
+        out[R_G1 + j] = (a0 + a1) * (1.f - h1 * h1);
+        out[R_G2 + j] = e2;
+    }
+    if (j < 32) {   // the first warp of the sample's two (OUT <= 96)
+        float l = s.y[n * MAXOUT + j] + s.y[n * MAXOUT + 32 + j] + (64 + j < OUT ? s.y[n * MAXOUT + 64 + j] : 0.f);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (valid && j == 0) out[R_LOSS] = l / (float)B;
+    }
+}
+static_assert(OUT % 3 == 0 && HID % 2 == 0, "unrolled sums");
+
+// k_mlp_grad: dW = sum over the samples of (error) x (input of the layer), 16 x
+// 16 entries a block (4 a thread), samples staged 32 at a time; the first
+// input column's blocks also sum the bias, the last block the loss.  Fixed
+// order: deterministic.
+constexpr int GT = 16, GN = 32;
+__host__ __device__ constexpr int tiles(int n) { return (n + GT - 1) / GT; }
+constexpr int T1 = tiles(HID) * tiles(IN), T2 = tiles(HID) * tiles(HID), T3 = tiles(OUT) * tiles(HID);
+
+__global__ void __launch_bounds__(64)
+k_mlp_grad(const float *X, const int *idx, const float *rec, int B, float *grad, float *loss) {
+    __shared__ float E[GN][GT], I[GN][GT];
+    const int t = threadIdx.x;
+    int tile = blockIdx.x;
+    if (tile == T1 + T2 + T3) {   // loss: 64 partial sums, then in order
+        float l = 0.f;
+        for (int n = t; n < B; n += 64) l += rec[(size_t)n * REC + R_LOSS];
+        float *part = &E[0][0];
+        part[t] = l;
         __syncthreads();
+        if (t == 0) {
+            float a = 0.f;
+            for (int i = 0; i < 64; ++i) a += part[i];
+            *loss = a;
+        }
+        return;
     }
-    float *out = partial + (size_t)blockIdx.x * (NPARAM + 1);
-    if (threadIdx.x == 0) out[NPARAM] = red[0] / (float)B;
-    // layer 3: dW3[o][j] = sum_n g3[n][o] h2[n][j], db3
-    for (int p = threadIdx.x; p < OUT * HID; p += blockDim.x) {
-        const int o = p / HID, j = p - (p / HID) * HID;
-        float a = 0.f;
-        for (int n = 0; n < SPB; ++n) a = fmaf(g3[n * OUT + o], s.h2[n * HID + j], a);
-        out[OFF_W3 + p] = a;
+    int rows, cols, re, ri, ow, ob;   // outputs, inputs, where errors and inputs lie in a record, in grad
+    if (tile < T1) { rows = HID; cols = IN; re = R_G1; ri = -1; ow = OFF_W1; ob = OFF_B1; }
+    else if (tile < T1 + T2) { tile -= T1; rows = HID; cols = HID; re = R_G2; ri = R_H1; ow = OFF_W2; ob = OFF_B2; }
+    else { tile -= T1 + T2; rows = OUT; cols = HID; re = R_G3; ri = R_H2; ow = OFF_W3; ob = OFF_B3; }
+    const int tc = tiles(cols), r0 = (tile / tc) * GT, c0 = (tile - (tile / tc) * tc) * GT;
+    const int r = (t >> 3) * 2, c = (t & 7) * 2;   // this thread's 2 x 2 entries
+    float a[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, bias[2] = {0.f, 0.f};
+    for (int b0 = 0; b0 < B; b0 += GN) {
+        float e[GN * GT / 64], in[GN * GT / 64];
+#pragma unroll
+        for (int i = 0; i < GN * GT / 64; ++i) {
+            const int q = t + 64 * i, n = b0 + q / GT, k = q % GT;
+            e[i] = n < B && r0 + k < rows ? rec[(size_t)n * REC + re + r0 + k] : 0.f;
+            in[i] = n < B && c0 + k < cols
+                        ? (ri < 0 ? X[(size_t)(idx ? idx[n] : n) * IN + c0 + k] : rec[(size_t)n * REC + ri + c0 + k])
+                        : 0.f;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < GN * GT / 64; ++i) {
+            const int q = t + 64 * i;
+            E[q / GT][q % GT] = e[i];
+            I[q / GT][q % GT] = in[i];
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int n = 0; n < GN; ++n) {
+            const float2 ev = *reinterpret_cast<const float2 *>(&E[n][r]), iv = *reinterpret_cast<const float2 *>(&I[n][c]);
+            a[0][0] = fmaf(ev.x, iv.x, a[0][0]);
+            a[0][1] = fmaf(ev.x, iv.y, a[0][1]);
+            a[1][0] = fmaf(ev.y, iv.x, a[1][0]);
+            a[1][1] = fmaf(ev.y, iv.y, a[1][1]);
+            bias[0] += ev.x;
+            bias[1] += ev.y;
+        }
     }
-    for (int o = threadIdx.x; o < OUT; o += blockDim.x) {
-        float a = 0.f;
-        for (int n = 0; n < SPB; ++n) a += g3[n * OUT + o];
-        out[OFF_B3 + o] = a;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        if (r0 + r + i >= rows) continue;
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (c0 + c + k < cols) grad[ow + (r0 + r + i) * cols + c0 + c + k] = a[i][k];
+        if (c0 == 0 && c == 0) grad[ob + r0 + r + i] = bias[i];
     }
-    // g2 = (g3 W3) * (1 - h2^2)
-    for (int q = threadIdx.x; q < SPB * HID; q += blockDim.x) {
-        const int n = q / HID, j = q - (q / HID) * HID;
-        float a = 0.f;
-        for (int o = 0; o < OUT; ++o) a = fmaf(g3[n * OUT + o], s.W3[o * HID + j], a);
-        const float h = s.h2[q];
-        g2[q] = a * (1.f - h * h);
-    }
-    __syncthreads();
-    for (int p = threadIdx.x; p < HID * HID; p += blockDim.x) {
-        const int j = p / HID, k = p - (p / HID) * HID;
-        float a = 0.f;
-        for (int n = 0; n < SPB; ++n) a = fmaf(g2[n * HID + j], s.h1[n * HID + k], a);
-        out[OFF_W2 + p] = a;
-    }
-    for (int j = threadIdx.x; j < HID; j += blockDim.x) {
-        float a = 0.f;
-        for (int n = 0; n < SPB; ++n) a += g2[n * HID + j];
-        out[OFF_B2 + j] = a;
-    }
-    // g1 = (g2 W2) * (1 - h1^2)
-    for (int q = threadIdx.x; q < SPB * HID; q += blockDim.x) {
-        const int n = q / HID, j = q - (q / HID) * HID;
-        float a = 0.f;
-        for (int k = 0; k < HID; ++k) a = fmaf(g2[n * HID + k], s.W2[k * HID + j], a);
-        const float h = s.h1[q];
-        g1[q] = a * (1.f - h * h);
-    }
-    __syncthreads();
-    for (int p = threadIdx.x; p < HID * IN; p += blockDim.x) {
-        const int j = p / IN, k = p - (p / IN) * IN;
-        float a = 0.f;
-        for (int n = 0; n < SPB; ++n) a = fmaf(g1[n * HID + j], s.x[n * IN + k], a);
-        out[OFF_W1 + p] = a;
-    }
-    for (int j = threadIdx.x; j < HID; j += blockDim.x) {
-        float a = 0.f;
-        for (int n = 0; n < SPB; ++n) a += g1[n * HID + j];
-        out[OFF_B1 + j] = a;
-    }
-}
-
-// grad[p] = sum over CTAs (in order) of partial[c][p]; loss likewise
-__global__ void k_mlp_reduce(const float *partial, int nblocks, float *grad, float *loss) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > NPARAM) return;
-    float a = 0.f;
-    for (int c = 0; c < nblocks; ++c) a += partial[(size_t)c * (NPARAM + 1) + p];
-    if (p < NPARAM) grad[p] = a;
-    else *loss = a;
 }
 
 __global__ void k_mlp_adam(float *params, float *m, float *v, const float *grad, float lr, float b1, float b2,
@@ -237,10 +335,10 @@ __global__ void k_mlp_to_bf16(const float *params, __nv_bfloat16 *wb) {
 __global__ void __launch_bounds__(THREADS)
 k_mlp_guess(const __nv_bfloat16 *wb, const float *params, const float *c2feat, const double *ru, int ne,
             double *x0u) {
-    extern __shared__ float smf[];
-    MlpSmem s(smf);
-    float *nrm = smf + MlpSmem::floats();     // [SPB]
-    load_net(wb, params, s);
+    extern __shared__ __align__(16) float smf[];
+    const MlpSmem<SPB> s(smf);
+    float *nrm = smf + MlpSmem<SPB>::floats();     // [SPB]
+    load_net(wb, params, s.w, s.b1, s.b2, s.b3);
     const int n0 = blockIdx.x * SPB, ns = min(SPB, ne - n0);
     if (threadIdx.x < SPB) {
         double a = 0.0;
@@ -252,18 +350,19 @@ k_mlp_guess(const __nv_bfloat16 *wb, const float *params, const float *c2feat, c
         nrm[threadIdx.x] = (float)sqrt(a);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < SPB * IN; i += blockDim.x) {
-        const int n = i / IN, k = i - (i / IN) * IN;
+    for (int i = threadIdx.x; i < SPB * KP; i += blockDim.x) {
+        const int n = i / KP, k = i - n * KP;
         float x = 0.f;
-        if (n < ns) {
+        if (n < ns && k < IN) {
             if (k < OUT) x = c2feat[(size_t)(n0 + n) * OUT + k];
             else if (nrm[n] > 0.f) x = (float)(ru[(size_t)(n0 + n) * OUT + (k - OUT)] / (double)nrm[n]);
         }
         s.x[i] = x;
     }
     __syncthreads();
-    forward_tile(s, ns);
-    for (int i = threadIdx.x; i < ns * OUT; i += blockDim.x) x0u[(size_t)n0 * OUT + i] = (double)nrm[i / OUT] * s.y[i];
+    forward_tile<SPB, 4>(s);
+    for (int i = threadIdx.x; i < ns * OUT; i += blockDim.x)
+        x0u[(size_t)n0 * OUT + i] = (double)nrm[i / OUT] * s.y[i / OUT * MAXOUT + i % OUT];
 }
 
 // training rows: X = [c2feat, r_u/||r_u||] (FP32) and, when y is given,
@@ -284,15 +383,15 @@ __global__ void k_mlp_rows(const float *c2feat, const double *ru, const double *
     }
 }
 
-size_t fwd_smem() { return MlpSmem::floats() * sizeof(float); }
-size_t guess_smem() { return (MlpSmem::floats() + SPB) * sizeof(float); }
-size_t bwd_smem() { return (MlpSmem::floats() + 2 * SPB * HID + THREADS) * sizeof(float); }
+size_t fwd_smem() { return MlpSmem<SPB>::floats() * sizeof(float); }
+size_t guess_smem() { return (MlpSmem<SPB>::floats() + SPB) * sizeof(float); }
+size_t samples_smem() { return (MlpSmem<SPT>::floats() + SPT * (MAXOUT + HID)) * sizeof(float); }
 
 bool attrs_done = false;
 int set_attrs() {
     if (attrs_done) return GDG_OK;
     if (cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd_smem()) != cudaSuccess ||
-        cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem()) != cudaSuccess ||
+        cudaFuncSetAttribute(k_mlp_samples, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)samples_smem()) != cudaSuccess ||
         cudaFuncSetAttribute(k_mlp_guess, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)guess_smem()) != cudaSuccess)
         return GDG_ECUDA;
     attrs_done = true;
@@ -327,7 +426,7 @@ extern "C" int gdg_mlp_forward(const uint16_t *w_bf16, const float *params, cons
 }
 
 extern "C" long long gdg_mlp_partial_len(int B) {
-    return B <= 0 ? 0 : (long long)((B + SPB - 1) / SPB) * (NPARAM + 1);
+    return B <= 0 ? 0 : (long long)((B + PART - 1) / PART) * (NPARAM + 1);
 }
 
 extern "C" int gdg_mlp_backward(const uint16_t *w_bf16, const float *params, const float *X, const float *T,
@@ -335,10 +434,9 @@ extern "C" int gdg_mlp_backward(const uint16_t *w_bf16, const float *params, con
     if (!w_bf16 || !params || !X || !T || !partial || !grad || !loss || B <= 0) return GDG_EINVAL;
     if (set_attrs()) return GDG_ECUDA;
     cudaStream_t s = (cudaStream_t)stream;
-    const int grid = (B + SPB - 1) / SPB;
-    k_mlp_backward<<<grid, THREADS, bwd_smem(), s>>>(reinterpret_cast<const __nv_bfloat16 *>(w_bf16), params, X,
-                                                     T, idx, B, partial);
-    k_mlp_reduce<<<(NPARAM + 1 + 255) / 256, 256, 0, s>>>(partial, grid, grad, loss);
+    k_mlp_samples<<<(B + SPT - 1) / SPT, TTHREADS, samples_smem(), s>>>(
+        reinterpret_cast<const __nv_bfloat16 *>(w_bf16), params, X, T, idx, B, partial);
+    k_mlp_grad<<<T1 + T2 + T3 + 1, 64, 0, s>>>(X, idx, partial, B, grad, loss);
     return cudaGetLastError() == cudaSuccess ? GDG_OK : GDG_ECUDA;
 }
 
