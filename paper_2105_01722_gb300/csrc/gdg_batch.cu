@@ -179,7 +179,7 @@ extern "C" int gdg_batch_create(const gdg_problem *pbs, int count, gdg_batch **o
         if (pbs[i].coef == GDG_COEF_CONST) {
             if (!c->mp.parity) { gdg_batch_destroy(b); return berr(nullptr, GDG_EUNSUPPORTED, "modal basis without parity"); }
             P.kind = 0;
-            P.lam2 = c->d_lam2;
+            P.lams = c->d_lams;
             P.sb = gdg_const_buffers(c);
             mps[i] = c->mp;
             for (int t = 0; t * b->tile < c->ne; ++t) mod_items.push_back(make_int2(i, t));
@@ -256,7 +256,7 @@ extern "C" int gdg_batch_step(gdg_batch *b, double *const *u, double *const *v, 
     auto enter = [&]() -> int {
         for (int i = 0; i < b->count; ++i) {
             gdg_ctx *c = b->ctx[i];
-            const int e = c->pb.coef == GDG_COEF_CONST ? gdg_const_enter(c, u[i], v[i], s)
+            const int e = c->pb.coef == GDG_COEF_CONST ? gdg_const_enter(c, u[i], v[i], dt[i], s)
                                                        : gdg_var_enter(c, u[i], v[i], s);
             if (e) return berr(b, e, "enter: " + c->err);
         }

@@ -13,8 +13,8 @@
 //                                 mixed solves' 27 KB allow 8 blocks, and the
 //                                 precomputed-inverse route streams its
 //                                 operators and wants every warp it can get);
-//                                 the modal body reads y_n and the
-//                                 accumulator where it uses them (LEAN).
+//                                 the modal body reads y_n where it
+//                                 uses it (LEAN).
 #pragma once
 
 #include "gdg_checks.cuh"
@@ -29,7 +29,7 @@ enum { BATCH_HI = 0, BATCH_MID = 1, BATCH_LO = 2, BATCH_VARIANTS = 3 };
 struct BatchProb {
     int kind;                 // 0 modal route (constant coefficients), 1 element solves
     const ModalParams *mp;    // kind 0: device copy of the problem's modal parameters
-    const double *lam2;       // kind 0
+    const double *lams;       // kind 0: the stages' tables (gdg_ctx::d_lams)
     VarParams vp;             // kind 1
     StepBuffers sb;
     double dt;
@@ -101,7 +101,7 @@ __host__ __device__ constexpr size_t batch_modal_doubles(int n1) {
 
 template <int N1, int STAGE, bool LEAN>
 __device__ __forceinline__ void batch_mod_item(const BatchProb *__restrict__ probs, int2 w, int &cur, double *smem) {
-    constexpr int MODE = STAGE == 1 ? M_S1 : (STAGE == 4 ? M_S4 : M_S23);
+    constexpr int MODE = STAGE == 1 ? M_S1 : M_S23;
     const BatchProb &P = probs[w.x];
     ModalParams *s_mp = reinterpret_cast<ModalParams *>(smem + batch_modal_doubles(N1));
     if (w.x != cur) {
@@ -109,8 +109,9 @@ __device__ __forceinline__ void batch_mod_item(const BatchProb *__restrict__ pro
         cur = w.x;
     }
     const StageRoles<STAGE> r(P.sb, P.dt);
-    const StageBufs bb{r.yU, r.yV, P.sb.nU, P.sb.nV, P.sb.aU, P.sb.aV, r.oU, r.oV, r.trin, r.trout, P.lam2};
-    stage2h_body<N1, MODE, LEAN>(*s_mp, bb, r.cA, r.cY, w.y, smem);
+    const StageBufs bb{r.yU, r.yV, P.sb.nU, P.sb.nV, STAGE == 4 ? P.sb.nU : r.oU, STAGE == 4 ? P.sb.nV : r.oV,
+                       r.trin, r.trout, P.lams + (STAGE - 1) * 4 * N1 * N1};
+    stage2h_body<N1, MODE, LEAN>(*s_mp, bb, P.dt / (RK_STAGES + 1 - STAGE), w.y, smem);
 }
 
 __host__ __device__ constexpr int batch_min_blocks(int n1, int variant) {

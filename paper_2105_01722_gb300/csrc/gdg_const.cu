@@ -42,7 +42,7 @@ constexpr int TPB1 = 128;  // threads per block, 1-D kernels (one element per th
 
 template <int N1, int MODE>
 __global__ void __launch_bounds__(MAXB2)
-k_stage2(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, double cY) {
+k_stage2(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) {
     extern __shared__ double smem[];
     const int t = threadIdx.x;
     const int le = t / N1, l = t - le * N1;
@@ -103,34 +103,18 @@ k_stage2(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, d
         for (int k = 0; k < N1; ++k) {
             const double Yu = b.yU[row + k], Yv = b.yV[row + k];
             const double ru = mp.d[0].gL[k] * gxm + mp.d[0].gR[k] * gxp + gLy * fy[k] + gRy * fy[N1 + k];
-            const double rv = L0[k] * Yu + mp.d[0].eL[k] * qxm + mp.d[0].eR[k] * qxp +
-                              eLy * fy[2 * N1 + k] + eRy * fy[3 * N1 + k];
-            const double ku = Yv + L1[k] * ru;
-            const double kv = rv;
+            const double rv = mp.d[0].eL[k] * qxm + mp.d[0].eR[k] * qxp + eLy * fy[2 * N1 + k] + eRy * fy[3 * N1 + k];
             if (MODE == M_RHS) {
-                b.oU[row + k] = ku;
-                b.oV[row + k] = kv;
-            } else if (MODE == M_S1) {
-                b.aU[row + k] = cA * ku;
-                b.aV[row + k] = cA * kv;
-                Ru[k] = Yu + cY * ku;
-                Rv[k] = Yv + cY * kv;
-            } else if (MODE == M_S23) {
-                b.aU[row + k] += cA * ku;
-                b.aV[row + k] += cA * kv;
-                Ru[k] = b.nU[row + k] + cY * ku;
-                Rv[k] = b.nV[row + k] + cY * kv;
-            } else {
-                Ru[k] = b.nU[row + k] + b.aU[row + k] + cA * ku;
-                Rv[k] = b.nV[row + k] + b.aV[row + k] + cA * kv;
+                Ru[k] = Yv + L1[k] * ru;
+                Rv[k] = L0[k] * Yu + rv;
+            } else {   // L0, L1 carry sc
+                const double Nu = MODE == M_S1 ? Yu : b.nU[row + k], Nv = MODE == M_S1 ? Yv : b.nV[row + k];
+                Ru[k] = fma(sc, Yv, fma(L1[k], ru, Nu));
+                Rv[k] = fma(L0[k], Yu, fma(sc, rv, Nv));
             }
         }
-        if (MODE != M_RHS) {
-            double *dU = (MODE == M_S4) ? b.nU : b.oU;
-            double *dV = (MODE == M_S4) ? b.nV : b.oV;
 #pragma unroll
-            for (int k = 0; k < N1; ++k) { dU[row + k] = Ru[k]; dV[row + k] = Rv[k]; }
-        }
+        for (int k = 0; k < N1; ++k) { b.oU[row + k] = Ru[k]; b.oV[row + k] = Rv[k]; }
     }
     if (MODE == M_RHS) return;   // uniform across the block
 
@@ -172,17 +156,17 @@ k_stage2(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, d
 
 template <int N1, int MODE, int ALT>
 __global__ void __launch_bounds__(MAXB2)
-k_stage2p(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, double cY) {
+k_stage2p(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) {
     extern __shared__ double smem[];
-    stage2p_body<N1, MODE, ALT>(mp, b, cA, cY, blockIdx.x, smem);
+    stage2p_body<N1, MODE, ALT>(mp, b, sc, blockIdx.x, smem);
 }
 
 // half-line variant (two threads per line), bit-identical results
 template <int N1, int MODE>
 __global__ void __launch_bounds__(MAXB2)
-k_stage2h(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, double cY) {
+k_stage2h(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) {
     extern __shared__ double smem[];
-    stage2h_body<N1, MODE>(mp, b, cA, cY, blockIdx.x, smem);
+    stage2h_body<N1, MODE>(mp, b, sc, blockIdx.x, smem);
 }
 
 // Field-split variant of stage2p_body.  The block's first W = 32 ceil(epb N1 / 32)
@@ -239,43 +223,28 @@ __device__ __forceinline__ void s2f_fluxes(const ModalParams &mp, const StageBuf
 // lift, diagonal solve and RK update of one field of line l, then the line's
 // row traces of that field and its row of the transpose tile
 template <int N1, int MODE, int FIELD>
-__device__ __forceinline__ void s2f_update(const ModalParams &mp, const StageBufs &b, double cA, double cY,
-                                           int e, int l, size_t row, const double *fy, double *tile, double XA,
-                                           double XB, double (&R)[N1], const double (&Y)[N1],
-                                           const double (&Nn)[N1], const double (&Aa)[N1]) {
+__device__ __forceinline__ void s2f_update(const ModalParams &mp, const StageBufs &b, double sc, int e, int l, size_t row,
+                                           const double *fy, double *tile, double XA, double XB, double (&R)[N1],
+                                           const double (&Y)[N1], const double (&Nn)[N1]) {
     constexpr int NE = (N1 + 1) / 2;
     double *oF = FIELD == 0 ? b.oU : b.oV;
-    double *aF = FIELD == 0 ? b.aU : b.aV;
-    double *nF = FIELD == 0 ? b.nU : b.nV;
     const double *L = b.lam2 + l * N1;
     const double *P1 = b.lam2 + 2 * N1 * N1 + l * N1, *P2 = b.lam2 + 3 * N1 * N1 + l * N1;
-    const double hy = mp.d[1].ceL[l];
+    const double cey = MODE == M_RHS ? mp.d[1].ceL[l] : sc * mp.d[1].ceL[l];
+    if (MODE != M_RHS && FIELD == 1) { XA *= sc; XB *= sc; }
     const double *F = fy + (FIELD == 0 ? 0 : 2 * N1) + (l < NE ? 0 : N1);
 #pragma unroll
-    for (int k = 0; k < N1; ++k) {
-        const double x = k < NE ? XA : XB;
-        double kf;
-        if (FIELD == 0) {
-            kf = fma(P1[k], x, fma(P2[k], F[k], Y[k]));
-        } else {
-            kf = fma(L[k], Y[k], fma(mp.d[0].ceL[k], x, hy * F[k]));
-        }
-        if (MODE == M_RHS) {
-            oF[row + k] = kf;
-        } else if (MODE == M_S1) {
-            aF[row + k] = kf;
-            R[k] = fma(cY, kf, R[k]);
-        } else if (MODE == M_S23) {
-            aF[row + k] = fma(2.0, kf, Aa[k]);
-            R[k] = fma(cY, kf, Nn[k]);
-        } else {
-            R[k] = fma(cA, Aa[k] + kf, Nn[k]);
-        }
+    for (int k = 0; k < N1; ++k) {   // the field's half of stage_entry (the other half is not used)
+        const double x = k < NE ? XA : XB, n = MODE == M_S1 ? R[k] : Nn[k];
+        double unused;
+        if (FIELD == 0)
+            stage_entry<MODE>(sc, 0.0, P1[k], P2[k], 0.0, 0.0, x, 0.0, F[k], 0.0, 0.0, Y[k], n, 0.0, R[k], unused);
+        else
+            stage_entry<MODE>(sc, L[k], 0.0, 0.0, mp.d[0].ceL[k], cey, 0.0, x, 0.0, F[k], Y[k], 0.0, 0.0, n, unused, R[k]);
     }
-    if (MODE == M_RHS) return;
-    double *dF = MODE == M_S4 ? nF : oF;
 #pragma unroll
-    for (int k = 0; k < N1; ++k) dF[row + k] = R[k];
+    for (int k = 0; k < N1; ++k) oF[row + k] = R[k];
+    if (MODE == M_RHS) return;
     double se = 0, so = 0;
 #pragma unroll
     for (int k = 0; k < N1; ++k) {
@@ -307,7 +276,7 @@ __device__ __forceinline__ void s2f_columns(const ModalParams &mp, const StageBu
 
 template <int N1, int MODE, int ALT>
 __global__ void __launch_bounds__(2 * MAXB2)
-k_stage2f(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, double cY) {
+k_stage2f(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) {
     extern __shared__ double smem[];
     const int epb = mp.epb;
     const int W = ((epb * N1 + 31) / 32) * 32;
@@ -320,19 +289,16 @@ k_stage2f(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, 
     double *fy = smem + le * (4 * N1);
     double *tile = smem + epb * 4 * N1 + le * (2 * N1 * (N1 + 1));
     const size_t row = ((size_t)(valid ? e : 0) * N1 + l) * N1;
-    // own field's stage input R (and y_n, accumulator), the other field's Y
-    double R[N1], Y[N1], Nn[N1], Aa[N1];
+    // own field's stage input R (and y_n), the other field's Y
+    double R[N1], Y[N1], Nn[N1];
     if (valid) {
         const double *own = fu ? b.yU : b.yV, *oth = fu ? b.yV : b.yU;
-        const double *nF = fu ? b.nU : b.nV, *aF = fu ? b.aU : b.aV;
+        const double *nF = fu ? b.nU : b.nV;
 #pragma unroll
         for (int k = 0; k < N1; ++k) {
             R[k] = own[row + k];
             Y[k] = oth[row + k];
-            if (MODE == M_S23 || MODE == M_S4) {
-                Nn[k] = nF[row + k];
-                Aa[k] = aF[row + k];
-            }
+            if (MODE == M_S23) Nn[k] = nF[row + k];
         }
     }
     double XA = 0, XB = 0;
@@ -342,8 +308,8 @@ k_stage2f(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, 
     }
     __syncthreads();
     if (valid) {
-        if (fu) s2f_update<N1, MODE, 0>(mp, b, cA, cY, e, l, row, fy, tile, XA, XB, R, Y, Nn, Aa);
-        else s2f_update<N1, MODE, 1>(mp, b, cA, cY, e, l, row, fy, tile, XA, XB, R, Y, Nn, Aa);
+        if (fu) s2f_update<N1, MODE, 0>(mp, b, sc, e, l, row, fy, tile, XA, XB, R, Y, Nn);
+        else s2f_update<N1, MODE, 1>(mp, b, sc, e, l, row, fy, tile, XA, XB, R, Y, Nn);
     }
     if (MODE == M_RHS) return;
     __syncthreads();
@@ -461,12 +427,12 @@ __device__ void neighbour_blocks(const ModalParams &mp, int epb, int *s_nb, int 
 }
 
 // one RK stage of stage2p_body on register state: R (stage input, becomes
-// the next stage's input), Nn (y_n), Aa (accumulator), per field
-template <int N1, int MODE, int ALT>
+// the stage's output), N (y_n), per field
+template <int N1, int ALT>
 __device__ __forceinline__ void stage2r(const ModalParams &mp, const double *lam2, const double *trin,
-                                        double *trout, double cA, double cY, int e, int l, bool valid,
+                                        double *trout, double sc, int e, int l, bool valid,
                                         double *fy, double *tile, double (&Ru)[N1], double (&Rv)[N1],
-                                        double (&Nu)[N1], double (&Nv)[N1], double (&Au)[N1], double (&Av)[N1]) {
+                                        const double (&Nu)[N1], const double (&Nv)[N1]) {
     constexpr int NE = (N1 + 1) / 2;
     const int nx = mp.nx, ny = mp.ny;
     const int ex = valid ? e % nx : 0, ey = valid ? e / nx : 0;
@@ -513,32 +479,17 @@ __device__ __forceinline__ void stage2r(const ModalParams &mp, const double *lam
     if (valid) {
         const double *L0 = lam2 + l * N1;
         const double *P1 = lam2 + 2 * N1 * N1 + l * N1, *P2 = lam2 + 3 * N1 * N1 + l * N1;
-        const double cey = mp.d[1].ceL[l];
+        const double cey = sc * mp.d[1].ceL[l];
+        QA *= sc;
+        QB *= sc;
         const double *FG = fy + (l < NE ? 0 : N1);
         const double *FQ = fy + (l < NE ? 2 * N1 : 3 * N1);
 #pragma unroll
         for (int k = 0; k < N1; ++k) {
             const double Yu = Ru[k], Yv = Rv[k];
             const double xg = k < NE ? GA : GB, xq = k < NE ? QA : QB;
-            const double ku = fma(P1[k], xg, fma(P2[k], FG[k], Yv));
-            const double rv = fma(L0[k], Yu, fma(mp.d[0].ceL[k], xq, cey * FQ[k]));
-            const double kv = rv;
-            if (MODE == M_S1) {
-                Au[k] = ku;
-                Av[k] = kv;
-                Ru[k] = fma(cY, ku, Yu);
-                Rv[k] = fma(cY, kv, Yv);
-            } else if (MODE == M_S23) {
-                Au[k] = fma(2.0, ku, Au[k]);
-                Av[k] = fma(2.0, kv, Av[k]);
-                Ru[k] = fma(cY, ku, Nu[k]);
-                Rv[k] = fma(cY, kv, Nv[k]);
-            } else {
-                Ru[k] = fma(cA, Au[k] + ku, Nu[k]);
-                Rv[k] = fma(cA, Av[k] + kv, Nv[k]);
-                Nu[k] = Ru[k];
-                Nv[k] = Rv[k];
-            }
+            stage_entry<M_S23>(sc, L0[k], P1[k], P2[k], mp.d[0].ceL[k], cey, xg, xq, FG[k], FQ[k], Yu, Yv, Nu[k], Nv[k],
+                               Ru[k], Rv[k]);
         }
         double ve = 0, vo_ = 0, de = 0, do_ = 0;
 #pragma unroll
@@ -574,12 +525,12 @@ __device__ __forceinline__ void stage2r(const ModalParams &mp, const double *lam
 // traces of y_n on entry and of the result on exit (as enqueue_rk4_step).
 // blockDim.x = epb * N1 (epb <= MAXB2 / N1); sync: sync_words(gridDim.x)
 // words (see neighbour_sync).
-// Registers are allocated per SM sub-partition (16,384 each): at <= 168 per
-// thread three warps fit in one, at 169..176 only two, so the cap keeps
-// 12 instead of 8 warps of the grid resident per SM.
+// Registers are allocated per SM sub-partition (16,384 each): at <= 128 per
+// thread four warps fit in one, so the cap keeps 16 warps of the grid resident
+// per SM (a line's state is 4 N1 doubles, 72 registers at N1 = 9).
 template <int N1, int ALT>
-__global__ void __maxnreg__(168)
-k_step2r(const __grid_constant__ ModalParams mp, const double *lam2, double *nU, double *nV, double *tr0,
+__global__ void __maxnreg__(128)
+k_step2r(const __grid_constant__ ModalParams mp, const double *lams, double *nU, double *nV, double *tr0,
          double *tr1, double dt, int nsteps, unsigned *sync, unsigned long long limit_ns) {
     extern __shared__ double smem[];
     __shared__ int s_ok;
@@ -596,32 +547,29 @@ k_step2r(const __grid_constant__ ModalParams mp, const double *lam2, double *nU,
     neighbour_blocks(mp, epb, s_nb, &s_cnt);
     __syncthreads();
     const int nnb = s_cnt;
-    double Ru[N1], Rv[N1], Nu[N1], Nv[N1], Au[N1], Av[N1];
+    double Ru[N1], Rv[N1], Nu[N1], Nv[N1];
 #pragma unroll
     for (int k = 0; k < N1; ++k) {
-        Nu[k] = valid ? nU[row + k] : 0.0;
-        Nv[k] = valid ? nV[row + k] : 0.0;
-        Ru[k] = Nu[k];
-        Rv[k] = Nv[k];
-        Au[k] = 0.0;
-        Av[k] = 0.0;
+        Ru[k] = valid ? nU[row + k] : 0.0;
+        Rv[k] = valid ? nV[row + k] : 0.0;
     }
     unsigned round = 0;
     for (int step = 0; step < nsteps; ++step) {
-        stage2r<N1, M_S1, ALT>(mp, lam2, tr0, tr1, dt / 6.0, 0.5 * dt, e, l, valid, fy, tile, Ru, Rv, Nu, Nv, Au, Av);
-        if (!neighbour_sync(sync, s_nb, nnb, ++round, limit_ns, &s_ok)) return;
-        stage2r<N1, M_S23, ALT>(mp, lam2, tr1, tr0, dt / 3.0, 0.5 * dt, e, l, valid, fy, tile, Ru, Rv, Nu, Nv, Au, Av);
-        if (!neighbour_sync(sync, s_nb, nnb, ++round, limit_ns, &s_ok)) return;
-        stage2r<N1, M_S23, ALT>(mp, lam2, tr0, tr1, dt / 3.0, dt, e, l, valid, fy, tile, Ru, Rv, Nu, Nv, Au, Av);
-        if (!neighbour_sync(sync, s_nb, nnb, ++round, limit_ns, &s_ok)) return;
-        stage2r<N1, M_S4, ALT>(mp, lam2, tr1, tr0, dt / 6.0, 0.0, e, l, valid, fy, tile, Ru, Rv, Nu, Nv, Au, Av);
-        if (step + 1 < nsteps && !neighbour_sync(sync, s_nb, nnb, ++round, limit_ns, &s_ok)) return;
+#pragma unroll
+        for (int k = 0; k < N1; ++k) { Nu[k] = Ru[k]; Nv[k] = Rv[k]; }
+        for (int st = 0; st < RK_STAGES; ++st) {
+            const bool even = (st & 1) == 0;
+            stage2r<N1, ALT>(mp, lams + (size_t)st * 4 * N1 * N1, even ? tr0 : tr1, even ? tr1 : tr0,
+                             dt / (RK_STAGES - st), e, l, valid, fy, tile, Ru, Rv, Nu, Nv);
+            if (st + 1 == RK_STAGES && step + 1 == nsteps) break;
+            if (!neighbour_sync(sync, s_nb, nnb, ++round, limit_ns, &s_ok)) return;
+        }
     }
     if (valid) {
 #pragma unroll
         for (int k = 0; k < N1; ++k) {
-            nU[row + k] = Nu[k];
-            nV[row + k] = Nv[k];
+            nU[row + k] = Ru[k];
+            nV[row + k] = Rv[k];
         }
     }
 }
@@ -813,7 +761,7 @@ __global__ void k_sum_partials(int n, const double *partial, double *out) {
 
 template <int N1, int MODE>
 __global__ void __launch_bounds__(TPB1)
-k_stage1(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, double cY) {
+k_stage1(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= mp.ne) return;
     const int nx = mp.nx;
@@ -840,27 +788,21 @@ k_stage1(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, d
     for (int k = 0; k < N1; ++k) {
         const double Yu = b.yU[row + k], Yv = b.yV[row + k];
         const double ru = mp.d[0].gL[k] * gm + mp.d[0].gR[k] * gp;
-        const double rv = b.lam2[k] * Yu + mp.d[0].eL[k] * qm + mp.d[0].eR[k] * qp;
-        const double ku = Yv + b.lam2[N1 + k] * ru, kv = rv;
-        if (MODE == M_RHS) { b.oU[row + k] = ku; b.oV[row + k] = kv; }
-        else if (MODE == M_S1) {
-            b.aU[row + k] = cA * ku; b.aV[row + k] = cA * kv;
-            Ru[k] = Yu + cY * ku; Rv[k] = Yv + cY * kv;
-        } else if (MODE == M_S23) {
-            b.aU[row + k] += cA * ku; b.aV[row + k] += cA * kv;
-            Ru[k] = b.nU[row + k] + cY * ku; Rv[k] = b.nV[row + k] + cY * kv;
-        } else {
-            Ru[k] = b.nU[row + k] + b.aU[row + k] + cA * ku;
-            Rv[k] = b.nV[row + k] + b.aV[row + k] + cA * kv;
+        const double rv = mp.d[0].eL[k] * qm + mp.d[0].eR[k] * qp;
+        if (MODE == M_RHS) {
+            b.oU[row + k] = Yv + b.lam2[N1 + k] * ru;
+            b.oV[row + k] = b.lam2[k] * Yu + rv;
+        } else {   // lam2 carries sc
+            const double Nu = MODE == M_S1 ? Yu : b.nU[row + k], Nv = MODE == M_S1 ? Yv : b.nV[row + k];
+            Ru[k] = fma(sc, Yv, fma(b.lam2[N1 + k], ru, Nu));
+            Rv[k] = fma(b.lam2[k], Yu, fma(sc, rv, Nv));
         }
     }
     if (MODE == M_RHS) return;
-    double *dU = (MODE == M_S4) ? b.nU : b.oU;
-    double *dV = (MODE == M_S4) ? b.nV : b.oV;
     double vL = 0, vR = 0, dL = 0, dR = 0;
 #pragma unroll
     for (int k = 0; k < N1; ++k) {
-        dU[row + k] = Ru[k]; dV[row + k] = Rv[k];
+        b.oU[row + k] = Ru[k]; b.oV[row + k] = Rv[k];
         vL += mp.d[0].eL[k] * Rv[k]; vR += mp.d[0].eR[k] * Rv[k];
         dL += mp.d[0].gL[k] * Ru[k]; dR += mp.d[0].gR[k] * Ru[k];
     }
@@ -929,17 +871,16 @@ size_t smem_traces2(int n1, int epb) { return (size_t)epb * (2 * n1 * (n1 + 1)) 
 size_t smem_sep2(int n1, int epb) { return (size_t)(4 * n1 * n1 + epb * 2 * n1 * (n1 + 1)) * sizeof(double); }
 
 template <int N1>
-void launch_stage2(int mode, const ModalParams &mp, const StageBufs &b, double cA, double cY, cudaStream_t s) {
+void launch_stage2(int mode, const ModalParams &mp, const StageBufs &b, double sc, cudaStream_t s) {
     dim3 grid((mp.ne + mp.epb - 1) / mp.epb), block(mp.epb * N1);
     size_t sm = smem_stage2(N1, mp.epb);
     if (mp.parity && mp.split == 1) {
         const dim3 gh((mp.ne + mp.epbh - 1) / mp.epbh), bh(mp.epbh * 2 * N1);
         const size_t smh = smem_stage2(N1, mp.epbh);
         switch (mode) {
-        case M_RHS: k_stage2h<N1, M_RHS><<<gh, bh, smh, s>>>(mp, b, cA, cY); break;
-        case M_S1: k_stage2h<N1, M_S1><<<gh, bh, smh, s>>>(mp, b, cA, cY); break;
-        case M_S23: k_stage2h<N1, M_S23><<<gh, bh, smh, s>>>(mp, b, cA, cY); break;
-        default: k_stage2h<N1, M_S4><<<gh, bh, smh, s>>>(mp, b, cA, cY); break;
+        case M_RHS: k_stage2h<N1, M_RHS><<<gh, bh, smh, s>>>(mp, b, sc); break;
+        case M_S1: k_stage2h<N1, M_S1><<<gh, bh, smh, s>>>(mp, b, sc); break;
+        default: k_stage2h<N1, M_S23><<<gh, bh, smh, s>>>(mp, b, sc); break;
         }
         return;
     }
@@ -947,10 +888,9 @@ void launch_stage2(int mode, const ModalParams &mp, const StageBufs &b, double c
         const dim3 bf(2 * (((mp.epb * N1 + 31) / 32) * 32));
         switch (mode) {
 #define GDG_K2F(m) (mp.alt ? k_stage2f<N1, m, 1> : k_stage2f<N1, m, 0>)
-        case M_RHS: GDG_K2F(M_RHS)<<<grid, bf, sm, s>>>(mp, b, cA, cY); break;
-        case M_S1: GDG_K2F(M_S1)<<<grid, bf, sm, s>>>(mp, b, cA, cY); break;
-        case M_S23: GDG_K2F(M_S23)<<<grid, bf, sm, s>>>(mp, b, cA, cY); break;
-        default: GDG_K2F(M_S4)<<<grid, bf, sm, s>>>(mp, b, cA, cY); break;
+        case M_RHS: GDG_K2F(M_RHS)<<<grid, bf, sm, s>>>(mp, b, sc); break;
+        case M_S1: GDG_K2F(M_S1)<<<grid, bf, sm, s>>>(mp, b, sc); break;
+        default: GDG_K2F(M_S23)<<<grid, bf, sm, s>>>(mp, b, sc); break;
 #undef GDG_K2F
         }
         return;
@@ -958,48 +898,45 @@ void launch_stage2(int mode, const ModalParams &mp, const StageBufs &b, double c
     if (mp.parity) {
         switch (mode) {
 #define GDG_K2P(m) (mp.alt ? k_stage2p<N1, m, 1> : k_stage2p<N1, m, 0>)
-        case M_RHS: GDG_K2P(M_RHS)<<<grid, block, sm, s>>>(mp, b, cA, cY); break;
-        case M_S1: GDG_K2P(M_S1)<<<grid, block, sm, s>>>(mp, b, cA, cY); break;
-        case M_S23: GDG_K2P(M_S23)<<<grid, block, sm, s>>>(mp, b, cA, cY); break;
-        default: GDG_K2P(M_S4)<<<grid, block, sm, s>>>(mp, b, cA, cY); break;
+        case M_RHS: GDG_K2P(M_RHS)<<<grid, block, sm, s>>>(mp, b, sc); break;
+        case M_S1: GDG_K2P(M_S1)<<<grid, block, sm, s>>>(mp, b, sc); break;
+        default: GDG_K2P(M_S23)<<<grid, block, sm, s>>>(mp, b, sc); break;
 #undef GDG_K2P
         }
         return;
     }
     switch (mode) {
-    case M_RHS: k_stage2<N1, M_RHS><<<grid, block, sm, s>>>(mp, b, cA, cY); break;
-    case M_S1: k_stage2<N1, M_S1><<<grid, block, sm, s>>>(mp, b, cA, cY); break;
-    case M_S23: k_stage2<N1, M_S23><<<grid, block, sm, s>>>(mp, b, cA, cY); break;
-    default: k_stage2<N1, M_S4><<<grid, block, sm, s>>>(mp, b, cA, cY); break;
+    case M_RHS: k_stage2<N1, M_RHS><<<grid, block, sm, s>>>(mp, b, sc); break;
+    case M_S1: k_stage2<N1, M_S1><<<grid, block, sm, s>>>(mp, b, sc); break;
+    default: k_stage2<N1, M_S23><<<grid, block, sm, s>>>(mp, b, sc); break;
     }
 }
 
 template <int N1>
-void launch_stage1(int mode, const ModalParams &mp, const StageBufs &b, double cA, double cY, cudaStream_t s) {
+void launch_stage1(int mode, const ModalParams &mp, const StageBufs &b, double sc, cudaStream_t s) {
     dim3 grid((mp.ne + TPB1 - 1) / TPB1), block(TPB1);
     switch (mode) {
-    case M_RHS: k_stage1<N1, M_RHS><<<grid, block, 0, s>>>(mp, b, cA, cY); break;
-    case M_S1: k_stage1<N1, M_S1><<<grid, block, 0, s>>>(mp, b, cA, cY); break;
-    case M_S23: k_stage1<N1, M_S23><<<grid, block, 0, s>>>(mp, b, cA, cY); break;
-    default: k_stage1<N1, M_S4><<<grid, block, 0, s>>>(mp, b, cA, cY); break;
+    case M_RHS: k_stage1<N1, M_RHS><<<grid, block, 0, s>>>(mp, b, sc); break;
+    case M_S1: k_stage1<N1, M_S1><<<grid, block, 0, s>>>(mp, b, sc); break;
+    default: k_stage1<N1, M_S23><<<grid, block, 0, s>>>(mp, b, sc); break;
     }
 }
 
-void launch_stage_raw(const gdg_ctx *ctx, int mode, const StageBufs &b, double cA, double cY, cudaStream_t s) {
+void launch_stage_raw(const gdg_ctx *ctx, int mode, const StageBufs &b, double sc, cudaStream_t s) {
     const int n1 = ctx->n1;
     if (ctx->dim == 3) {
-        gdg3_stage(ctx->mp, n1, mode, b, cA, cY, s);
+        gdg3_stage(ctx->mp, n1, mode, b, sc, s);
         return;
     }
     if (ctx->dim == 2) {
         switch (n1) {
-#define X(n) case n: launch_stage2<n>(mode, ctx->mp, b, cA, cY, s); break;
+#define X(n) case n: launch_stage2<n>(mode, ctx->mp, b, sc, s); break;
             GDG_N1_CASES(X)
 #undef X
         }
     } else {
         switch (n1) {
-#define X(n) case n: launch_stage1<n>(mode, ctx->mp, b, cA, cY, s); break;
+#define X(n) case n: launch_stage1<n>(mode, ctx->mp, b, sc, s); break;
             GDG_N1_CASES(X)
 #undef X
         }
@@ -1067,8 +1004,8 @@ void launch_sep_raw(const gdg_ctx *ctx, const double *in0, const double *in1, do
     }
 }
 
-void launch_stage(gdg_ctx *ctx, int mode, const StageBufs &b, double cA, double cY, cudaStream_t s) {
-    GDG_PROF(ctx, GDG_K_STAGE, s, launch_stage_raw(ctx, mode, b, cA, cY, s));
+void launch_stage(gdg_ctx *ctx, int mode, const StageBufs &b, double sc, cudaStream_t s) {
+    GDG_PROF(ctx, GDG_K_STAGE, s, launch_stage_raw(ctx, mode, b, sc, s));
 }
 void launch_traces(gdg_ctx *ctx, const double *yU, const double *yV, double *tr, cudaStream_t s) {
     GDG_PROF(ctx, GDG_K_TRACES, s, launch_traces_raw(ctx, yU, yV, tr, s));
@@ -1079,7 +1016,7 @@ void launch_sep(gdg_ctx *ctx, const double *in0, const double *in1, double *out0
 }
 
 double *buf(gdg_ctx *ctx, int i) { return ctx->d_state + (size_t)i * ctx->ndof; }
-enum { B_NU = 0, B_NV, B_AU, B_AV, B_XU, B_XV, B_YU, B_YV, B_KU, B_KV, B_COUNT };
+enum { B_NU = 0, B_NV, B_XU, B_XV, B_YU, B_YV, B_KU, B_KV, B_COUNT };
 
 // The persistent step needs every CTA of its grid resident at once.  Its
 // elements per block: the per-stage kernels' choice if that grid fits,
@@ -1132,11 +1069,11 @@ template <int N1>
 void launch_persist_n(gdg_ctx *ctx, double dt, int nsteps, cudaStream_t s) {
     const ModalParams &mp = ctx->mp;
     const dim3 grid((mp.ne + mp.epbp - 1) / mp.epbp), block(mp.epbp * N1);
-    const double *lam2 = ctx->d_lam2;
+    const double *lams = ctx->d_lams;
     double *nU = buf(ctx, B_NU), *nV = buf(ctx, B_NV), *tr0 = ctx->d_tr, *tr1 = ctx->d_tr + ctx->tr_len;
     unsigned *sync = ctx->d_sync;
     unsigned long long lim = ctx->wait_limit_ns;
-    void *args[] = {(void *)&mp, (void *)&lam2, (void *)&nU, (void *)&nV, (void *)&tr0, (void *)&tr1,
+    void *args[] = {(void *)&mp, (void *)&lams, (void *)&nU, (void *)&nV, (void *)&tr0, (void *)&tr1,
                     (void *)&dt, (void *)&nsteps, (void *)&sync, (void *)&lim};
     cudaLaunchCooperativeKernel(mp.alt ? (const void *)k_step2r<N1, 1> : (const void *)k_step2r<N1, 0>, grid, block,
                                 args, smem_stage2(N1, mp.epbp), s);
@@ -1185,27 +1122,21 @@ int set_smem_limits() {
     cudaFuncSetAttribute(k_stage2<n, M_RHS>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage2<n, M_S1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);   \
     cudaFuncSetAttribute(k_stage2<n, M_S23>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
-    cudaFuncSetAttribute(k_stage2<n, M_S4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);   \
     cudaFuncSetAttribute(k_stage2p<n, M_RHS, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
     cudaFuncSetAttribute(k_stage2p<n, M_S1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage2p<n, M_S23, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
-    cudaFuncSetAttribute(k_stage2p<n, M_S4, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage2p<n, M_RHS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
     cudaFuncSetAttribute(k_stage2p<n, M_S1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage2p<n, M_S23, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
-    cudaFuncSetAttribute(k_stage2p<n, M_S4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage2h<n, M_RHS>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
     cudaFuncSetAttribute(k_stage2h<n, M_S1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage2h<n, M_S23>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
-    cudaFuncSetAttribute(k_stage2h<n, M_S4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage2f<n, M_RHS, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
     cudaFuncSetAttribute(k_stage2f<n, M_S1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage2f<n, M_S23, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
-    cudaFuncSetAttribute(k_stage2f<n, M_S4, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage2f<n, M_RHS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
     cudaFuncSetAttribute(k_stage2f<n, M_S1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage2f<n, M_S23, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
-    cudaFuncSetAttribute(k_stage2f<n, M_S4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_traces2<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);        \
     cudaFuncSetAttribute(k_sep2<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     GDG_N1_CASES(X)
@@ -1249,26 +1180,37 @@ int choose_epb(int ne, int n1, int sms, int tpe) {
     return best;
 }
 
-// one RK4 step on the internal modal state (y_n in B_N*, traces of y_n in tr0)
-void enqueue_rk4_step(gdg_ctx *ctx, double dt, cudaStream_t s) {
+// the tables of the four RK stages for the step size dt: d_lam2 times dt/4,
+// dt/3, dt/2, dt (the context keeps them until dt changes)
+__global__ void k_stage_tables(int n, const double *lam2, double dt, double *lams) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < RK_STAGES * n) lams[i] = lam2[i % n] * (dt / (RK_STAGES - i / n));
+}
+
+void stage_tables(gdg_ctx *ctx, double dt, cudaStream_t s) {
+    if (ctx->lams_dt == dt) return;
+    const int n = ctx->lam_len;
+    k_stage_tables<<<(RK_STAGES * n + 255) / 256, 256, 0, s>>>(n, ctx->d_lam2, dt, ctx->d_lams);
+    ctx->lams_dt = dt;
+}
+
+// stage st (0..3) of an RK4 step on the internal modal state (y_n in B_N*,
+// traces of y_n in tr0): the inputs are y_n, X, Y, X, the outputs X, Y, X, y_n
+void enqueue_rk4_stage(gdg_ctx *ctx, int st, double dt, cudaStream_t s) {
     double *tr0 = ctx->d_tr, *tr1 = ctx->d_tr + ctx->tr_len;
-    const double *lam2 = ctx->d_lam2;
+    const int in = st == 0 ? B_NU : st == 2 ? B_YU : B_XU, out = st == 3 ? B_NU : st == 1 ? B_YU : B_XU;
     StageBufs b{};
     b.nU = buf(ctx, B_NU); b.nV = buf(ctx, B_NV);
-    b.aU = buf(ctx, B_AU); b.aV = buf(ctx, B_AV);
-    b.lam2 = lam2;
-    // stage 1: Y1 = y_n -> acc = dt/6 k1, X = y_n + dt/2 k1
-    b.yU = b.nU; b.yV = b.nV; b.oU = buf(ctx, B_XU); b.oV = buf(ctx, B_XV); b.trin = tr0; b.trout = tr1;
-    launch_stage(ctx, M_S1, b, dt / 6.0, 0.5 * dt, s);
-    // stage 2: k2 = f(X) -> acc += dt/3 k2, Y = y_n + dt/2 k2
-    b.yU = buf(ctx, B_XU); b.yV = buf(ctx, B_XV); b.oU = buf(ctx, B_YU); b.oV = buf(ctx, B_YV); b.trin = tr1; b.trout = tr0;
-    launch_stage(ctx, M_S23, b, dt / 3.0, 0.5 * dt, s);
-    // stage 3: k3 = f(Y) -> acc += dt/3 k3, X = y_n + dt k3
-    b.yU = buf(ctx, B_YU); b.yV = buf(ctx, B_YV); b.oU = buf(ctx, B_XU); b.oV = buf(ctx, B_XV); b.trin = tr0; b.trout = tr1;
-    launch_stage(ctx, M_S23, b, dt / 3.0, dt, s);
-    // stage 4: k4 = f(X) -> y_n += acc + dt/6 k4 (traces of y_{n+1} to tr0)
-    b.yU = buf(ctx, B_XU); b.yV = buf(ctx, B_XV); b.oU = nullptr; b.oV = nullptr; b.trin = tr1; b.trout = tr0;
-    launch_stage(ctx, M_S4, b, dt / 6.0, 0.0, s);
+    b.yU = buf(ctx, in); b.yV = buf(ctx, in + 1);
+    b.oU = buf(ctx, out); b.oV = buf(ctx, out + 1);
+    b.trin = st & 1 ? tr1 : tr0;
+    b.trout = st & 1 ? tr0 : tr1;
+    b.lam2 = ctx->d_lams + (size_t)st * ctx->lam_len;
+    launch_stage(ctx, st == 0 ? M_S1 : M_S23, b, rk_factor(st, dt), s);
+}
+
+void enqueue_rk4_step(gdg_ctx *ctx, double dt, cudaStream_t s) {
+    for (int st = 0; st < RK_STAGES; ++st) enqueue_rk4_stage(ctx, st, dt, s);
 }
 
 // ---------------------------------------------- nodal-state route ------
@@ -1280,21 +1222,13 @@ void enqueue_rk4_step(gdg_ctx *ctx, double dt, cudaStream_t s) {
 // transforms more per stage; it exists to measure the two routes against
 // each other.
 
-// RK4 combination on nodal vectors (the modal route's coefficients: the
-// accumulator holds k1 + 2 k2 + 2 k3, stage 4 forms y_n + cA (acc + k4))
-__global__ void k_rk_nodal(size_t n, int mode, double *nU, double *nV, const double *kU, const double *kV,
-                           double *aU, double *aV, double *yU, double *yV, double cA, double cY) {
+// RK4 combination on nodal vectors in the nested form of the modal route:
+// stage output y_n + sc k (the last one into y_n)
+__global__ void k_rk_nodal(size_t n, const double *nU, const double *nV, const double *kU, const double *kV, double *oU,
+                           double *oV, double sc) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const double ku = kU[i], kv = kV[i];
-        if (mode == M_S1) {
-            aU[i] = ku; aV[i] = kv;
-            yU[i] = fma(cY, ku, nU[i]); yV[i] = fma(cY, kv, nV[i]);
-        } else if (mode == M_S23) {
-            aU[i] = fma(2.0, ku, aU[i]); aV[i] = fma(2.0, kv, aV[i]);
-            yU[i] = fma(cY, ku, nU[i]); yV[i] = fma(cY, kv, nV[i]);
-        } else {
-            nU[i] = fma(cA, aU[i] + ku, nU[i]); nV[i] = fma(cA, aV[i] + kv, nV[i]);
-        }
+        oU[i] = fma(sc, kU[i], nU[i]);
+        oV[i] = fma(sc, kV[i], nV[i]);
     }
 }
 
@@ -1304,9 +1238,7 @@ void enqueue_rk4_step_nodal(gdg_ctx *ctx, double *u, double *v, double dt, cudaS
     const size_t n = (size_t)ctx->ndof;
     const int threads = 256, blocks = (int)std::min<size_t>((n + threads - 1) / threads, 4096);
     double *yU = buf(ctx, B_YU), *yV = buf(ctx, B_YV), *kU = buf(ctx, B_NU), *kV = buf(ctx, B_NV);
-    const double cY[4] = {0.5 * dt, 0.5 * dt, dt, 0.0};
-    const int mode[4] = {M_S1, M_S23, M_S23, M_S4};
-    for (int st = 0; st < 4; ++st) {
+    for (int st = 0; st < RK_STAGES; ++st) {
         const double *inU = st == 0 ? u : yU, *inV = st == 0 ? v : yV;
         launch_sep(ctx, inU, inV, buf(ctx, B_XU), buf(ctx, B_XV), T_P, nullptr, -1, s);
         launch_traces(ctx, buf(ctx, B_XU), buf(ctx, B_XV), ctx->d_tr, s);
@@ -1314,10 +1246,10 @@ void enqueue_rk4_step_nodal(gdg_ctx *ctx, double *u, double *v, double dt, cudaS
         b.yU = buf(ctx, B_XU); b.yV = buf(ctx, B_XV);
         b.oU = buf(ctx, B_KU); b.oV = buf(ctx, B_KV);
         b.trin = ctx->d_tr; b.lam2 = ctx->d_lam2;
-        launch_stage(ctx, M_RHS, b, 0.0, 0.0, s);
+        launch_stage(ctx, M_RHS, b, 0.0, s);
         launch_sep(ctx, buf(ctx, B_KU), buf(ctx, B_KV), kU, kV, T_PSI, nullptr, -1, s);
-        k_rk_nodal<<<blocks, threads, 0, s>>>(n, mode[st], u, v, kU, kV, buf(ctx, B_AU), buf(ctx, B_AV), yU, yV,
-                                              dt / 6.0, cY[st]);
+        const bool last = st + 1 == RK_STAGES;
+        k_rk_nodal<<<blocks, threads, 0, s>>>(n, u, v, kU, kV, last ? u : yU, last ? v : yV, rk_factor(st, dt));
     }
 }
 
@@ -1404,23 +1336,12 @@ int halo_exchange(gdg_ctx *ctx, double *T, cudaStream_t s) {
 // traces of y_{n+1}: the next gdg_step call recomputes them)
 int rk4_step_halo(gdg_ctx *ctx, double dt, bool last, cudaStream_t s) {
     double *tr0 = ctx->d_tr, *tr1 = ctx->d_tr + ctx->tr_len;
-    StageBufs b{};
-    b.nU = buf(ctx, B_NU); b.nV = buf(ctx, B_NV);
-    b.aU = buf(ctx, B_AU); b.aV = buf(ctx, B_AV);
-    b.lam2 = ctx->d_lam2;
-    int st;
-    b.yU = b.nU; b.yV = b.nV; b.oU = buf(ctx, B_XU); b.oV = buf(ctx, B_XV); b.trin = tr0; b.trout = tr1;
-    launch_stage(ctx, M_S1, b, dt / 6.0, 0.5 * dt, s);
-    if ((st = halo_exchange(ctx, tr1, s))) return st;
-    b.yU = buf(ctx, B_XU); b.yV = buf(ctx, B_XV); b.oU = buf(ctx, B_YU); b.oV = buf(ctx, B_YV); b.trin = tr1; b.trout = tr0;
-    launch_stage(ctx, M_S23, b, dt / 3.0, 0.5 * dt, s);
-    if ((st = halo_exchange(ctx, tr0, s))) return st;
-    b.yU = buf(ctx, B_YU); b.yV = buf(ctx, B_YV); b.oU = buf(ctx, B_XU); b.oV = buf(ctx, B_XV); b.trin = tr0; b.trout = tr1;
-    launch_stage(ctx, M_S23, b, dt / 3.0, dt, s);
-    if ((st = halo_exchange(ctx, tr1, s))) return st;
-    b.yU = buf(ctx, B_XU); b.yV = buf(ctx, B_XV); b.oU = nullptr; b.oV = nullptr; b.trin = tr1; b.trout = tr0;
-    launch_stage(ctx, M_S4, b, dt / 6.0, 0.0, s);
-    return last ? GDG_OK : halo_exchange(ctx, tr0, s);
+    for (int st = 0; st < RK_STAGES; ++st) {
+        enqueue_rk4_stage(ctx, st, dt, s);
+        if (last && st + 1 == RK_STAGES) break;
+        if (const int rc = halo_exchange(ctx, st & 1 ? tr0 : tr1, s)) return rc;
+    }
+    return GDG_OK;
 }
 
 }  // namespace
@@ -1567,8 +1488,10 @@ int gdg_const_setup(gdg_ctx *ctx) {
     const long long ghost = (mp.halo_lo || mp.halo_hi) ? (long long)ctx->nx * 8 * n1 : 0;
     ctx->tr_len += 2 * ghost;
     ctx->red_len = 1024;
+    ctx->lam_len = (int)l2.size();
     int st;
-    if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&ctx->d_mats, tables.size() * sizeof(double)), "alloc")) ||
+    if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&ctx->d_lams, RK_STAGES * l2.size() * sizeof(double)), "alloc")) ||
+        (st = gdg_cuda_check(ctx, cudaMalloc((void **)&ctx->d_mats, tables.size() * sizeof(double)), "alloc")) ||
         (st = gdg_cuda_check(ctx, cudaMalloc((void **)&ctx->d_lam2, l2.size() * sizeof(double)), "alloc")) ||
         (st = gdg_cuda_check(ctx, cudaMalloc((void **)&ctx->d_state, (size_t)B_COUNT * ctx->ndof * sizeof(double)), "alloc")) ||
         (st = gdg_cuda_check(ctx, cudaMalloc((void **)&ctx->d_tr_alloc, (size_t)2 * ctx->tr_len * sizeof(double)), "alloc")) ||
@@ -1598,6 +1521,8 @@ void gdg_const_free(gdg_ctx *ctx) {
     ctx->graph.exec = nullptr;
     cudaFree(ctx->d_mats);
     cudaFree(ctx->d_lam2);
+    cudaFree(ctx->d_lams);
+    ctx->d_lams = nullptr;
     cudaFree(ctx->d_state);
     cudaFree(ctx->d_tr_alloc);
     cudaFree(ctx->d_red);
@@ -1622,7 +1547,7 @@ int gdg_const_rhs(gdg_ctx *ctx, const double *u, const double *v, double *du, do
     b.yU = buf(ctx, B_XU); b.yV = buf(ctx, B_XV);
     b.oU = buf(ctx, B_KU); b.oV = buf(ctx, B_KV);
     b.trin = ctx->d_tr; b.lam2 = ctx->d_lam2;
-    launch_stage(ctx, M_RHS, b, 0.0, 0.0, s);
+    launch_stage(ctx, M_RHS, b, 0.0, s);
     launch_sep(ctx, buf(ctx, B_KU), buf(ctx, B_KV), du, dv, T_PSI, nullptr, -1, s);
     return gdg_cuda_check(ctx, cudaGetLastError(), "gdg_rhs launch");
 }
@@ -1648,28 +1573,20 @@ int tune_stage_kernel(gdg_ctx *ctx, double dt, cudaStream_t s, const double *u, 
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    StageBufs b{};
-    b.nU = buf(ctx, B_NU); b.nV = buf(ctx, B_NV);
-    b.aU = buf(ctx, B_AU); b.aV = buf(ctx, B_AV);
-    b.lam2 = ctx->d_lam2;
-    b.yU = b.nU; b.yV = b.nV; b.oU = buf(ctx, B_XU); b.oV = buf(ctx, B_XV);
-    b.trin = ctx->d_tr; b.trout = ctx->d_tr + ctx->tr_len;
-    // best of 5 repetitions of 4 launches each (stage-1 and stage-2/3 kinds
-    // alternately; these write only X, the accumulator and the second trace
-    // buffer, which the step's first stage overwrites); another variant must
-    // beat the one-line kernel by 1 % to replace it
+    // best of 5 repetitions of 3 launches each (stages 1 to 3; these write only
+    // X, Y and the trace buffers, and the traces of y_n are rebuilt below);
+    // another variant must beat the one-line kernel by 1 % to replace it
     float best[4] = {1e30f, 1e30f, 1e30f, 1e30f};
     for (int split = 0; split < 3; ++split) {
         mp.split = split;
         for (int rep = 0; rep < 5; ++rep) {
             float ms = 0.f;
             cudaEventRecord(e0, s);
-            for (int i = 0; i < 4; ++i)
-                launch_stage_raw(ctx, (i & 1) ? M_S23 : M_S1, b, (i & 1) ? dt / 3.0 : dt / 6.0, 0.5 * dt, s);
+            for (int i = 0; i < 3; ++i) enqueue_rk4_stage(ctx, i, dt, s);
             cudaEventRecord(e1, s);
             cudaEventSynchronize(e1);
             cudaEventElapsedTime(&ms, e0, e1);
-            best[split] = std::min(best[split], ms);
+            best[split] = std::min(best[split], ms * (4.0f / 3.0f));
         }
     }
     if (persist_fits(ctx)) {   // one step = 4 stages per trial launch
@@ -1684,9 +1601,9 @@ int tune_stage_kernel(gdg_ctx *ctx, double dt, cudaStream_t s, const double *u, 
             best[3] = std::min(best[3], ms);
         }
         if (persist_failed(ctx, s)) best[3] = 1e30f;
-        launch_sep(ctx, u, v, buf(ctx, B_NU), buf(ctx, B_NV), T_P, nullptr, -1, s);
-        launch_traces(ctx, buf(ctx, B_NU), buf(ctx, B_NV), ctx->d_tr, s);
     }
+    launch_sep(ctx, u, v, buf(ctx, B_NU), buf(ctx, B_NV), T_P, nullptr, -1, s);
+    launch_traces(ctx, buf(ctx, B_NU), buf(ctx, B_NV), ctx->d_tr, s);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     int pick = 0;
@@ -1727,6 +1644,7 @@ extern "C" int gdg_get_stage_variant(const gdg_ctx *ctx, int *variant) {
 int gdg_const_step(gdg_ctx *ctx, double *u, double *v, double dt, int nsteps, cudaStream_t s) {
     int st;
     if (ctx->pb.route == GDG_ROUTE_NODAL) return step_nodal(ctx, u, v, dt, nsteps, s);
+    stage_tables(ctx, dt, s);
     launch_sep(ctx, u, v, buf(ctx, B_NU), buf(ctx, B_NV), T_P, nullptr, -1, s);
     launch_traces(ctx, buf(ctx, B_NU), buf(ctx, B_NV), ctx->d_tr, s);
     if ((st = gdg_cuda_check(ctx, cudaGetLastError(), "gdg_step prologue"))) return st;
@@ -1803,13 +1721,14 @@ int gdg_const_energy(gdg_ctx *ctx, const double *u, const double *v, double *E, 
 
 StepBuffers gdg_const_buffers(gdg_ctx *ctx) {
     StepBuffers b;
-    b.nU = buf(ctx, B_NU); b.nV = buf(ctx, B_NV); b.aU = buf(ctx, B_AU); b.aV = buf(ctx, B_AV);
+    b.nU = buf(ctx, B_NU); b.nV = buf(ctx, B_NV); b.aU = b.aV = nullptr;
     b.xU = buf(ctx, B_XU); b.xV = buf(ctx, B_XV); b.yU = buf(ctx, B_YU); b.yV = buf(ctx, B_YV);
     b.tr0 = ctx->d_tr; b.tr1 = ctx->d_tr + ctx->tr_len;
     return b;
 }
 
-int gdg_const_enter(gdg_ctx *ctx, const double *u, const double *v, cudaStream_t s) {
+int gdg_const_enter(gdg_ctx *ctx, const double *u, const double *v, double dt, cudaStream_t s) {
+    stage_tables(ctx, dt, s);
     launch_sep(ctx, u, v, buf(ctx, B_NU), buf(ctx, B_NV), T_P, nullptr, -1, s);
     launch_traces(ctx, buf(ctx, B_NU), buf(ctx, B_NV), ctx->d_tr, s);
     return gdg_cuda_check(ctx, cudaGetLastError(), "enter");
@@ -2131,7 +2050,7 @@ extern "C" int gdg_rhs_static(const gdg_problem *pb, const double *u, const doub
     launch_traces(&c, Yu, Yv, tr, s);
     StageBufs b{};
     b.yU = Yu; b.yV = Yv; b.oU = Ku; b.oV = Kv; b.trin = tr; b.lam2 = c.d_lam2;
-    launch_stage(&c, M_RHS, b, 0.0, 0.0, s);
+    launch_stage(&c, M_RHS, b, 0.0, s);
     launch_sep(&c, Ku, Kv, du, dv, T_PSI, nullptr, -1, s);
     c.d_mats = c.d_lam2 = nullptr;   // not owned
     return cudaGetLastError() == cudaSuccess ? GDG_OK : GDG_ECUDA;

@@ -79,7 +79,7 @@ __host__ __device__ constexpr int epb3c() { return MAXB3 / (N1 * N1) > 1 ? MAXB3
 
 template <int N1, int MODE>
 __global__ void __launch_bounds__(MAXB3)
-k_stage3(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, double cY) {
+k_stage3(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) {
     constexpr int NT = N1 * N1, NA = N1 * N1 * N1;
     extern __shared__ double smem[];
     const int epb = blockDim.x / NT;
@@ -129,34 +129,19 @@ k_stage3(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, d
             const double Yu = b.yU[row + k], Yv = b.yV[row + k];
             const double ru = mp.d[0].gL[k] * Gxm + mp.d[0].gR[k] * Gxp + gLy * F[4 * NT + ty] +
                               gRy * F[6 * NT + ty] + gLz * F[8 * NT + tz] + gRz * F[10 * NT + tz];
-            const double rv = L0[k] * Yu + mp.d[0].eL[k] * Qxm + mp.d[0].eR[k] * Qxp + eLy * F[5 * NT + ty] +
+            const double rv = mp.d[0].eL[k] * Qxm + mp.d[0].eR[k] * Qxp + eLy * F[5 * NT + ty] +
                               eRy * F[7 * NT + ty] + eLz * F[9 * NT + tz] + eRz * F[11 * NT + tz];
-            const double ku = Yv + L1[k] * ru;
-            const double kv = rv;
             if (MODE == M_RHS) {
-                b.oU[row + k] = ku;
-                b.oV[row + k] = kv;
-            } else if (MODE == M_S1) {
-                b.aU[row + k] = cA * ku;
-                b.aV[row + k] = cA * kv;
-                Ru[k] = Yu + cY * ku;
-                Rv[k] = Yv + cY * kv;
-            } else if (MODE == M_S23) {
-                b.aU[row + k] += cA * ku;
-                b.aV[row + k] += cA * kv;
-                Ru[k] = b.nU[row + k] + cY * ku;
-                Rv[k] = b.nV[row + k] + cY * kv;
-            } else {
-                Ru[k] = b.nU[row + k] + b.aU[row + k] + cA * ku;
-                Rv[k] = b.nV[row + k] + b.aV[row + k] + cA * kv;
+                Ru[k] = Yv + L1[k] * ru;
+                Rv[k] = L0[k] * Yu + rv;
+            } else {   // L0, L1 carry sc
+                const double Nu = MODE == M_S1 ? Yu : b.nU[row + k], Nv = MODE == M_S1 ? Yv : b.nV[row + k];
+                Ru[k] = fma(sc, Yv, fma(L1[k], ru, Nu));
+                Rv[k] = fma(L0[k], Yu, fma(sc, rv, Nv));
             }
         }
-        if (MODE != M_RHS) {
-            double *dU = (MODE == M_S4) ? b.nU : b.oU;
-            double *dV = (MODE == M_S4) ? b.nV : b.oV;
 #pragma unroll
-            for (int k = 0; k < N1; ++k) { dU[row + k] = Ru[k]; dV[row + k] = Rv[k]; }
-        }
+        for (int k = 0; k < N1; ++k) { b.oU[row + k] = Ru[k]; b.oV[row + k] = Rv[k]; }
     }
     if (MODE == M_RHS) return;   // uniform across the block
 
@@ -182,9 +167,8 @@ k_stage3(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, d
 }
 
 // The u lifts are folded with the diagonal solve (rows 2-4 of lam2: hgL of
-// each direction over lambda) and RK4 accumulates k1 + 2 k2 + 2 k3 (stages
-// 1-3 ignore cA; stage 4 forms y_n + cA (acc + k4), cA = dt/6), as the 2-D
-// parity kernels do.
+// each direction over lambda) and RK4 runs in nested form with the stage's
+// factor folded into the tables, as in the 2-D parity kernels (stage2p_body).
 // Parity version of k_stage3 (modes ordered even first in every direction:
 // eR = s eL and gR = s gL, s = +1 for the NE = (N1+1)/2 even modes, -1 for
 // the odd ones).  Phase 1 keeps, per direction and transverse mode pair, the
@@ -224,7 +208,7 @@ __device__ __forceinline__ void traces3_yz_p(const ModalParams &mp, const double
 
 template <int N1, int MODE, int ALT>
 __global__ void __launch_bounds__(MAXB3, 3)
-k_stage3p(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, double cY) {
+k_stage3p(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) {
     constexpr int NT = N1 * N1, NA = N1 * N1 * N1, NE = (N1 + 1) / 2;
     constexpr int EPB = epb3c<N1>(), BD = EPB * NT;   // blockDim.x == BD (launch_stage3)
     extern __shared__ double smem[];
@@ -238,7 +222,10 @@ k_stage3p(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, 
     double *F = smem + le * smem3_doubles<N1>();
     double *tU = F + 12 * NT, *tV = tU + NA;
     double *ce = smem + EPB * smem3_doubles<N1>();   // [3][N1]: c^2 eL / 2 of x, y, z
-    if (t < N1) { ce[t] = mp.d[0].ceL[t]; ce[N1 + t] = mp.d[1].ceL[t]; ce[2 * N1 + t] = mp.d[2].ceL[t]; }
+    if (t < 3 * N1) {   // c^2 eL / 2 of x, y, z, times the stage's factor
+        const double v = t < N1 ? mp.d[0].ceL[t] : t < 2 * N1 ? mp.d[1].ceL[t - N1] : mp.d[2].ceL[t - 2 * N1];
+        ce[t] = MODE == M_RHS ? v : sc * v;
+    }
     const int ex = valid ? e % mp.nx : 0, ey = valid ? (e / mp.nx) % mp.ny : 0, ez = valid ? e / (mp.nx * mp.ny) : 0;
 
     if (valid) {   // fluxes of the three face pairs at this thread's transverse mode pair
@@ -274,15 +261,31 @@ k_stage3p(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, 
     // line per thread would stride them by N1).  Entry q = (m3 N1 + m2) N1 +
     // m1 of element le2 finds its line's fluxes in that element's F; each
     // entry's arithmetic is the same sequence of operations in either order.
-    // The stage's arrays do not overlap: with restrict the next entry's loads
-    // may be issued before this entry's stores.
-    const double *__restrict__ pyU = b.yU, *__restrict__ pyV = b.yV;
-    double *__restrict__ paU = b.aU, *__restrict__ paV = b.aV, *__restrict__ pnU = b.nU, *__restrict__ pnV = b.nV;
-    double *__restrict__ poU = b.oU, *__restrict__ poV = b.oV;
+    // An entry's input and y_n are read before its output is stored, and no
+    // other entry reads it: the output may be y_n itself (the last stage).
+    const double *pyU = b.yU, *pyV = b.yV, *pnU = b.nU, *pnV = b.nV;
     const double *__restrict__ lam = b.lam2;
     const size_t base = (size_t)blockIdx.x * EPB * NA;
+    const long long left = ((long long)mp.ne - (long long)blockIdx.x * EPB) * NA;   // entries of the block's elements
+    constexpr int GRP = 3;   // entries whose loads are in flight together
 #pragma unroll
-    for (int s = 0; s < N1; ++s) {
+    for (int s0 = 0; s0 < N1; s0 += GRP) {
+    double Yr[2 * GRP], Nr[2 * GRP];
+#pragma unroll
+    for (int i = 0; i < GRP; ++i) {
+        const bool in = s0 + i < N1 && t + (s0 + i) * BD < left;
+        const size_t g = base + t + (s0 + i) * BD;
+        Yr[i] = in ? pyU[g] : 0.0;
+        Yr[GRP + i] = in ? pyV[g] : 0.0;
+        if (MODE == M_S23) {
+            Nr[i] = in ? pnU[g] : 0.0;
+            Nr[GRP + i] = in ? pnV[g] : 0.0;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < GRP; ++i) {
+        const int s = s0 + i;
+        if (s >= N1) continue;
         const int idx = t + s * BD;
         const int le2 = idx / NA, q = idx - le2 * NA;
         if (blockIdx.x * EPB + le2 >= mp.ne) continue;
@@ -290,7 +293,7 @@ k_stage3p(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, 
         const int m3 = line / N1, m2 = line - m3 * N1;
         double *F2 = smem + le2 * smem3_doubles<N1>();
         const size_t g = base + idx;
-        const double Yu = pyU[g], Yv = pyV[g];
+        const double Yu = Yr[i], Yv = Yr[GRP + i];
         const double xg = F2[(k < NE ? 0 : 1) * NT + line], xq = F2[(k < NE ? 2 : 3) * NT + line];
         const double FGy = F2[(4 + (m2 < NE ? 0 : 1)) * NT + m3 * N1 + k];   // at ty = m3 N1 + m1
         const double FQy = F2[(6 + (m2 < NE ? 0 : 1)) * NT + m3 * N1 + k];
@@ -298,33 +301,20 @@ k_stage3p(const __grid_constant__ ModalParams mp, const StageBufs b, double cA, 
         const double FQz = F2[(10 + (m3 < NE ? 0 : 1)) * NT + m2 * N1 + k];
         // k_u = V + Lambda^+ r_u with the three rank-one lifts folded into
         // rows 2-4 of lam2 (hgL / lambda per direction): three FMAs
-        const double ku = fma(lam[2 * NA + q], xg, fma(lam[3 * NA + q], FGy, fma(lam[4 * NA + q], FGz, Yv)));
-        const double rv = fma(lam[q], Yu, fma(ce[k], xq, fma(ce[N1 + m2], FQy, ce[2 * N1 + m3] * FQz)));
-        const double kv = rv;
-        double Ru, Rv;
         if (MODE == M_RHS) {
-            poU[g] = ku;
-            poV[g] = kv;
+            b.oU[g] = fma(lam[2 * NA + q], xg, fma(lam[3 * NA + q], FGy, fma(lam[4 * NA + q], FGz, Yv)));
+            b.oV[g] = fma(lam[q], Yu, fma(ce[k], xq, fma(ce[N1 + m2], FQy, ce[2 * N1 + m3] * FQz)));
             continue;
-        } else if (MODE == M_S1) {   // accumulator k1 + 2 k2 + 2 k3, scaled by dt/6 at stage 4
-            paU[g] = ku;
-            paV[g] = kv;
-            Ru = fma(cY, ku, Yu);
-            Rv = fma(cY, kv, Yv);
-        } else if (MODE == M_S23) {
-            paU[g] = fma(2.0, ku, paU[g]);
-            paV[g] = fma(2.0, kv, paV[g]);
-            Ru = fma(cY, ku, pnU[g]);
-            Rv = fma(cY, kv, pnV[g]);
-        } else {
-            Ru = fma(cA, paU[g] + ku, pnU[g]);
-            Rv = fma(cA, paV[g] + kv, pnV[g]);
         }
-        if (MODE == M_S4) { pnU[g] = Ru; pnV[g] = Rv; }
-        else { poU[g] = Ru; poV[g] = Rv; }
+        const double Nu = MODE == M_S1 ? Yu : Nr[i], Nv = MODE == M_S1 ? Yv : Nr[GRP + i];
+        const double Ru = fma(sc, Yv, fma(lam[2 * NA + q], xg, fma(lam[3 * NA + q], FGy, fma(lam[4 * NA + q], FGz, Nu))));
+        const double Rv = fma(lam[q], Yu, fma(ce[k], xq, fma(ce[N1 + m2], FQy, fma(ce[2 * N1 + m3], FQz, Nv))));
+        b.oU[g] = Ru;
+        b.oV[g] = Rv;
         double *tU2 = F2 + 12 * NT;
         tU2[q] = Ru;
         tU2[NA + q] = Rv;
+    }
     }
     if (MODE == M_RHS) return;   // uniform across the block
     __syncthreads();
@@ -530,34 +520,32 @@ size_t smem_traces3(int n1) { return (size_t)epb3(n1) * 2 * n1 * n1 * n1 * sizeo
 size_t smem_sep3(int n1) { return (size_t)(6 * n1 * n1 + epb3(n1) * n1 * n1 * n1) * sizeof(double); }
 
 template <int N1>
-void launch_stage3(int mode, const ModalParams &mp, const StageBufs &b, double cA, double cY, cudaStream_t s) {
+void launch_stage3(int mode, const ModalParams &mp, const StageBufs &b, double sc, cudaStream_t s) {
     const int epb = epb3(N1);
     const dim3 grid((mp.ne + epb - 1) / epb), block(epb * N1 * N1);
     const size_t sm = smem_stage3(N1);
     if (mp.parity) {
         switch (mode) {
 #define GDG_K3P(m) (mp.alt ? k_stage3p<N1, m, 1> : k_stage3p<N1, m, 0>)
-        case M_RHS: GDG_K3P(M_RHS)<<<grid, block, sm, s>>>(mp, b, cA, cY); break;
-        case M_S1: GDG_K3P(M_S1)<<<grid, block, sm, s>>>(mp, b, cA, cY); break;
-        case M_S23: GDG_K3P(M_S23)<<<grid, block, sm, s>>>(mp, b, cA, cY); break;
-        default: GDG_K3P(M_S4)<<<grid, block, sm, s>>>(mp, b, cA, cY); break;
+        case M_RHS: GDG_K3P(M_RHS)<<<grid, block, sm, s>>>(mp, b, sc); break;
+        case M_S1: GDG_K3P(M_S1)<<<grid, block, sm, s>>>(mp, b, sc); break;
+        default: GDG_K3P(M_S23)<<<grid, block, sm, s>>>(mp, b, sc); break;
 #undef GDG_K3P
         }
         return;
     }
     switch (mode) {
-    case M_RHS: k_stage3<N1, M_RHS><<<grid, block, sm, s>>>(mp, b, cA, cY); break;
-    case M_S1: k_stage3<N1, M_S1><<<grid, block, sm, s>>>(mp, b, cA, cY); break;
-    case M_S23: k_stage3<N1, M_S23><<<grid, block, sm, s>>>(mp, b, cA, cY); break;
-    default: k_stage3<N1, M_S4><<<grid, block, sm, s>>>(mp, b, cA, cY); break;
+    case M_RHS: k_stage3<N1, M_RHS><<<grid, block, sm, s>>>(mp, b, sc); break;
+    case M_S1: k_stage3<N1, M_S1><<<grid, block, sm, s>>>(mp, b, sc); break;
+    default: k_stage3<N1, M_S23><<<grid, block, sm, s>>>(mp, b, sc); break;
     }
 }
 
 }  // namespace
 
-void gdg3_stage(const ModalParams &mp, int n1, int mode, const StageBufs &b, double cA, double cY, cudaStream_t s) {
+void gdg3_stage(const ModalParams &mp, int n1, int mode, const StageBufs &b, double sc, cudaStream_t s) {
     switch (n1) {
-#define X(n) case n: launch_stage3<n>(mode, mp, b, cA, cY, s); break;
+#define X(n) case n: launch_stage3<n>(mode, mp, b, sc, s); break;
         GDG_N1_CASES3(X)
 #undef X
     }
@@ -600,15 +588,12 @@ void gdg3_set_smem_limits() {
     cudaFuncSetAttribute(k_stage3<n, M_RHS>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
     cudaFuncSetAttribute(k_stage3<n, M_S1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage3<n, M_S23>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
-    cudaFuncSetAttribute(k_stage3<n, M_S4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage3p<n, M_RHS, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
     cudaFuncSetAttribute(k_stage3p<n, M_S1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage3p<n, M_S23, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
-    cudaFuncSetAttribute(k_stage3p<n, M_S4, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage3p<n, M_RHS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
     cudaFuncSetAttribute(k_stage3p<n, M_S1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage3p<n, M_S23, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
-    cudaFuncSetAttribute(k_stage3p<n, M_S4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_traces3<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);       \
     cudaFuncSetAttribute(k_sep3<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     GDG_N1_CASES3(X)

@@ -39,27 +39,31 @@ struct ModalParams {
     int halo_lo, halo_hi; // y sides whose neighbour traces arrive in ghost rows (partitioned mesh)
 };
 
-// RK4 stage modes of the stage kernels
+// RK4 stage modes of the stage kernels.  Element solves (classic RK4):
 enum {
     M_RHS = 0,   // write k = f(Y)
     M_S1 = 1,    // acc = cA k; Y' = Y + cY k         (Y = y_n)
     M_S23 = 2,   // acc += cA k; Y' = y_n + cY k
     M_S4 = 3     // y_n += acc + cA k
 };
+// Modal route (nested form, see stage2p_body): M_RHS; M_S1 (Y = y_n) and M_S23
+// write y_n + sc k(Y), the last stage into y_n itself.
+constexpr int RK_STAGES = 4;
+inline double rk_factor(int stage, double dt) { return dt / (RK_STAGES - stage); }   // stage 0..3: dt/4 .. dt
 
 // Buffers of one modal RK stage launch.
 struct StageBufs {
     const double *yU, *yV;   // stage input (modal)
-    double *nU, *nV;         // y_n
-    double *aU, *aV;         // RK accumulator
-    double *oU, *oV;         // next stage input, or k (M_RHS)
+    const double *nU, *nV;   // y_n
+    double *oU, *oV;         // stage output, or k (M_RHS)
     const double *trin;      // traces of the stage input
-    double *trout;           // traces of the next stage input
-    const double *lam2;      // [2][n1^d] : -c2 * lambda, 1/lambda (0 on mode 0); 2-D: [4][n1^2]
+    double *trout;           // traces of the output
+    const double *lam2;      // [2][n1^d] : -c2 * lambda, 1/lambda (0 on mode 0); 2-D: [4][n1^2], 3-D: [5][n1^3];
+                             // all times sc in the stage modes
 };
 
 // 3-D modal-route launches (gdg_const3.cu), n1 = N+1 in 2..10
-void gdg3_stage(const ModalParams &mp, int n1, int mode, const StageBufs &b, double cA, double cY, cudaStream_t s);
+void gdg3_stage(const ModalParams &mp, int n1, int mode, const StageBufs &b, double sc, cudaStream_t s);
 void gdg3_traces(const ModalParams &mp, int n1, const double *yU, const double *yV, double *tr, cudaStream_t s);
 void gdg3_sep(int n1, int ne, const double *in0, const double *in1, double *out0, double *out1, const double *Bx,
               const double *By, const double *Bz, const double *D, const double *Cx, const double *Cy,
@@ -104,7 +108,10 @@ struct gdg_ctx {
     double *d_mats = nullptr;     // device tables: per direction P = Psi^T M, Psi, Psi^T (n1*n1 each)
     double *d_lam2 = nullptr;     // per mode: -c2*lambda, 1/lambda (0 for mode 0); 2-D also P1, P2
                                   // (the u lifts over lambda, see stage2p_body)
-    double *d_state = nullptr;    // modal work: yn(2 fields), acc(2), YA(2), YB(2), K(2)
+    double *d_lams = nullptr;     // d_lam2 times the factor of each RK stage, for the step size lams_dt
+    double lams_dt = 0.0;
+    int lam_len = 0;              // doubles in d_lam2
+    double *d_state = nullptr;    // modal work: yn(2 fields), YA(2), YB(2), K(2)
     double *d_tr = nullptr;       // two trace buffers (past the lower ghost row when halo sides exist)
     long long tr_len = 0;         // doubles per trace buffer (ghost rows included)
     double *d_tr_alloc = nullptr; // allocation holding d_tr
@@ -169,13 +176,13 @@ int gdg_var_step_stats(gdg_ctx *ctx, gdg_pcg_stats *su, gdg_pcg_stats *sv);
 // Buffers of one problem's RK4 state as used by the stage kernels (the
 // batched launcher drives several problems' stages from one kernel).
 struct StepBuffers {
-    double *nU, *nV, *aU, *aV, *xU, *xV, *yU, *yV;   // y_n, accumulator, two stage inputs
+    double *nU, *nV, *aU, *aV, *xU, *xV, *yU, *yV;   // y_n, accumulator (element solves), two stage inputs
     double *tr0, *tr1;                               // traces of y_n / odd stages, even stages
 };
 StepBuffers gdg_const_buffers(gdg_ctx *ctx);
 StepBuffers gdg_var_buffers(gdg_ctx *ctx);
 // nodal (u, v) -> internal state and its traces; internal state -> nodal
-int gdg_const_enter(gdg_ctx *ctx, const double *u, const double *v, cudaStream_t s);
+int gdg_const_enter(gdg_ctx *ctx, const double *u, const double *v, double dt, cudaStream_t s);
 int gdg_const_leave(gdg_ctx *ctx, double *u, double *v, cudaStream_t s);
 int gdg_var_enter(gdg_ctx *ctx, const double *u, const double *v, cudaStream_t s);
 int gdg_var_leave(gdg_ctx *ctx, double *u, double *v, cudaStream_t s);

@@ -52,6 +52,22 @@ __device__ __forceinline__ void flux2(double vi, double di, double vo, double dO
     q2 = fma(t2, d1, di - dO);
 }
 
+// One modal entry of a stage (see stage2p_body): the new (u, v) from the stage
+// input (Yu, Yv) and y_n (Nu, Nv), or k itself (M_RHS).  L0, P1, P2, cey, xq
+// carry the stage's factor sc unless M_RHS.
+template <int MODE>
+__device__ __forceinline__ void stage_entry(double sc, double L0, double P1, double P2, double cex, double cey,
+                                            double xg, double xq, double FG, double FQ, double Yu, double Yv, double Nu,
+                                            double Nv, double &Ru, double &Rv) {
+    if (MODE == M_RHS) {
+        Ru = fma(P1, xg, fma(P2, FG, Yv));
+        Rv = fma(L0, Yu, fma(cex, xq, cey * FQ));
+    } else {
+        Ru = fma(sc, Yv, fma(P1, xg, fma(P2, FG, Nu)));
+        Rv = fma(L0, Yu, fma(cex, xq, fma(cey, FQ, Nv)));
+    }
+}
+
 // Body of the parity stage kernel for element tile `etile` (blockDim.x / N1
 // elements per block).  Parity version of the generic stage: the GD element is symmetric under r -> 1-r,
 // so every modified-basis vector is even or odd: Psi[N-i][k] = s_k Psi[i][k].
@@ -64,12 +80,18 @@ __device__ __forceinline__ void flux2(double vi, double di, double vo, double dO
 // The u lifts enter only through k_u = V + Lambda^+ r_u, so they are folded
 // with the diagonal solve: P1[l][k] = hgL_x[k] / lambda[l][k] and
 // P2[l][k] = hgL_y[l] / lambda[l][k] (lam2 rows 2 and 3; 0 on the constant
-// mode), two FMAs per entry.  RK4 accumulates k1 + 2 k2 + 2 k3 (stages 1-3
-// ignore cA) and stage 4 forms y_n + cA (acc + k4) with cA = dt/6, the
-// order of the classic formula y_n + dt/6 (k1 + 2 k2 + 2 k3 + k4).
+// mode), two FMAs per entry.
+// RK4 in nested form: the semi-discretisation is linear and autonomous, so one
+// classic RK4 step is the Taylor polynomial of degree 4, and with L y = k(y)
+//   w1 = y + dt/4 L y,  w2 = y + dt/3 L w1,  w3 = y + dt/2 L w2,  y' = y + dt L w3
+// gives it without an accumulator: a stage reads its input and y_n and writes
+// its output, three passes over the state instead of five, and keeps 4 N1
+// doubles of a line instead of 6 N1.  The stage's factor sc = dt/4 .. dt is
+// folded into its copy of the tables (lam2 rows 0, 2, 3) and the fluxes of v,
+// so an entry takes 6 FMAs for both fields (10 operations with k formed first).
 template <int N1, int MODE, int ALT>
-__device__ __forceinline__ void stage2p_body(const ModalParams &mp, const StageBufs &b, double cA, double cY,
-                                             int etile, double *smem) {
+__device__ __forceinline__ void stage2p_body(const ModalParams &mp, const StageBufs &b, double sc, int etile,
+                                             double *smem) {
     constexpr int NE = (N1 + 1) / 2;
     const int epb = blockDim.x / N1;
     const int t = threadIdx.x;
@@ -85,17 +107,15 @@ __device__ __forceinline__ void stage2p_body(const ModalParams &mp, const StageB
 
     // issue every row load of this stage before the barrier so their latency
     // overlaps the flux work (a few warps per SM only at small element counts)
-    double Ru[N1], Rv[N1], Nu[N1], Nv[N1], Au[N1], Av[N1];
+    double Ru[N1], Rv[N1], Nu[N1], Nv[N1];
     if (valid) {
 #pragma unroll
         for (int k = 0; k < N1; ++k) {
             Ru[k] = b.yU[row + k];
             Rv[k] = b.yV[row + k];
-            if (MODE == M_S23 || MODE == M_S4) {
+            if (MODE == M_S23) {
                 Nu[k] = b.nU[row + k];
                 Nv[k] = b.nV[row + k];
-                Au[k] = b.aU[row + k];
-                Av[k] = b.aV[row + k];
             }
         }
     }
@@ -146,41 +166,19 @@ __device__ __forceinline__ void stage2p_body(const ModalParams &mp, const StageB
     if (valid) {
         const double *L0 = b.lam2 + l * N1;
         const double *P1 = b.lam2 + 2 * N1 * N1 + l * N1, *P2 = b.lam2 + 3 * N1 * N1 + l * N1;
-        const double cey = mp.d[1].ceL[l];
+        const double cey = MODE == M_RHS ? mp.d[1].ceL[l] : sc * mp.d[1].ceL[l];
+        if (MODE != M_RHS) { QA *= sc; QB *= sc; }
         const double *FG = fy + (l < NE ? 0 : N1);
         const double *FQ = fy + (l < NE ? 2 * N1 : 3 * N1);
 #pragma unroll
         for (int k = 0; k < N1; ++k) {
             const double Yu = Ru[k], Yv = Rv[k];
             const double xg = k < NE ? GA : GB, xq = k < NE ? QA : QB;
-            // k_u = V + Lambda^+ r_u with the rank-one lifts folded into P1, P2
-            const double ku = fma(P1[k], xg, fma(P2[k], FG[k], Yv));
-            const double rv = fma(L0[k], Yu, fma(mp.d[0].ceL[k], xq, cey * FQ[k]));
-            const double kv = rv;
-            if (MODE == M_RHS) {
-                b.oU[row + k] = ku;
-                b.oV[row + k] = kv;
-            } else if (MODE == M_S1) {   // accumulator k1 + 2 k2 + 2 k3, scaled by dt/6 at stage 4
-                b.aU[row + k] = ku;
-                b.aV[row + k] = kv;
-                Ru[k] = fma(cY, ku, Yu);
-                Rv[k] = fma(cY, kv, Yv);
-            } else if (MODE == M_S23) {
-                b.aU[row + k] = fma(2.0, ku, Au[k]);
-                b.aV[row + k] = fma(2.0, kv, Av[k]);
-                Ru[k] = fma(cY, ku, Nu[k]);
-                Rv[k] = fma(cY, kv, Nv[k]);
-            } else {
-                Ru[k] = fma(cA, Au[k] + ku, Nu[k]);
-                Rv[k] = fma(cA, Av[k] + kv, Nv[k]);
-            }
+            stage_entry<MODE>(sc, L0[k], P1[k], P2[k], mp.d[0].ceL[k], cey, xg, xq, FG[k], FQ[k], Yu, Yv,
+                              MODE == M_S1 ? Yu : Nu[k], MODE == M_S1 ? Yv : Nv[k], Ru[k], Rv[k]);
         }
-        if (MODE != M_RHS) {
-            double *dU = (MODE == M_S4) ? b.nU : b.oU;
-            double *dV = (MODE == M_S4) ? b.nV : b.oV;
 #pragma unroll
-            for (int k = 0; k < N1; ++k) { dU[row + k] = Ru[k]; dV[row + k] = Rv[k]; }
-        }
+        for (int k = 0; k < N1; ++k) { b.oU[row + k] = Ru[k]; b.oV[row + k] = Rv[k]; }
     }
     if (MODE == M_RHS) return;
 
@@ -228,12 +226,12 @@ __device__ __forceinline__ unsigned pair_mask() {
     return lanes >= 32 ? 0xffffffffu : ((1u << lanes) - 1u);
 }
 
-// LEAN: y_n and the RK accumulator are read where the update uses them
-// instead of with the stage input (same operations and results; 40 fewer
-// live registers at S23 / S4, for kernels held to a low register count).
+// LEAN: y_n is read where the update uses it instead of with the stage input
+// (same operations and results; 20 fewer live registers, for kernels held to a
+// low register count).
 template <int N1, int MODE, bool LEAN = false>
-__device__ __forceinline__ void stage2h_body(const ModalParams &mp, const StageBufs &b, double cA, double cY,
-                                             int etile, double *smem) {
+__device__ __forceinline__ void stage2h_body(const ModalParams &mp, const StageBufs &b, double sc, int etile,
+                                             double *smem) {
     constexpr int NE = (N1 + 1) / 2;   // even modes; the odd half has N1 - NE <= NE entries
     const int epb = blockDim.x / (2 * N1);
     const int t = threadIdx.x;
@@ -250,18 +248,16 @@ __device__ __forceinline__ void stage2h_body(const ModalParams &mp, const StageB
     const double b2 = mp.beta2, t2 = mp.tau2;
     const size_t row = ((size_t)(valid ? e : 0) * N1 + l) * N1 + k0;
 
-    double Ru[NE], Rv[NE], Nu[NE], Nv[NE], Au[NE], Av[NE];
+    double Ru[NE], Rv[NE], Nu[NE], Nv[NE];
     if (valid) {
 #pragma unroll
         for (int kk = 0; kk < NE; ++kk) {
             if (kk < nk) {
                 Ru[kk] = b.yU[row + kk];
                 Rv[kk] = b.yV[row + kk];
-                if (!LEAN && (MODE == M_S23 || MODE == M_S4)) {
+                if (!LEAN && MODE == M_S23) {
                     Nu[kk] = b.nU[row + kk];
                     Nv[kk] = b.nV[row + kk];
-                    Au[kk] = b.aU[row + kk];
-                    Av[kk] = b.aV[row + kk];
                 }
             }
         }
@@ -324,7 +320,8 @@ __device__ __forceinline__ void stage2h_body(const ModalParams &mp, const StageB
     if (valid) {
         const double *L0 = b.lam2 + l * N1 + k0;
         const double *P1 = b.lam2 + 2 * N1 * N1 + l * N1 + k0, *P2 = b.lam2 + 3 * N1 * N1 + l * N1 + k0;
-        const double cey = mp.d[1].ceL[l];
+        const double cey = MODE == M_RHS ? mp.d[1].ceL[l] : sc * mp.d[1].ceL[l];
+        const double sxq = MODE == M_RHS ? xq : xq * sc;
         const double *FG = fy + (l < NE ? 0 : N1) + k0;
         const double *FQ = fy + (l < NE ? 2 * N1 : 3 * N1) + k0;
         const double *cex = mp.d[0].ceL + k0;
@@ -332,42 +329,17 @@ __device__ __forceinline__ void stage2h_body(const ModalParams &mp, const StageB
         for (int kk = 0; kk < NE; ++kk) {
             if (kk < nk) {
                 const double Yu = Ru[kk], Yv = Rv[kk];
-                const double ku = fma(P1[kk], xg, fma(P2[kk], FG[kk], Yv));
-                const double rv = fma(L0[kk], Yu, fma(cex[kk], xq, cey * FQ[kk]));
-                const double kv = rv;
-                const size_t o = row + kk;
-                if (LEAN && (MODE == M_S23 || MODE == M_S4)) {
-                    Nu[kk] = b.nU[o];
-                    Nv[kk] = b.nV[o];
-                    Au[kk] = b.aU[o];
-                    Av[kk] = b.aV[o];
+                if (LEAN && MODE == M_S23) {
+                    Nu[kk] = b.nU[row + kk];
+                    Nv[kk] = b.nV[row + kk];
                 }
-                if (MODE == M_RHS) {
-                    b.oU[o] = ku;
-                    b.oV[o] = kv;
-                } else if (MODE == M_S1) {
-                    b.aU[o] = ku;
-                    b.aV[o] = kv;
-                    Ru[kk] = fma(cY, ku, Yu);
-                    Rv[kk] = fma(cY, kv, Yv);
-                } else if (MODE == M_S23) {
-                    b.aU[o] = fma(2.0, ku, Au[kk]);
-                    b.aV[o] = fma(2.0, kv, Av[kk]);
-                    Ru[kk] = fma(cY, ku, Nu[kk]);
-                    Rv[kk] = fma(cY, kv, Nv[kk]);
-                } else {
-                    Ru[kk] = fma(cA, Au[kk] + ku, Nu[kk]);
-                    Rv[kk] = fma(cA, Av[kk] + kv, Nv[kk]);
-                }
+                stage_entry<MODE>(sc, L0[kk], P1[kk], P2[kk], cex[kk], cey, xg, sxq, FG[kk], FQ[kk], Yu, Yv,
+                                  MODE == M_S1 ? Yu : Nu[kk], MODE == M_S1 ? Yv : Nv[kk], Ru[kk], Rv[kk]);
             }
         }
-        if (MODE != M_RHS) {
-            double *dU = (MODE == M_S4) ? b.nU : b.oU;
-            double *dV = (MODE == M_S4) ? b.nV : b.oV;
 #pragma unroll
-            for (int kk = 0; kk < NE; ++kk)
-                if (kk < nk) { dU[row + kk] = Ru[kk]; dV[row + kk] = Rv[kk]; }
-        }
+        for (int kk = 0; kk < NE; ++kk)
+            if (kk < nk) { b.oU[row + kk] = Ru[kk]; b.oV[row + kk] = Rv[kk]; }
     }
     if (MODE == M_RHS) return;
 
