@@ -574,61 +574,18 @@ k_step2r(const __grid_constant__ ModalParams mp, const double *lams, double *nU,
     }
 }
 
-// traces of a modal state (start of gdg_step and gdg_rhs)
-template <int N1>
-__global__ void __launch_bounds__(MAXB2)
-k_traces2(const __grid_constant__ ModalParams mp, const double *yU, const double *yV, double *trout) {
-    extern __shared__ double smem[];
-    const int t = threadIdx.x;
-    const int le = t / N1, l = t - le * N1;
-    const int e = blockIdx.x * (int)(blockDim.x / N1) + le;
-    const bool valid = e < mp.ne;
-    double *tile = smem + le * (2 * N1 * (N1 + 1));
-    if (valid) {
-        const size_t row = ((size_t)e * N1 + l) * N1;
-        double vL = 0, vR = 0, dL = 0, dR = 0;
-#pragma unroll
-        for (int k = 0; k < N1; ++k) {
-            const double u = yU[row + k], v = yV[row + k];
-            vL += mp.d[0].eL[k] * v;
-            vR += mp.d[0].eR[k] * v;
-            dL += mp.d[0].gL[k] * u;
-            dR += mp.d[0].gR[k] * u;
-            tile[l * (N1 + 1) + k] = u;
-            tile[N1 * (N1 + 1) + l * (N1 + 1) + k] = v;
-        }
-        trout[tix2<N1>(e, 0, 0, l)] = vL;
-        trout[tix2<N1>(e, 0, 1, l)] = dL;
-        trout[tix2<N1>(e, 1, 0, l)] = vR;
-        trout[tix2<N1>(e, 1, 1, l)] = dR;
-    }
-    __syncthreads();
-    if (valid) {
-        const int k = l;
-        double vL = 0, vR = 0, dL = 0, dR = 0;
-#pragma unroll
-        for (int j = 0; j < N1; ++j) {
-            const double u = tile[j * (N1 + 1) + k], v = tile[N1 * (N1 + 1) + j * (N1 + 1) + k];
-            vL += mp.d[1].eL[j] * v;
-            vR += mp.d[1].eR[j] * v;
-            dL += mp.d[1].gL[j] * u;
-            dR += mp.d[1].gR[j] * u;
-        }
-        trout[tix2<N1>(e, 2, 0, k)] = vL;
-        trout[tix2<N1>(e, 2, 1, k)] = dL;
-        trout[tix2<N1>(e, 3, 0, k)] = vR;
-        trout[tix2<N1>(e, 3, 1, k)] = dR;
-    }
-}
-
 // Separable element transform: out = (Cy (x) Cx) diag(D) (By (x) Bx) in,
 // with C and D optional (nullptr).  Matrices are n1 x n1 row-major,
 // (A (x) B)[(l,k),(j,i)] = A[l][j] B[k][i].  Two fields per call (U and V
-// share the matrices).
-template <int N1>
+// share the matrices); tr (modal output (U, V)): also its face traces.
+// KB: the kind of B (line_transform); C is of kind 2 when B is of kind 3.
+// Bound by the FP64 pipe: 97 x 70 elements, N1 = 9, both fields: 39 us in with the traces, 29 us out (dense lines
+// 42 us, and 15 us for the traces in a kernel of their own).
+template <int N1, int KB>
 __global__ void __launch_bounds__(MAXB2)
-k_sep2(int ne, const double *in0, const double *in1, double *out0, double *out1,
-       const double *Bx, const double *By, const double *D, const double *Cx, const double *Cy) {
+k_sep2(const __grid_constant__ ModalParams mp, const double *in0, const double *in1, double *out0, double *out1,
+       const double *Bx, const double *By, const double *D, const double *Cx, const double *Cy, double *tr) {
+    constexpr int KC = KB == 3 ? 2 : 0;
     extern __shared__ double smem[];
     double *sB = smem;                 // Bx, By, Cx, Cy
     double *tiles = smem + 4 * N1 * N1;
@@ -640,82 +597,71 @@ k_sep2(int ne, const double *in0, const double *in1, double *out0, double *out1,
     }
     const int le = t / N1, l = t - le * N1;
     const int e = blockIdx.x * (int)(blockDim.x / N1) + le;
-    const bool valid = e < ne;
+    const bool valid = e < mp.ne;
     double *tile = tiles + le * (2 * N1 * (N1 + 1));
     const int nf = in1 ? 2 : 1;
+    const size_t row = ((size_t)(valid ? e : 0) * N1 + l) * N1;
+    double x[N1], y[N1];
+    // (1) rows: T[j][k] = sum_i Bx[k][i] in[j][i]   (thread = row j)
     __syncthreads();
+#pragma unroll 1
     for (int f = 0; f < nf; ++f) {
         const double *in = f ? in1 : in0;
+        double *T = tile + f * N1 * (N1 + 1);
+        if (!valid) continue;
+#pragma unroll
+        for (int i = 0; i < N1; ++i) x[i] = in[row + i];
+        line_transform<N1, KB>(sB, x, [&](int k, double v) { T[l * (N1 + 1) + k] = v; });
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int f = 0; f < nf; ++f) {
         double *out = f ? out1 : out0;
         double *T = tile + f * N1 * (N1 + 1);
-        // (1) rows: T[j][k] = sum_i Bx[k][i] in[j][i]   (thread = row j)
-        if (valid) {
-            double x[N1];
-            const size_t row = ((size_t)e * N1 + l) * N1;
+        if (!valid) continue;
+        // (2) columns: Z[m][k] = D[m][k] * sum_j By[m][j] T[j][k]   (thread = column k = l)
 #pragma unroll
-            for (int i = 0; i < N1; ++i) x[i] = in[row + i];
-#pragma unroll
-            for (int k = 0; k < N1; ++k) {
-                double s = 0;
-#pragma unroll
-                for (int i = 0; i < N1; ++i) s += sB[k * N1 + i] * x[i];
-                T[l * (N1 + 1) + k] = s;
+        for (int j = 0; j < N1; ++j) x[j] = T[j * (N1 + 1) + l];
+        if (!Cx) {   // the tile keeps the column for the x faces; the y faces come from it here
+            LineTraces<N1, KB != 0> tc(f ? mp.d[1].eL : mp.d[1].gL, f ? mp.d[1].eR : mp.d[1].gR);
+            line_transform<N1, KB>(sB + N1 * N1, x, [&](int m, double v) {
+                T[m * (N1 + 1) + l] = v;
+                out[((size_t)e * N1 + m) * N1 + l] = v;
+                if (tr) tc.add(m, v);
+            });
+            if (tr) {
+                tr[tix2<N1>(e, 2, 1 - f, l)] = tc.left();
+                tr[tix2<N1>(e, 3, 1 - f, l)] = tc.right();
             }
-        }
-        __syncthreads();
-        // (2) columns: Z[m][k] = D[m][k] * sum_j By[m][j] T[j][k]   (thread = column k)
-        double z[N1];
-        if (valid) {
-            const int k = l;
-            double c[N1];
-#pragma unroll
-            for (int j = 0; j < N1; ++j) c[j] = T[j * (N1 + 1) + k];
-#pragma unroll
-            for (int m = 0; m < N1; ++m) {
-                double s = 0;
-#pragma unroll
-                for (int j = 0; j < N1; ++j) s += sB[N1 * N1 + m * N1 + j] * c[j];
-                if (D) s *= D[m * N1 + k];
-                z[m] = s;
-            }
-        }
-        if (!Cx) {
-            if (valid) {
-                const int k = l;
-#pragma unroll
-                for (int m = 0; m < N1; ++m) out[((size_t)e * N1 + m) * N1 + k] = z[m];
-            }
-            __syncthreads();
             continue;
         }
-        // (3) columns again with Cy: W[r][k] = sum_m Cy[r][m] Z[m][k]; store to T
-        __syncthreads();
-        if (valid) {
-            const int k = l;
+        line_transform<N1, KB>(sB + N1 * N1, x, [&](int m, double v) { T[m * (N1 + 1) + l] = D ? v * D[m * N1 + l] : v; });
+        // (3) columns again with Cy: W[r][k] = sum_m Cy[r][m] Z[m][k], in the thread's own column of T
 #pragma unroll
-            for (int r = 0; r < N1; ++r) {
-                double s = 0;
+        for (int m = 0; m < N1; ++m) y[m] = T[m * (N1 + 1) + l];
+        line_transform<N1, KC>(sB + 3 * N1 * N1, y, [&](int r, double v) { T[r * (N1 + 1) + l] = v; });
+    }
+    if (!Cx && !tr) return;   // uniform
+    __syncthreads();
+#pragma unroll 1
+    for (int f = 0; f < nf; ++f) {
+        double *T = tile + f * N1 * (N1 + 1);
+        if (!valid) continue;
+        if (Cx) {   // (4) rows with Cx: out[r][q] = sum_k Cx[q][k] W[r][k]   (thread = row r), through the tile
+            double *out = f ? out1 : out0;
 #pragma unroll
-                for (int m = 0; m < N1; ++m) s += sB[3 * N1 * N1 + r * N1 + m] * z[m];
-                T[r * (N1 + 1) + k] = s;
-            }
+            for (int k = 0; k < N1; ++k) x[k] = T[l * (N1 + 1) + k];
+            line_transform<N1, KC>(sB + 2 * N1 * N1, x, [&](int q, double v) {
+                T[l * (N1 + 1) + q] = v;
+                out[row + q] = v;
+            });
+        } else {    // x faces
+            LineTraces<N1, KB != 0> tc(f ? mp.d[0].eL : mp.d[0].gL, f ? mp.d[0].eR : mp.d[0].gR);
+#pragma unroll
+            for (int k = 0; k < N1; ++k) tc.add(k, T[l * (N1 + 1) + k]);
+            tr[tix2<N1>(e, 0, 1 - f, l)] = tc.left();
+            tr[tix2<N1>(e, 1, 1 - f, l)] = tc.right();
         }
-        __syncthreads();
-        // (4) rows with Cx: out[r][q] = sum_k Cx[q][k] W[r][k]   (thread = row r)
-        if (valid) {
-            double w[N1];
-#pragma unroll
-            for (int k = 0; k < N1; ++k) w[k] = T[l * (N1 + 1) + k];
-            const size_t row = ((size_t)e * N1 + l) * N1;
-#pragma unroll
-            for (int q = 0; q < N1; ++q) {
-                double s = 0;
-#pragma unroll
-                for (int k = 0; k < N1; ++k) s += sB[2 * N1 * N1 + q * N1 + k] * w[k];
-                out[row + q] = s;
-            }
-        }
-        __syncthreads();
     }
 }
 
@@ -867,7 +813,6 @@ __global__ void k_sep1(int ne, const double *in0, const double *in1, double *out
 #define GDG_N1_CASES_P(X) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10)
 
 size_t smem_stage2(int n1, int epb) { return (size_t)epb * (4 * n1 + 2 * n1 * (n1 + 1)) * sizeof(double); }
-size_t smem_traces2(int n1, int epb) { return (size_t)epb * (2 * n1 * (n1 + 1)) * sizeof(double); }
 size_t smem_sep2(int n1, int epb) { return (size_t)(4 * n1 * n1 + epb * 2 * n1 * (n1 + 1)) * sizeof(double); }
 
 template <int N1>
@@ -943,44 +888,23 @@ void launch_stage_raw(const gdg_ctx *ctx, int mode, const StageBufs &b, double s
     }
 }
 
-void launch_traces_raw(const gdg_ctx *ctx, const double *yU, const double *yV, double *tr, cudaStream_t s) {
-    const int n1 = ctx->n1;
-    if (ctx->dim == 3) {
-        gdg3_traces(ctx->mp, n1, yU, yV, tr, s);
-        return;
-    }
-    if (ctx->dim == 2) {
-        const int epb = ctx->mp.epb;
-        dim3 grid((ctx->ne + epb - 1) / epb), block(epb * n1);
-        switch (n1) {
-#define X(n) case n: k_traces2<n><<<grid, block, smem_traces2(n, epb), s>>>(ctx->mp, yU, yV, tr); break;
-            GDG_N1_CASES(X)
-#undef X
-        }
-    } else {
-        dim3 grid((ctx->ne + TPB1 - 1) / TPB1), block(TPB1);
-        switch (n1) {
-#define X(n) case n: k_traces1<n><<<grid, block, 0, s>>>(ctx->mp, yU, yV, tr); break;
-            GDG_N1_CASES(X)
-#undef X
-        }
-    }
-}
-
 // table offsets inside ctx->d_mats: [dir][P, Psi, PsiT][n1*n1]
 const double *mat(const gdg_ctx *ctx, int dir, int which) {
     return ctx->d_mats + ((size_t)dir * 3 + which) * ctx->n1 * ctx->n1;
 }
 enum { T_P = 0, T_PSI = 1, T_PSIT = 2 };
 
-// out = (C) diag(D) (B) in, over both fields when in1 != nullptr
+// out = (C) diag(D) (B) in, over both fields when in1 != nullptr; tr: the face
+// traces of the modal result (out0, out1) too (B = T_P)
 void launch_sep_raw(const gdg_ctx *ctx, const double *in0, const double *in1, double *out0, double *out1,
-                int B, const double *D, int C, cudaStream_t s) {
+                    int B, const double *D, int C, double *tr, cudaStream_t s) {
     const int n1 = ctx->n1;
+    // with parity every use is nodes to modes (P, Psi^T), then modes to nodes (Psi) or nothing
+    const int kind = !ctx->mp.parity ? 0 : B == T_PSI ? 2 : B == T_P ? 1 : 3;
     if (ctx->dim == 3) {
-        gdg3_sep(n1, ctx->ne, in0, in1, out0, out1, mat(ctx, 0, B), mat(ctx, 1, B), mat(ctx, 2, B), D,
+        gdg3_sep(ctx->mp, n1, kind, in0, in1, out0, out1, mat(ctx, 0, B), mat(ctx, 1, B), mat(ctx, 2, B), D,
                  C >= 0 ? mat(ctx, 0, C) : nullptr, C >= 0 ? mat(ctx, 1, C) : nullptr,
-                 C >= 0 ? mat(ctx, 2, C) : nullptr, s);
+                 C >= 0 ? mat(ctx, 2, C) : nullptr, tr, s);
         return;
     }
     if (ctx->dim == 2) {
@@ -989,7 +913,7 @@ void launch_sep_raw(const gdg_ctx *ctx, const double *in0, const double *in1, do
         const double *Bx = mat(ctx, 0, B), *By = mat(ctx, 1, B);
         const double *Cx = C >= 0 ? mat(ctx, 0, C) : nullptr, *Cy = C >= 0 ? mat(ctx, 1, C) : nullptr;
         switch (n1) {
-#define X(n) case n: k_sep2<n><<<grid, block, smem_sep2(n, epb), s>>>(ctx->ne, in0, in1, out0, out1, Bx, By, D, Cx, Cy); break;
+#define X(n) case n: (kind == 0 ? k_sep2<n, 0> : kind == 1 ? k_sep2<n, 1> : kind == 2 ? k_sep2<n, 2> : k_sep2<n, 3>)<<<grid, block, smem_sep2(n, epb), s>>>(ctx->mp, in0, in1, out0, out1, Bx, By, D, Cx, Cy, tr); break;
             GDG_N1_CASES(X)
 #undef X
         }
@@ -997,7 +921,7 @@ void launch_sep_raw(const gdg_ctx *ctx, const double *in0, const double *in1, do
         dim3 grid((ctx->ne + TPB1 - 1) / TPB1), block(TPB1);
         const double *Bm = mat(ctx, 0, B), *Cm = C >= 0 ? mat(ctx, 0, C) : nullptr;
         switch (n1) {
-#define X(n) case n: k_sep1<n><<<grid, block, 0, s>>>(ctx->ne, in0, in1, out0, out1, Bm, D, Cm); break;
+#define X(n) case n: k_sep1<n><<<grid, block, 0, s>>>(ctx->ne, in0, in1, out0, out1, Bm, D, Cm); if (tr) k_traces1<n><<<grid, block, 0, s>>>(ctx->mp, out0, out1, tr); break;
             GDG_N1_CASES(X)
 #undef X
         }
@@ -1007,12 +931,13 @@ void launch_sep_raw(const gdg_ctx *ctx, const double *in0, const double *in1, do
 void launch_stage(gdg_ctx *ctx, int mode, const StageBufs &b, double sc, cudaStream_t s) {
     GDG_PROF(ctx, GDG_K_STAGE, s, launch_stage_raw(ctx, mode, b, sc, s));
 }
-void launch_traces(gdg_ctx *ctx, const double *yU, const double *yV, double *tr, cudaStream_t s) {
-    GDG_PROF(ctx, GDG_K_TRACES, s, launch_traces_raw(ctx, yU, yV, tr, s));
-}
 void launch_sep(gdg_ctx *ctx, const double *in0, const double *in1, double *out0, double *out1,
                 int B, const double *D, int C, cudaStream_t s) {
-    GDG_PROF(ctx, GDG_K_TRANSFORM, s, launch_sep_raw(ctx, in0, in1, out0, out1, B, D, C, s));
+    GDG_PROF(ctx, GDG_K_TRANSFORM, s, launch_sep_raw(ctx, in0, in1, out0, out1, B, D, C, nullptr, s));
+}
+// nodal (u, v) to the modal state (mU, mV) and its traces
+void launch_enter(gdg_ctx *ctx, const double *u, const double *v, double *mU, double *mV, double *tr, cudaStream_t s) {
+    GDG_PROF(ctx, GDG_K_TRANSFORM, s, launch_sep_raw(ctx, u, v, mU, mV, T_P, nullptr, -1, tr, s));
 }
 
 double *buf(gdg_ctx *ctx, int i) { return ctx->d_state + (size_t)i * ctx->ndof; }
@@ -1137,8 +1062,10 @@ int set_smem_limits() {
     cudaFuncSetAttribute(k_stage2f<n, M_RHS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
     cudaFuncSetAttribute(k_stage2f<n, M_S1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage2f<n, M_S23, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
-    cudaFuncSetAttribute(k_traces2<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);        \
-    cudaFuncSetAttribute(k_sep2<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_sep2<n, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);        \
+    cudaFuncSetAttribute(k_sep2<n, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);        \
+    cudaFuncSetAttribute(k_sep2<n, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);        \
+    cudaFuncSetAttribute(k_sep2<n, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     GDG_N1_CASES(X)
 #undef X
 #define X(n)                                                                                   \
@@ -1240,8 +1167,7 @@ void enqueue_rk4_step_nodal(gdg_ctx *ctx, double *u, double *v, double dt, cudaS
     double *yU = buf(ctx, B_YU), *yV = buf(ctx, B_YV), *kU = buf(ctx, B_NU), *kV = buf(ctx, B_NV);
     for (int st = 0; st < RK_STAGES; ++st) {
         const double *inU = st == 0 ? u : yU, *inV = st == 0 ? v : yV;
-        launch_sep(ctx, inU, inV, buf(ctx, B_XU), buf(ctx, B_XV), T_P, nullptr, -1, s);
-        launch_traces(ctx, buf(ctx, B_XU), buf(ctx, B_XV), ctx->d_tr, s);
+        launch_enter(ctx, inU, inV, buf(ctx, B_XU), buf(ctx, B_XV), ctx->d_tr, s);
         StageBufs b{};
         b.yU = buf(ctx, B_XU); b.yV = buf(ctx, B_XV);
         b.oU = buf(ctx, B_KU); b.oV = buf(ctx, B_KV);
@@ -1426,6 +1352,14 @@ int gdg_const_setup(gdg_ctx *ctx) {
         std::vector<double> Psi(nn), M(nn);
         for (int i = 0; i < n1; ++i)
             for (int k = 0; k < n1; ++k) Psi[i * n1 + k] = ctx->Psih[i * n1 + perm[k]] / sq;
+        if (mp.parity)   // exactly even and odd modes: the transforms read one half of each
+            for (int k = 0; k < n1; ++k)
+                for (int i = 0; i <= (n1 - 1) / 2; ++i) {
+                    const double sgn = k < (n1 + 1) / 2 ? 1.0 : -1.0;
+                    const double a = 0.5 * (Psi[i * n1 + k] + sgn * Psi[(n1 - 1 - i) * n1 + k]);
+                    Psi[i * n1 + k] = a;
+                    Psi[(n1 - 1 - i) * n1 + k] = sgn * a;
+                }
         for (int i = 0; i < nn; ++i) M[i] = H * ctx->Mh[i];
         lam[d].resize(n1);
         for (int k = 0; k < n1; ++k) lam[d][k] = ctx->lamh[perm[k]] / (H * H);
@@ -1536,8 +1470,7 @@ void gdg_const_free(gdg_ctx *ctx) {
 
 int gdg_const_rhs(gdg_ctx *ctx, const double *u, const double *v, double *du, double *dv, cudaStream_t s) {
     // modal state of (u, v), its traces, k = f(Y) in modal form, back to nodal
-    launch_sep(ctx, u, v, buf(ctx, B_XU), buf(ctx, B_XV), T_P, nullptr, -1, s);
-    launch_traces(ctx, buf(ctx, B_XU), buf(ctx, B_XV), ctx->d_tr, s);
+    launch_enter(ctx, u, v, buf(ctx, B_XU), buf(ctx, B_XV), ctx->d_tr, s);
     if (has_halo(ctx)) {
         if (!ctx->halo_fn) return gdg_set_err(ctx, GDG_EINVAL, "gdg_rhs: halo sides need gdg_set_halo first");
         const int st = halo_exchange(ctx, ctx->d_tr, s);
@@ -1602,8 +1535,7 @@ int tune_stage_kernel(gdg_ctx *ctx, double dt, cudaStream_t s, const double *u, 
         }
         if (persist_failed(ctx, s)) best[3] = 1e30f;
     }
-    launch_sep(ctx, u, v, buf(ctx, B_NU), buf(ctx, B_NV), T_P, nullptr, -1, s);
-    launch_traces(ctx, buf(ctx, B_NU), buf(ctx, B_NV), ctx->d_tr, s);
+    launch_enter(ctx, u, v, buf(ctx, B_NU), buf(ctx, B_NV), ctx->d_tr, s);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     int pick = 0;
@@ -1645,8 +1577,7 @@ int gdg_const_step(gdg_ctx *ctx, double *u, double *v, double dt, int nsteps, cu
     int st;
     if (ctx->pb.route == GDG_ROUTE_NODAL) return step_nodal(ctx, u, v, dt, nsteps, s);
     stage_tables(ctx, dt, s);
-    launch_sep(ctx, u, v, buf(ctx, B_NU), buf(ctx, B_NV), T_P, nullptr, -1, s);
-    launch_traces(ctx, buf(ctx, B_NU), buf(ctx, B_NV), ctx->d_tr, s);
+    launch_enter(ctx, u, v, buf(ctx, B_NU), buf(ctx, B_NV), ctx->d_tr, s);
     if ((st = gdg_cuda_check(ctx, cudaGetLastError(), "gdg_step prologue"))) return st;
     if (has_halo(ctx)) {   // partitioned mesh: stages launched one by one, exchanges between them
         if (!ctx->halo_fn) return gdg_set_err(ctx, GDG_EINVAL, "gdg_step: halo sides need gdg_set_halo first");
@@ -1729,8 +1660,7 @@ StepBuffers gdg_const_buffers(gdg_ctx *ctx) {
 
 int gdg_const_enter(gdg_ctx *ctx, const double *u, const double *v, double dt, cudaStream_t s) {
     stage_tables(ctx, dt, s);
-    launch_sep(ctx, u, v, buf(ctx, B_NU), buf(ctx, B_NV), T_P, nullptr, -1, s);
-    launch_traces(ctx, buf(ctx, B_NU), buf(ctx, B_NV), ctx->d_tr, s);
+    launch_enter(ctx, u, v, buf(ctx, B_NU), buf(ctx, B_NV), ctx->d_tr, s);
     return gdg_cuda_check(ctx, cudaGetLastError(), "enter");
 }
 
@@ -2046,8 +1976,7 @@ extern "C" int gdg_rhs_static(const gdg_problem *pb, const double *u, const doub
     c.d_lam2 = base + 6 * nn;
     double *Yu = base + ntab, *Yv = Yu + ndof, *Ku = Yv + ndof, *Kv = Ku + ndof, *tr = Kv + ndof;
     set_smem_limits();
-    launch_sep(&c, u, v, Yu, Yv, T_P, nullptr, -1, s);
-    launch_traces(&c, Yu, Yv, tr, s);
+    launch_enter(&c, u, v, Yu, Yv, tr, s);
     StageBufs b{};
     b.yU = Yu; b.yV = Yv; b.oU = Ku; b.oV = Kv; b.trin = tr; b.lam2 = c.d_lam2;
     launch_stage(&c, M_RHS, b, 0.0, s);

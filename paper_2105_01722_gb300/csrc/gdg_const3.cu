@@ -336,49 +336,17 @@ k_stage3p(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) 
     }
 }
 
-// traces of a modal state (start of gdg_step and gdg_rhs)
-template <int N1>
-__global__ void __launch_bounds__(MAXB3)
-k_traces3(const __grid_constant__ ModalParams mp, const double *yU, const double *yV, double *trout) {
-    constexpr int NT = N1 * N1, NA = N1 * N1 * N1;
-    extern __shared__ double smem[];
-    const int epb = blockDim.x / NT;
-    const int t = threadIdx.x;
-    const int le = t / NT, r = t - le * NT;
-    const int a = r / N1, c = r - (r / N1) * N1;
-    const int e = blockIdx.x * epb + le;
-    const bool valid = e < mp.ne;
-    double *tU = smem + le * 2 * NA, *tV = tU + NA;
-    if (valid) {
-        const int line = a * N1 + c;
-        const size_t row = ((size_t)e * NT + line) * N1;
-        double vL = 0, vR = 0, dL = 0, dR = 0;
-#pragma unroll
-        for (int k = 0; k < N1; ++k) {
-            const double u = yU[row + k], v = yV[row + k];
-            vL += mp.d[0].eL[k] * v;
-            vR += mp.d[0].eR[k] * v;
-            dL += mp.d[0].gL[k] * u;
-            dR += mp.d[0].gR[k] * u;
-            tU[line * N1 + k] = u;
-            tV[line * N1 + k] = v;
-        }
-        trout[tix3<N1>(e, 0, 0, line)] = vL;
-        trout[tix3<N1>(e, 0, 1, line)] = dL;
-        trout[tix3<N1>(e, 1, 0, line)] = vR;
-        trout[tix3<N1>(e, 1, 1, line)] = dR;
-    }
-    __syncthreads();
-    if (valid) traces3_yz<N1>(mp, tU, tV, e, a, c, trout);
-}
-
 // Separable element transform out = (Cz (x) Cy (x) Cx) diag(D) (Bz (x) By (x) Bx) in
 // (C, D optional); per field, passes along x, y, z through an element tile.
-template <int N1>
+// tr (modal output (U, V)): also its face traces.  KB: the kind of B
+// (line_transform); C is of kind 2 when B is of kind 3.  Bound by the FP64
+// pipe: 32^3 elements, N1 = 9, both fields: see gdg_step's table of times.
+template <int N1, int KB>
 __global__ void __launch_bounds__(MAXB3)
-k_sep3(int ne, const double *in0, const double *in1, double *out0, double *out1, const double *Bx,
-       const double *By, const double *Bz, const double *D, const double *Cx, const double *Cy, const double *Cz) {
-    constexpr int NT = N1 * N1, NA = N1 * N1 * N1;
+k_sep3(const __grid_constant__ ModalParams mp, const double *in0, const double *in1, double *out0, double *out1,
+       const double *Bx, const double *By, const double *Bz, const double *D, const double *Cx, const double *Cy,
+       const double *Cz, double *tr) {
+    constexpr int NT = N1 * N1, NA = N1 * N1 * N1, KC = KB == 3 ? 2 : 0;
     extern __shared__ double smem[];
     double *sM = smem;            // Bx, By, Bz, Cx, Cy, Cz
     const int t = threadIdx.x;
@@ -392,99 +360,88 @@ k_sep3(int ne, const double *in0, const double *in1, double *out0, double *out1,
     const int le = t / NT, r = t - le * NT;
     const int a = r / N1, c = r - (r / N1) * N1;
     const int e = blockIdx.x * epb + le;
-    const bool valid = e < ne;
+    const bool valid = e < mp.ne;
     double *T = smem + 6 * NT + le * NA;
     const int nf = in1 ? 2 : 1;
-    __syncthreads();
+    const size_t base = (size_t)blockIdx.x * epb * NA;           // the block's elements are consecutive
+    const int count = min(epb, mp.ne - (int)blockIdx.x * epb) * NA;
+    double *Tb = smem + 6 * NT;
     for (int f = 0; f < nf; ++f) {
         const double *in = f ? in1 : in0;
         double *out = f ? out1 : out0;
-        double x[N1], y[N1];
+        double x[N1];
+        // the tiles, coalesced (a line per thread would stride the loads by N1)
+        for (int i = t; i < count; i += blockDim.x) Tb[i] = in[base + i];
+        __syncthreads();
         // (1) x: thread = line (k = a, j = c)
         if (valid) {
-            const size_t row = ((size_t)e * NT + a * N1 + c) * N1;
 #pragma unroll
-            for (int i = 0; i < N1; ++i) x[i] = in[row + i];
-#pragma unroll
-            for (int q = 0; q < N1; ++q) {
-                double s = 0;
-#pragma unroll
-                for (int i = 0; i < N1; ++i) s += sM[q * N1 + i] * x[i];
-                T[(a * N1 + c) * N1 + q] = s;
-            }
+            for (int i = 0; i < N1; ++i) x[i] = T[(a * N1 + c) * N1 + i];
+            line_transform<N1, KB>(sM, x, [&](int q, double v) { T[(a * N1 + c) * N1 + q] = v; });
         }
         __syncthreads();
         // (2) y: thread = (k = a, i = c), column over j
         if (valid) {
 #pragma unroll
             for (int j = 0; j < N1; ++j) x[j] = T[(a * N1 + j) * N1 + c];
-#pragma unroll
-            for (int m = 0; m < N1; ++m) {
-                double s = 0;
-#pragma unroll
-                for (int j = 0; j < N1; ++j) s += sM[NT + m * N1 + j] * x[j];
-                T[(a * N1 + m) * N1 + c] = s;
-            }
+            line_transform<N1, KB>(sM + NT, x, [&](int m, double v) { T[(a * N1 + m) * N1 + c] = v; });
         }
         __syncthreads();
         // (3) z: thread = (j = a, i = c), column over k; then D
         if (valid) {
 #pragma unroll
             for (int k = 0; k < N1; ++k) x[k] = T[(k * N1 + a) * N1 + c];
-#pragma unroll
-            for (int m = 0; m < N1; ++m) {
-                double s = 0;
-#pragma unroll
-                for (int k = 0; k < N1; ++k) s += sM[2 * NT + m * N1 + k] * x[k];
-                if (D) s *= D[(m * N1 + a) * N1 + c];
-                y[m] = s;
+            LineTraces<N1, KB != 0> tc(f ? mp.d[2].eL : mp.d[2].gL, f ? mp.d[2].eR : mp.d[2].gR);
+            line_transform<N1, KB>(sM + 2 * NT, x, [&](int m, double v) {
+                T[(m * N1 + a) * N1 + c] = D ? v * D[(m * N1 + a) * N1 + c] : v;
+                if (tr) tc.add(m, v);
+            });
+            if (tr) {
+                tr[tix3<N1>(e, 4, 1 - f, a * N1 + c)] = tc.left();
+                tr[tix3<N1>(e, 5, 1 - f, a * N1 + c)] = tc.right();
             }
         }
-        if (!Cx) {
-            if (valid) {
+        if (!Cx) {   // out, coalesced from the tiles, and the traces of the other faces
+            __syncthreads();
+            for (int i = t; i < count; i += blockDim.x) out[base + i] = Tb[i];
+            if (tr && valid) {
+                LineTraces<N1, KB != 0> tx(f ? mp.d[0].eL : mp.d[0].gL, f ? mp.d[0].eR : mp.d[0].gR);
+                LineTraces<N1, KB != 0> ty(f ? mp.d[1].eL : mp.d[1].gL, f ? mp.d[1].eR : mp.d[1].gR);
 #pragma unroll
-                for (int m = 0; m < N1; ++m) out[((size_t)e * NT + m * N1 + a) * N1 + c] = y[m];
+                for (int k = 0; k < N1; ++k) {
+                    tx.add(k, T[(a * N1 + c) * N1 + k]);
+                    ty.add(k, T[(a * N1 + k) * N1 + c]);
+                }
+                tr[tix3<N1>(e, 0, 1 - f, a * N1 + c)] = tx.left();
+                tr[tix3<N1>(e, 1, 1 - f, a * N1 + c)] = tx.right();
+                tr[tix3<N1>(e, 2, 1 - f, a * N1 + c)] = ty.left();
+                tr[tix3<N1>(e, 3, 1 - f, a * N1 + c)] = ty.right();
             }
             __syncthreads();
             continue;
         }
-        // (4) Cz along z (same thread layout), back into the thread's own column of the tile
+        // (4) Cz along z (same thread layout), in the thread's own column of the tile
         if (valid) {
 #pragma unroll
-            for (int r2 = 0; r2 < N1; ++r2) {
-                double s = 0;
-#pragma unroll
-                for (int m = 0; m < N1; ++m) s += sM[5 * NT + r2 * N1 + m] * y[m];
-                T[(r2 * N1 + a) * N1 + c] = s;
-            }
+            for (int k = 0; k < N1; ++k) x[k] = T[(k * N1 + a) * N1 + c];
+            line_transform<N1, KC>(sM + 5 * NT, x, [&](int m, double v) { T[(m * N1 + a) * N1 + c] = v; });
         }
         __syncthreads();
         // (5) Cy along y: thread = (k = a, i = c)
         if (valid) {
 #pragma unroll
             for (int j = 0; j < N1; ++j) x[j] = T[(a * N1 + j) * N1 + c];
-#pragma unroll
-            for (int m = 0; m < N1; ++m) {
-                double s = 0;
-#pragma unroll
-                for (int j = 0; j < N1; ++j) s += sM[4 * NT + m * N1 + j] * x[j];
-                T[(a * N1 + m) * N1 + c] = s;
-            }
+            line_transform<N1, KC>(sM + 4 * NT, x, [&](int m, double v) { T[(a * N1 + m) * N1 + c] = v; });
         }
         __syncthreads();
         // (6) Cx along x: thread = line (k = a, j = c)
         if (valid) {
-            const size_t row = ((size_t)e * NT + a * N1 + c) * N1;
 #pragma unroll
             for (int i = 0; i < N1; ++i) x[i] = T[(a * N1 + c) * N1 + i];
-#pragma unroll
-            for (int q = 0; q < N1; ++q) {
-                double s = 0;
-#pragma unroll
-                for (int i = 0; i < N1; ++i) s += sM[3 * NT + q * N1 + i] * x[i];
-                out[row + q] = s;
-            }
+            line_transform<N1, KC>(sM + 3 * NT, x, [&](int q, double v) { T[(a * N1 + c) * N1 + q] = v; });
         }
+        __syncthreads();
+        for (int i = t; i < count; i += blockDim.x) out[base + i] = Tb[i];
         __syncthreads();
     }
 }
@@ -516,7 +473,6 @@ __global__ void k_energy_partial3(int ne, const double *yU, const double *yV, co
 int epb3(int n1) { return std::max(1, MAXB3 / (n1 * n1)); }
 // per element the fluxes and the tile; per block the parity kernel's c^2 eL / 2 table
 size_t smem_stage3(int n1) { return ((size_t)epb3(n1) * (12 * n1 * n1 + 2 * n1 * n1 * n1) + 3 * n1) * sizeof(double); }
-size_t smem_traces3(int n1) { return (size_t)epb3(n1) * 2 * n1 * n1 * n1 * sizeof(double); }
 size_t smem_sep3(int n1) { return (size_t)(6 * n1 * n1 + epb3(n1) * n1 * n1 * n1) * sizeof(double); }
 
 template <int N1>
@@ -551,23 +507,13 @@ void gdg3_stage(const ModalParams &mp, int n1, int mode, const StageBufs &b, dou
     }
 }
 
-void gdg3_traces(const ModalParams &mp, int n1, const double *yU, const double *yV, double *tr, cudaStream_t s) {
+void gdg3_sep(const ModalParams &mp, int n1, int kind, const double *in0, const double *in1, double *out0, double *out1,
+              const double *Bx, const double *By, const double *Bz, const double *D, const double *Cx, const double *Cy,
+              const double *Cz, double *tr, cudaStream_t s) {
     const int epb = epb3(n1);
     const dim3 grid((mp.ne + epb - 1) / epb), block(epb * n1 * n1);
     switch (n1) {
-#define X(n) case n: k_traces3<n><<<grid, block, smem_traces3(n), s>>>(mp, yU, yV, tr); break;
-        GDG_N1_CASES3(X)
-#undef X
-    }
-}
-
-void gdg3_sep(int n1, int ne, const double *in0, const double *in1, double *out0, double *out1, const double *Bx,
-              const double *By, const double *Bz, const double *D, const double *Cx, const double *Cy,
-              const double *Cz, cudaStream_t s) {
-    const int epb = epb3(n1);
-    const dim3 grid((ne + epb - 1) / epb), block(epb * n1 * n1);
-    switch (n1) {
-#define X(n) case n: k_sep3<n><<<grid, block, smem_sep3(n), s>>>(ne, in0, in1, out0, out1, Bx, By, Bz, D, Cx, Cy, Cz); break;
+#define X(n) case n: (kind == 0 ? k_sep3<n, 0> : kind == 1 ? k_sep3<n, 1> : kind == 2 ? k_sep3<n, 2> : k_sep3<n, 3>)<<<grid, block, smem_sep3(n), s>>>(mp, in0, in1, out0, out1, Bx, By, Bz, D, Cx, Cy, Cz, tr); break;
         GDG_N1_CASES3(X)
 #undef X
     }
@@ -594,8 +540,10 @@ void gdg3_set_smem_limits() {
     cudaFuncSetAttribute(k_stage3p<n, M_RHS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
     cudaFuncSetAttribute(k_stage3p<n, M_S1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage3p<n, M_S23, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
-    cudaFuncSetAttribute(k_traces3<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);       \
-    cudaFuncSetAttribute(k_sep3<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_sep3<n, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);       \
+    cudaFuncSetAttribute(k_sep3<n, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);       \
+    cudaFuncSetAttribute(k_sep3<n, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);       \
+    cudaFuncSetAttribute(k_sep3<n, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     GDG_N1_CASES3(X)
 #undef X
 }

@@ -64,10 +64,9 @@ struct StageBufs {
 
 // 3-D modal-route launches (gdg_const3.cu), n1 = N+1 in 2..10
 void gdg3_stage(const ModalParams &mp, int n1, int mode, const StageBufs &b, double sc, cudaStream_t s);
-void gdg3_traces(const ModalParams &mp, int n1, const double *yU, const double *yV, double *tr, cudaStream_t s);
-void gdg3_sep(int n1, int ne, const double *in0, const double *in1, double *out0, double *out1, const double *Bx,
-              const double *By, const double *Bz, const double *D, const double *Cx, const double *Cy,
-              const double *Cz, cudaStream_t s);
+void gdg3_sep(const ModalParams &mp, int n1, int kind, const double *in0, const double *in1, double *out0, double *out1,
+              const double *Bx, const double *By, const double *Bz, const double *D, const double *Cx, const double *Cy,
+              const double *Cz, double *tr, cudaStream_t s);
 void gdg3_energy_partial(int n1, int ne, const double *yU, const double *yV, const double *lam2, double *partial,
                          int blocks, cudaStream_t s);
 void gdg3_set_smem_limits();

@@ -52,6 +52,90 @@ __device__ __forceinline__ void flux2(double vi, double di, double vo, double dO
     q2 = fma(t2, d1, di - dO);
 }
 
+// y = A x for one line of an element transform, A row-major in shared memory.
+// KIND 0: any matrix.  The modes are even or odd under r -> 1-r where the
+// basis has that symmetry (parity contexts; the even ones, NE = ceil(N1/2),
+// first), so a line splits in node pairs and each output is a sum of about
+// N1/2 products: 41 FMAs and 8 additions instead of 81 at N1 = 9.
+// KIND 1: nodes to modes by P = Psi^T M, row q of A even or odd in i.  Rows
+// q > 0 sum to zero (M 1 is the constant mode), so they are applied to the
+// differences from a middle node: the rounding of the table then meets the
+// variation along the line, not the values, which the high modes (times lambda
+// afterwards) would show.  KIND 3: the same by Psi^T, whose rows do not sum to
+// zero, from the plain sums and differences of the pairs.  KIND 2: modes to
+// nodes (column k even or odd in i), a pair from its even and odd parts.
+// emit(i, y[i]) as each is formed: a store there keeps the loads of the
+// matrix from being moved up into a hundred registers.
+template <int N1, int KIND, typename EMIT>
+__device__ __forceinline__ void line_transform(const double *A, const double (&x)[N1], EMIT emit) {
+    constexpr int NE = (N1 + 1) / 2, H = N1 / 2;   // H pairs, and the middle node when N1 is odd
+    if (KIND == 1 || KIND == 3) {
+        const double ref = KIND == 1 ? x[(N1 - 1) / 2] : 0.0;
+        double sm[NE], df[H > 0 ? H : 1];
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            sm[i] = KIND == 1 ? (x[i] - ref) + (x[N1 - 1 - i] - ref) : x[i] + x[N1 - 1 - i];
+            df[i] = x[i] - x[N1 - 1 - i];
+        }
+        if (N1 & 1) sm[NE - 1] = KIND == 1 ? 0.0 : x[H];
+#pragma unroll
+        for (int q = 0; q < N1; ++q) {
+            double s = 0.0;
+            if (KIND == 1 && q == 0) {   // the constant mode: the only one that sees ref
+#pragma unroll
+                for (int i = 0; i < H; ++i) s = fma(A[i], x[i] + x[N1 - 1 - i], s);
+                if (N1 & 1) s = fma(A[H], x[H], s);
+            } else {
+#pragma unroll
+                for (int i = 0; i < (q < NE && KIND == 3 ? NE : H); ++i)
+                    s = fma(A[q * N1 + i], q < NE ? sm[i] : df[i < H ? i : 0], s);
+            }
+            emit(q, s);
+        }
+    } else if (KIND == 2) {
+#pragma unroll
+        for (int i = 0; i < NE; ++i) {
+            double ev = 0.0, od = 0.0;
+#pragma unroll
+            for (int k = 0; k < NE; ++k) ev = fma(A[i * N1 + k], x[k], ev);
+            if (i < H) {
+#pragma unroll
+                for (int k = NE; k < N1; ++k) od = fma(A[i * N1 + k], x[k], od);
+                emit(N1 - 1 - i, ev - od);
+            }
+            emit(i, i < H ? ev + od : ev);
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < N1; ++q) {
+            double s = 0.0;
+#pragma unroll
+            for (int i = 0; i < N1; ++i) s = fma(A[q * N1 + i], x[i], s);
+            emit(q, s);
+        }
+    }
+}
+
+// the two face traces of a modal line (values: L, R = eL, eR; outward slopes:
+// gL, gR), its entries added in any order
+template <int N1, bool PAR>
+struct LineTraces {
+    const double *L, *R;
+    double a = 0.0, b = 0.0;   // parity: even and odd parts; else left and right
+    __device__ LineTraces(const double *L_, const double *R_) : L(L_), R(R_) {}
+    __device__ __forceinline__ void add(int k, double y) {
+        if (PAR) {
+            if (k < (N1 + 1) / 2) a = fma(L[k], y, a);
+            else b = fma(L[k], y, b);
+        } else {
+            a = fma(L[k], y, a);
+            b = fma(R[k], y, b);
+        }
+    }
+    __device__ __forceinline__ double left() const { return PAR ? a + b : a; }
+    __device__ __forceinline__ double right() const { return PAR ? a - b : b; }
+};
+
 // One modal entry of a stage (see stage2p_body): the new (u, v) from the stage
 // input (Yu, Yv) and y_n (Nu, Nv), or k itself (M_RHS).  L0, P1, P2, cey, xq
 // carry the stage's factor sc unless M_RHS.
