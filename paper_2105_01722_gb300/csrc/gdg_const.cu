@@ -705,9 +705,10 @@ __global__ void k_sum_partials(int n, const double *partial, double *out) {
 
 // ------------------------------------------------------------ 1-D --------
 
-template <int N1, int MODE>
+// k = f(Y) of gdg_rhs (time steps run in k_run1)
+template <int N1>
 __global__ void __launch_bounds__(TPB1)
-k_stage1(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) {
+k_stage1(const __grid_constant__ ModalParams mp, const StageBufs b) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= mp.ne) return;
     const int nx = mp.nx;
@@ -729,31 +730,137 @@ k_stage1(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) {
     } else { vo = -vi; dO = -di; }
     flux(vi, di, vo, dO, mp.beta, mp.tau, mp.c2, mp.alt, 1, en >= nx, gp, qp);
     const size_t row = (size_t)e * N1;
-    double Ru[N1], Rv[N1];
 #pragma unroll
     for (int k = 0; k < N1; ++k) {
         const double Yu = b.yU[row + k], Yv = b.yV[row + k];
         const double ru = mp.d[0].gL[k] * gm + mp.d[0].gR[k] * gp;
         const double rv = mp.d[0].eL[k] * qm + mp.d[0].eR[k] * qp;
-        if (MODE == M_RHS) {
-            b.oU[row + k] = Yv + b.lam2[N1 + k] * ru;
-            b.oV[row + k] = b.lam2[k] * Yu + rv;
-        } else {   // lam2 carries sc
-            const double Nu = MODE == M_S1 ? Yu : b.nU[row + k], Nv = MODE == M_S1 ? Yv : b.nV[row + k];
-            Ru[k] = fma(sc, Yv, fma(b.lam2[N1 + k], ru, Nu));
-            Rv[k] = fma(b.lam2[k], Yu, fma(sc, rv, Nv));
+        b.oU[row + k] = Yv + b.lam2[N1 + k] * ru;
+        b.oV[row + k] = b.lam2[k] * Yu + rv;
+    }
+}
+
+// Time steps of a 1-D mesh: a block holds a window of W elements in shared
+// memory and registers, one thread per element and mode, and advances it
+// `steps` RK4 steps without leaving the SM.  A block owns `own` elements;
+// where the window does not reach the whole mesh it adds 4 `steps` elements on
+// either side, since a stage carries information one element far: what the
+// window's open ends get wrong has not reached the owned ones when the launch
+// ends.  So one launch replaces 4 `steps` of them (and, for a mesh of one
+// window, every launch of the call: 16 elements, 16 steps 480 -> 45 us, the
+// 64 stages 0.6 us each where a launch took 7.5).
+// `first`: u, v are nodal and enter through P; `last`: they leave through Psi;
+// else modal.  Bound by the latency of a stage's chain (update, trace sums,
+// fluxes: FP64 issues a warp instruction every 64 cycles of a sub-partition).
+constexpr int RUN1_WHOLE = 32;   // largest mesh run by one block: above, windows on more SMs are faster
+constexpr int RUN1_STEPS = 2;    // steps a launch: window overlap (8 elements a step) against launches
+constexpr int RUN1_MAXT = 1024;
+
+__host__ __device__ constexpr size_t run1_doubles(int n1, int W) {
+    return (size_t)W * (2 * n1 + 8) + 2 * n1 * n1 + 4 * n1 + RK_STAGES * 2 * n1;
+}
+
+template <int N1>
+__global__ void __launch_bounds__(RUN1_MAXT)
+k_run1(const __grid_constant__ ModalParams mp, const double *P, const double *Psi, const double *lams, const double *u,
+       const double *v, double *ou, double *ov, double dt, int steps, int own, int halo, int first, int last) {
+    extern __shared__ double smem[];
+    const int t = threadIdx.x, nt = blockDim.x, nx = mp.nx;
+    const int b0 = blockIdx.x * own, nown = min(own, nx - b0);
+    // the window [lo, lo + W) of the (periodically continued) line
+    const int lo = mp.per_x ? b0 - halo : max(0, b0 - halo);
+    const int W = (mp.per_x ? b0 + nown + halo : min(nx, b0 + nown + halo)) - lo;
+    double *wU = smem, *wV = wU + W * N1, *tr = wV + W * N1, *fl = tr + 4 * W;   // fl: gm, gp, qm, qp
+    double *sP = fl + 4 * W, *sPsi = sP + N1 * N1, *vec = sPsi + N1 * N1, *lam = vec + 4 * N1;
+    for (int i = t; i < N1 * N1; i += nt) { sP[i] = P[i]; sPsi[i] = Psi[i]; }
+    for (int i = t; i < N1; i += nt) {   // trace vectors: vL, vR, dL, dR
+        vec[i] = mp.d[0].eL[i];
+        vec[N1 + i] = mp.d[0].eR[i];
+        vec[2 * N1 + i] = mp.d[0].gL[i];
+        vec[3 * N1 + i] = mp.d[0].gR[i];
+    }
+    for (int i = t; i < RK_STAGES * 2 * N1; i += nt) lam[i] = lams[i];
+    const int e = t / N1, k = t - e * N1;
+    const bool on = e < W;
+    int ge = lo + (on ? e : 0);
+    if (mp.per_x) ge = (ge % nx + nx) % nx;
+    GDG_CHECK_INDEX(ge, 0, mp.ne, GDG_SITE_STAGE1_NB + 0, 0);
+    double Yu = on ? u[(size_t)ge * N1 + k] : 0.0, Yv = on ? v[(size_t)ge * N1 + k] : 0.0;
+    if (on) { wU[t] = Yu; wV[t] = Yv; }
+    __syncthreads();
+    if (first) {
+        Yu = Yv = 0.0;
+        if (on) {
+#pragma unroll
+            for (int i = 0; i < N1; ++i) {
+                Yu = fma(sP[k * N1 + i], wU[e * N1 + i], Yu);
+                Yv = fma(sP[k * N1 + i], wV[e * N1 + i], Yv);
+            }
+        }
+        __syncthreads();
+        if (on) { wU[t] = Yu; wV[t] = Yv; }
+        __syncthreads();
+    }
+    const double gLk = vec[2 * N1 + k], gRk = vec[3 * N1 + k], eLk = vec[k], eRk = vec[N1 + k];
+    for (int step = 0; step < steps; ++step) {
+        const double Nu = Yu, Nv = Yv;
+        for (int st = 0; st < RK_STAGES; ++st) {
+            // traces of the stage input: four sums an element
+            for (int i = t; i < 4 * W; i += nt) {
+                const int ee = i >> 2, j = i & 3;
+                const double *w = (j < 2 ? wV : wU) + ee * N1, *c = vec + j * N1;
+                double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+                for (int m = 0; m + 1 < N1; m += 2) {
+                    s0 = fma(c[m], w[m], s0);
+                    s1 = fma(c[m + 1], w[m + 1], s1);
+                }
+                if (N1 & 1) s0 = fma(c[N1 - 1], w[N1 - 1], s0);
+                tr[i] = s0 + s1;
+            }
+            __syncthreads();
+            for (int i = t; i < 2 * W; i += nt) {   // fluxes of the minus (0) and plus (1) face
+                const int ee = i >> 1, side = i & 1;
+                const double vi = tr[4 * ee + side], di = tr[4 * ee + 2 + side];
+                int nb = ee + 2 * side - 1;
+                bool wall = false;
+                if (nb < 0 || nb >= W) {   // the mesh's end, or the window's (whose values are not used)
+                    if (mp.per_x && W == nx && halo == 0) nb = nb < 0 ? W - 1 : 0;
+                    else { wall = true; nb = ee; }
+                }
+                const double vo = wall ? -vi : tr[4 * nb + 1 - side], dO = wall ? -di : tr[4 * nb + 3 - side];
+                double g, q;
+                flux(vi, di, vo, dO, mp.beta, mp.tau, mp.c2, mp.alt, side, wall, g, q);
+                fl[4 * ee + side] = g;
+                fl[4 * ee + 2 + side] = q;
+            }
+            __syncthreads();
+            if (on) {
+                const double sc = dt / (RK_STAGES - st), *f = fl + 4 * e, *L = lam + st * 2 * N1;
+                const double ru = fma(gLk, f[0], gRk * f[1]), rv = fma(eLk, f[2], eRk * f[3]);
+                const double nu = fma(sc, Yv, fma(L[N1 + k], ru, Nu));
+                Yv = fma(L[k], Yu, fma(sc, rv, Nv));
+                Yu = nu;
+                wU[t] = Yu;
+                wV[t] = Yv;
+            }
+            __syncthreads();
         }
     }
-    if (MODE == M_RHS) return;
-    double vL = 0, vR = 0, dL = 0, dR = 0;
+    if (on && e >= b0 - lo && e < b0 - lo + nown) {
+        if (last) {
+            double a = 0.0, c = 0.0;
 #pragma unroll
-    for (int k = 0; k < N1; ++k) {
-        b.oU[row + k] = Ru[k]; b.oV[row + k] = Rv[k];
-        vL += mp.d[0].eL[k] * Rv[k]; vR += mp.d[0].eR[k] * Rv[k];
-        dL += mp.d[0].gL[k] * Ru[k]; dR += mp.d[0].gR[k] * Ru[k];
+            for (int m = 0; m < N1; ++m) {
+                a = fma(sPsi[k * N1 + m], wU[e * N1 + m], a);
+                c = fma(sPsi[k * N1 + m], wV[e * N1 + m], c);
+            }
+            Yu = a;
+            Yv = c;
+        }
+        ou[(size_t)ge * N1 + k] = Yu;
+        ov[(size_t)ge * N1 + k] = Yv;
     }
-    b.trout[tix1(e, 0, 0)] = vL; b.trout[tix1(e, 0, 1)] = dL;
-    b.trout[tix1(e, 1, 0)] = vR; b.trout[tix1(e, 1, 1)] = dR;
 }
 
 template <int N1>
@@ -858,13 +965,8 @@ void launch_stage2(int mode, const ModalParams &mp, const StageBufs &b, double s
 }
 
 template <int N1>
-void launch_stage1(int mode, const ModalParams &mp, const StageBufs &b, double sc, cudaStream_t s) {
-    dim3 grid((mp.ne + TPB1 - 1) / TPB1), block(TPB1);
-    switch (mode) {
-    case M_RHS: k_stage1<N1, M_RHS><<<grid, block, 0, s>>>(mp, b, sc); break;
-    case M_S1: k_stage1<N1, M_S1><<<grid, block, 0, s>>>(mp, b, sc); break;
-    default: k_stage1<N1, M_S23><<<grid, block, 0, s>>>(mp, b, sc); break;
-    }
+void launch_stage1(const ModalParams &mp, const StageBufs &b, cudaStream_t s) {
+    k_stage1<N1><<<(mp.ne + TPB1 - 1) / TPB1, TPB1, 0, s>>>(mp, b);
 }
 
 void launch_stage_raw(const gdg_ctx *ctx, int mode, const StageBufs &b, double sc, cudaStream_t s) {
@@ -881,7 +983,7 @@ void launch_stage_raw(const gdg_ctx *ctx, int mode, const StageBufs &b, double s
         }
     } else {
         switch (n1) {
-#define X(n) case n: launch_stage1<n>(mode, ctx->mp, b, sc, s); break;
+#define X(n) case n: launch_stage1<n>(ctx->mp, b, s); break;
             GDG_N1_CASES(X)
 #undef X
         }
@@ -1068,6 +1170,9 @@ int set_smem_limits() {
     cudaFuncSetAttribute(k_sep2<n, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     GDG_N1_CASES(X)
 #undef X
+#define X(n) cudaFuncSetAttribute(k_run1<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    GDG_N1_CASES(X)
+#undef X
 #define X(n)                                                                                   \
     cudaFuncSetAttribute(k_step2r<n, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);    \
     cudaFuncSetAttribute(k_step2r<n, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
@@ -1138,6 +1243,49 @@ void enqueue_rk4_stage(gdg_ctx *ctx, int st, double dt, cudaStream_t s) {
 
 void enqueue_rk4_step(gdg_ctx *ctx, double dt, cudaStream_t s) {
     for (int st = 0; st < RK_STAGES; ++st) enqueue_rk4_stage(ctx, st, dt, s);
+}
+
+// nsteps of a 1-D mesh on the nodal (u, v) in place (k_run1)
+template <int N1>
+void run1_n(gdg_ctx *ctx, double *u, double *v, double dt, int nsteps, cudaStream_t s) {
+    const ModalParams &mp = ctx->mp;
+    const double *P = mat(ctx, 0, T_P), *Psi = mat(ctx, 0, T_PSI);
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+    const bool whole = mp.ne <= RUN1_WHOLE;
+    const int halo = whole ? 0 : RK_STAGES * RUN1_STEPS;
+    const int own = whole ? mp.ne : std::min(std::max(8, (mp.ne + sms - 1) / sms), RUN1_MAXT / N1 - 2 * halo);
+    const int grid = (mp.ne + own - 1) / own, threads = (((own + 2 * halo) * N1 + 31) / 32) * 32;
+    const size_t sm = run1_doubles(N1, own + 2 * halo) * sizeof(double);
+    const double *iu = u, *iv = v;
+    for (int done = 0; done < nsteps;) {
+        const int k = std::min(whole ? 4096 : RUN1_STEPS, nsteps - done);
+        const bool first = done == 0, last = done + k == nsteps;
+        done += k;
+        // a window reads its neighbours' elements: never written in place by the same launch
+        const int out = iu == buf(ctx, B_XU) ? B_YU : B_XU;
+        const bool nodal = last && (whole || !first);
+        double *ou = nodal ? u : buf(ctx, out), *ov = nodal ? v : buf(ctx, out + 1);
+        GDG_PROF(ctx, GDG_K_STAGE, s, (k_run1<N1><<<grid, threads, sm, s>>>(mp, P, Psi, ctx->d_lams, iu, iv, ou, ov, dt, k,
+                                                                            own, halo, first, nodal)));
+        iu = ou;
+        iv = ov;
+    }
+    if (iu != u) launch_sep(ctx, iu, iv, u, v, T_PSI, nullptr, -1, s);
+}
+
+int step_1d(gdg_ctx *ctx, double *u, double *v, double dt, int nsteps, cudaStream_t s) {
+    if (nsteps <= 0) {   // as the other routes: through the modified basis and back
+        launch_sep(ctx, u, v, buf(ctx, B_NU), buf(ctx, B_NV), T_P, nullptr, -1, s);
+        launch_sep(ctx, buf(ctx, B_NU), buf(ctx, B_NV), u, v, T_PSI, nullptr, -1, s);
+        return gdg_cuda_check(ctx, cudaGetLastError(), "gdg_step (1-D)");
+    }
+    switch (ctx->n1) {
+#define X(n) case n: run1_n<n>(ctx, u, v, dt, nsteps, s); break;
+        GDG_N1_CASES(X)
+#undef X
+    }
+    return gdg_cuda_check(ctx, cudaGetLastError(), "gdg_step (1-D)");
 }
 
 // ---------------------------------------------- nodal-state route ------
@@ -1577,6 +1725,7 @@ int gdg_const_step(gdg_ctx *ctx, double *u, double *v, double dt, int nsteps, cu
     int st;
     if (ctx->pb.route == GDG_ROUTE_NODAL) return step_nodal(ctx, u, v, dt, nsteps, s);
     stage_tables(ctx, dt, s);
+    if (ctx->dim == 1) return step_1d(ctx, u, v, dt, nsteps, s);
     launch_enter(ctx, u, v, buf(ctx, B_NU), buf(ctx, B_NV), ctx->d_tr, s);
     if ((st = gdg_cuda_check(ctx, cudaGetLastError(), "gdg_step prologue"))) return st;
     if (has_halo(ctx)) {   // partitioned mesh: stages launched one by one, exchanges between them
