@@ -574,6 +574,122 @@ k_step2r(const __grid_constant__ ModalParams mp, const double *lams, double *nU,
     }
 }
 
+// The persistent step with one thread per modal entry, for meshes whose
+// entries all fit the GPU at once.  A warp gets one FP64 instruction every 64
+// cycles whatever the other sub-partitions do, and a line of N1 = 9 entries is
+// about 130 of them: with few elements on an SM k_step2r is that chain, 4 us and
+// more a stage.  Here a stage is 5 (fluxes) + 2 + 8 (update) + 6 (traces)
+// instructions a warp, for about a quarter more FP64 instructions an element.
+// Every entry's arithmetic is stage2r's, operation for operation: bit-identical
+// results.  Threads of an element: NS = N1^2 rounded up to an even number, so
+// that the pairs of threads that swap a value share a warp.  N1 = 8..10 (4 N1
+// face points and 8 N1 half sums fit the threads of an element).
+constexpr int STEP2E_MINBLOCKS = 5, STEP2E_MAXT = 256;
+__host__ __device__ constexpr int step2e_stride(int n1) { return (n1 * n1 + 1) & ~1; }
+__host__ __device__ constexpr size_t step2e_doubles(int n1, int epb) {
+    return (size_t)epb * (16 * n1 + 2 * n1 * (n1 + 1)) + 4 * n1;
+}
+
+template <int N1, int ALT>
+__global__ void __launch_bounds__(STEP2E_MAXT, STEP2E_MINBLOCKS)
+k_step2e(const __grid_constant__ ModalParams mp, const double *lams, double *nU, double *nV, double *tr0, double *tr1,
+         double dt, int nsteps, int epb, unsigned *sync, unsigned long long limit_ns) {
+    constexpr int NA = N1 * N1, NE = (N1 + 1) / 2, NS = step2e_stride(N1);
+    extern __shared__ double smem[];
+    __shared__ int s_ok, s_cnt;
+    __shared__ int s_nb[4 * (STEP2E_MAXT / NS)];
+    const int t = threadIdx.x, le = t / NS, q = t - le * NS, l = q / N1, k = q - l * N1;
+    const int e = blockIdx.x * epb + le;
+    const bool valid = le < epb && e < mp.ne, entry = valid && q < NA;
+    double *F = smem + (le < epb ? le : 0) * (16 * N1 + 2 * N1 * (N1 + 1));   // [2][GA, GB, QA, QB][N1]
+    double *O = F + 8 * N1;                                                   // own traces [4 faces][v, d][N1]
+    double *tile = O + 8 * N1;
+    double *vec = smem + epb * (16 * N1 + 2 * N1 * (N1 + 1));                 // gL, eL of x, then of y
+    if (t < N1) {
+        vec[t] = mp.d[0].gL[t];
+        vec[N1 + t] = mp.d[0].eL[t];
+        vec[2 * N1 + t] = mp.d[1].gL[t];
+        vec[3 * N1 + t] = mp.d[1].eL[t];
+    }
+    neighbour_blocks(mp, epb, s_nb, &s_cnt);
+    // this thread's face point: direction fd, transverse mode fm, side; the neighbour across it
+    const int fd = q / (2 * N1), fm = (q - fd * 2 * N1) >> 1, side = q & 1;
+    const bool face = valid && q < 4 * N1;
+    int nb = -1;
+    if (face) {
+        const int n = fd ? mp.ny : mp.nx, per = fd ? mp.per_y : mp.per_x, ex = e % mp.nx, ey = e / mp.nx;
+        int x = (fd ? ey : ex) + 2 * side - 1;
+        if (per) x = x < 0 ? x + n : x >= n ? x - n : x;
+        if (x >= 0 && x < n) {
+            nb = fd ? x * mp.nx + ex : ey * mp.nx + x;
+            GDG_CHECK_ELEM2(nb, mp, GDG_SITE_STAGE2R_NB + 2 * fd + side);
+        }
+    }
+    // ... and half sum: direction td, transverse mode tm, field tf (0: slope of u, 1: value of v), parity tp
+    const int td = q / (4 * N1), tm = (q - td * 4 * N1) >> 2, tf = (q >> 1) & 1, tp = q & 1;
+    const bool sum = valid && q < 8 * N1;
+    const size_t at = (size_t)(valid ? e : 0) * NA + (q < NA ? q : 0);
+    double Ru = entry ? nU[at] : 0.0, Rv = entry ? nV[at] : 0.0;
+    if (sum) O[q] = __ldcg(tr0 + tix2<N1>(e, 0, 0, 0) + q);
+    __syncthreads();
+    const int nnb = s_cnt;
+    const double cex = mp.d[0].ceL[k], cey = mp.d[1].ceL[l < N1 ? l : 0];
+    const double *w = vec + (2 * td + tf) * N1;
+    unsigned round = 0;
+    for (int step = 0; step < nsteps; ++step) {
+        const double Nu = Ru, Nv = Rv;
+        for (int st = 0; st < RK_STAGES; ++st) {
+            const double *trin = st & 1 ? tr1 : tr0, *lam = lams + (size_t)st * 4 * NA;
+            double *trout = st & 1 ? tr0 : tr1;
+            const double sc = dt / (RK_STAGES - st);
+            double g = 0.0, qq = 0.0;
+            if (face) {
+                const int f = 2 * fd + side;
+                const double vi = O[(2 * f) * N1 + fm], di = O[(2 * f + 1) * N1 + fm];
+                const double vo = nb < 0 ? -vi : __ldcg(trin + tix2<N1>(nb, f ^ 1, 0, fm));
+                const double dO = nb < 0 ? -di : __ldcg(trin + tix2<N1>(nb, f ^ 1, 1, fm));
+                flux2(vi, di, vo, dO, mp.beta2, mp.tau2, ALT, side, nb < 0, g, qq);
+            }
+            const double go = __shfl_xor_sync(0xffffffffu, g, 1), qo = __shfl_xor_sync(0xffffffffu, qq, 1);
+            if (face) {   // the minus side keeps the sums, the plus side minus - plus
+                F[(4 * fd + side) * N1 + fm] = side ? go - g : g + go;
+                F[(4 * fd + 2 + side) * N1 + fm] = side ? qo - qq : qq + qo;
+            }
+            __syncthreads();
+            if (entry) {
+                const int px = k < NE ? 0 : 1, py = l < NE ? 0 : 1;
+                stage_entry<M_S23>(sc, lam[q], lam[2 * NA + q], lam[3 * NA + q], cex, sc * cey, F[px * N1 + l],
+                                   F[(2 + px) * N1 + l] * sc, F[(4 + py) * N1 + k], F[(6 + py) * N1 + k], Ru, Rv, Nu, Nv, Ru,
+                                   Rv);
+                tile[l * (N1 + 1) + k] = Ru;
+                tile[N1 * (N1 + 1) + l * (N1 + 1) + k] = Rv;
+            }
+            __syncthreads();
+            double s = 0.0;
+            if (sum) {
+                const double *T = tile + tf * N1 * (N1 + 1) + (td ? tm : tm * (N1 + 1));
+                const int inc = td ? N1 + 1 : 1, j0 = tp ? NE : 0, j1 = tp ? N1 : NE;
+#pragma unroll
+                for (int i = 0; i < NE; ++i)
+                    if (j0 + i < j1) s = fma(w[j0 + i], T[(j0 + i) * inc], s);
+            }
+            const double so = __shfl_xor_sync(0xffffffffu, s, 1);
+            if (sum) {   // left face: even + odd, right face: even - odd
+                const double v = tp ? so - s : s + so;
+                const int i = ((2 * td + tp) * 2 + 1 - tf) * N1 + tm;
+                O[i] = v;
+                trout[tix2<N1>(e, 0, 0, 0) + i] = v;
+            }
+            if (st + 1 == RK_STAGES && step + 1 == nsteps) break;
+            if (!neighbour_sync(sync, s_nb, nnb, ++round, limit_ns, &s_ok)) return;
+        }
+    }
+    if (entry) {
+        nU[at] = Ru;
+        nV[at] = Rv;
+    }
+}
+
 // Separable element transform: out = (Cy (x) Cx) diag(D) (By (x) Bx) in,
 // with C and D optional (nullptr).  Matrices are n1 x n1 row-major,
 // (A (x) B)[(l,k),(j,i)] = A[l][j] B[k][i].  Two fields per call (U and V
@@ -1078,6 +1194,39 @@ int persist_epb_n(const gdg_ctx *ctx) {
     return best;
 }
 
+// Elements per block of the entry-per-thread persistent step: the fewest warps
+// on the busiest SM among the choices whose grid is resident at once; 0 if none.
+template <int N1>
+int step2e_epb_n(const gdg_ctx *ctx) {
+    const ModalParams &mp = ctx->mp;
+    int coop = 0, sms = 0, best = 0;
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+    if (!coop || sms <= 0) return 0;
+    long long fewest = 0;
+    for (int epb = 1; epb * step2e_stride(N1) <= STEP2E_MAXT; ++epb) {
+        const int warps = (epb * step2e_stride(N1) + 31) / 32;
+        const long long blocks = (mp.ne + epb - 1) / epb, busiest = (blocks + sms - 1) / sms * warps;
+        int nb = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, mp.alt ? k_step2e<N1, 1> : k_step2e<N1, 0>, warps * 32,
+                                                          step2e_doubles(N1, epb) * sizeof(double)) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        if ((long long)nb * sms >= blocks && (!best || busiest < fewest)) { best = epb; fewest = busiest; }
+    }
+    return best;
+}
+
+int step2e_epb(const gdg_ctx *ctx) {
+    switch (ctx->n1) {
+    case 8: return step2e_epb_n<8>(ctx);
+    case 9: return step2e_epb_n<9>(ctx);
+    case 10: return step2e_epb_n<10>(ctx);
+    }
+    return 0;
+}
+
 int persist_epb(const gdg_ctx *ctx) {
     if (ctx->dim != 2 || !ctx->mp.parity || !ctx->d_sync) return 0;
     switch (ctx->n1) {
@@ -1089,11 +1238,37 @@ int persist_epb(const gdg_ctx *ctx) {
 }
 bool persist_fits(gdg_ctx *ctx) {
     ctx->mp.epbp = persist_epb(ctx);
+    ctx->epbe = ctx->mp.epbp > 0 ? step2e_epb(ctx) : 0;
     return ctx->mp.epbp > 0;
+}
+
+// The entry-per-thread persistent step wherever its grid fits.  32 steps, p = 5,
+// N1 = 9, k_step2r against k_step2e: 8^2 elements 677 and 487 us, 16^2 820 and
+// 545, 24^2 838 and 672, 32^2 1017 and 955, 44^2 1246..1433 and 1240; N1 = 10:
+// 32^2 1045 and 1050 (the one size where neither is faster), 40^2 1315 and 1303.
+template <int N1>
+bool launch_step2e_n(gdg_ctx *ctx, double dt, int nsteps, cudaStream_t s) {
+    if constexpr (N1 >= 8 && N1 <= 10) {
+        const ModalParams &mp = ctx->mp;
+        int epb = ctx->epbe;
+        if (epb < 1) return false;
+        const dim3 grid((mp.ne + epb - 1) / epb), block(((epb * step2e_stride(N1) + 31) / 32) * 32);
+        const double *lams = ctx->d_lams;
+        double *nU = buf(ctx, B_NU), *nV = buf(ctx, B_NV), *tr0 = ctx->d_tr, *tr1 = ctx->d_tr + ctx->tr_len;
+        unsigned *sync = ctx->d_sync;
+        unsigned long long lim = ctx->wait_limit_ns;
+        void *args[] = {(void *)&mp, (void *)&lams, (void *)&nU, (void *)&nV, (void *)&tr0, (void *)&tr1,
+                        (void *)&dt, (void *)&nsteps, (void *)&epb, (void *)&sync, (void *)&lim};
+        cudaLaunchCooperativeKernel(mp.alt ? (const void *)k_step2e<N1, 1> : (const void *)k_step2e<N1, 0>, grid, block,
+                                    args, step2e_doubles(N1, epb) * sizeof(double), s);
+        return true;
+    }
+    return false;
 }
 
 template <int N1>
 void launch_persist_n(gdg_ctx *ctx, double dt, int nsteps, cudaStream_t s) {
+    if (launch_step2e_n<N1>(ctx, dt, nsteps, s)) return;
     const ModalParams &mp = ctx->mp;
     const dim3 grid((mp.ne + mp.epbp - 1) / mp.epbp), block(mp.epbp * N1);
     const double *lams = ctx->d_lams;
@@ -1113,7 +1288,8 @@ void launch_persist(gdg_ctx *ctx, double dt, int nsteps, cudaStream_t s) {
     // at most 2^16 steps per launch keeps the barrier counters far from overflow
     for (int done = 0; done < nsteps;) {
         const int k = std::min(nsteps - done, 1 << 16);
-        cudaMemsetAsync(ctx->d_sync, 0, sync_words((ctx->mp.ne + ctx->mp.epbp - 1) / ctx->mp.epbp) * sizeof(unsigned), s);
+        const int epb = ctx->epbe > 0 ? ctx->epbe : ctx->mp.epbp;
+        cudaMemsetAsync(ctx->d_sync, 0, sync_words((ctx->mp.ne + epb - 1) / epb) * sizeof(unsigned), s);
         switch (ctx->n1) {
 #define X(n) case n: GDG_PROF(ctx, GDG_K_STAGE, s, launch_persist_n<n>(ctx, dt, k, s)); break;
             GDG_N1_CASES_P(X)

@@ -123,6 +123,7 @@ struct gdg_ctx {
     double *h_red = nullptr;      // pinned host scalar(s)
     cudaStream_t cap_stream = nullptr;
     GraphCache graph;
+    int epbe = 0;                 // elements per block of the entry-per-thread persistent step (0: not used)
     bool stage_tuned = false;     // stage kernel variant chosen (first gdg_step)
     unsigned *d_sync = nullptr;   // grid barrier of the persistent step: arrivals, give-up flag
     unsigned long long wait_limit_ns = 1000000000ull;   // bound on any device-side wait
