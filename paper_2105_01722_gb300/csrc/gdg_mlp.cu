@@ -58,24 +58,34 @@ struct MlpSmem {
 };
 static_assert(SWEND % 8 == 0, "16-byte aligned floats behind the weights");
 
-// weights and biases into shared memory (rows of 2-byte pairs: IN, HID are even)
+__device__ __forceinline__ void copy_async(void *dst, const void *src) {   // 4 bytes
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copies_done() {   // the caller's next barrier shows them to the block
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+}
+
+// weights and biases into shared memory (rows of 2-byte pairs: IN, HID are even);
+// the caller waits with copies_done and a barrier
 __device__ __forceinline__ void load_net(const __nv_bfloat16 *wb, const float *params, __nv_bfloat16 *w, float *b1,
                                          float *b2, float *b3) {
     if (reinterpret_cast<uintptr_t>(wb) & 3) {   // BF16s that do not start on a word: one at a time
         for (int i = threadIdx.x; i < HID * KP; i += blockDim.x)
             w[i] = i % KP < IN ? wb[i / KP * IN + i % KP] : __float2bfloat16(0.f);
         for (int i = threadIdx.x; i < (HID + OUT) * HID; i += blockDim.x) w[SW2 + i / HID * S2 + i % HID] = wb[WB_W2 + i];
-    }
-    const unsigned *src = reinterpret_cast<const unsigned *>(wb);
-    unsigned *dst = reinterpret_cast<unsigned *>(w);
-    const bool words = !(reinterpret_cast<uintptr_t>(wb) & 3);
-    for (int i = threadIdx.x; words && i < HID * KP / 2; i += blockDim.x) {
-        const int j = i / (KP / 2), k = i - j * (KP / 2);
-        dst[i] = k < IN / 2 ? src[j * (IN / 2) + k] : 0u;
-    }
-    for (int i = threadIdx.x; words && i < (HID + OUT) * (HID / 2); i += blockDim.x) {   // W2 and W3: rows of HID
-        const int j = i / (HID / 2), k = i - j * (HID / 2);
-        dst[SW2 / 2 + j * (S2 / 2) + k] = src[WB_W2 / 2 + i];
+    } else {   // word by word, asynchronously: every copy in flight at once, no register round trip
+        const unsigned *src = reinterpret_cast<const unsigned *>(wb);
+        unsigned *dst = reinterpret_cast<unsigned *>(w);
+        for (int i = threadIdx.x; i < HID * KP / 2; i += blockDim.x) {
+            const int j = i / (KP / 2), k = i - j * (KP / 2);
+            if (k < IN / 2) copy_async(dst + i, src + j * (IN / 2) + k);
+            else dst[i] = 0u;
+        }
+        for (int i = threadIdx.x; i < (HID + OUT) * (HID / 2); i += blockDim.x) {   // W2 and W3: rows of HID
+            const int j = i / (HID / 2), k = i - j * (HID / 2);
+            copy_async(dst + SW2 / 2 + j * (S2 / 2) + k, src + WB_W2 / 2 + i);
+        }
     }
     for (int i = threadIdx.x; i < HID; i += blockDim.x) {
         b1[i] = params[OFF_B1 + i];
@@ -151,6 +161,7 @@ k_mlp_forward(const __nv_bfloat16 *wb, const float *params, const float *X, int 
         const int n = i / KP, k = i - n * KP;
         s.x[i] = n < ns && k < IN ? X[(size_t)(n0 + n) * IN + k] : 0.f;
     }
+    copies_done();
     __syncthreads();
     forward_tile<SPB, 4>(s);
     for (int i = threadIdx.x; i < ns * OUT; i += blockDim.x) Y[(size_t)n0 * OUT + i] = s.y[i / OUT * MAXOUT + i % OUT];
@@ -158,7 +169,8 @@ k_mlp_forward(const __nv_bfloat16 *wb, const float *params, const float *X, int 
 
 // One minibatch: two kernels.  (One block of 32 samples computing its share of
 // every gradient left 144 of 152 SMs idle at 256 samples, and its weight reads,
-// 64 floats apart, hit one bank: 103 us; now 10 us for both.)
+// 64 floats apart, hit one bank: 103 us.  An iteration of 256 samples, both
+// kernels and Adam: 100 us then, 36 with plain loads of the weights, 29.6 now.)
 //
 // k_mlp_samples: 2 samples a block, so that 256 samples use 128 SMs.  Record of
 // a sample in `rec`: h1, h2, g1, g2, g3 (the errors before the layers'
@@ -180,6 +192,7 @@ k_mlp_samples(const __nv_bfloat16 *wb, const float *params, const float *X, cons
         const int n = i / KP, k = i - n * KP;
         s.x[i] = n0 + n < B && k < IN ? X[(size_t)(idx ? idx[n0 + n] : n0 + n) * IN + k] : 0.f;
     }
+    copies_done();
     __syncthreads();
     forward_tile<SPT, 1>(s);
     const int n = threadIdx.x >> 6, j = threadIdx.x & 63;
@@ -231,28 +244,33 @@ k_mlp_samples(const __nv_bfloat16 *wb, const float *params, const float *X, cons
 static_assert(OUT % 3 == 0 && HID % 2 == 0, "unrolled sums");
 
 // k_mlp_grad: dW = sum over the samples of (error) x (input of the layer), 16 x
-// 16 entries a block (4 a thread), samples staged 32 at a time; the first
-// input column's blocks also sum the bias, the last block the loss.  Fixed
-// order: deterministic.
-constexpr int GT = 16, GN = 32;
+// 16 entries a block.  Four groups of 64 threads (4 entries a thread) take the
+// samples 32 at a time in turn, the next 32 on their way from L2 meanwhile (a
+// single group spent 8 load latencies in a row at 256 samples: 26 us); the
+// groups' sums are added in order.  The first input column's blocks also sum
+// the bias, the last block the loss.  Fixed order: deterministic.
+constexpr int GT = 16, GN = 32, GG = 4;
 __host__ __device__ constexpr int tiles(int n) { return (n + GT - 1) / GT; }
 constexpr int T1 = tiles(HID) * tiles(IN), T2 = tiles(HID) * tiles(HID), T3 = tiles(OUT) * tiles(HID);
 
-__global__ void __launch_bounds__(64)
+__global__ void __launch_bounds__(64 * GG)
 k_mlp_grad(const float *X, const int *idx, const float *rec, int B, float *grad, float *loss) {
-    __shared__ float E[GN][GT], I[GN][GT];
-    const int t = threadIdx.x;
+    constexpr int LD = GN * GT / 64;   // values of a stage per thread
+    __shared__ float E[GG][GN][GT], I[GG][GN][GT];
+    __shared__ float part[GG][GT * GT + GT];
+    const int g = threadIdx.x >> 6, t = threadIdx.x & 63;
     int tile = blockIdx.x;
-    if (tile == T1 + T2 + T3) {   // loss: 64 partial sums, then in order
+    if (tile == T1 + T2 + T3) {   // loss: partial sums, then in order
         float l = 0.f;
-        for (int n = t; n < B; n += 64) l += rec[(size_t)n * REC + R_LOSS];
-        float *part = &E[0][0];
-        part[t] = l;
+        for (int n = threadIdx.x; n < B; n += 64 * GG) l += rec[(size_t)n * REC + R_LOSS];
+        part[0][threadIdx.x] = l;
         __syncthreads();
-        if (t == 0) {
+        if (threadIdx.x < 32) {
             float a = 0.f;
-            for (int i = 0; i < 64; ++i) a += part[i];
-            *loss = a;
+            for (int i = 0; i < 64 * GG / 32; ++i) a += part[0][threadIdx.x + 32 * i];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (threadIdx.x == 0) *loss = a;
         }
         return;
     }
@@ -263,27 +281,31 @@ k_mlp_grad(const float *X, const int *idx, const float *rec, int B, float *grad,
     const int tc = tiles(cols), r0 = (tile / tc) * GT, c0 = (tile - (tile / tc) * tc) * GT;
     const int r = (t >> 3) * 2, c = (t & 7) * 2;   // this thread's 2 x 2 entries
     float a[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, bias[2] = {0.f, 0.f};
-    for (int b0 = 0; b0 < B; b0 += GN) {
-        float e[GN * GT / 64], in[GN * GT / 64];
+    float e[LD], in[LD];
+    const int k = t % GT, n1 = t / GT;             // this thread's loads: column k of samples n1 + 4 i
+    auto load = [&](int b0) {
 #pragma unroll
-        for (int i = 0; i < GN * GT / 64; ++i) {
-            const int q = t + 64 * i, n = b0 + q / GT, k = q % GT;
+        for (int i = 0; i < LD; ++i) {
+            const int n = b0 + n1 + (64 / GT) * i;
             e[i] = n < B && r0 + k < rows ? rec[(size_t)n * REC + re + r0 + k] : 0.f;
             in[i] = n < B && c0 + k < cols
                         ? (ri < 0 ? X[(size_t)(idx ? idx[n] : n) * IN + c0 + k] : rec[(size_t)n * REC + ri + c0 + k])
                         : 0.f;
         }
+    };
+    load(g * GN);
+    for (int b0 = 0; b0 < B; b0 += GG * GN) {
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < GN * GT / 64; ++i) {
-            const int q = t + 64 * i;
-            E[q / GT][q % GT] = e[i];
-            I[q / GT][q % GT] = in[i];
+        for (int i = 0; i < LD; ++i) {
+            E[g][n1 + (64 / GT) * i][k] = e[i];
+            I[g][n1 + (64 / GT) * i][k] = in[i];
         }
         __syncthreads();
+        if (b0 + GG * GN < B) load(b0 + GG * GN + g * GN);
 #pragma unroll 8
         for (int n = 0; n < GN; ++n) {
-            const float2 ev = *reinterpret_cast<const float2 *>(&E[n][r]), iv = *reinterpret_cast<const float2 *>(&I[n][c]);
+            const float2 ev = *reinterpret_cast<const float2 *>(&E[g][n][r]), iv = *reinterpret_cast<const float2 *>(&I[g][n][c]);
             a[0][0] = fmaf(ev.x, iv.x, a[0][0]);
             a[0][1] = fmaf(ev.x, iv.y, a[0][1]);
             a[1][0] = fmaf(ev.y, iv.x, a[1][0]);
@@ -294,11 +316,22 @@ k_mlp_grad(const float *X, const int *idx, const float *rec, int B, float *grad,
     }
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-        if (r0 + r + i >= rows) continue;
 #pragma unroll
-        for (int k = 0; k < 2; ++k)
-            if (c0 + c + k < cols) grad[ow + (r0 + r + i) * cols + c0 + c + k] = a[i][k];
-        if (c0 == 0 && c == 0) grad[ob + r0 + r + i] = bias[i];
+        for (int q = 0; q < 2; ++q) part[g][(r + i) * GT + c + q] = a[i][q];
+        if (c == 0) part[g][GT * GT + r + i] = bias[i];
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < GT * GT + GT; q += 64 * GG) {
+        float s = part[0][q];
+#pragma unroll
+        for (int i = 1; i < GG; ++i) s += part[i][q];
+        const int row = q < GT * GT ? q / GT : q - GT * GT, col = q % GT;
+        if (r0 + row >= rows) continue;
+        if (q < GT * GT) {
+            if (c0 + col < cols) grad[ow + (r0 + row) * cols + c0 + col] = s;
+        } else if (c0 == 0) {
+            grad[ob + r0 + row] = s;
+        }
     }
 }
 
@@ -359,6 +392,7 @@ k_mlp_guess(const __nv_bfloat16 *wb, const float *params, const float *c2feat, c
         }
         s.x[i] = x;
     }
+    copies_done();
     __syncthreads();
     forward_tile<SPB, 4>(s);
     for (int i = threadIdx.x; i < ns * OUT; i += blockDim.x)
@@ -436,7 +470,7 @@ extern "C" int gdg_mlp_backward(const uint16_t *w_bf16, const float *params, con
     cudaStream_t s = (cudaStream_t)stream;
     k_mlp_samples<<<(B + SPT - 1) / SPT, TTHREADS, samples_smem(), s>>>(
         reinterpret_cast<const __nv_bfloat16 *>(w_bf16), params, X, T, idx, B, partial);
-    k_mlp_grad<<<T1 + T2 + T3 + 1, 64, 0, s>>>(X, idx, partial, B, grad, loss);
+    k_mlp_grad<<<T1 + T2 + T3 + 1, 64 * GG, 0, s>>>(X, idx, partial, B, grad, loss);
     return cudaGetLastError() == cudaSuccess ? GDG_OK : GDG_ECUDA;
 }
 
