@@ -863,30 +863,34 @@ k_stage1(const __grid_constant__ ModalParams mp, const StageBufs b) {
 // either side, since a stage carries information one element far: what the
 // window's open ends get wrong has not reached the owned ones when the launch
 // ends.  So one launch replaces 4 `steps` of them (and, for a mesh of one
-// window, every launch of the call: 16 elements, 16 steps 480 -> 45 us, the
-// 64 stages 0.6 us each where a launch took 7.5).
+// window, every launch of the call: 16 elements, p = 3, N1 = 9, 16 steps 480 ->
+// 101 us, 1.6 us a stage where a launch took 7.5).
 // `first`: u, v are nodal and enter through P; `last`: they leave through Psi;
 // else modal.  Bound by the latency of a stage's chain (update, trace sums,
-// fluxes: FP64 issues a warp instruction every 64 cycles of a sub-partition).
+// fluxes: a warp gets an FP64 instruction every 64 cycles, some 20 of them and
+// three barriers).  Even and odd modes apart: 113 -> 101 us.
 constexpr int RUN1_WHOLE = 32;   // largest mesh run by one block: above, windows on more SMs are faster
 constexpr int RUN1_STEPS = 2;    // steps a launch: window overlap (8 elements a step) against launches
 constexpr int RUN1_MAXT = 1024;
 
 __host__ __device__ constexpr size_t run1_doubles(int n1, int W) {
-    return (size_t)W * (2 * n1 + 8) + 2 * n1 * n1 + 4 * n1 + RK_STAGES * 2 * n1;
+    return (size_t)W * (2 * n1 + 8) + 2 * n1 * n1 + 4 * n1 + RK_STAGES * 3 * n1;
 }
 
-template <int N1>
+// PAR: modes even or odd, even ones first (as in the 2-D kernels): a face pair
+// lifts onto an entry with one product and a trace pair is one sum in two parts.
+template <int N1, bool PAR>
 __global__ void __launch_bounds__(RUN1_MAXT)
 k_run1(const __grid_constant__ ModalParams mp, const double *P, const double *Psi, const double *lams, const double *u,
        const double *v, double *ou, double *ov, double dt, int steps, int own, int halo, int first, int last) {
+    constexpr int NE = (N1 + 1) / 2;
     extern __shared__ double smem[];
-    const int t = threadIdx.x, nt = blockDim.x, nx = mp.nx;
+    const int t = threadIdx.x, nt = blockDim.x, nx = mp.nx, lane = t & 31, warp0 = t & ~31;
     const int b0 = blockIdx.x * own, nown = min(own, nx - b0);
     // the window [lo, lo + W) of the (periodically continued) line
     const int lo = mp.per_x ? b0 - halo : max(0, b0 - halo);
     const int W = (mp.per_x ? b0 + nown + halo : min(nx, b0 + nown + halo)) - lo;
-    double *wU = smem, *wV = wU + W * N1, *tr = wV + W * N1, *fl = tr + 4 * W;   // fl: gm, gp, qm, qp
+    double *wU = smem, *wV = wU + W * N1, *tr = wV + W * N1, *fl = tr + 4 * W;   // tr: vL, vR, dL, dR
     double *sP = fl + 4 * W, *sPsi = sP + N1 * N1, *vec = sPsi + N1 * N1, *lam = vec + 4 * N1;
     for (int i = t; i < N1 * N1; i += nt) { sP[i] = P[i]; sPsi[i] = Psi[i]; }
     for (int i = t; i < N1; i += nt) {   // trace vectors: vL, vR, dL, dR
@@ -895,7 +899,7 @@ k_run1(const __grid_constant__ ModalParams mp, const double *P, const double *Ps
         vec[2 * N1 + i] = mp.d[0].gL[i];
         vec[3 * N1 + i] = mp.d[0].gR[i];
     }
-    for (int i = t; i < RK_STAGES * 2 * N1; i += nt) lam[i] = lams[i];
+    for (int i = t; i < RK_STAGES * 3 * N1; i += nt) lam[i] = lams[i];
     const int e = t / N1, k = t - e * N1;
     const bool on = e < W;
     int ge = lo + (on ? e : 0);
@@ -904,39 +908,55 @@ k_run1(const __grid_constant__ ModalParams mp, const double *P, const double *Ps
     double Yu = on ? u[(size_t)ge * N1 + k] : 0.0, Yv = on ? v[(size_t)ge * N1 + k] : 0.0;
     if (on) { wU[t] = Yu; wV[t] = Yv; }
     __syncthreads();
-    if (first) {
+    if (first) {   // rows k > 0 of P sum to zero: from differences (line_transform, KIND 1)
         Yu = Yv = 0.0;
         if (on) {
+            const double ru = k ? wU[e * N1 + N1 / 2] : 0.0, rv = k ? wV[e * N1 + N1 / 2] : 0.0;
 #pragma unroll
             for (int i = 0; i < N1; ++i) {
-                Yu = fma(sP[k * N1 + i], wU[e * N1 + i], Yu);
-                Yv = fma(sP[k * N1 + i], wV[e * N1 + i], Yv);
+                Yu = fma(sP[k * N1 + i], wU[e * N1 + i] - ru, Yu);
+                Yv = fma(sP[k * N1 + i], wV[e * N1 + i] - rv, Yv);
             }
         }
         __syncthreads();
         if (on) { wU[t] = Yu; wV[t] = Yv; }
         __syncthreads();
     }
-    const double gLk = vec[2 * N1 + k], gRk = vec[3 * N1 + k], eLk = vec[k], eRk = vec[N1 + k];
+    const double gLk = vec[2 * N1 + k], gRk = vec[3 * N1 + k], eLk = vec[k], eRk = vec[N1 + k], ceL = mp.d[0].ceL[k];
     for (int step = 0; step < steps; ++step) {
         const double Nu = Yu, Nv = Yv;
         for (int st = 0; st < RK_STAGES; ++st) {
-            // traces of the stage input: four sums an element
-            for (int i = t; i < 4 * W; i += nt) {
-                const int ee = i >> 2, j = i & 3;
-                const double *w = (j < 2 ? wV : wU) + ee * N1, *c = vec + j * N1;
-                double s0 = 0.0, s1 = 0.0;
+            const double sc = dt / (RK_STAGES - st);
+            // traces of the stage input, four sums an element (PAR: even and odd
+            // parts, swapped between neighbouring lanes)
+            for (int i0 = warp0; i0 < 4 * W; i0 += nt) {   // (warps without a sum skip it)
+                const int i = i0 + lane, ee = min(i, 4 * W - 1) >> 2, f = (i >> 1) & 1, par = i & 1;   // f: 0 v, 1 u
+                const double *w = (f ? wU : wV) + ee * N1, *c = vec + (2 * f + (PAR ? 0 : par)) * N1;
+                double s = 0.0;
+                if (PAR) {
+                    const int m0 = par ? NE : 0, m1 = par ? N1 : NE;
 #pragma unroll
-                for (int m = 0; m + 1 < N1; m += 2) {
-                    s0 = fma(c[m], w[m], s0);
-                    s1 = fma(c[m + 1], w[m + 1], s1);
+                    for (int m = 0; m < NE; ++m)
+                        if (m0 + m < m1) s = fma(c[m0 + m], w[m0 + m], s);
+                    const double o = __shfl_xor_sync(0xffffffffu, s, 1);
+                    s = o + (par ? -s : s);
+                } else {
+                    double s1 = 0.0;
+#pragma unroll
+                    for (int m = 0; m + 1 < N1; m += 2) {
+                        s = fma(c[m], w[m], s);
+                        s1 = fma(c[m + 1], w[m + 1], s1);
+                    }
+                    if (N1 & 1) s = fma(c[N1 - 1], w[N1 - 1], s);
+                    s += s1;
                 }
-                if (N1 & 1) s0 = fma(c[N1 - 1], w[N1 - 1], s0);
-                tr[i] = s0 + s1;
+                if (i < 4 * W) tr[i] = s;
             }
             __syncthreads();
-            for (int i = t; i < 2 * W; i += nt) {   // fluxes of the minus (0) and plus (1) face
-                const int ee = i >> 1, side = i & 1;
+            // fluxes of the minus (0) and plus (1) face (PAR: doubled, their sums
+            // and differences, those of v times sc)
+            for (int i0 = warp0; i0 < 2 * W; i0 += nt) {
+                const int i = i0 + lane, ee = min(i, 2 * W - 1) >> 1, side = i & 1;
                 const double vi = tr[4 * ee + side], di = tr[4 * ee + 2 + side];
                 int nb = ee + 2 * side - 1;
                 bool wall = false;
@@ -946,16 +966,32 @@ k_run1(const __grid_constant__ ModalParams mp, const double *P, const double *Ps
                 }
                 const double vo = wall ? -vi : tr[4 * nb + 1 - side], dO = wall ? -di : tr[4 * nb + 3 - side];
                 double g, q;
-                flux(vi, di, vo, dO, mp.beta, mp.tau, mp.c2, mp.alt, side, wall, g, q);
-                fl[4 * ee + side] = g;
-                fl[4 * ee + 2 + side] = q;
+                if (PAR) {
+                    flux2(vi, di, vo, dO, mp.beta2, mp.tau2, mp.alt, side, wall, g, q);
+                    const double go = __shfl_xor_sync(0xffffffffu, g, 1), qo = __shfl_xor_sync(0xffffffffu, q, 1);
+                    g = go + (side ? -g : g);
+                    q = sc * (qo + (side ? -q : q));
+                } else {
+                    flux(vi, di, vo, dO, mp.beta, mp.tau, mp.c2, mp.alt, side, wall, g, q);
+                }
+                if (i < 2 * W) {
+                    fl[4 * ee + side] = g;
+                    fl[4 * ee + 2 + side] = q;
+                }
             }
             __syncthreads();
             if (on) {
-                const double sc = dt / (RK_STAGES - st), *f = fl + 4 * e, *L = lam + st * 2 * N1;
-                const double ru = fma(gLk, f[0], gRk * f[1]), rv = fma(eLk, f[2], eRk * f[3]);
-                const double nu = fma(sc, Yv, fma(L[N1 + k], ru, Nu));
-                Yv = fma(L[k], Yu, fma(sc, rv, Nv));
+                const double *f = fl + 4 * e, *L = lam + st * 3 * N1;
+                double nu;
+                if (PAR) {
+                    const int px = k < NE ? 0 : 1;
+                    nu = fma(sc, Yv, fma(L[2 * N1 + k], f[px], Nu));
+                    Yv = fma(L[k], Yu, fma(ceL, f[2 + px], Nv));
+                } else {
+                    const double ru = fma(gLk, f[0], gRk * f[1]), rv = fma(eLk, f[2], eRk * f[3]);
+                    nu = fma(sc, Yv, fma(L[N1 + k], ru, Nu));
+                    Yv = fma(L[k], Yu, fma(sc, rv, Nv));
+                }
                 Yu = nu;
                 wU[t] = Yu;
                 wV[t] = Yv;
@@ -994,10 +1030,11 @@ __global__ void k_traces1(const __grid_constant__ ModalParams mp, const double *
     trout[tix1(e, 1, 0)] = vR; trout[tix1(e, 1, 1)] = dR;
 }
 
-// out = C diag(D) B in  (1-D, two fields)
+// out = C diag(D) B in  (1-D, two fields); diff: B = P, whose rows k > 0 sum to
+// zero and are applied to differences (line_transform, KIND 1)
 template <int N1>
 __global__ void k_sep1(int ne, const double *in0, const double *in1, double *out0, double *out1,
-                       const double *B, const double *D, const double *C) {
+                       const double *B, const double *D, const double *C, bool diff) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= ne) return;
     const int nf = in1 ? 2 : 1;
@@ -1010,8 +1047,9 @@ __global__ void k_sep1(int ne, const double *in0, const double *in1, double *out
 #pragma unroll
         for (int k = 0; k < N1; ++k) {
             double s = 0;
+            const double ref = diff && k ? x[N1 / 2] : 0.0;
 #pragma unroll
-            for (int i = 0; i < N1; ++i) s += B[k * N1 + i] * x[i];
+            for (int i = 0; i < N1; ++i) s = fma(B[k * N1 + i], x[i] - ref, s);
             z[k] = D ? s * D[k] : s;
         }
         if (!C) {
@@ -1139,7 +1177,7 @@ void launch_sep_raw(const gdg_ctx *ctx, const double *in0, const double *in1, do
         dim3 grid((ctx->ne + TPB1 - 1) / TPB1), block(TPB1);
         const double *Bm = mat(ctx, 0, B), *Cm = C >= 0 ? mat(ctx, 0, C) : nullptr;
         switch (n1) {
-#define X(n) case n: k_sep1<n><<<grid, block, 0, s>>>(ctx->ne, in0, in1, out0, out1, Bm, D, Cm); if (tr) k_traces1<n><<<grid, block, 0, s>>>(ctx->mp, out0, out1, tr); break;
+#define X(n) case n: k_sep1<n><<<grid, block, 0, s>>>(ctx->ne, in0, in1, out0, out1, Bm, D, Cm, B == T_P); if (tr) k_traces1<n><<<grid, block, 0, s>>>(ctx->mp, out0, out1, tr); break;
             GDG_N1_CASES(X)
 #undef X
         }
@@ -1346,7 +1384,9 @@ int set_smem_limits() {
     cudaFuncSetAttribute(k_sep2<n, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     GDG_N1_CASES(X)
 #undef X
-#define X(n) cudaFuncSetAttribute(k_run1<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+#define X(n)                                                                                    \
+    cudaFuncSetAttribute(k_run1<n, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);   \
+    cudaFuncSetAttribute(k_run1<n, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     GDG_N1_CASES(X)
 #undef X
 #define X(n)                                                                                   \
@@ -1442,7 +1482,7 @@ void run1_n(gdg_ctx *ctx, double *u, double *v, double dt, int nsteps, cudaStrea
         const int out = iu == buf(ctx, B_XU) ? B_YU : B_XU;
         const bool nodal = last && (whole || !first);
         double *ou = nodal ? u : buf(ctx, out), *ov = nodal ? v : buf(ctx, out + 1);
-        GDG_PROF(ctx, GDG_K_STAGE, s, (k_run1<N1><<<grid, threads, sm, s>>>(mp, P, Psi, ctx->d_lams, iu, iv, ou, ov, dt, k,
+        GDG_PROF(ctx, GDG_K_STAGE, s, ((mp.parity ? k_run1<N1, true> : k_run1<N1, false>)<<<grid, threads, sm, s>>>(mp, P, Psi, ctx->d_lams, iu, iv, ou, ov, dt, k,
                                                                             own, halo, first, nodal)));
         iu = ou;
         iv = ov;
@@ -1660,7 +1700,7 @@ int gdg_const_setup(gdg_ctx *ctx) {
                 if (std::fabs(ctx->Psih[(n1 - 1 - i) * n1 + k] - sgn * ctx->Psih[i * n1 + k]) > 1e-9 * big) clean = false;
             (sgn > 0 ? even : odd).push_back(k);
         }
-        mp.parity = clean && (int)even.size() == (n1 + 1) / 2 && even[0] == 0 && ctx->dim >= 2;
+        mp.parity = clean && (int)even.size() == (n1 + 1) / 2 && even[0] == 0;
         if (mp.parity) {
             for (int k = 0; k < (int)even.size(); ++k) perm[k] = even[k];
             for (int k = 0; k < (int)odd.size(); ++k) perm[even.size() + k] = odd[k];
@@ -1720,18 +1760,19 @@ int gdg_const_setup(gdg_ctx *ctx) {
     mp.epbh = ctx->dim == 2 ? choose_epb(ctx->ne, n1, sms, 2 * n1) : 1;
     mp.split = 0;   // decided by timing at the first gdg_step (one-line kernel on partitioned meshes)
     const int ents = ctx->dim == 3 ? nn * n1 : (ctx->dim == 2 ? nn : n1);
-    // rows: -c^2 lambda, 1/lambda (0 on the constant mode); 2-D and 3-D also
-    // the u lifts folded with the diagonal solve, one row per direction:
+    // rows: -c^2 lambda, 1/lambda (0 on the constant mode), and the u lifts folded with the diagonal solve, one row per direction:
     // P1 = hgL_x/lambda, P2 = hgL_y/lambda (, P3 = hgL_z/lambda), which the
     // parity stage kernels apply
-    std::vector<double> l2((size_t)(ctx->dim == 2 ? 4 : (ctx->dim == 3 ? 5 : 2)) * ents, 0.0);
+    std::vector<double> l2((size_t)(ctx->dim + 2) * ents, 0.0);
     for (int m = 0; m < ents; ++m) {
         double L = ctx->dim == 3   ? lam[0][m % n1] + lam[1][(m / n1) % n1] + lam[2][m / nn]
                    : ctx->dim == 2 ? lam[0][m % n1] + lam[1][m / n1]
                                    : lam[0][m];
         l2[m] = -ctx->pb.c2 * L;
         l2[ents + m] = m == 0 ? 0.0 : 1.0 / L;
-        if (ctx->dim == 2) {
+        if (ctx->dim == 1) {
+            l2[2 * ents + m] = l2[ents + m] * mp.d[0].hgL[m];
+        } else if (ctx->dim == 2) {
             l2[2 * ents + m] = l2[ents + m] * mp.d[0].hgL[m % n1];
             l2[3 * ents + m] = l2[ents + m] * mp.d[1].hgL[m / n1];
         } else if (ctx->dim == 3) {   // m = (mz n1 + my) n1 + mx
