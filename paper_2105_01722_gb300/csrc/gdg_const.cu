@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "gdg_checks.cuh"
+#include "gdg_fxline.cuh"
 #include "gdg_internal.h"
 #include "gdg_stage_const.cuh"
 
@@ -690,13 +691,87 @@ k_step2e(const __grid_constant__ ModalParams mp, const double *lams, double *nU,
     }
 }
 
+// Nodes to modes or modes to nodes on the integer pipe (gdg_fxline.cuh), a line
+// of one field of an element a thread: rows through the table of x, then
+// columns through that of y.  tr (modal output (U, V)): also its face traces.
+// 97 x 70 elements, N1 = 9, both fields: 18 us in with the traces and 15 us out,
+// where FP64 lines by node pairs took 39 and 29 (its pipe was the bound).  Now
+// latency between barriers (issue 30 to 36 %) and, for the traces, the FP64 pipe.
+constexpr int FX2_THREADS = 128;
+template <int N1> __host__ __device__ constexpr int fx2_tile() { return N1 * (N1 | 1); }   // odd row stride: no bank conflicts
+
+template <int N1, int KIND>
+__global__ void __launch_bounds__(FX2_THREADS)
+k_fx2(const __grid_constant__ ModalParams mp, const __grid_constant__ FxLines<N1, 2> A, const double *in0,
+      const double *in1, double *out0, double *out1, double *tr, int epb) {
+    constexpr int NA = N1 * N1, LS = N1 | 1, TILE = fx2_tile<N1>();
+    extern __shared__ long long fx_tiles[];   // [field][element][TILE]
+    __shared__ int smax[FX2_THREADS / N1], sbits[FX2_THREADS / N1];
+    const int nf = in1 ? 2 : 1, groups = nf * epb;
+    const int t = threadIdx.x, g = t / N1, l = t - g * N1, f = g >= epb ? 1 : 0;
+    const int e = blockIdx.x * epb + g - f * epb;
+    const bool valid = g < groups && e < mp.ne;
+    const size_t base = (size_t)blockIdx.x * epb * NA;
+    const int count = min(epb, mp.ne - (int)blockIdx.x * epb) * NA;
+    if (t < groups) smax[t] = sbits[t] = 0;
+    for (int k = 0; k < nf; ++k)
+        for (int i = t; i < count; i += blockDim.x)
+            fx_tiles[k * epb * TILE + i + i / N1 * (LS - N1)] = __double_as_longlong((k ? in1 : in0)[base + i]);
+    __syncthreads();
+    long long *T = fx_tiles + g * TILE;
+    int h[N1], x[N1];
+    if (valid) {
+        int m = 0;
+#pragma unroll
+        for (int i = 0; i < N1; ++i) m = max(m, fx_expo(__longlong_as_double(T[l * LS + i])));
+        atomicMax(&smax[g], m);
+    }
+    __syncthreads();
+    const int emax = valid ? smax[g] : 0;
+    if (valid) {
+#pragma unroll
+        for (int i = 0; i < N1; ++i) fx_limbs(__longlong_as_double(T[l * LS + i]), emax, h[i], x[i]);
+        int m = 0;
+        fx_line<N1, KIND>(A.a[0], h, x, [&](int q, long long Y) { T[l * LS + q] = Y; m |= fx_bits(Y); });
+        atomicOr(&sbits[g], m);
+    }
+    __syncthreads();
+    if (valid) {
+        const int len = fx_length(sbits[g]);
+#pragma unroll
+        for (int i = 0; i < N1; ++i) fx_limbs(T[i * LS + l] << (62 - len), h[i], x[i]);
+        const int q0 = (emax - 1022) + (A.pe[0] + len - 57) + A.pe[1] - 57;
+        const bool nan = emax == 0x7ff, plain = !nan && fx_plain(q0);
+        LineTraces<N1, true> ty(f ? mp.d[1].eL : mp.d[1].gL, nullptr);
+        fx_line<N1, KIND>(A.a[1], h, x, [&](int q, long long Y) {
+            const double v = fx_double(Y, q0, plain, nan);
+            T[q * LS + l] = __double_as_longlong(v);
+            if (KIND == FX_TO_MODES && tr) ty.add(q, v);
+        });
+        if (KIND == FX_TO_MODES && tr) {
+            tr[tix2<N1>(e, 2, 1 - f, l)] = ty.left();
+            tr[tix2<N1>(e, 3, 1 - f, l)] = ty.right();
+        }
+    }
+    __syncthreads();
+    for (int k = 0; k < nf; ++k)
+        for (int i = t; i < count; i += blockDim.x)
+            (k ? out1 : out0)[base + i] = __longlong_as_double(fx_tiles[k * epb * TILE + i + i / N1 * (LS - N1)]);
+    if (KIND == FX_TO_MODES && tr && valid) {
+        LineTraces<N1, true> tx(f ? mp.d[0].eL : mp.d[0].gL, nullptr);
+#pragma unroll
+        for (int k = 0; k < N1; ++k) tx.add(k, __longlong_as_double(T[l * LS + k]));
+        tr[tix2<N1>(e, 0, 1 - f, l)] = tx.left();
+        tr[tix2<N1>(e, 1, 1 - f, l)] = tx.right();
+    }
+}
+
 // Separable element transform: out = (Cy (x) Cx) diag(D) (By (x) Bx) in,
-// with C and D optional (nullptr).  Matrices are n1 x n1 row-major,
+// with C and D optional (nullptr; KB == 3 has C).  Matrices are n1 x n1 row-major,
 // (A (x) B)[(l,k),(j,i)] = A[l][j] B[k][i].  Two fields per call (U and V
 // share the matrices); tr (modal output (U, V)): also its face traces.
-// KB: the kind of B (line_transform); C is of kind 2 when B is of kind 3.
-// Bound by the FP64 pipe: 97 x 70 elements, N1 = 9, both fields: 39 us in with the traces, 29 us out (dense lines
-// 42 us, and 15 us for the traces in a kernel of their own).
+// KB: the kind of B (line_transform); C is of kind 2 when B is of kind 3.  Bound
+// by the FP64 pipe; with parity P and Psi alone go through k_fx2.
 template <int N1, int KB>
 __global__ void __launch_bounds__(MAXB2)
 k_sep2(const __grid_constant__ ModalParams mp, const double *in0, const double *in1, double *out0, double *out1,
@@ -739,7 +814,7 @@ k_sep2(const __grid_constant__ ModalParams mp, const double *in0, const double *
 #pragma unroll
         for (int j = 0; j < N1; ++j) x[j] = T[j * (N1 + 1) + l];
         if (!Cx) {   // the tile keeps the column for the x faces; the y faces come from it here
-            LineTraces<N1, KB != 0> tc(f ? mp.d[1].eL : mp.d[1].gL, f ? mp.d[1].eR : mp.d[1].gR);
+            LineTraces<N1, false> tc(f ? mp.d[1].eL : mp.d[1].gL, f ? mp.d[1].eR : mp.d[1].gR);
             line_transform<N1, KB>(sB + N1 * N1, x, [&](int m, double v) {
                 T[m * (N1 + 1) + l] = v;
                 out[((size_t)e * N1 + m) * N1 + l] = v;
@@ -772,7 +847,7 @@ k_sep2(const __grid_constant__ ModalParams mp, const double *in0, const double *
                 out[row + q] = v;
             });
         } else {    // x faces
-            LineTraces<N1, KB != 0> tc(f ? mp.d[0].eL : mp.d[0].gL, f ? mp.d[0].eR : mp.d[0].gR);
+            LineTraces<N1, false> tc(f ? mp.d[0].eL : mp.d[0].gL, f ? mp.d[0].eR : mp.d[0].gR);
 #pragma unroll
             for (int k = 0; k < N1; ++k) tc.add(k, T[l * (N1 + 1) + k]);
             tr[tix2<N1>(e, 0, 1 - f, l)] = tc.left();
@@ -908,7 +983,7 @@ k_run1(const __grid_constant__ ModalParams mp, const double *P, const double *Ps
     double Yu = on ? u[(size_t)ge * N1 + k] : 0.0, Yv = on ? v[(size_t)ge * N1 + k] : 0.0;
     if (on) { wU[t] = Yu; wV[t] = Yv; }
     __syncthreads();
-    if (first) {   // rows k > 0 of P sum to zero: from differences (line_transform, KIND 1)
+    if (first) {   // rows k > 0 of P sum to zero: from differences (fx_line has the reason)
         Yu = Yv = 0.0;
         if (on) {
             const double ru = k ? wU[e * N1 + N1 / 2] : 0.0, rv = k ? wV[e * N1 + N1 / 2] : 0.0;
@@ -1031,7 +1106,7 @@ __global__ void k_traces1(const __grid_constant__ ModalParams mp, const double *
 }
 
 // out = C diag(D) B in  (1-D, two fields); diff: B = P, whose rows k > 0 sum to
-// zero and are applied to differences (line_transform, KIND 1)
+// zero and are applied to differences (fx_line has the reason)
 template <int N1>
 __global__ void k_sep1(int ne, const double *in0, const double *in1, double *out0, double *out1,
                        const double *B, const double *D, const double *C, bool diff) {
@@ -1150,6 +1225,119 @@ const double *mat(const gdg_ctx *ctx, int dir, int which) {
 }
 enum { T_P = 0, T_PSI = 1, T_PSIT = 2 };
 
+// hi + lo, lo below half a unit of hi: the setup's sums to twice the precision
+// (volatile: no fused multiply-add may take the place of a product and a sum)
+struct Twofold {
+    double hi = 0.0, lo = 0.0;
+    void add(double x) {
+        volatile double s = hi + x;
+        const volatile double b = s - hi, e1 = s - b, e2 = x - b;
+        lo += (hi - e1) + e2;
+        hi = s;
+    }
+    void mad(double a, double b) {
+        const volatile double p = a * b;
+        add(p);
+        lo += std::fma(a, b, -p);
+    }
+    void mad(const Twofold &a, double b) {
+        mad(a.hi, b);
+        lo += a.lo * b;
+    }
+    Twofold settled() const {
+        Twofold r;
+        r.hi = hi;
+        r.add(lo);
+        return r;
+    }
+};
+
+// Modes of the unit element from eigenvectors of clean parity (columns, even
+// ones first): exactly even and odd, the first one exactly constant, and
+// orthonormal in M to beyond double precision by one Newton step, so that a
+// transform and its inverse differ by their own rounding only.  P = Psi^T M.
+void parity_modes(int n1, std::vector<double> &M, const std::vector<double> &V, std::vector<Twofold> &Psi,
+                  std::vector<Twofold> &P) {
+    const int ne = (n1 + 1) / 2, nn = n1 * n1;
+    std::vector<double> A(nn), S(nn);
+    for (int i = 0; i < nn; ++i) S[i] = 0.5 * (M[i] + M[nn - 1 - i]);   // M itself is symmetric under r -> 1 - r
+    M = S;
+    double sum = 0.0;
+    for (int i = 0; i < nn; ++i) sum += M[i];
+    for (int k = 0; k < n1; ++k)
+        for (int i = 0; i < n1; ++i)
+            A[i * n1 + k] = k == 0 ? 1.0 / std::sqrt(sum) : 0.5 * (V[i * n1 + k] + (k < ne ? 1.0 : -1.0) * V[(n1 - 1 - i) * n1 + k]);
+    // R = A^T M A - 1; A -= A R / 2, but all of a mode's part along the constant one
+    std::vector<Twofold> W(nn);
+    for (int a = 0; a < n1; ++a)
+        for (int k = 0; k < n1; ++k) {
+            for (int b = 0; b < n1; ++b) W[a * n1 + k].mad(M[a * n1 + b], A[b * n1 + k]);
+            W[a * n1 + k] = W[a * n1 + k].settled();
+        }
+    Psi.assign(nn, Twofold());
+    P.assign(nn, Twofold());
+    for (int i = 0; i < nn; ++i) Psi[i].hi = A[i];
+    for (int k = 0; k < n1; ++k)
+        for (int j = 0; j < n1; ++j) {
+            if ((j < ne) != (k < ne) || (k == 0 && j != 0)) continue;
+            Twofold r;
+            for (int a = 0; a < n1; ++a) r.mad(W[a * n1 + k], A[a * n1 + j]);
+            if (j == k) r.add(-1.0);
+            const double c = (j == 0 && k != 0 ? -1.0 : -0.5) * (r.hi + r.lo);
+            for (int i = 0; i < n1; ++i) Psi[i * n1 + k].mad(c, A[i * n1 + j]);
+        }
+    for (int k = 0; k < n1; ++k)   // from one half, so that both are alike to the last bit
+        for (int i = 0; i < n1; ++i) {
+            Twofold t = Psi[std::min(i, n1 - 1 - i) * n1 + k].settled();
+            if (i > n1 - 1 - i && k >= ne) { t.hi = -t.hi; t.lo = -t.lo; }
+            Psi[i * n1 + k] = t;
+        }
+    for (int k = 0; k < n1; ++k)
+        for (int i = 0; i < n1; ++i) {
+            for (int a = 0; a < n1; ++a) P[k * n1 + i].mad(Psi[a * n1 + k], M[a * n1 + i]);
+            P[k * n1 + i] = P[k * n1 + i].settled();
+        }
+}
+
+// one transform table as integers (FxLines): P's rows by their first halves,
+// or the first half of Psi's rows
+void fx_line_table(const std::vector<Twofold> &A, int n1, bool to_modes, int2 *a, int &pe) {
+    const int ne = (n1 + 1) / 2;
+    double big = 0.0, sum = 0.0;   // largest entry, largest sum of a row
+    for (int q = 0; q < n1; ++q) {
+        double s = 0.0;
+        for (int i = 0; i < n1; ++i) {
+            big = std::max(big, std::fabs(A[q * n1 + i].hi));
+            s += std::fabs(A[q * n1 + i].hi);
+        }
+        sum = std::max(sum, s);
+    }
+    big = std::max(big, 0.125 * sum);
+    pe = big > 0.0 && std::isfinite(big) ? std::ilogb(big) + 1 : 0;
+    for (int k = 0; k < n1 * ne; ++k) {
+        const Twofold &t = A[to_modes ? k / ne * n1 + k % ne : k];
+        const double hi = std::scalbn(t.hi, 57 - pe), whole = std::rint(hi);
+        const long long v = (long long)whole + std::llrint((hi - whole) + std::scalbn(t.lo, 57 - pe));
+        const long long lo = ((v + (1ll << 28)) & ((1ll << 29) - 1)) - (1ll << 28);
+        a[k] = make_int2((int)((v - lo) >> 29), (int)lo);
+    }
+}
+
+template <int N1>
+void launch_fx2(const gdg_ctx *ctx, int kind, const double *in0, const double *in1, double *out0, double *out1,
+                double *tr, cudaStream_t s) {
+    constexpr int LEN = N1 * ((N1 + 1) / 2);
+    FxLines<N1, 2> A;
+    for (int d = 0; d < 2; ++d) {
+        std::copy(ctx->fx.a[d][kind - 1], ctx->fx.a[d][kind - 1] + LEN, A.a[d]);
+        A.pe[d] = ctx->fx.pe[d][kind - 1];
+    }
+    // blocks of up to 128 threads, smaller where that leaves SMs without one
+    const int nf = in1 ? 2 : 1, sms = 152, epb = std::max(1, std::min(FX2_THREADS / (2 * N1), ctx->ne / (2 * sms)));
+    (kind == FX_TO_MODES ? k_fx2<N1, FX_TO_MODES> : k_fx2<N1, FX_TO_NODES>)<<<(ctx->ne + epb - 1) / epb, nf * epb * N1,
+        (size_t)nf * epb * fx2_tile<N1>() * sizeof(double), s>>>(ctx->mp, A, in0, in1, out0, out1, tr, epb);
+}
+
 // out = (C) diag(D) (B) in, over both fields when in1 != nullptr; tr: the face
 // traces of the modal result (out0, out1) too (B = T_P)
 void launch_sep_raw(const gdg_ctx *ctx, const double *in0, const double *in1, double *out0, double *out1,
@@ -1157,6 +1345,20 @@ void launch_sep_raw(const gdg_ctx *ctx, const double *in0, const double *in1, do
     const int n1 = ctx->n1;
     // with parity every use is nodes to modes (P, Psi^T), then modes to nodes (Psi) or nothing
     const int kind = !ctx->mp.parity ? 0 : B == T_PSI ? 2 : B == T_P ? 1 : 3;
+    if (kind == FX_TO_MODES || kind == FX_TO_NODES) {
+        if (ctx->dim == 3) {
+            gdg3_fx(ctx->mp, n1, kind, ctx->fx, in0, in1, out0, out1, tr, s);
+            return;
+        }
+        if (ctx->dim == 2) {
+            switch (n1) {
+#define X(n) case n: launch_fx2<n>(ctx, kind, in0, in1, out0, out1, tr, s); break;
+                GDG_N1_CASES(X)
+#undef X
+            }
+            return;
+        }
+    }
     if (ctx->dim == 3) {
         gdg3_sep(ctx->mp, n1, kind, in0, in1, out0, out1, mat(ctx, 0, B), mat(ctx, 1, B), mat(ctx, 2, B), D,
                  C >= 0 ? mat(ctx, 0, C) : nullptr, C >= 0 ? mat(ctx, 1, C) : nullptr,
@@ -1169,7 +1371,7 @@ void launch_sep_raw(const gdg_ctx *ctx, const double *in0, const double *in1, do
         const double *Bx = mat(ctx, 0, B), *By = mat(ctx, 1, B);
         const double *Cx = C >= 0 ? mat(ctx, 0, C) : nullptr, *Cy = C >= 0 ? mat(ctx, 1, C) : nullptr;
         switch (n1) {
-#define X(n) case n: (kind == 0 ? k_sep2<n, 0> : kind == 1 ? k_sep2<n, 1> : kind == 2 ? k_sep2<n, 2> : k_sep2<n, 3>)<<<grid, block, smem_sep2(n, epb), s>>>(ctx->mp, in0, in1, out0, out1, Bx, By, D, Cx, Cy, tr); break;
+#define X(n) case n: (kind == 0 ? k_sep2<n, 0> : k_sep2<n, 3>)<<<grid, block, smem_sep2(n, epb), s>>>(ctx->mp, in0, in1, out0, out1, Bx, By, D, Cx, Cy, tr); break;
             GDG_N1_CASES(X)
 #undef X
         }
@@ -1379,8 +1581,6 @@ int set_smem_limits() {
     cudaFuncSetAttribute(k_stage2f<n, M_S1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage2f<n, M_S23, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
     cudaFuncSetAttribute(k_sep2<n, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);        \
-    cudaFuncSetAttribute(k_sep2<n, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);        \
-    cudaFuncSetAttribute(k_sep2<n, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);        \
     cudaFuncSetAttribute(k_sep2<n, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     GDG_N1_CASES(X)
 #undef X
@@ -1708,36 +1908,46 @@ int gdg_const_setup(gdg_ctx *ctx) {
             for (int k = 0; k < n1; ++k) perm[k] = k;
         }
     }
+    std::vector<Twofold> unitPsi(nn), unitP(nn);
+    if (mp.parity) {
+        std::vector<double> M(ctx->Mh), V(nn);
+        for (int i = 0; i < n1; ++i)
+            for (int k = 0; k < n1; ++k) V[i * n1 + k] = ctx->Psih[i * n1 + perm[k]];
+        parity_modes(n1, M, V, unitPsi, unitP);
+    }
     std::vector<double> tables((size_t)3 * 3 * nn, 0.0);
     std::vector<double> lam[3];
     for (int d = 0; d < ctx->dim; ++d) {
         const double H = (ctx->pb.hi[d] - ctx->pb.lo[d]) / ctx->pb.n_elem[d];
         const double sq = std::sqrt(H);
-        std::vector<double> Psi(nn), M(nn);
-        for (int i = 0; i < n1; ++i)
-            for (int k = 0; k < n1; ++k) Psi[i * n1 + k] = ctx->Psih[i * n1 + perm[k]] / sq;
-        if (mp.parity)   // exactly even and odd modes: the transforms read one half of each
+        double *P = &tables[((size_t)d * 3 + T_P) * nn];
+        double *Psi = &tables[((size_t)d * 3 + T_PSI) * nn];
+        double *PT = &tables[((size_t)d * 3 + T_PSIT) * nn];
+        if (mp.parity) {   // Psi = unit Psi / sqrt(H), P = Psi^T (H M)
+            std::vector<Twofold> fPsi(nn), fP(nn);
+            for (int i = 0; i < nn; ++i) {
+                fPsi[i].hi = unitPsi[i].hi / sq;
+                fPsi[i].lo = (std::fma(-fPsi[i].hi, sq, unitPsi[i].hi) + unitPsi[i].lo) / sq;
+                fP[i].mad(unitP[i], sq);
+                fP[i] = fP[i].settled();
+                Psi[i] = fPsi[i].hi;
+                P[i] = fP[i].hi;
+            }
+            fx_line_table(fP, n1, true, ctx->fx.a[d][FX_TO_MODES - 1], ctx->fx.pe[d][FX_TO_MODES - 1]);
+            fx_line_table(fPsi, n1, false, ctx->fx.a[d][FX_TO_NODES - 1], ctx->fx.pe[d][FX_TO_NODES - 1]);
+        } else {
+            for (int i = 0; i < nn; ++i) Psi[i] = ctx->Psih[i] / sq;
             for (int k = 0; k < n1; ++k)
-                for (int i = 0; i <= (n1 - 1) / 2; ++i) {
-                    const double sgn = k < (n1 + 1) / 2 ? 1.0 : -1.0;
-                    const double a = 0.5 * (Psi[i * n1 + k] + sgn * Psi[(n1 - 1 - i) * n1 + k]);
-                    Psi[i * n1 + k] = a;
-                    Psi[(n1 - 1 - i) * n1 + k] = sgn * a;
+                for (int i = 0; i < n1; ++i) {
+                    double s = 0;
+                    for (int a = 0; a < n1; ++a) s += Psi[a * n1 + k] * (H * ctx->Mh[a * n1 + i]);
+                    P[k * n1 + i] = s;             // Psi^T M
                 }
-        for (int i = 0; i < nn; ++i) M[i] = H * ctx->Mh[i];
+        }
+        for (int k = 0; k < n1; ++k)
+            for (int i = 0; i < n1; ++i) PT[k * n1 + i] = Psi[i * n1 + k];
         lam[d].resize(n1);
         for (int k = 0; k < n1; ++k) lam[d][k] = ctx->lamh[perm[k]] / (H * H);
-        double *P = &tables[((size_t)d * 3 + T_P) * nn];
-        double *Ps = &tables[((size_t)d * 3 + T_PSI) * nn];
-        double *PT = &tables[((size_t)d * 3 + T_PSIT) * nn];
-        for (int k = 0; k < n1; ++k)
-            for (int i = 0; i < n1; ++i) {
-                double s = 0;
-                for (int a = 0; a < n1; ++a) s += Psi[a * n1 + k] * M[a * n1 + i];
-                P[k * n1 + i] = s;             // Psi^T M
-                Ps[i * n1 + k] = Psi[i * n1 + k];
-                PT[k * n1 + i] = Psi[i * n1 + k];
-            }
         ModalDir &md = mp.d[d];
         for (int k = 0; k < n1; ++k) {
             md.eL[k] = Psi[0 * n1 + k];

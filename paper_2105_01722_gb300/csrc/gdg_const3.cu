@@ -7,6 +7,7 @@
 #include <algorithm>
 
 #include "gdg_checks.cuh"
+#include "gdg_fxline.cuh"
 #include "gdg_internal.h"
 #include "gdg_stage_const.cuh"
 
@@ -336,11 +337,104 @@ k_stage3p(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) 
     }
 }
 
+// Nodes to modes or modes to nodes on the integer pipe (gdg_fxline.cuh), one
+// line of an element a thread and pass; tr (modal output (U, V)): also its face
+// traces.  32^3 elements, N1 = 9, both fields: 572 us in with the traces (FP64
+// pipe 66 %, those sums and the conversions to doubles; issue 40 %) and 483 us
+// out (issue 44 %), where FP64 lines by node pairs took 2115 and 1641.
+template <int N1, int KIND>
+__global__ void __launch_bounds__(MAXB3, 4)
+k_fx3(const __grid_constant__ ModalParams mp, const __grid_constant__ FxLines<N1, 3> A, const double *in0,
+      const double *in1, double *out0, double *out1, double *tr) {
+    constexpr int NT = N1 * N1, NA = N1 * N1 * N1, EPB = epb3c<N1>();
+    extern __shared__ long long fx_tiles[];
+    __shared__ int slot[2][3][EPB];   // per field and element: largest exponent, bits after x, after y
+    const int t = threadIdx.x, le = t / NT, r = t - le * NT, a = r / N1, c = r - a * N1;
+    const int e = blockIdx.x * EPB + le;
+    const bool valid = e < mp.ne;     // blockDim.x == EPB * NT
+    const size_t base = (size_t)blockIdx.x * EPB * NA;           // the block's elements are consecutive
+    const int count = min(EPB, mp.ne - (int)blockIdx.x * EPB) * NA;
+    long long *T = fx_tiles + le * NA;
+    for (int i = t; i < 6 * EPB; i += blockDim.x) (&slot[0][0][0])[i] = 0;
+    const int nf = in1 ? 2 : 1;
+#pragma unroll 1
+    for (int f = 0; f < nf; ++f) {
+        const double *in = f ? in1 : in0;
+        double *out = f ? out1 : out0;
+        for (int i = t; i < count; i += blockDim.x) fx_tiles[i] = __double_as_longlong(in[base + i]);
+        __syncthreads();
+        int h[N1], l[N1];
+        // (1) x: thread = line (m3 = a, m2 = c)
+        long long *line = T + r * N1;
+        if (valid) {
+            int m = 0;
+#pragma unroll
+            for (int i = 0; i < N1; ++i) m = max(m, fx_expo(__longlong_as_double(line[i])));
+            atomicMax(&slot[f][0][le], m);
+        }
+        __syncthreads();
+        const int emax = slot[f][0][le];
+        if (valid) {
+#pragma unroll
+            for (int i = 0; i < N1; ++i) fx_limbs(__longlong_as_double(line[i]), emax, h[i], l[i]);
+            int m = 0;
+            fx_line<N1, KIND>(A.a[0], h, l, [&](int q, long long Y) { line[q] = Y; m |= fx_bits(Y); });
+            atomicOr(&slot[f][1][le], m);
+        }
+        __syncthreads();
+        // (2) y: thread = (m3 = a, m1 = c)
+        const int len1 = fx_length(slot[f][1][le]);
+        line = T + a * NT + c;
+        if (valid) {
+#pragma unroll
+            for (int i = 0; i < N1; ++i) fx_limbs(line[i * N1] << (62 - len1), h[i], l[i]);
+            int m = 0;
+            fx_line<N1, KIND>(A.a[1], h, l, [&](int q, long long Y) { line[q * N1] = Y; m |= fx_bits(Y); });
+            atomicOr(&slot[f][2][le], m);
+        }
+        __syncthreads();
+        // (3) z: thread = (m2 = a, m1 = c)
+        const int len2 = fx_length(slot[f][2][le]);
+        line = T + r;
+        if (valid) {
+#pragma unroll
+            for (int i = 0; i < N1; ++i) fx_limbs(line[i * NT] << (62 - len2), h[i], l[i]);
+            const int q0 = (emax - 1022) + (A.pe[0] + len1 - 57) + (A.pe[1] + len2 - 57) + A.pe[2] - 57;
+            const bool nan = emax == 0x7ff, plain = !nan && fx_plain(q0);
+            LineTraces<N1, true> tz(f ? mp.d[2].eL : mp.d[2].gL, nullptr);
+            fx_line<N1, KIND>(A.a[2], h, l, [&](int q, long long Y) {
+                const double v = fx_double(Y, q0, plain, nan);
+                line[q * NT] = __double_as_longlong(v);
+                if (KIND == FX_TO_MODES && tr) tz.add(q, v);
+            });
+            if (KIND == FX_TO_MODES && tr) {
+                tr[tix3<N1>(e, 4, 1 - f, r)] = tz.left();
+                tr[tix3<N1>(e, 5, 1 - f, r)] = tz.right();
+            }
+        }
+        __syncthreads();
+        for (int i = t; i < count; i += blockDim.x) out[base + i] = __longlong_as_double(fx_tiles[i]);
+        if (KIND == FX_TO_MODES && tr && valid) {   // the traces of the x and y faces
+            LineTraces<N1, true> tx(f ? mp.d[0].eL : mp.d[0].gL, nullptr), ty(f ? mp.d[1].eL : mp.d[1].gL, nullptr);
+#pragma unroll
+            for (int k = 0; k < N1; ++k) {
+                tx.add(k, __longlong_as_double(T[r * N1 + k]));
+                ty.add(k, __longlong_as_double(T[(a * N1 + k) * N1 + c]));
+            }
+            tr[tix3<N1>(e, 0, 1 - f, r)] = tx.left();
+            tr[tix3<N1>(e, 1, 1 - f, r)] = tx.right();
+            tr[tix3<N1>(e, 2, 1 - f, r)] = ty.left();
+            tr[tix3<N1>(e, 3, 1 - f, r)] = ty.right();
+        }
+        if (f + 1 < nf) __syncthreads();
+    }
+}
+
 // Separable element transform out = (Cz (x) Cy (x) Cx) diag(D) (Bz (x) By (x) Bx) in
 // (C, D optional); per field, passes along x, y, z through an element tile.
 // tr (modal output (U, V)): also its face traces.  KB: the kind of B
 // (line_transform); C is of kind 2 when B is of kind 3.  Bound by the FP64
-// pipe: 32^3 elements, N1 = 9, both fields: see gdg_step's table of times.
+// pipe; with parity P and Psi alone go through k_fx3.
 template <int N1, int KB>
 __global__ void __launch_bounds__(MAXB3)
 k_sep3(const __grid_constant__ ModalParams mp, const double *in0, const double *in1, double *out0, double *out1,
@@ -391,7 +485,7 @@ k_sep3(const __grid_constant__ ModalParams mp, const double *in0, const double *
         if (valid) {
 #pragma unroll
             for (int k = 0; k < N1; ++k) x[k] = T[(k * N1 + a) * N1 + c];
-            LineTraces<N1, KB != 0> tc(f ? mp.d[2].eL : mp.d[2].gL, f ? mp.d[2].eR : mp.d[2].gR);
+            LineTraces<N1, false> tc(f ? mp.d[2].eL : mp.d[2].gL, f ? mp.d[2].eR : mp.d[2].gR);
             line_transform<N1, KB>(sM + 2 * NT, x, [&](int m, double v) {
                 T[(m * N1 + a) * N1 + c] = D ? v * D[(m * N1 + a) * N1 + c] : v;
                 if (tr) tc.add(m, v);
@@ -405,8 +499,8 @@ k_sep3(const __grid_constant__ ModalParams mp, const double *in0, const double *
             __syncthreads();
             for (int i = t; i < count; i += blockDim.x) out[base + i] = Tb[i];
             if (tr && valid) {
-                LineTraces<N1, KB != 0> tx(f ? mp.d[0].eL : mp.d[0].gL, f ? mp.d[0].eR : mp.d[0].gR);
-                LineTraces<N1, KB != 0> ty(f ? mp.d[1].eL : mp.d[1].gL, f ? mp.d[1].eR : mp.d[1].gR);
+                LineTraces<N1, false> tx(f ? mp.d[0].eL : mp.d[0].gL, f ? mp.d[0].eR : mp.d[0].gR);
+                LineTraces<N1, false> ty(f ? mp.d[1].eL : mp.d[1].gL, f ? mp.d[1].eR : mp.d[1].gR);
 #pragma unroll
                 for (int k = 0; k < N1; ++k) {
                     tx.add(k, T[(a * N1 + c) * N1 + k]);
@@ -513,7 +607,29 @@ void gdg3_sep(const ModalParams &mp, int n1, int kind, const double *in0, const 
     const int epb = epb3(n1);
     const dim3 grid((mp.ne + epb - 1) / epb), block(epb * n1 * n1);
     switch (n1) {
-#define X(n) case n: (kind == 0 ? k_sep3<n, 0> : kind == 1 ? k_sep3<n, 1> : kind == 2 ? k_sep3<n, 2> : k_sep3<n, 3>)<<<grid, block, smem_sep3(n), s>>>(mp, in0, in1, out0, out1, Bx, By, Bz, D, Cx, Cy, Cz, tr); break;
+#define X(n) case n: (kind == 0 ? k_sep3<n, 0> : k_sep3<n, 3>)<<<grid, block, smem_sep3(n), s>>>(mp, in0, in1, out0, out1, Bx, By, Bz, D, Cx, Cy, Cz, tr); break;
+        GDG_N1_CASES3(X)
+#undef X
+    }
+}
+
+template <int N1>
+void launch_fx3(const ModalParams &mp, int kind, const FxTables &t, const double *in0, const double *in1, double *out0,
+                double *out1, double *tr, cudaStream_t s) {
+    constexpr int EPB = epb3c<N1>(), LEN = N1 * ((N1 + 1) / 2);
+    FxLines<N1, 3> A;
+    for (int d = 0; d < 3; ++d) {
+        std::copy(t.a[d][kind - 1], t.a[d][kind - 1] + LEN, A.a[d]);
+        A.pe[d] = t.pe[d][kind - 1];
+    }
+    (kind == FX_TO_MODES ? k_fx3<N1, FX_TO_MODES> : k_fx3<N1, FX_TO_NODES>)<<<(mp.ne + EPB - 1) / EPB, EPB * N1 * N1,
+        (size_t)EPB * N1 * N1 * N1 * sizeof(double), s>>>(mp, A, in0, in1, out0, out1, tr);
+}
+
+void gdg3_fx(const ModalParams &mp, int n1, int kind, const FxTables &t, const double *in0, const double *in1, double *out0,
+             double *out1, double *tr, cudaStream_t s) {
+    switch (n1) {
+#define X(n) case n: launch_fx3<n>(mp, kind, t, in0, in1, out0, out1, tr, s); break;
         GDG_N1_CASES3(X)
 #undef X
     }
@@ -541,8 +657,6 @@ void gdg3_set_smem_limits() {
     cudaFuncSetAttribute(k_stage3p<n, M_S1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);  \
     cudaFuncSetAttribute(k_stage3p<n, M_S23, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
     cudaFuncSetAttribute(k_sep3<n, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);       \
-    cudaFuncSetAttribute(k_sep3<n, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);       \
-    cudaFuncSetAttribute(k_sep3<n, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);       \
     cudaFuncSetAttribute(k_sep3<n, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     GDG_N1_CASES3(X)
 #undef X

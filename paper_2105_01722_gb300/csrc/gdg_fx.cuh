@@ -1,9 +1,9 @@
 // FP64-accurate dot products on the integer pipe.
 //
 // GB300 issues one FP64 warp instruction per SM every 16 cycles and one
-// 32 x 32 + 64-bit integer multiply-add (IMAD.WIDE) every 0.54 (both measured
+// 32 x 32 + 64-bit integer multiply-add (IMAD.WIDE) every 1.06 (both measured
 // with instruction chains, 4 to 32 warps per SM).  A product of two 58-bit
-// integers in two 29-bit limbs each is four of the latter: 2.2 cycles where
+// integers in two 29-bit limbs each is four of the latter: 4.2 cycles where
 // an FP64 FMA costs 16.  The element matrices of the variable-coefficient
 // path are fixed after setup, so they are kept as such integers:
 //

@@ -62,13 +62,24 @@ struct StageBufs {
                              // all times sc in the stage modes
 };
 
-// 3-D modal-route launches (gdg_const3.cu), n1 = N+1 in 2..10
+// The transform tables as 58-bit integers, two 29-bit limbs each (gdg_fxline.cuh):
+// per direction P and Psi, the halves that parity leaves, and their exponents.
+constexpr int FX_TAB_LEN = 128;   // n1 = 16: 16 x 8
+struct FxTables {
+    int2 a[3][2][FX_TAB_LEN];
+    int pe[3][2];
+};
+
+// 3-D modal-route launches (gdg_const3.cu), n1 = N+1 in 2..10; kind: 0 dense
+// matrices, 1 nodes to modes (P), 2 modes to nodes (Psi), 3 Psi^T first
 void gdg3_stage(const ModalParams &mp, int n1, int mode, const StageBufs &b, double sc, cudaStream_t s);
 void gdg3_sep(const ModalParams &mp, int n1, int kind, const double *in0, const double *in1, double *out0, double *out1,
               const double *Bx, const double *By, const double *Bz, const double *D, const double *Cx, const double *Cy,
               const double *Cz, double *tr, cudaStream_t s);
 void gdg3_energy_partial(int n1, int ne, const double *yU, const double *yV, const double *lam2, double *partial,
                          int blocks, cudaStream_t s);
+void gdg3_fx(const ModalParams &mp, int n1, int kind, const FxTables &t, const double *in0, const double *in1, double *out0,
+             double *out1, double *tr, cudaStream_t s);
 void gdg3_set_smem_limits();
 
 struct GraphCache {
@@ -105,6 +116,7 @@ struct gdg_ctx {
     // constant-coefficient Cartesian (diagonalised route)
     ModalParams mp{};
     double *d_mats = nullptr;     // device tables: per direction P = Psi^T M, Psi, Psi^T (n1*n1 each)
+    FxTables fx{};                // the same as integers (with parity)
     double *d_lam2 = nullptr;     // per mode: -c2*lambda, 1/lambda (0 for mode 0); 2-D also P1, P2
                                   // (the u lifts over lambda, see stage2p_body)
     double *d_lams = nullptr;     // d_lam2 times the factor of each RK stage, for the step size lams_dt

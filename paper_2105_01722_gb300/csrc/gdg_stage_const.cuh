@@ -57,39 +57,27 @@ __device__ __forceinline__ void flux2(double vi, double di, double vo, double dO
 // basis has that symmetry (parity contexts; the even ones, NE = ceil(N1/2),
 // first), so a line splits in node pairs and each output is a sum of about
 // N1/2 products: 41 FMAs and 8 additions instead of 81 at N1 = 9.
-// KIND 1: nodes to modes by P = Psi^T M, row q of A even or odd in i.  Rows
-// q > 0 sum to zero (M 1 is the constant mode), so they are applied to the
-// differences from a middle node: the rounding of the table then meets the
-// variation along the line, not the values, which the high modes (times lambda
-// afterwards) would show.  KIND 3: the same by Psi^T, whose rows do not sum to
-// zero, from the plain sums and differences of the pairs.  KIND 2: modes to
-// nodes (column k even or odd in i), a pair from its even and odd parts.
+// KIND 3: nodes to modes by Psi^T, row q even or odd in i, from the plain sums
+// and differences of the pairs.  KIND 2: modes to nodes (column k even or odd in
+// i), a pair from its even and odd parts.
 // emit(i, y[i]) as each is formed: a store there keeps the loads of the
 // matrix from being moved up into a hundred registers.
 template <int N1, int KIND, typename EMIT>
 __device__ __forceinline__ void line_transform(const double *A, const double (&x)[N1], EMIT emit) {
     constexpr int NE = (N1 + 1) / 2, H = N1 / 2;   // H pairs, and the middle node when N1 is odd
-    if (KIND == 1 || KIND == 3) {
-        const double ref = KIND == 1 ? x[(N1 - 1) / 2] : 0.0;
+    if (KIND == 3) {
         double sm[NE], df[H > 0 ? H : 1];
 #pragma unroll
         for (int i = 0; i < H; ++i) {
-            sm[i] = KIND == 1 ? (x[i] - ref) + (x[N1 - 1 - i] - ref) : x[i] + x[N1 - 1 - i];
+            sm[i] = x[i] + x[N1 - 1 - i];
             df[i] = x[i] - x[N1 - 1 - i];
         }
-        if (N1 & 1) sm[NE - 1] = KIND == 1 ? 0.0 : x[H];
+        if (N1 & 1) sm[NE - 1] = x[H];
 #pragma unroll
         for (int q = 0; q < N1; ++q) {
             double s = 0.0;
-            if (KIND == 1 && q == 0) {   // the constant mode: the only one that sees ref
 #pragma unroll
-                for (int i = 0; i < H; ++i) s = fma(A[i], x[i] + x[N1 - 1 - i], s);
-                if (N1 & 1) s = fma(A[H], x[H], s);
-            } else {
-#pragma unroll
-                for (int i = 0; i < (q < NE && KIND == 3 ? NE : H); ++i)
-                    s = fma(A[q * N1 + i], q < NE ? sm[i] : df[i < H ? i : 0], s);
-            }
+            for (int i = 0; i < (q < NE ? NE : H); ++i) s = fma(A[q * N1 + i], q < NE ? sm[i] : df[i < H ? i : 0], s);
             emit(q, s);
         }
     } else if (KIND == 2) {
