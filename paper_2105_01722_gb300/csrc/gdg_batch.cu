@@ -172,7 +172,7 @@ extern "C" int gdg_batch_create(const gdg_problem *pbs, int count, gdg_batch **o
     std::vector<ModalParams> mps(count);
     std::vector<int2> var_items, mod_items;
     for (int i = 0; i < count; ++i) {
-        if ((st = gdg_create(&pbs[i], &b->ctx[i]))) { gdg_batch_destroy(b); return st; }
+        if ((st = gdg_create_ctx(&pbs[i], true, &b->ctx[i]))) { gdg_batch_destroy(b); return st; }
         gdg_ctx *c = b->ctx[i];
         BatchProb &P = b->h_probs[i];
         std::memset(&P, 0, sizeof(P));
@@ -187,7 +187,7 @@ extern "C" int gdg_batch_create(const gdg_problem *pbs, int count, gdg_batch **o
             P.kind = 1;
             P.vp = c->var->vp;
             P.sb = gdg_var_buffers(c);
-            b->smem = std::max(b->smem, c->var->smem_stage);
+            b->smem = std::max(b->smem, c->var->smem_pcg);
             for (int e = 0; e < c->ne; ++e) var_items.push_back(make_int2(i, e));
         }
     }

@@ -85,7 +85,7 @@ __device__ __forceinline__ void batch_var_item(const BatchProb *__restrict__ pro
         __syncthreads();
         cur = w.x;
     }
-    var_stage_body<N1, MODE>(s_vp, s_b, s_c[0], s_c[1], w.y, smem);
+    var_stage_body<N1, ROUTE_ANY>(s_vp, s_b, MODE, s_c[0], s_c[1], w.y, smem);
 }
 
 // elements of one modal work item: the half-line body (two threads per

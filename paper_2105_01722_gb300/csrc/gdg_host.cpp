@@ -425,7 +425,7 @@ static int validate(const gdg_problem *pb, std::string &why) {
     return GDG_OK;
 }
 
-extern "C" int gdg_create(const gdg_problem *pb, gdg_ctx **out) {
+int gdg_create_ctx(const gdg_problem *pb, bool batched, gdg_ctx **out) {
     if (!out) return GDG_EINVAL;
     *out = nullptr;
     std::string why;
@@ -436,6 +436,7 @@ extern "C" int gdg_create(const gdg_problem *pb, gdg_ctx **out) {
     }
     gdg_ctx *ctx = new (std::nothrow) gdg_ctx();
     if (!ctx) return GDG_ENOMEM;
+    ctx->batched = batched;
     ctx->pb = *pb;
     ctx->pb.x_nodes = ctx->pb.y_nodes = ctx->pb.c2_nodes = nullptr;
     ctx->dim = pb->dim;
@@ -471,6 +472,8 @@ extern "C" int gdg_create(const gdg_problem *pb, gdg_ctx **out) {
     *out = ctx;
     return GDG_OK;
 }
+
+extern "C" int gdg_create(const gdg_problem *pb, gdg_ctx **out) { return gdg_create_ctx(pb, false, out); }
 
 extern "C" int gdg_destroy(gdg_ctx *ctx) {
     if (!ctx) return GDG_EINVAL;

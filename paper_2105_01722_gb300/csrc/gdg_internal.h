@@ -141,6 +141,7 @@ struct gdg_ctx {
     unsigned long long wait_limit_ns = 1000000000ull;   // bound on any device-side wait
 
     VarData *var = nullptr;
+    bool batched = false;         // a member of a batch: its stages run in the batch's kernel
     Profiler prof;
     double *d_io = nullptr;       // device copies for gdg_step_host (2 fields)
 };
@@ -152,6 +153,9 @@ struct gdg_ctx {
         stmt;                                                          \
         if (gdg_ev0_) (ctx)->prof.end((kind), gdg_ev0_, (s));           \
     } while (0)
+
+// gdg_create, and the same for a member of a batch
+int gdg_create_ctx(const gdg_problem *pb, bool batched, gdg_ctx **out);
 
 // error helpers
 int gdg_set_err(gdg_ctx *ctx, int status, const std::string &msg);

@@ -18,9 +18,12 @@
 //
 // Kernels (one CTA per element):
 //   k_var_geom    quadrature assembly of M_J, S_c2, w and face data
-//   k_var_traces  v and n.grad u at the face quadrature points
-//   k_var_stage   fluxes + lifts + stiffness + both PCG solves (matrices in
-//                 shared memory) + RK combine + traces of the next stage input
+//   k_var_facemat, k_fm_pack  face operators, as integers
+//   k_fx_pack     element matrices as packed triangles of integers
+//   k_var_invert  element inverses (GDG_SOLVE_INVERSE)
+//   k_var_traces  face lines of a given state
+//   k_var_stage   fluxes + lifts + stiffness + both solves (matrices in shared
+//                 memory) + RK combine + face lines of the next stage input
 //   k_var_pcg     one element PCG (gdg_pcg)
 //   k_var_energy  per-element V^T M V + U^T S U
 #include <algorithm>
@@ -254,6 +257,8 @@ int gdg_var_setup(gdg_ctx *ctx) {
     P.tab = D->d_tab; P.S = D->d_S; P.M = D->d_M; P.w = D->d_w; P.pre = D->d_pre; P.face = D->d_face;
     P.stats = D->d_stats;
     P.mixed = ctx->pb.precision == GDG_MIXED;
+    P.inverse = ctx->pb.solver == GDG_SOLVE_INVERSE;
+    P.staged = P.inverse && !ctx->batched;
     P.refine_max = ctx->pb.refine_max > 0 ? ctx->pb.refine_max : 8;
     P.refine_rtol = (float)(ctx->pb.refine_rtol > 0.0 ? ctx->pb.refine_rtol : 1e-5);
     D->smem_geom = geom_smem(n1, Q);
@@ -261,7 +266,8 @@ int gdg_var_setup(gdg_ctx *ctx) {
     switch (n1) {
 #define X(n)                                                                                   \
     case n:                                                                                    \
-        D->smem_stage = D->smem_pcg = StageSmem<n>::bytes();                                     \
+        D->smem_pcg = StageSmem<n, false>::bytes();                                              \
+        D->smem_stage = P.staged ? StageSmem<n, true>::bytes() : D->smem_pcg;                   \
         set_attrs<n>();                                                                        \
         break;
         GDG_VAR_CASES(X)
@@ -289,7 +295,7 @@ int gdg_var_setup(gdg_ctx *ctx) {
         (st = gdg_cuda_check(ctx, cudaMemcpy(D->d_Psx, psx.data(), psx.size() * sizeof(int2), cudaMemcpyHostToDevice), "upload Psi")))
         return st;
     switch (n1) {
-#define X(n) case n: k_fm_pack<n><<<ctx->ne, nthreads_for(n * n)>>>(D->d_FM, slope_exp, D->d_FMq); break;
+#define X(n) case n: k_fm_pack<n><<<ctx->ne, nthreads_for(n * n)>>>(D->d_FM, slope_exp, P.staged, D->d_FMq); break;
         GDG_VAR_CASES(X)
 #undef X
     }
@@ -322,7 +328,6 @@ int gdg_var_setup(gdg_ctx *ctx) {
 #undef X
     }
     P.dS = D->d_dS;
-    P.inverse = ctx->pb.solver == GDG_SOLVE_INVERSE;
     const size_t fxm = (size_t)ctx->ne * fx_tri_len(NA);   // one set of packed integer matrices
     const int sets = P.inverse ? 4 : 2;
     if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_fx, sets * fxm * sizeof(int2)), "alloc integer matrices")) ||

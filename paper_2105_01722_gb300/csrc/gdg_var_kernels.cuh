@@ -30,8 +30,9 @@ struct VarParams {
     // (fx_tri_len entries an element) and the exponents d of their rows [ne][N1*N1]
     FxMatrix Sx, Mx;             // S_c2, M_J
     FxMatrix Ax, Vx;             // (S_c2 + w w^T)^-1 - 1 1^T (k_var_invert), M_J^-1 (GDG_SOLVE_INVERSE)
-    const int2 *FM;              // [ne][4 faces][6 N1 columns][3 N1 rows] face operators (k_var_facemat)
+    const int2 *FM;              // [ne][4 faces] operators, [6 N1 columns][3 N1 rows]; inverse route [3][3 N1 rows][2 N1] (k_fm_pack)
     const short2 *FMq;           // [ne][4 faces][3 N1] exponents of a row's v columns and u columns
+    int staged;                  // FM's layout: lift_lines_staged's (stages of the inverse route outside batches)
     int slope_exp;               // the u slopes along a face normal count as 2^-slope_exp of the u values
     const int2 *Psx;             // Psi in units of 2^(Ps_exp - 57), rows and columns summing to at most 2^57
     int Ps_exp;
@@ -880,24 +881,44 @@ __device__ __forceinline__ double source_amplitude(const VarParams &P, const Var
 
 __global__ void k_set_time(double *time, double t0) { *time = t0; }
 
-// Shared memory of one element's block, in doubles: the packed matrix, Psi, w
-// and one scratch region for the phases of a stage in turn: the lifts (limbs of
-// the face lines, line integrals), the solves (vectors and limb vectors; the
-// FP32 vectors in the place of p and Ap), the new state whose face lines go out.
-template <int N1>
+// Shared memory of one element's block, in doubles: the packed matrix (or, for
+// the lifts of the inverse route, face operators), Psi, w and one scratch region
+// for the phases of a stage in turn: the lifts (limbs of the face lines, line
+// integrals), the solves (vectors and limb vectors; the FP32 vectors in the place
+// of p and Ap), the new state whose face lines go out.  INV: the inverse route
+// alone, which keeps a limb vector or the line integrals beside the matrix, all
+// else in its place: 27.6 KB at N1 = 9, 8 blocks an SM, where the rest needs 31.4
+// KB and 7.
+template <int N1, bool INV>
 struct StageSmem {
     static constexpr int NA = N1 * N1;
     static constexpr int NP = (NA + 1) & ~1;   // limb vectors start on 16 bytes
     static constexpr int SCR = 36 * N1 > 6 * NP ? (36 * N1 + 1) & ~1 : 6 * NP;
-    static constexpr int LEN = fx_tri_len(NA) + 2 * NP + SCR + 24;   // 31.4 KB at N1 = 9: 7 blocks an SM
+    static constexpr int FACE = 18 * NA;       // a face's operator
+    static constexpr int LINES = INV ? 24 * N1 : 0;   // limbs of the face lines, beside the face operators
+    static constexpr int ARENA = fx_tri_len(NA) > FACE + LINES ? fx_tri_len(NA) : FACE + LINES;
+    static constexpr int SLOTS = (ARENA - LINES) / FACE < 2 ? 1 : 2;
+    static constexpr int SIDE = NP > 12 * N1 ? NP : 12 * N1;
+    static constexpr int LEN = ARENA + (INV ? SIDE : 2 * NP + SCR) + 24;
     int2 *A, *Ps, *lines, *X, *X2;
     int *slot;
     double *L, *U, *V, *w, *r, *z, *p, *Ap, *red;
     float *Ps32, *t1, *t2, *red32;
     __device__ StageSmem(double *base) {
         A = reinterpret_cast<int2 *>(base);
-        Ps = A + fx_tri_len(NA);
-        w = base + fx_tri_len(NA) + NP;
+        red = base + LEN - 24;                            // 8 doubles
+        slot = reinterpret_cast<int *>(red + 8);          // 16 ints
+        red32 = reinterpret_cast<float *>(red + 16);      // 16 floats
+        if (INV) {
+            lines = A + SLOTS * FACE;
+            L = base + ARENA;
+            X = A + ARENA;
+            U = base;
+            V = base + NP;
+            return;
+        }
+        Ps = A + ARENA;
+        w = base + ARENA + NP;
         double *scr = w + NP;
         lines = reinterpret_cast<int2 *>(scr);
         L = scr + 24 * N1;
@@ -912,9 +933,6 @@ struct StageSmem {
         Ps32 = reinterpret_cast<float *>(Ap);
         U = scr;
         V = scr + NP;
-        red = scr + SCR;                                  // 8 doubles
-        slot = reinterpret_cast<int *>(red + 8);          // 16 ints
-        red32 = reinterpret_cast<float *>(red + 16);      // 16 floats
     }
     static constexpr size_t bytes() { return sizeof(double) * (size_t)LEN; }
     __device__ __forceinline__ FxSystem system(const FxMatrix &m, int e) const {
@@ -1026,8 +1044,16 @@ k_var_facemat(VarParams P, double *__restrict__ FM) {
     }
 }
 
-// The face operators as integers, in place (one thread per row r of a face,
-// which alone reads and writes that row).  A row's columns fall in two groups,
+// The columns of a face in three parts of 2 N1: the v lines of both sides, the
+// element's own u lines, the neighbour's (column c as in k_var_facemat).
+template <int N1> __device__ __forceinline__ int line_third(int c) { return c % (3 * N1) < N1 ? 0 : c < 3 * N1 ? 1 : 2; }
+template <int N1> __device__ __forceinline__ int line_place(int c) {
+    return c % (3 * N1) < N1 ? c / (3 * N1) * N1 + c % N1 : c % (3 * N1) - N1;
+}
+
+// The face operators as integers, in place, face by face.  `staged`: [part][row]
+// [2 N1] in place of [6 N1][row], so that a row's part is read 16 bytes at a time
+// (lift_lines_staged).  A row's columns fall in two groups,
 // each in units of 2^(q - 57): the v lines and the u lines, whose vectors get
 // a block exponent each (u and v may differ by any factor).  The u group holds
 // values along the face and slopes across it; the slopes count as
@@ -1038,27 +1064,32 @@ __device__ __forceinline__ bool slope_line(int f, int m) { return f < 2 ? m == 1
 
 template <int N1>
 __global__ void __launch_bounds__(nthreads_for(N1 * N1))
-k_fm_pack(double *FM, int slope_exp, short2 *FMq) {
-    constexpr int NL = 3 * N1;
+k_fm_pack(double *FM, int slope_exp, int staged, short2 *FMq) {
+    constexpr int NL = 3 * N1, FACE = 2 * NL * NL;
+    __shared__ double in[FACE];
     const int e = blockIdx.x;
-    for (int task = threadIdx.x; task < 4 * NL; task += blockDim.x) {
-        const int f = task / NL, r = task - (task / NL) * NL;
-        double *col = FM + ((size_t)e * 4 + f) * 2 * NL * NL + r;
-        int qv = -FX_NAN, qu = -FX_NAN;
-        for (int c = 0; c < 2 * NL; ++c) {
-            const int m = (c % NL) / N1;
-            const int k = fx_key(col[(size_t)c * NL], slope_line<N1>(f, m) ? slope_exp : 0) - 1022;   // |v| < 2^k
-            if (m == 0) qv = max(qv, k); else qu = max(qu, k);
+    for (int f = 0; f < 4; ++f) {
+        double *face = FM + ((size_t)e * 4 + f) * FACE;
+        for (int i = threadIdx.x; i < FACE; i += blockDim.x) in[i] = face[i];
+        __syncthreads();
+        for (int r = threadIdx.x; r < NL; r += blockDim.x) {
+            int qv = -FX_NAN, qu = -FX_NAN;
+            for (int c = 0; c < 2 * NL; ++c) {
+                const int m = (c % NL) / N1;
+                const int k = fx_key(in[c * NL + r], slope_line<N1>(f, m) ? slope_exp : 0) - 1022;   // |v| < 2^k
+                if (m == 0) qv = max(qv, k); else qu = max(qu, k);
+            }
+            qv = max(-16000, min(qv, 16000));
+            qu = max(-16000, min(qu, 16000));
+            FMq[((size_t)e * 4 + f) * NL + r] = make_short2((short)qv, (short)qu);
+            for (int c = 0; c < 2 * NL; ++c) {
+                const int m = (c % NL) / N1;
+                const int to = staged ? (line_third<N1>(c) * NL + r) * 2 * N1 + line_place<N1>(c) : c * NL + r;
+                reinterpret_cast<int2 *>(face)[to] =
+                    fx_split(fx_int(in[c * NL + r], (m == 0 ? qv : qu) + 1022, slope_line<N1>(f, m) ? slope_exp : 0));
+            }
         }
-        qv = max(-16000, min(qv, 16000));
-        qu = max(-16000, min(qu, 16000));
-        FMq[((size_t)e * 4 + f) * NL + r] = make_short2((short)qv, (short)qu);
-        for (int c = 0; c < 2 * NL; ++c) {
-            const int m = (c % NL) / N1;
-            double *v = col + (size_t)c * NL;
-            const int2 a = fx_split(fx_int(*v, (m == 0 ? qv : qu) + 1022, slope_line<N1>(f, m) ? slope_exp : 0));
-            *reinterpret_cast<int2 *>(v) = a;
-        }
+        __syncthreads();
     }
 }
 
@@ -1128,6 +1159,105 @@ __device__ __forceinline__ void lift_lines(const VarParams &P, int e, const doub
     __syncthreads();
 }
 
+// start the copy of the operator of face f into its slot of the matrix's place
+template <int N1, typename SMEM>
+__device__ __forceinline__ void load_face(const VarParams &P, const SMEM &s, int e, int f) {
+    constexpr int FACE = SMEM::FACE;
+    const int2 *src = P.FM + ((size_t)e * 4 + f) * FACE;
+    int2 *dst = s.A + f % SMEM::SLOTS * FACE;
+    for (int i = 2 * threadIdx.x; i < FACE; i += 2 * blockDim.x) cp_async_16(dst + i, src + i);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+
+// The same in the inverse route, whose operators all stream through: the face
+// operators come through the matrix's place in shared memory, as many at a time
+// as fit (the first ones on their way when this starts).  A row's three parts go
+// to three lanes of a warp, ten rows a warp; the exact sums of the two u parts
+// are added before they are rounded.  128^2 elements, four steps with element
+// inverses: 8.55 -> 7.50 ms, with the eighth block an SM that the smaller scratch
+// allows (staged alone 7.92).  In the iterative
+// routes, where S would have to be read again for the solve, the direct form is
+// the faster one: a step of 128^2 elements 9.5 against 9.8 ms.
+template <int N1, typename SMEM>
+__device__ __forceinline__ void lift_lines_staged(const VarParams &P, const SMEM &s, int e, const double *trin) {
+    constexpr int NL = 3 * N1, BD = nthreads_for(N1 * N1), PER = (4 * NL + BD - 1) / BD, WARPS = BD / 32;
+    constexpr int FACE = SMEM::FACE, SLOTS = SMEM::SLOTS;
+    const int t = threadIdx.x;
+    int *slot = s.slot;
+    double own[PER], nbl[PER];
+    int kv = -FX_NAN, ku = -FX_NAN;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int q = t + BD * i;
+        own[i] = nbl[i] = 0.0;
+        if (q < 4 * NL) {
+            const int f = q / NL, c = q - f * NL;
+            int fo;
+            const int nb = neighbour(P, e, f, fo);
+            own[i] = trin[lix<N1>(e, 0) + q];
+            if (nb >= 0) nbl[i] = trin[lix<N1>(nb, fo) + c];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int q = t + BD * i, f = q / NL, m = (q - f * NL) / N1;
+        if (q < 4 * NL) {
+            const int sh = slope_line<N1>(f, m) ? -P.slope_exp : 0;
+            const int k = max(fx_key(own[i], sh), fx_key(nbl[i], sh));
+            if (m == 0) kv = max(kv, k); else ku = max(ku, k);
+        }
+    }
+    kv = __reduce_max_sync(0xffffffffu, kv);
+    ku = __reduce_max_sync(0xffffffffu, ku);
+    if ((t & 31) == 0) { slot[8 + (t >> 5)] = kv; slot[12 + (t >> 5)] = ku; }   // set 1
+    __syncthreads();
+    for (int w = 0; w < WARPS; ++w) { kv = max(kv, slot[8 + w]); ku = max(ku, slot[12 + w]); }
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int q = t + BD * i;
+        if (q < 4 * NL) {
+            const int f = q / NL, c = q - f * NL, m = c / N1;
+            const int sh = slope_line<N1>(f, m) ? -P.slope_exp : 0, k = m == 0 ? kv : ku;
+            int2 *x = s.lines + f * 6 * N1;
+            x[line_third<N1>(c) * 2 * N1 + line_place<N1>(c)] = fx_split(fx_int(own[i], k, sh));
+            x[line_third<N1>(c + NL) * 2 * N1 + line_place<N1>(c + NL)] = fx_split(fx_int(nbl[i], k, sh));   // zero on a Dirichlet side
+        }
+    }
+    const int lane = t & 31, part = lane % 3;
+#pragma unroll 1
+    for (int f = 0; f < 4; ++f) {
+        if (f + 1 < SLOTS) asm volatile("cp.async.wait_group %0;\n" ::"n"(SLOTS > 1 ? SLOTS - 1 : 0) : "memory");   // the first of SLOTS
+        else cp_async_wait_all();
+        __syncthreads();   // face f has arrived, and every thread is past face f - 1
+        if (SLOTS > 1 && f >= 1 && f - 1 + SLOTS < 4) load_face<N1>(P, s, e, f - 1 + SLOTS);
+#pragma unroll 1
+        for (int row0 = 10 * (t >> 5); row0 < NL; row0 += 10 * WARPS) {
+            const int row = min(row0 + lane / 3, NL - 1);
+            const short2 q = P.FMq[((size_t)e * 4 + f) * NL + row];
+            const int4 *a = reinterpret_cast<const int4 *>(s.A + f % SLOTS * FACE + (part * NL + row) * 2 * N1);
+            const int4 *x = reinterpret_cast<const int4 *>(s.lines + (f * 3 + part) * 2 * N1);
+            FxSum sum;
+#pragma unroll
+            for (int i = 0; i < N1; ++i) {
+                const int4 av = a[i], xv = x[i];
+                sum.mad(make_int2(av.x, av.y), xv.x, xv.y);
+                sum.mad(make_int2(av.z, av.w), xv.z, xv.w);
+            }
+            long long T = sum.top();
+            const long long nbr = __shfl_down_sync(0xffffffffu, T, 1);
+            if (part == 1) T += nbr;
+            const double y = fx_value(T, fx_top_exp(part ? ku : kv) + (part ? q.y : q.x), part ? ku : kv);
+            const double u = __shfl_down_sync(0xffffffffu, y, 1);
+            if (part == 0 && lane < 30 && row0 + lane / 3 < NL) s.L[f * NL + row] = y + u;
+        }
+        if (SLOTS == 1 && f < 3) {
+            __syncthreads();
+            load_face<N1>(P, s, e, f + 1);
+        }
+    }
+    __syncthreads();
+}
+
 // r_u, r_v (r_v without the stiffness term) at node t from the face line integrals
 template <int N1>
 __device__ __forceinline__ void lift_assemble(const double *L, const Tabs &T, int t, double &ru, double &rv) {
@@ -1145,14 +1275,26 @@ __device__ __forceinline__ void lift_assemble(const double *L, const Tabs &T, in
 
 // Psi into shared memory, as integers or, for the inner solves, in FP32
 template <int N1>
-__device__ __forceinline__ void load_psi(const VarParams &P, const StageSmem<N1> &s) {
+__device__ __forceinline__ void load_psi(const VarParams &P, const StageSmem<N1, false> &s) {
     if (threadIdx.x < N1 * N1) s.Ps[threadIdx.x] = P.Psx[threadIdx.x];
+}
+
+// The route of a stage.  ROUTE_ANY reads it from the problem (batches; FP64 PCG,
+// which is as fast so: 9.52 ms a step of 128^2 elements, alone 9.56); the mixed
+// form by itself spills less at 80 registers (128 x 120 elements, p = 3, a step
+// 6.41 -> 6.26 ms), the inverse route has its own layout of shared memory.
+enum { ROUTE_ANY, ROUTE_MIXED, ROUTE_INVERSE };
+template <int ROUTE> __device__ __forceinline__ bool route_inverse(const VarParams &P) {
+    return ROUTE == ROUTE_ANY ? P.inverse != 0 : ROUTE == ROUTE_INVERSE;
+}
+template <int ROUTE> __device__ __forceinline__ bool route_mixed(const VarParams &P) {
+    return ROUTE == ROUTE_ANY ? P.mixed != 0 : ROUTE == ROUTE_MIXED;
 }
 
 // solve one of the element's systems (W: the u_t system, + w w^T) from the
 // right-hand side b; x: the guess (unless zero) and the result
-template <int N1>
-__device__ __forceinline__ void solve(const VarParams &P, const StageSmem<N1> &s, const Tabs &T, int e, bool W, double w,
+template <int N1, int ROUTE>
+__device__ __forceinline__ void solve(const VarParams &P, const StageSmem<N1, false> &s, const Tabs &T, int e, bool W, double w,
                                       double b, double &x, bool zero, bool guess, int *iters, int *sweeps, int *fell,
                                       double *rel, bool want_rel) {
     constexpr int NA = N1 * N1;
@@ -1161,7 +1303,7 @@ __device__ __forceinline__ void solve(const VarParams &P, const StageSmem<N1> &s
     const FxSystem f = s.system(W ? P.Sx : P.Mx, e);
     const FxPrecond pre{s.Ps, P.Ps_exp, W ? (on ? P.dS[(size_t)e * NA + t] : 0.0) : P.pre[(size_t)e * 4 + 3],
                         P.precond == GDG_PC_NONE};
-    if (P.mixed) {
+    if (route_mixed<ROUTE>(P)) {
         Inner32 in;
         in.sc = __int_as_float(max(1, min(254, 127 + f.d)) << 23);
         in.d = (float)pre.d;
@@ -1185,29 +1327,46 @@ __device__ __forceinline__ void solve(const VarParams &P, const StageSmem<N1> &s
 }
 
 // One element's RK stage (one block of nthreads_for(N1*N1) threads).
-template <int N1, int MODE>
-__device__ __forceinline__ void var_stage_body(const VarParams &P, const VarBufs &b, double cA, double cY, int e,
+template <int N1, int ROUTE>
+__device__ __forceinline__ void var_stage_body(const VarParams &P, const VarBufs &b, int mode, double cA, double cY, int e,
                                                double *smraw) {
     constexpr int NA = N1 * N1;
-    const StageSmem<N1> s(smraw);
+    const StageSmem<N1, ROUTE == ROUTE_INVERSE> s(smraw);
     const int t = threadIdx.x;
+    const bool inverse = route_inverse<ROUTE>(P), mixed = route_mixed<ROUTE>(P);
     const bool on = t < NA;
     const size_t at = (size_t)e * NA + (on ? t : 0);
-    load_fx<N1>(s.A, P.Sx, e);
-    const Tabs T = tabs_at(P.tab, P.Q, N1);
-    const double Yu = on ? b.yU[at] : 0.0, Yv = on ? b.yV[at] : 0.0, w = on ? P.w[at] : 0.0;
-    double ru = 0.0, rv = 0.0, x = 0.0;
-    if (on) s.w[t] = w;
-    if (!P.inverse) load_psi<N1>(P, s);
     const bool guess = b.part == 2;
+    constexpr bool staged = ROUTE == ROUTE_INVERSE;   // (a problem of inverses in a batch: P.staged is 0)
+    if constexpr (staged) {
+#pragma unroll
+        for (int f = 0; f < s.SLOTS; ++f) load_face<N1>(P, s, e, f);
+    } else {
+        load_fx<N1>(s.A, P.Sx, e);
+    }
+    const Tabs T = tabs_at(P.tab, P.Q, N1);
+    const double Yu = on ? b.yU[at] : 0.0, Yv = on ? b.yV[at] : 0.0;
+    double ru = 0.0, rv = 0.0, x = 0.0, w = 0.0;
+    if constexpr (ROUTE != ROUTE_INVERSE) {
+        w = on ? P.w[at] : 0.0;
+        if (on) s.w[t] = w;
+        if (!inverse) load_psi<N1>(P, s);
+    }
+    if constexpr (staged) {
+        lift_lines_staged<N1>(P, s, e, b.trin);
+        load_fx<N1>(s.A, P.Sx, e);
+        if (on) lift_assemble<N1>(s.L, T, t, ru, rv);
+    }
     fx_arrived();
     if (!guess) {
         const double SU = fx_matvec<NA>(s.system(P.Sx, e), Yu, 0);
-        __syncthreads();
-        if (P.inverse && b.part != 1) load_fx<N1>(s.A, P.Ax, e);   // on its way during the lifts
-        lift_lines<N1>(P, e, b.trin, s.lines, s.slot, s.L);
+        __syncthreads();   // the matrix and the vector are read
+        if (inverse && b.part != 1) load_fx<N1>(s.A, P.Ax, e);   // on its way during the lifts
+        if constexpr (!staged) {
+            lift_lines<N1>(P, e, b.trin, s.lines, s.slot, s.L);
+            if (on) lift_assemble<N1>(s.L, T, t, ru, rv);
+        }
         if (on) {
-            lift_assemble<N1>(s.L, T, t, ru, rv);
             rv -= SU;
             if (e == P.src_e) rv += source_amplitude(P, b) * P.src_w[t];
         }
@@ -1221,7 +1380,7 @@ __device__ __forceinline__ void var_stage_body(const VarParams &P, const VarBufs
         rv = b.rv[at];
         x = b.x0u[at];
     }
-    if (P.inverse) {   // dU/dt = V + (S_c2 + w w^T)^-1 r_u (k_var_invert), dV/dt = M_J^-1 r_v
+    if (inverse) {   // dU/dt = V + (S_c2 + w w^T)^-1 r_u (k_var_invert), dV/dt = M_J^-1 r_v
 #pragma unroll 1
         for (int sys = 0; sys < 2; ++sys) {
             fx_arrived();
@@ -1235,16 +1394,16 @@ __device__ __forceinline__ void var_stage_body(const VarParams &P, const VarBufs
             x = y;             // dV/dt after the second pass
         }
         if (t == 0 && P.stats) atomicAdd(&P.stats[6], 1ull);
-    } else {
+    } else if constexpr (ROUTE != ROUTE_INVERSE) {
         int it[2], sw[2], fell = 0;
         bool bad[2];
 #pragma unroll 1
         for (int sys = 0; sys < 2; ++sys) {   // the u_t system from r_u, then the v_t system from r_v
             double rel = 0.0;
-            if (P.mixed && on) s.Ps32[t] = (float)T.Ps[t];
+            if (mixed && on) s.Ps32[t] = (float)T.Ps[t];
             if (sys) fx_arrived();
-            solve<N1>(P, s, T, e, sys == 0, w, ru, x, sys || !guess, guess && !sys, &it[sys], &sw[sys], &fell, &rel, false);
-            bad[sys] = (P.mixed ? sw[sys] >= P.refine_max : it[sys] >= P.maxit) && rel > P.rtol;
+            solve<N1, ROUTE>(P, s, T, e, sys == 0, w, ru, x, sys || !guess, guess && !sys, &it[sys], &sw[sys], &fell, &rel, false);
+            bad[sys] = (mixed ? sw[sys] >= P.refine_max : it[sys] >= P.maxit) && rel > P.rtol;
             __syncthreads();
             if (sys == 0) {
                 load_fx<N1>(s.A, P.Mx, e);
@@ -1272,15 +1431,15 @@ __device__ __forceinline__ void var_stage_body(const VarParams &P, const VarBufs
     if (on) {
         const double ku = rv, kv = x;
         double nu = 0.0, nv = 0.0;
-        if (MODE == M_RHS) {
+        if (mode == M_RHS) {
             b.oU[at] = ku;
             b.oV[at] = kv;
-        } else if (MODE == M_S1) {
+        } else if (mode == M_S1) {
             b.aU[at] = cA * ku;
             b.aV[at] = cA * kv;
             nu = Yu + cY * ku;
             nv = Yv + cY * kv;
-        } else if (MODE == M_S23) {
+        } else if (mode == M_S23) {
             b.aU[at] += cA * ku;
             b.aV[at] += cA * kv;
             nu = b.nU[at] + cY * ku;
@@ -1289,38 +1448,40 @@ __device__ __forceinline__ void var_stage_body(const VarParams &P, const VarBufs
             nu = b.nU[at] + b.aU[at] + cA * ku;
             nv = b.nV[at] + b.aV[at] + cA * kv;
         }
-        if (MODE != M_RHS) {
-            (MODE == M_S4 ? b.nU : b.oU)[at] = nu;
-            (MODE == M_S4 ? b.nV : b.oV)[at] = nv;
+        if (mode != M_RHS) {
+            (mode == M_S4 ? b.nU : b.oU)[at] = nu;
+            (mode == M_S4 ? b.nV : b.oV)[at] = nv;
             s.U[t] = nu;
             s.V[t] = nv;
         }
     }
     // the source block (the only reader of the source time) starts the next step
-    if (MODE == M_S4 && e == P.src_e && t == 0) *P.time += b.tstage;
-    if (MODE == M_RHS) return;
+    if (mode == M_S4 && e == P.src_e && t == 0) *P.time += b.tstage;
+    if (mode == M_RHS) return;
     __syncthreads();
     face_lines<N1>(s.U, s.V, T, b.trout + lix<N1>(e, 0), t, blockDim.x);
 }
 
-// Resident blocks promised to ptxas for the stage kernel: the 7 that the shared
-// memory of a block of at most 3 warps allows, 4 for larger elements.
-__host__ __device__ constexpr int var_stage_min_blocks(int n1) { return nthreads_for(n1 * n1) <= 96 ? 7 : 4; }
+// Resident blocks promised to ptxas for the stage kernel: the 7 (inverse route 8)
+// that the shared memory of a block of at most 3 warps allows, 4 for larger elements.
+__host__ __device__ constexpr int var_stage_min_blocks(int n1, int route) {
+    return nthreads_for(n1 * n1) <= 96 ? (route == ROUTE_INVERSE ? 8 : 7) : 4;
+}
 
-template <int N1, int MODE>
-__global__ void __launch_bounds__(nthreads_for(N1 * N1), var_stage_min_blocks(N1))
-k_var_stage(VarParams P, VarBufs b, double cA, double cY) {
+template <int N1, int ROUTE>
+__global__ void __launch_bounds__(nthreads_for(N1 * N1), var_stage_min_blocks(N1, ROUTE))
+k_var_stage(const __grid_constant__ VarParams P, const __grid_constant__ VarBufs b, int mode, double cA, double cY) {
     extern __shared__ __align__(16) double smraw[];
-    var_stage_body<N1, MODE>(P, b, cA, cY, blockIdx.x, smraw);
+    var_stage_body<N1, ROUTE>(P, b, mode, cA, cY, blockIdx.x, smraw);
 }
 
 // standalone element PCG (gdg_pcg): which = 0 M, 1 S (+ w w^T)
 template <int N1>
-__global__ void __launch_bounds__(nthreads_for(N1 * N1), var_stage_min_blocks(N1))
+__global__ void __launch_bounds__(nthreads_for(N1 * N1), var_stage_min_blocks(N1, ROUTE_ANY))
 k_var_pcg(VarParams P, int which, const double *bvec, double *xvec, int *iters, double *rel, int *sweeps) {
     constexpr int NA = N1 * N1;
     extern __shared__ __align__(16) double smraw[];
-    const StageSmem<N1> s(smraw);
+    const StageSmem<N1, false> s(smraw);
     const int e = blockIdx.x, t = threadIdx.x;
     const bool on = t < NA;
     const size_t at = (size_t)e * NA + (on ? t : 0);
@@ -1335,7 +1496,7 @@ k_var_pcg(VarParams P, int which, const double *bvec, double *xvec, int *iters, 
     }
     load_psi<N1>(P, s);
     fx_arrived();
-    solve<N1>(P, s, T, e, which != 0, w, b, x, false, false, &it, &sw, &fell, &rr, true);
+    solve<N1, ROUTE_ANY>(P, s, T, e, which != 0, w, b, x, false, false, &it, &sw, &fell, &rr, true);
     if (on) xvec[at] = x;
     if (t == 0) {
         iters[e] = it;

@@ -12,20 +12,15 @@ struct VarLaunch {
     // by every context: always raised to the device's opt-in maximum so that a
     // context with smaller needs cannot lower it under another one.
     static void attrs(int lim) {
-        cudaFuncSetAttribute(k_var_stage<N1, M_RHS>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_var_stage<N1, M_S1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_var_stage<N1, M_S23>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_var_stage<N1, M_S4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_var_stage<N1, ROUTE_ANY>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_var_stage<N1, ROUTE_MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_var_stage<N1, ROUTE_INVERSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_var_pcg<N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     }
     static void stage(const VarParams &P, size_t sm, int mode, const VarBufs &b, double cA, double cY, cudaStream_t s) {
         const dim3 grid(P.ne), block(nthreads_for(N1 * N1));   // one block per element
-        switch (mode) {
-        case M_RHS: k_var_stage<N1, M_RHS><<<grid, block, sm, s>>>(P, b, cA, cY); break;
-        case M_S1: k_var_stage<N1, M_S1><<<grid, block, sm, s>>>(P, b, cA, cY); break;
-        case M_S23: k_var_stage<N1, M_S23><<<grid, block, sm, s>>>(P, b, cA, cY); break;
-        default: k_var_stage<N1, M_S4><<<grid, block, sm, s>>>(P, b, cA, cY); break;
-        }
+        (P.staged ? k_var_stage<N1, ROUTE_INVERSE> : P.mixed ? k_var_stage<N1, ROUTE_MIXED> : k_var_stage<N1, ROUTE_ANY>)
+            <<<grid, block, sm, s>>>(P, b, mode, cA, cY);
     }
     static void pcg(const VarParams &P, size_t sm, int which, const double *b, double *x, int *iters, double *rel,
                     int *sweeps, cudaStream_t s) {
