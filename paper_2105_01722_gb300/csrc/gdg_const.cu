@@ -1635,8 +1635,13 @@ __global__ void k_stage_tables(int n, const double *lam2, double dt, double *lam
     if (i < RK_STAGES * n) lams[i] = lam2[i % n] * (dt / (RK_STAGES - i / n));
 }
 
+// A captured call only records the kernel, and a replay rewrites the tables at any
+// later time: from the first capture on they are written at every call.
 void stage_tables(gdg_ctx *ctx, double dt, cudaStream_t s) {
-    if (ctx->lams_dt == dt) return;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(s, &cs);
+    if (cs != cudaStreamCaptureStatusNone) ctx->lams_captured = true;
+    if (!ctx->lams_captured && ctx->lams_dt == dt) return;
     const int n = ctx->lam_len;
     k_stage_tables<<<(RK_STAGES * n + 255) / 256, 256, 0, s>>>(n, ctx->d_lam2, dt, ctx->d_lams);
     ctx->lams_dt = dt;

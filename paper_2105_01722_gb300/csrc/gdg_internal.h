@@ -121,6 +121,7 @@ struct gdg_ctx {
                                   // (the u lifts over lambda, see stage2p_body)
     double *d_lams = nullptr;     // d_lam2 times the factor of each RK stage, for the step size lams_dt
     double lams_dt = 0.0;
+    bool lams_captured = false;   // a captured graph writes d_lams too: lams_dt says nothing
     int lam_len = 0;              // doubles in d_lam2
     double *d_state = nullptr;    // modal work: yn(2 fields), YA(2), YB(2), K(2)
     double *d_tr = nullptr;       // two trace buffers (past the lower ghost row when halo sides exist)

@@ -103,3 +103,31 @@ def test_transforms_by_node_pairs(n, N, p):
     ctx.mass_solve(gdg.OP_M, b, b)
     assert torch.equal(x, b)
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [(16,), (12, 9), (3, 2, 2)])
+def test_step_sizes_of_a_captured_graph(n):
+    """A captured step replayed between steps of another size, against contexts
+    that see one size each."""
+    N, dt = 8, (0.01 / (max(n) * 8), 0.02 / (max(n) * 8))
+    ctx, plain = _context(n, N, 5, "upwind", (False,) * len(n)), _context(n, N, 5, "upwind", (False,) * len(n))
+    u, v = _state(n, N, 5)
+    a, b = u.clone(), v.clone()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        for w in (dt[0], dt[1], dt[0]):   # (the first call of a context times its kernels)
+            ctx.step(u, v, 0.0, w, 1, stream=s)
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            ctx.step(u, v, 0.0, dt[1], 1, stream=s)
+        ctx.step(u, v, 0.0, dt[0], 1, stream=s)
+        g.replay()
+        ctx.step(u, v, 0.0, dt[0], 1, stream=s)
+        s.synchronize()
+    for w in (dt[0], dt[1], dt[0], dt[0], dt[1], dt[0]):
+        plain.step(a, b, 0.0, w, 1)
+    torch.cuda.synchronize()
+    assert _rel((u, v), (a, b)) < 6 * TOL
+    ctx.close()
+    plain.close()
