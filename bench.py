@@ -113,7 +113,10 @@ def var_counts(n1, it_u, it_v, form, sweeps_u=0.0, sweeps_v=0.0):
     bytes: the FP64 element matrices (PCG: S_c2 and M_J, 2 NA^2 * 8; mixed:
     their FP32 copies plus the FP64 matrices once per sweep; inverse: the
     folded operators 189 NA * 8) plus the face operators (72 n1^2 * 8) and
-    the state."""
+    the state.
+    These are the counts of the forms in floating point, kept as the measure;
+    the kernels form most products on integers, read each matrix as a packed
+    triangle of 8-byte integers, and apply the inverses unfolded."""
     NA = n1 * n1
     face = 144 * n1 * n1 + 16 * NA
     it_cost = 2 * NA * NA + 8 * n1 ** 3 + 12 * NA

@@ -62,13 +62,12 @@ enum { GDG_COEF_CONST = 0, GDG_COEF_NODAL = 1 };
  * 7.1), or precomputed element inverses (GDG_COEF_NODAL only): the
  * precomputed-inverse route that Section 3.1 discusses, applied to the
  * time-independent element systems of Section 7.1.  gdg_create forms
- * (S_c2 + w w^T)^-1 and M_J^-1 per element by Cholesky and folds them with
- * the face lifts and the stiffness matrix into G_u = (S_c2 + w w^T)^-1 R_u,
- * G_v = M_J^-1 R_v and K = M_J^-1 S_c2 (R_u, R_v: the lifts of the face line
- * integrals into r_u, r_v; (12 (N+1) + (N+1)^2) (N+1)^2 more doubles per
- * element are kept, the inverses are freed after setup); every stage then
- * applies them instead of running PCG.  FP64 only (GDG_EUNSUPPORTED with
- * GDG_MIXED); gdg_pcg still runs PCG on such a context. */
+ * (S_c2 + w w^T)^-1 and M_J^-1 per element by Cholesky and keeps them as packed
+ * triangles of integers ((N+1)^2 ((N+1)^2 + 1) / 2 x 8 bytes each per element);
+ * every stage then applies them instead of running PCG.  FP64 only
+ * (GDG_EUNSUPPORTED with GDG_MIXED); gdg_pcg still runs PCG on such a context.
+ * Products with the element matrices and inverses run on 58-bit integers with
+ * exact sums in every form, as accurate as FP64 sums (gdg_fx.cuh). */
 enum { GDG_SOLVE_DIAG = 0, GDG_SOLVE_PCG = 1, GDG_SOLVE_INVERSE = 2 };
 /* PCG preconditioner: frozen-coefficient diagonalisation, none (plain CG),
  * or the zero fill-in incomplete Cholesky factors of Section 7.1, which the
@@ -76,8 +75,8 @@ enum { GDG_SOLVE_DIAG = 0, GDG_SOLVE_PCG = 1, GDG_SOLVE_INVERSE = 2 };
  * element; gdg_create returns GDG_EUNSUPPORTED). */
 enum { GDG_PC_FDM = 0, GDG_PC_NONE = 1, GDG_PC_IC0 = 2 };
 /* Arithmetic of the element solves.  GDG_FP64 everywhere, or (GDG_SOLVE_PCG
- * only) FP32 inner PCG with FP64 iterative refinement of every solve (FP64
- * state, residuals, lifts, norms and energy; same FP64 stopping test).
+ * only) FP32 inner PCG (its products with the element matrix on integers of 29
+ * and 28 bits) with FP64 iterative refinement of every solve (FP64 state, residuals, lifts, norms and energy; same FP64 stopping test).
  * Constant-coefficient contexts are FP64 only (GDG_EUNSUPPORTED otherwise):
  * their diagonal solves have no iteration to refine. */
 enum { GDG_FP64 = 0, GDG_MIXED = 1 };
@@ -385,7 +384,7 @@ int gdg_set_halo(gdg_ctx *ctx, double *send_lo, double *send_hi, double *recv_lo
 int gdg_mlp_forward(const uint16_t *w_bf16, const float *params, const float *X, int B, float *Y,
                     void *stream);
 
-/* Floats of the per-CTA partial buffer gdg_mlp_backward needs for B samples. */
+/* Floats of the scratch buffer gdg_mlp_backward needs for B samples (activations and errors). */
 long long gdg_mlp_partial_len(int B);
 
 /*
