@@ -1159,7 +1159,7 @@ k_fm_pack(double *FM, int slope_exp, int staged, short2 *FMq) {
 // line integrals L[f][m][j] of the element's four faces from its own face
 // lines and its neighbours' (lines: 24 N1 limb pairs of shared scratch).
 // A row's 6 N1 coefficients go to two threads, one for the own and one for the
-// neighbour's lines, whose exact sums are then added.  Bound by the 46.7 KB of
+// neighbour's lines, whose sums are then added.  Bound by the 46.7 KB of
 // face operators an element reads (N1 = 9).
 template <int N1>
 __device__ __forceinline__ void lift_lines(const VarParams &P, int e, const double *trin, int2 *lines, int *slot,
@@ -1235,8 +1235,8 @@ __device__ __forceinline__ void load_face(const VarParams &P, const SMEM &s, int
 // The same in the inverse route, whose operators all stream through: the face
 // operators come through the matrix's place in shared memory, as many at a time
 // as fit (the first ones on their way when this starts).  A row's three parts go
-// to three lanes of a warp, ten rows a warp; the exact sums of the two u parts
-// are added before they are rounded.  128^2 elements, four steps with element
+// to three lanes of a warp, ten rows a warp.  The own and the neighbour's lines are
+// rounded apart and then added, as in lift_lines: the same bits.  128^2 elements, four steps with element
 // inverses: 8.55 -> 7.50 ms, with the eighth block an SM that the smaller scratch
 // allows (staged alone 7.92).  In the iterative
 // routes, where S would have to be read again for the solve, the direct form is
@@ -1300,13 +1300,18 @@ __device__ __forceinline__ void lift_lines_staged(const VarParams &P, const SMEM
             const int4 *a = reinterpret_cast<const int4 *>(s.A + f % SLOTS * FACE + (part * NL + row) * 2 * N1);
             const int4 *x = reinterpret_cast<const int4 *>(s.lines + (f * 3 + part) * 2 * N1);
             FxSum sum;
+            long long own = 0;
 #pragma unroll
-            for (int i = 0; i < N1; ++i) {
-                const int4 av = a[i], xv = x[i];
-                sum.mad(make_int2(av.x, av.y), xv.x, xv.y);
-                sum.mad(make_int2(av.z, av.w), xv.z, xv.w);
+            for (int c = 0; c < 2 * N1; ++c) {
+                if (c == N1 && part == 0) {   // the own v lines end here
+                    own = sum.top();
+                    sum = FxSum();
+                }
+                const int4 av = a[c / 2], xv = x[c / 2];
+                if (c & 1) sum.mad(make_int2(av.z, av.w), xv.z, xv.w);
+                else sum.mad(make_int2(av.x, av.y), xv.x, xv.y);
             }
-            long long T = sum.top();
+            long long T = own + sum.top();
             const long long nbr = __shfl_down_sync(0xffffffffu, T, 1);
             if (part == 1) T += nbr;
             const double y = fx_value(T, fx_top_exp(part ? ku : kv) + (part ? q.y : q.x), part ? ku : kv);
