@@ -15,10 +15,16 @@
 //   sums     of limb products, 2^56 each, over at most 100 terms: below 2^63,
 //            exact and the same in any order.
 //
-// The rounding of a_ij and X_j (half a unit of 2^-57 of the largest) takes the
-// place of the rounding of every partial sum in FP64: the error of a product
-// with the element matrices, in the 2-norm against extended precision, is
-// 0.1 to 0.8 of that of the FP64 sum (p = 3, 5, 7, smooth and random vectors).
+// The rounding of a_ij and X_j (half a unit of 2^-57 of the largest) and, once a
+// row, of the sum (half a unit of 2^-56) takes the place of the rounding of every
+// partial sum in FP64, all of them to nearest: a sum cut off downwards would
+// err to one side at every stage, and sums over the mesh that the method conserves
+// would drift.  The error of a product with the element matrices and inverses, in
+// the 2-norm against extended precision, is on average 0.15 to 0.85 of that of the
+// FP64 sum for random and smooth vectors and pulses of a third of the element's
+// width (N = 4 to 9, p = 1 to 7); entries far below the largest keep fewer bits than a
+// double, so on pulses of a tenth of its width it is 0.3 to 1.1 of it on
+// average, and up to 4 times it in one vector.
 // A vector with an infinity or NaN gives NaN; entries below 2^-57 of the
 // largest, and subnormal ones, count as zero.
 #pragma once
@@ -61,10 +67,12 @@ __device__ __forceinline__ double fx_scale(long long T, int q) {
     return q > -1023 && q < 1024 ? v * fx_pow2(q) : scalbn(v, q);
 }
 
-// the exact sum of limb products
+// The sum of limb products, exact until top() or next() rounds it to nearest: m1
+// starts at half a unit of the result.
 struct FxSum {
+    static constexpr int TOP = FX_LIMB - 1, NEXT = FX_LIMB - 2;
     long long hh, m1, m2, ll;
-    __device__ FxSum() : hh(0), m1(0), m2(0), ll(0) {}
+    __device__ explicit FxSum(int half = TOP) : hh(0), m1(1ll << half), m2(0), ll(0) {}
     __device__ __forceinline__ void mad(int2 a, int2 x) {
         hh += (long long)a.x * x.x;
         m1 += (long long)a.x * x.y;
@@ -72,11 +80,11 @@ struct FxSum {
         ll += (long long)a.y * x.y;
     }
     __device__ __forceinline__ void mad(int2 a, int xh, int xl) { mad(a, make_int2(xh, xl)); }
-    // the sum in units of 2^58 (floor)
+    // the sum in units of 2^58
     __device__ __forceinline__ long long top() const {
         return hh + (((m1 >> 1) + (m2 >> 1) + (ll >> (FX_LIMB + 1))) >> (FX_LIMB - 1));
     }
-    // the sum in units of 2^57, as the next limbs of a chain of contractions
+    // the sum (from FxSum(NEXT)) in units of 2^57, as the next limbs of a chain of contractions
     // whose matrix rows sum to at most 1 (|sum| <= 2^114, few terms: m1 + m2 fits)
     __device__ __forceinline__ int2 next() const {
         return fx_split(hh + hh + ((m1 + m2 + (ll >> FX_LIMB)) >> (FX_LIMB - 1)));

@@ -355,7 +355,7 @@ __device__ __forceinline__ double fx_precondition(const FxSystem &f, const FxPre
     if (on) f.X[t] = fx_split(fx_int(r, e1));
     __syncthreads();
     if (on) {   // x modes: sum_i r[j][i] Psi[i][k]
-        FxSum s;
+        FxSum s(FxSum::NEXT);
 #pragma unroll
         for (int q = 0; q < N1; ++q) s.mad(p.Ps[q * N1 + c], f.X[a * N1 + q]);
         f.X2[t] = s.next();
@@ -372,7 +372,7 @@ __device__ __forceinline__ double fx_precondition(const FxSystem &f, const FxPre
     if (on) f.X[t] = fx_split(fx_int(v, e2));
     __syncthreads();
     if (on) {   // back in x: sum_k t[l][k] Psi[i][k]
-        FxSum s;
+        FxSum s(FxSum::NEXT);
 #pragma unroll
         for (int q = 0; q < N1; ++q) s.mad(p.Ps[c * N1 + q], f.X[a * N1 + q]);
         f.X2[t] = s.next();
