@@ -62,7 +62,8 @@ enum { GDG_COEF_CONST = 0, GDG_COEF_NODAL = 1 };
  * 7.1), or precomputed element inverses (GDG_COEF_NODAL only): the
  * precomputed-inverse route that Section 3.1 discusses, applied to the
  * time-independent element systems of Section 7.1.  gdg_create forms
- * (S_c2 + w w^T)^-1 and M_J^-1 per element by Cholesky and keeps them as packed
+ * (S_c2 + sigma w w^T)^-1 and M_J^-1 per element by Cholesky (sigma on the scale
+ * of S_c2; every sigma > 0 gives the same dU/dt) and keeps them as packed
  * triangles of integers ((N+1)^2 ((N+1)^2 + 1) / 2 x 8 bytes each per element);
  * every stage then applies them instead of running PCG.  FP64 only
  * (GDG_EUNSUPPORTED with GDG_MIXED); gdg_pcg still runs PCG on such a context.

@@ -333,7 +333,7 @@ int gdg_var_setup(gdg_ctx *ctx) {
     if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_fx, sets * fxm * sizeof(int2)), "alloc integer matrices")) ||
         (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_fxd, sets * nd), "alloc exponents")))
         return st;
-    if (P.inverse) {   // element inverses (S_c2 + w w^T)^-1 and M_J^-1
+    if (P.inverse) {   // element inverses of the two systems
         const size_t nm = nd * NA;
         if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_Ainv, nm * sizeof(double)), "alloc Ainv")) ||
             (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_Minv, nm * sizeof(double)), "alloc Minv")))

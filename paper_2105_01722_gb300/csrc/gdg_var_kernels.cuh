@@ -29,7 +29,7 @@ struct VarParams {
     // the operators of the stage as integers (gdg_fx.cuh).  Element matrices: packed lower triangles
     // (fx_tri_len entries an element) and the exponents d of their rows [ne][N1*N1]
     FxMatrix Sx, Mx;             // S_c2, M_J
-    FxMatrix Ax, Vx;             // (S_c2 + w w^T)^-1 - 1 1^T (k_var_invert), M_J^-1 (GDG_SOLVE_INVERSE)
+    FxMatrix Ax, Vx;             // inverse of the u_t system (k_var_invert), M_J^-1 (GDG_SOLVE_INVERSE)
     const int2 *FM;              // [ne][4 faces] operators, [6 N1 columns][3 N1 rows]; inverse route [3][3 N1 rows][2 N1] (k_fm_pack)
     const short2 *FMq;           // [ne][4 faces][3 N1] exponents of a row's v columns and u columns
     int staged;                  // FM's layout: lift_lines_staged's (stages of the inverse route outside batches)
@@ -1448,7 +1448,7 @@ __device__ __forceinline__ void var_stage_body(const VarParams &P, const VarBufs
         rv = b.rv[at];
         x = b.x0u[at];
     }
-    if (inverse) {   // dU/dt = V + (S_c2 + w w^T)^-1 r_u (k_var_invert), dV/dt = M_J^-1 r_v
+    if (inverse) {   // dU/dt = V + (S_c2 + sigma w w^T)^-1 r_u (k_var_invert), dV/dt = M_J^-1 r_v
 #pragma unroll 1
         for (int sys = 0; sys < 2; ++sys) {
             fx_arrived();
@@ -1575,11 +1575,16 @@ k_var_pcg(VarParams P, int which, const double *bvec, double *xvec, int *iters, 
 
 // Element inverse at setup (GDG_SOLVE_INVERSE; the precomputed-inverse route
 // of Section 3.1 applied to the element systems of Section 7.1):
-// Dst[e] = (Src[e] + w_e w_e^T)^-1 - 1 1^T (w != nullptr) or Src[e]^-1.
-// The u_t system's right-hand sides have 1^T r_u = 0 (the constant test
-// function has no gradient), and w^T y = 1^T r_u for its solution y, since
-// (S + w w^T) 1 = w; subtracting 1 1^T takes the rounding of 1^T r_u out of
-// w^T y = 0 and changes nothing else (still symmetric, and positive
+// Dst[e] = (Src[e] + sigma w_e w_e^T)^-1 - (1/sigma) 1 1^T (w != nullptr) or
+// Src[e]^-1.  The u_t system's right-hand sides have 1^T r_u = 0 (the constant
+// test function has no gradient), so its solution y is the same for every weight
+// sigma > 0: (S + sigma w w^T) 1 = sigma w, hence w^T y = 1^T r_u / sigma = 0.
+// sigma, the power of two at or below the trace of S, puts the rank-one term among
+// the eigenvalues of S: the inverse is as well conditioned as S on the
+// functions without a constant part, whatever the size of c^2 (with sigma = 1 its
+// error grew with c^2, 1e-4 at c^2 = 1e8, where it is 1e-13 now, and the part
+// below could outweigh the rest of it).  Subtracting (1/sigma) 1 1^T takes the rounding of
+// 1^T r_u out of w^T y and changes nothing else (still symmetric, and positive
 // semidefinite).  By Cholesky
 // A = L L^T in shared memory and one forward + back substitution per column
 // of the identity (thread j solves column j); the result is made exactly
@@ -1593,9 +1598,15 @@ k_var_invert(const double *__restrict__ Src, const double *__restrict__ w, doubl
     const int e = blockIdx.x, t = threadIdx.x, nt = blockDim.x;
     const double *src = Src + (size_t)e * NA * NA;
     const double *we = w ? w + (size_t)e * NA : nullptr;
+    double sigma = 1.0;
+    if (we) {
+        double trace = 0.0;
+        for (int i = 0; i < NA; ++i) trace += src[i * (NA + 1)];
+        sigma = scalbn(1.0, ilogb(trace));
+    }
     for (int i = t; i < NA * NA; i += nt) {
         const int r = i / NA, c = i - (i / NA) * NA;
-        A[i] = src[i] + (we ? we[r] * we[c] : 0.0);
+        A[i] = src[i] + (we ? sigma * (we[r] * we[c]) : 0.0);
     }
     __syncthreads();
     // right-looking Cholesky, lower triangle in place
@@ -1645,7 +1656,7 @@ k_var_invert(const double *__restrict__ Src, const double *__restrict__ w, doubl
     double *dst = Dst + (size_t)e * NA * NA;
     for (int i = t; i < NA * NA; i += nt) {
         const int r = i / NA, c = i - (i / NA) * NA;
-        dst[i] = (r > c ? B[c * NA + r] : B[i]) - (we ? 1.0 : 0.0);
+        dst[i] = (r > c ? B[c * NA + r] : B[i]) - (we ? 1.0 / sigma : 0.0);
     }
 }
 

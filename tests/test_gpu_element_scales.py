@@ -1,0 +1,58 @@
+"""Element operators at scales other than 1: the mapped path through gdg_rhs, gdg_step and
+gdg_batch_step where c^2 is not of order 1."""
+import numpy as np
+import pytest
+
+from paper_2105_01722_gb300 import gdg, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _problem(n, N, p, c2_factor=1.0, size=1.0, **kw):
+    X, Y = inputs.mapped_nodes(n, N, 0.05)
+    return gdg.make_problem(2, n, N, p, coef=gdg.COEF_NODAL, x_nodes=X * size, y_nodes=Y * size,
+                            c2_nodes=inputs.c2_sine(X, Y) * c2_factor, **kw)
+
+
+def _gpu(a):
+    import torch
+    return torch.tensor(np.ascontiguousarray(a, dtype=np.float64).ravel(), device="cuda")
+
+
+# the wave equation is the same under c^2 -> s^2 c^2, v -> s v, t -> t / s; with s a power of two
+# every product, sum, quotient and square root of the inverse route scales by one too
+SCALES = [-10, 7, 10, 13]
+
+
+@pytest.mark.parametrize("k", SCALES)
+@pytest.mark.parametrize("N,p", [(7, 3), (8, 5), (9, 7)])
+def test_inverse_route_does_not_depend_on_the_unit_of_time(N, p, k):
+    """c^2 from 1e-6 to 7e7: the same bits, up to the scale, as with c^2 of order 1."""
+    import torch
+    n, na = (4, 4), 16 * (N + 1) ** 2
+    out = []
+    for s in (1.0, 2.0**k):
+        ctx = gdg.Context(_problem(n, N, p, c2_factor=s * s, solver=gdg.SOLVE_INVERSE))
+        u, v = _gpu(inputs.random_state((na,), 1)), _gpu(inputs.random_state((na,), 2)) * s
+        du, dv = torch.empty_like(u), torch.empty_like(u)
+        ctx.rhs(u, v, du, dv)
+        ctx.step(u, v, 0.0, 1e-3 / s, 2)
+        out.append([du / s, dv / s**2, u, v / s])
+        ctx.close()
+    for a, b in zip(*out):
+        assert bool(torch.isfinite(a).all()) and torch.equal(a, b)
+
+
+@pytest.mark.parametrize("k", SCALES)
+def test_batched_inverses_do_not_depend_on_the_unit_of_time(k):
+    import torch
+    out = []
+    for s in (1.0, 2.0**k):
+        batch = gdg.Batch([_problem((3, 2), 8, p, c2_factor=s * s, solver=gdg.SOLVE_INVERSE) for p in (3, 7)])
+        us = [_gpu(inputs.random_state((6 * 81,), 1 + i)) for i in range(2)]
+        vs = [_gpu(inputs.random_state((6 * 81,), 5 + i)) * s for i in range(2)]
+        batch.step(us, vs, [1e-3 / s] * 2, 2)
+        out.append(us + [v / s for v in vs])
+        batch.close()
+    for a, b in zip(*out):
+        assert bool(torch.isfinite(a).all()) and torch.equal(a, b)
