@@ -331,7 +331,7 @@ int gdg_var_setup(gdg_ctx *ctx) {
     const size_t fxm = (size_t)ctx->ne * fx_tri_len(NA);   // one set of packed integer matrices
     const int sets = P.inverse ? 4 : 2;
     if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_fx, sets * fxm * sizeof(int2)), "alloc integer matrices")) ||
-        (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_fxd, sets * nd), "alloc exponents")))
+        (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_fxd, sets * nd * sizeof(short)), "alloc exponents")))
         return st;
     if (P.inverse) {   // element inverses of the two systems
         const size_t nm = nd * NA;
@@ -353,7 +353,7 @@ int gdg_var_setup(gdg_ctx *ctx) {
     const double *const from[4] = {D->d_S, D->d_M, D->d_Ainv, D->d_Minv};
     for (int k = 0; k < sets; ++k) {
         int2 *A = D->d_fx + k * fxm;
-        signed char *d = D->d_fxd + k * nd;
+        short *d = D->d_fxd + k * nd;
         const int grid = (int)std::min<long long>(ctx->ne, 65535);
         switch (n1) {
 #define X(n) case n: k_fx_pack<n><<<grid, 128>>>(ctx->ne, from[k], A, d); break;

@@ -13,8 +13,9 @@
 // element matrices as integers (k_fx_pack)
 struct FxMatrix {
     const int2 *A;
-    const signed char *d;
+    const short *d;   // FX_BAD: the element's matrix is not finite, nor is any product with it
 };
+constexpr short FX_BAD = 0x7fff;
 
 struct VarParams {
     int nx, ny, ne, Q;
@@ -85,7 +86,7 @@ struct VarData {
     double *d_S = nullptr, *d_M = nullptr, *d_w = nullptr, *d_pre = nullptr, *d_face = nullptr;
     double *d_dS = nullptr;
     int2 *d_fx = nullptr;                        // packed integer matrices: S, M (, A^-1, M^-1)
-    signed char *d_fxd = nullptr;                // their row exponents
+    short *d_fxd = nullptr;                      // their row exponents
     double *d_FM = nullptr;                      // face operators (integers after k_fm_pack)
     short2 *d_FMq = nullptr;
     int2 *d_Psx = nullptr;
@@ -200,7 +201,7 @@ __device__ __forceinline__ T block_sum(T v, double *red) {
 // one element's matrix and the block's scratch
 struct FxSystem {
     const int2 *A;   // packed integers (shared)
-    int d;           // exponent of the thread's row
+    int d;           // exponent of the thread's row (FX_NAN: the matrix is not finite)
     int2 *X, *X2;    // limb vectors (shared, 16-byte aligned)
     int *slot;       // shared: two sets of 8 ints, used in turn
 };
@@ -326,7 +327,7 @@ __device__ __forceinline__ double fx_matvec(const FxSystem &f, double x, int set
         if (WIDE) fx_row_wide<NA>(f.A, row);
         else fx_row<NA>(f.A, [&](int2 a, int k) { row.s.mad(a, row.X[k]); });
     }
-    return fx_value(row.s.top(), fx_top_exp(emax) + f.d, emax);
+    return fx_value(row.s.top(), fx_top_exp(emax) + f.d, max(emax, f.d));
 }
 
 // Psi of the frozen-coefficient preconditioner as integers (shared), and the
@@ -999,7 +1000,8 @@ struct StageSmem {
     }
     static constexpr size_t bytes() { return sizeof(double) * (size_t)LEN; }
     __device__ __forceinline__ FxSystem system(const FxMatrix &m, int e) const {
-        return FxSystem{A, threadIdx.x < NA ? m.d[(size_t)e * NA + threadIdx.x] : 0, X, X2, slot};
+        const int d = threadIdx.x < NA ? m.d[(size_t)e * NA + threadIdx.x] : 0;
+        return FxSystem{A, d == FX_BAD ? FX_NAN : d, X, X2, slot};
     }
     __device__ __forceinline__ SolveBufs bufs() const { return SolveBufs{r, z, p, Ap, red, w}; }
 };
@@ -1661,25 +1663,39 @@ k_var_invert(const double *__restrict__ Src, const double *__restrict__ w, doubl
 }
 
 // Integer form of ne exactly symmetric NA x NA element matrices (gdg_fx.cuh):
-// packed lower triangles and row exponents, one block per element
+// packed lower triangles and row exponents, one block per element.  The exponents
+// of the rows are those of their diagonal entries, which bound every entry of
+// a positive semidefinite matrix; a matrix with a larger entry (of a folded
+// element, say) takes the exponent of its largest entry for every row.
 template <int N1>
-__global__ void k_fx_pack(int ne, const double *__restrict__ src, int2 *__restrict__ dst,
-                          signed char *__restrict__ dexp) {
+__global__ void k_fx_pack(int ne, const double *__restrict__ src, int2 *__restrict__ dst, short *__restrict__ dexp) {
     constexpr int NA = N1 * N1;
-    __shared__ int d[NA];
+    __shared__ int d[NA], largest, beyond;
     for (int e = blockIdx.x; e < ne; e += gridDim.x) {
         const double *A = src + (size_t)e * NA * NA;
-        for (int i = threadIdx.x; i < NA; i += blockDim.x) {
-            // A_ii < 2^k: half of it, rounded up
-            const int k = fx_expo(A[(size_t)i * NA + i]) - 1022;
-            d[i] = max(-120, min((k + 1) >> 1, 120));
-            dexp[(size_t)e * NA + i] = (signed char)d[i];
-        }
+        for (int i = threadIdx.x; i < NA; i += blockDim.x)
+            d[i] = (fx_expo(A[(size_t)i * NA + i]) - 1022 + 1) >> 1;   // A_ii < 2^k: half of k, rounded up
+        if (threadIdx.x == 0) largest = beyond = 0;
         __syncthreads();
+        int big = 0, over = 0;
+        for (int q = threadIdx.x; q < NA * NA; q += blockDim.x) {
+            const int k = fx_expo(A[q]);
+            big = max(big, k);
+            over |= k - 1022 > d[q / NA] + d[q % NA];
+        }
+        atomicMax(&largest, big);
+        atomicOr(&beyond, over);
+        __syncthreads();
+        const bool finite = largest != 0x7ff;
+        if (beyond)
+            for (int i = threadIdx.x; i < NA; i += blockDim.x) d[i] = (largest - 1022 + 1) >> 1;
+        __syncthreads();
+        for (int i = threadIdx.x; i < NA; i += blockDim.x) dexp[(size_t)e * NA + i] = finite ? (short)d[i] : FX_BAD;
         int2 *L = dst + (size_t)e * fx_tri_len(NA);
         for (int q = threadIdx.x; q < NA * NA; q += blockDim.x) {
             const int i = q / NA, k = q - (q / NA) * NA;
-            if (k <= i) L[i * (i + 1) / 2 + k] = fx_split(__double2ll_rn(scalbn(A[q], FX_ONE - d[i] - d[k])));
+            if (k <= i)
+                L[i * (i + 1) / 2 + k] = finite ? fx_split(__double2ll_rn(scalbn(A[q], FX_ONE - d[i] - d[k]))) : make_int2(0, 0);
         }
         if (NA * (NA + 1) / 2 < fx_tri_len(NA) && threadIdx.x == 0) L[NA * (NA + 1) / 2] = make_int2(0, 0);
         __syncthreads();

@@ -1,5 +1,5 @@
 """Element operators at scales other than 1: the mapped path through gdg_rhs, gdg_step and
-gdg_batch_step where c^2 is not of order 1."""
+gdg_batch_step where c^2 or the mesh is not of order 1, and where a matrix is not finite."""
 import numpy as np
 import pytest
 
@@ -56,3 +56,48 @@ def test_batched_inverses_do_not_depend_on_the_unit_of_time(k):
         batch.close()
     for a, b in zip(*out):
         assert bool(torch.isfinite(a).all()) and torch.equal(a, b)
+
+
+@pytest.mark.parametrize("k", [-133, 133])
+@pytest.mark.parametrize("form", ["pcg", "inverse"])
+@pytest.mark.parametrize("what", ["length", "time"])
+def test_far_scales(what, form, k):
+    """Meshes of 1e-40 and 1e40, c^2 of 1e-80 and 1e80: matrix entries far beyond 2^+-240, the same
+    bits as at scale 1.  (The iteration of the PCG form sees c^2 against its rank-one term: there the residuals
+    alone are the same.)"""
+    import torch
+    n, N, p = (3, 2), 8, 5
+    out = []
+    for s in (1.0, 2.0**k):
+        size, c2 = (s, 1.0) if what == "length" else (1.0, s * s)
+        rate = 1.0 / s if what == "length" else s            # time runs faster by this factor
+        ctx = gdg.Context(_problem(n, N, p, c2_factor=c2, size=size,
+                                   solver=gdg.SOLVE_INVERSE if form == "inverse" else gdg.SOLVE_PCG))
+        u, v = _gpu(inputs.random_state((6 * 81,), 1)), _gpu(inputs.random_state((6 * 81,), 2)) * rate
+        ru, rv, du, dv = (torch.empty_like(u) for _ in range(4))
+        ctx.residuals(u, v, ru, rv)
+        fields = [ru / rate / c2, rv / c2]
+        if form == "inverse" or what == "length":
+            ctx.rhs(u, v, du, dv)
+            fields += [du / rate, dv / rate / rate]
+        out.append(fields)
+        ctx.close()
+    for a, b in zip(*out):
+        assert bool(torch.isfinite(a).all()) and torch.equal(a, b)
+
+
+def test_inverses_that_are_not_finite_stay_visible():
+    """A node pushed through its neighbours folds an element: its matrices are not positive definite, the
+    Cholesky factors not finite, and neither are its time derivatives; the other elements' are."""
+    import torch
+    X, Y = inputs.cartesian_nodes((2, 2), 8)
+    X = X.copy()
+    X[0, 0, 4, 4] += 0.2
+    ctx = gdg.Context(gdg.make_problem(2, (2, 2), 8, 5, coef=gdg.COEF_NODAL, x_nodes=X, y_nodes=Y, c2_nodes=np.ones_like(X),
+                                       solver=gdg.SOLVE_INVERSE))
+    u, v = _gpu(inputs.random_state((4 * 81,), 5)), _gpu(inputs.random_state((4 * 81,), 6))
+    du, dv = torch.zeros_like(u), torch.zeros_like(u)
+    ctx.rhs(u, v, du, dv)
+    for f in (du.view(4, 81), dv.view(4, 81)):
+        assert not bool(torch.isfinite(f[0]).any()) and bool(torch.isfinite(f[1:]).all())
+    ctx.close()
