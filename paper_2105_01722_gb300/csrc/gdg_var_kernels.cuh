@@ -1144,18 +1144,26 @@ k_fm_pack(double *FM, int slope_exp, int staged, short2 *FMq) {
                 const int k = fx_key(in[c * NL + r], slope_line<N1>(f, m) ? slope_exp : 0) - 1022;   // |v| < 2^k
                 if (m == 0) qv = max(qv, k); else qu = max(qu, k);
             }
-            qv = max(-16000, min(qv, 16000));
-            qu = max(-16000, min(qu, 16000));
+            // Inf and NaN (c^2 interpolated below zero has no square root) mark the row: FX_BAD
+            qv = qv > FX_NAN / 2 ? FX_BAD : max(-16000, qv);
+            qu = qu > FX_NAN / 2 ? FX_BAD : max(-16000, qu);
             FMq[((size_t)e * 4 + f) * NL + r] = make_short2((short)qv, (short)qu);
             for (int c = 0; c < 2 * NL; ++c) {
                 const int m = (c % NL) / N1;
                 const int to = staged ? (line_third<N1>(c) * NL + r) * 2 * N1 + line_place<N1>(c) : c * NL + r;
                 reinterpret_cast<int2 *>(face)[to] =
-                    fx_split(fx_int(in[c * NL + r], (m == 0 ? qv : qu) + 1022, slope_line<N1>(f, m) ? slope_exp : 0));
+                    (m == 0 ? qv : qu) == FX_BAD
+                        ? make_int2(0, 0)
+                        : fx_split(fx_int(in[c * NL + r], (m == 0 ? qv : qu) + 1022, slope_line<N1>(f, m) ? slope_exp : 0));
             }
         }
         __syncthreads();
     }
+}
+
+// a row's sum T as a line integral; q: the exponent of its columns
+__device__ __forceinline__ double fx_face_value(long long T, int q, int emax) {
+    return fx_value(T, fx_top_exp(emax) + q, q == FX_BAD ? FX_NAN : emax);
 }
 
 // line integrals L[f][m][j] of the element's four faces from its own face
@@ -1217,7 +1225,7 @@ __device__ __forceinline__ void lift_lines(const VarParams &P, int e, const doub
         S += __shfl_xor_sync(0xffffffffu, S, 1);
         const short2 q = P.FMq[(size_t)e * 4 * NL + task];
         // one conversion a thread: the even one takes the v sum, the odd one the u sum
-        double y = side ? fx_value(S, fx_top_exp(ku) + q.y, ku) : fx_value(T, fx_top_exp(kv) + q.x, kv);
+        double y = side ? fx_face_value(S, q.y, ku) : fx_face_value(T, q.x, kv);
         y += __shfl_xor_sync(0xffffffffu, y, 1);
         if (side == 0 && task0 + (t >> 1) < 4 * NL) L[task] = y;
     }
@@ -1316,7 +1324,7 @@ __device__ __forceinline__ void lift_lines_staged(const VarParams &P, const SMEM
             long long T = own + sum.top();
             const long long nbr = __shfl_down_sync(0xffffffffu, T, 1);
             if (part == 1) T += nbr;
-            const double y = fx_value(T, fx_top_exp(part ? ku : kv) + (part ? q.y : q.x), part ? ku : kv);
+            const double y = fx_face_value(T, part ? q.y : q.x, part ? ku : kv);
             const double u = __shfl_down_sync(0xffffffffu, y, 1);
             if (part == 0 && lane < 30 && row0 + lane / 3 < NL) s.L[f * NL + row] = y + u;
         }

@@ -3,6 +3,7 @@ gdg_batch_step where c^2 or the mesh is not of order 1, and where a matrix is no
 import numpy as np
 import pytest
 
+from oracle import dg_var as dv
 from paper_2105_01722_gb300 import gdg, inputs
 
 pytestmark = pytest.mark.gpu
@@ -100,4 +101,29 @@ def test_inverses_that_are_not_finite_stay_visible():
     ctx.rhs(u, v, du, dv)
     for f in (du.view(4, 81), dv.view(4, 81)):
         assert not bool(torch.isfinite(f[0]).any()) and bool(torch.isfinite(f[1:]).all())
+    ctx.close()
+
+
+@pytest.mark.parametrize("form", ["pcg", "mixed", "inverse"])
+def test_face_operators_that_are_not_finite_stay_visible(form):
+    """Positive nodal c^2 whose interpolant dips below zero on two faces of one element: its local
+    wave speed is NaN there.  So are r_u in the element (the lifts of a face's line integrals reach every node,
+    if with factor zero) and r_v at the nodes of those faces, as in FP64 sums, and nothing else."""
+    import torch
+    n, N, p = (4, 1), 8, 5
+    X, Y = inputs.cartesian_nodes(n, N)
+    C2 = np.ones_like(X)
+    C2[0, 1, 0::2, :] = 1e-3          # element 1: dips between its rows, on its left and right faces
+    with np.errstate(invalid="ignore"):
+        c = dv.assemble(dv.VarProblem(n=n, N=N, p=p, X=X, Y=Y, C2=C2)).c
+    assert [bool(np.isnan(c[f]).any()) for f in dv.FACES] == [True, True, False, False]
+    assert not any(np.isnan(c[f][[0, 2, 3]]).any() for f in dv.FACES)
+    kw = {"pcg": {}, "mixed": {"precision": gdg.MIXED}, "inverse": {"solver": gdg.SOLVE_INVERSE}}[form]
+    ctx = gdg.Context(gdg.make_problem(2, n, N, p, coef=gdg.COEF_NODAL, x_nodes=X, y_nodes=Y, c2_nodes=C2, pcg_maxit=30, **kw))
+    u, v = _gpu(inputs.random_state((4, 81), 5)), _gpu(inputs.random_state((4, 81), 6))
+    ru, rv = torch.empty_like(u), torch.empty_like(u)
+    ctx.residuals(u, v, ru, rv)
+    ru, rv = (torch.isnan(f).cpu().numpy().reshape(4, 9, 9) for f in (ru, rv))
+    assert ru[1].all() and rv[1][:, [0, 8]].all() and not rv[1][:, 1:8].any()
+    assert not ru[[0, 2, 3]].any() and not rv[[0, 2, 3]].any()
     ctx.close()
