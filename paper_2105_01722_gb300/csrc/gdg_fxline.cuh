@@ -45,8 +45,11 @@ __device__ __forceinline__ long long fx_pair_value(long long hh, long long mid) 
     return hh + hh + ((mid + (1 << (FX_LIMB - 2))) >> (FX_LIMB - 1));
 }
 
-// limbs of X = Z 2^-5, |Z| < 2^62, the low one balanced
+// limbs of X = Z 2^-5, |Z| < 2^62, the low one balanced; X is rounded to nearest, halves
+// away from zero: entries of either sign are treated alike, and what is conserved
+// does not drift from transform to transform
 __device__ __forceinline__ void fx_limbs(long long Z, int &h, int &l) {
+    Z += 16 + (Z >> 63);
     const int hi = (int)(Z >> 32);
     h = (hi + 2) >> 2;
     l = (int)__funnelshift_r((unsigned)Z, (unsigned)hi, 2) >> 3;
