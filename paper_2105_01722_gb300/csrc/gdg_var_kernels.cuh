@@ -207,6 +207,7 @@ struct FxSystem {
 };
 
 constexpr int FX_NAN = 1 << 20;   // block exponent of a vector with an Inf or NaN
+#define FX_QNAN __longlong_as_double(0x7ff8000000000000ll)
 
 // exponent of v 2^shift for the maximum of a vector (zero and subnormals: below every other)
 __device__ __forceinline__ int fx_key(double v, int shift = 0) {
@@ -228,7 +229,7 @@ __device__ __forceinline__ int fx_block_max(int k, int *slot, int set) {
 
 // T 2^q, or NaN where the vector behind T had an Inf or NaN
 __device__ __forceinline__ double fx_value(long long T, int q, int emax) {
-    return emax >= FX_NAN / 2 ? __longlong_as_double(0x7ff8000000000000ll) : fx_scale(T, q);
+    return emax >= FX_NAN / 2 ? FX_QNAN : fx_scale(T, q);
 }
 
 // mad(entry (t, k), k) over row t of the packed matrix: the columns of earlier
@@ -528,7 +529,7 @@ __device__ __forceinline__ int pcg(const FxSystem &f, const FxPrecond &pre, cons
     rr = v.red[2];
     if (want_rel || it >= maxit) {   // the cap, or the caller's statistics
         __syncthreads();
-        if (t == 0) v.red[3] = b2 > 0.0 ? sqrt(rr) / sqrt(b2) : 0.0;
+        if (t == 0) v.red[3] = b2 == 0.0 ? 0.0 : sqrt(rr) / sqrt(b2);   // (NaN where b is)
         __syncthreads();
         *relres = v.red[3];
     } else {
@@ -699,7 +700,8 @@ __device__ __forceinline__ int refine(const FxSystem &f, const FxPrecond &pre, c
         ++sweeps;
     }
     *inner = its;
-    *relres = bnorm > 0.0 ? rn / bnorm : 0.0;
+    *relres = bnorm == 0.0 ? 0.0 : rn / bnorm;
+    if (!isfinite(rn)) x = *relres = FX_QNAN;   // no sweep runs on a NaN, and x may still be zero
     return sweeps;
 }
 
@@ -1481,7 +1483,8 @@ __device__ __forceinline__ void var_stage_body(const VarParams &P, const VarBufs
             if (mixed && on) s.Ps32[t] = (float)T.Ps[t];
             if (sys) fx_arrived();
             solve<N1, ROUTE>(P, s, T, e, sys == 0, w, ru, x, sys || !guess, guess && !sys, &it[sys], &sw[sys], &fell, &rel, false);
-            bad[sys] = (mixed ? sw[sys] >= P.refine_max : it[sys] >= P.maxit) && rel > P.rtol;
+            // (rel is formed at the cap and in the mixed form; a NaN is no convergence)
+            bad[sys] = !(rel <= P.rtol) && (!mixed || sw[sys] >= P.refine_max || isnan(rel));
             __syncthreads();
             if (sys == 0) {
                 load_fx<N1>(s.A, P.Mx, e);
