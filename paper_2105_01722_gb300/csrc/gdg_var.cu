@@ -50,6 +50,9 @@ size_t geom_smem(int N1, int Q) {
 }
 size_t traces_smem(int N1, int Q) { return sizeof(double) * ((size_t)tab_len(Q, N1) + 2 * N1 * N1 + 12 * N1); }
 
+// FP64 element matrices held at a time during the setup (5000 elements at N1 = 9; smaller meshes whole)
+constexpr size_t SETUP_BYTES = (size_t)512 << 20;
+
 size_t invert_smem(int N1) { return sizeof(double) * (2 * (size_t)N1 * N1 * N1 * N1 + (size_t)N1 * N1); }
 
 const VarOps &ops_of(int n1) {
@@ -201,9 +204,7 @@ int gdg_var_setup(gdg_ctx *ctx) {
     const size_t nd = (size_t)ctx->ndof;
     int st;
     D->tr_len = (long long)ctx->ne * 12 * n1;   // face lines: 4 faces x 3 N1 per element
-    if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_S, nd * NA * sizeof(double)), "alloc S")) ||
-        (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_M, nd * NA * sizeof(double)), "alloc M")) ||
-        (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_w, nd * sizeof(double)), "alloc w")) ||
+    if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_w, nd * sizeof(double)), "alloc w")) ||
         (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_pre, (size_t)ctx->ne * 4 * sizeof(double)), "alloc pre")) ||
         (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_face, (size_t)ctx->ne * 16 * Q * sizeof(double)), "alloc face")) ||
         (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_tab, tab.size() * sizeof(double)), "alloc tab")) ||
@@ -254,7 +255,7 @@ int gdg_var_setup(gdg_ctx *ctx) {
     P.rtol = ctx->pb.pcg_rtol;
     P.maxit = ctx->pb.pcg_maxit;
     P.precond = ctx->pb.precond;
-    P.tab = D->d_tab; P.S = D->d_S; P.M = D->d_M; P.w = D->d_w; P.pre = D->d_pre; P.face = D->d_face;
+    P.tab = D->d_tab; P.w = D->d_w; P.pre = D->d_pre; P.face = D->d_face;
     P.stats = D->d_stats;
     P.mixed = ctx->pb.precision == GDG_MIXED;
     P.inverse = ctx->pb.solver == GDG_SOLVE_INVERSE;
@@ -276,11 +277,37 @@ int gdg_var_setup(gdg_ctx *ctx) {
     if (D->smem_pcg > 220 * 1024 || D->smem_geom > 220 * 1024 ||
         (ctx->pb.solver == GDG_SOLVE_INVERSE && invert_smem(n1) > 220 * 1024))
         return gdg_set_err(ctx, GDG_EUNSUPPORTED, "element too large for shared memory (reduce nquad)");
+    // the element matrices: S, M (, the inverses of both systems) in FP64 for a part of the mesh at a time, then
+    // as packed integers, which are kept
     const double *Xd = D->d_nodes, *Yd = D->d_nodes + nd, *Cd = D->d_nodes + 2 * nd;
-    switch (n1) {
-#define X(n) case n: k_var_geom<n><<<ctx->ne, GEOM_THREADS, D->smem_geom>>>(P, Xd, Yd, Cd, D->d_S, D->d_M, D->d_w, D->d_pre, D->d_face); break;
-        GDG_VAR_CASES(X)
+    const size_t fxm = (size_t)ctx->ne * fx_tri_len(NA), full = (size_t)NA * NA;
+    const int sets = P.inverse ? 4 : 2;
+    const int most = (int)std::max<size_t>(1, std::min<size_t>(ctx->ne, SETUP_BYTES / (sets * full * sizeof(double))));
+    if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_fx, sets * fxm * sizeof(int2)), "alloc integer matrices")) ||
+        (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_fxd, sets * nd * sizeof(short)), "alloc exponents")) ||
+        (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_work, sets * most * full * sizeof(double)), "alloc matrices")))
+        return st;
+    FxMatrix *const fxs[4] = {&P.Sx, &P.Mx, &P.Ax, &P.Vx};
+    for (int k = 0; k < sets; ++k) *fxs[k] = FxMatrix{D->d_fx + k * fxm, D->d_fxd + k * nd};
+    for (int e0 = 0; e0 < ctx->ne; e0 += most) {
+        const int count = std::min(most, ctx->ne - e0);
+        double *const A[4] = {D->d_work, D->d_work + most * full, D->d_work + 2 * most * full, D->d_work + 3 * most * full};
+        const size_t ism = invert_smem(n1), v0 = (size_t)e0 * NA, m0 = (size_t)e0 * fx_tri_len(NA);
+        const int threads = nthreads_for(NA), grid = std::min(count, 65535);
+        switch (n1) {
+#define X(n)                                                                                                          \
+    case n:                                                                                                           \
+        k_var_geom<n><<<count, GEOM_THREADS, D->smem_geom>>>(P, e0, Xd, Yd, Cd, A[0], A[1], D->d_w, D->d_pre, D->d_face); \
+        if (P.inverse) {                                                                                              \
+            k_var_invert<n><<<count, threads, ism>>>(A[0], D->d_w + v0, A[2]);                                        \
+            k_var_invert<n><<<count, threads, ism>>>(A[1], nullptr, A[3]);                                            \
+        }                                                                                                             \
+        for (int k = 0; k < sets; ++k)                                                                                \
+            k_fx_pack<n><<<grid, 128>>>(count, A[k], D->d_fx + k * fxm + m0, D->d_fxd + k * nd + v0);                  \
+        break;
+            GDG_VAR_CASES(X)
 #undef X
+        }
     }
     // face operators: 4 faces x 6 N1 columns x 3 N1 rows per element, from the face data
     if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_FM, (size_t)ctx->ne * 72 * n1 * n1 * sizeof(double)), "alloc FM")))
@@ -328,46 +355,10 @@ int gdg_var_setup(gdg_ctx *ctx) {
 #undef X
     }
     P.dS = D->d_dS;
-    const size_t fxm = (size_t)ctx->ne * fx_tri_len(NA);   // one set of packed integer matrices
-    const int sets = P.inverse ? 4 : 2;
-    if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_fx, sets * fxm * sizeof(int2)), "alloc integer matrices")) ||
-        (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_fxd, sets * nd * sizeof(short)), "alloc exponents")))
-        return st;
-    if (P.inverse) {   // element inverses of the two systems
-        const size_t nm = nd * NA;
-        if ((st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_Ainv, nm * sizeof(double)), "alloc Ainv")) ||
-            (st = gdg_cuda_check(ctx, cudaMalloc((void **)&D->d_Minv, nm * sizeof(double)), "alloc Minv")))
-            return st;
-        const size_t ism = invert_smem(n1);
-        switch (n1) {
-#define X(n)                                                                                         \
-    case n:                                                                                          \
-        k_var_invert<n><<<ctx->ne, nthreads_for(n * n), ism>>>(D->d_S, D->d_w, D->d_Ainv);           \
-        k_var_invert<n><<<ctx->ne, nthreads_for(n * n), ism>>>(D->d_M, nullptr, D->d_Minv);          \
-        break;
-            GDG_VAR_CASES(X)
-#undef X
-        }
-    }
-    FxMatrix *const fxs[4] = {&P.Sx, &P.Mx, &P.Ax, &P.Vx};
-    const double *const from[4] = {D->d_S, D->d_M, D->d_Ainv, D->d_Minv};
-    for (int k = 0; k < sets; ++k) {
-        int2 *A = D->d_fx + k * fxm;
-        short *d = D->d_fxd + k * nd;
-        const int grid = (int)std::min<long long>(ctx->ne, 65535);
-        switch (n1) {
-#define X(n) case n: k_fx_pack<n><<<grid, 128>>>(ctx->ne, from[k], A, d); break;
-            GDG_VAR_CASES(X)
-#undef X
-        }
-        fxs[k]->A = A;
-        fxs[k]->d = d;
-    }
     st = gdg_cuda_check(ctx, cudaDeviceSynchronize(), "assembly");
     cudaFree(D->d_nodes);
-    cudaFree(D->d_Ainv);
-    cudaFree(D->d_Minv);
-    D->d_nodes = D->d_Ainv = D->d_Minv = nullptr;
+    cudaFree(D->d_work);
+    D->d_nodes = D->d_work = nullptr;
     if (st) return st;
     // the mapping must be orientation preserving: every frozen |J| mean > 0
     std::vector<double> pre((size_t)ctx->ne * 4);
@@ -381,7 +372,7 @@ int gdg_var_setup(gdg_ctx *ctx) {
 void gdg_var_free(gdg_ctx *ctx) {
     VarData *D = ctx->var;
     if (!D) return;
-    cudaFree(D->d_S); cudaFree(D->d_M); cudaFree(D->d_dS); cudaFree(D->d_Ainv); cudaFree(D->d_Minv); cudaFree(D->d_fx); cudaFree(D->d_fxd); cudaFree(D->d_FMq); cudaFree(D->d_Psx); cudaFree(D->d_FM); cudaFree(D->d_time); cudaFree(D->d_src); cudaFree(D->d_w); cudaFree(D->d_pre); cudaFree(D->d_face); cudaFree(D->d_affine);
+    cudaFree(D->d_dS); cudaFree(D->d_work); cudaFree(D->d_fx); cudaFree(D->d_fxd); cudaFree(D->d_FMq); cudaFree(D->d_Psx); cudaFree(D->d_FM); cudaFree(D->d_time); cudaFree(D->d_src); cudaFree(D->d_w); cudaFree(D->d_pre); cudaFree(D->d_face); cudaFree(D->d_affine);
     cudaFree(D->d_tab); cudaFree(D->d_nodes); cudaFree(D->d_state); cudaFree(D->d_tr);
     cudaFree(D->d_c2feat); cudaFree(D->d_wbf16); cudaFree(D->d_mlp);
     cudaFree(D->d_ru); cudaFree(D->d_rv); cudaFree(D->d_x0u);
@@ -489,7 +480,7 @@ int gdg_var_energy(gdg_ctx *ctx, const double *u, const double *v, double *E, cu
     VarData &D = *ctx->var;
     const dim3 grid(ctx->ne), block(nthreads_for(ctx->n1 * ctx->n1));
     switch (ctx->n1) {
-#define X(n) case n: k_var_energy<n><<<grid, block, 0, s>>>(D.vp, u, v, D.d_red); break;
+#define X(n) case n: k_var_energy<n><<<grid, block, StageSmem<n, true>::bytes(), s>>>(D.vp, u, v, D.d_red); break;
         GDG_VAR_CASES(X)
 #undef X
     }

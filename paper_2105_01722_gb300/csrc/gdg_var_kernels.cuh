@@ -25,7 +25,7 @@ struct VarParams {
     double rtol;
     int maxit, precond;   // GDG_PC_*
     const double *tab;    // B[Q][N1], D[Q][N1], wq[Q], dphiL[N1], dphiR[N1], Psi[N1][N1], lam[N1]
-    const double *S, *M, *w, *pre, *face;
+    const double *w, *pre, *face;
     const double *dS;            // [ne][N1*N1] frozen-coefficient preconditioner diagonal (S system)
     // the operators of the stage as integers (gdg_fx.cuh).  Element matrices: packed lower triangles
     // (fx_tri_len entries an element) and the exponents d of their rows [ne][N1*N1]
@@ -83,7 +83,7 @@ extern const VarOps var_ops_2, var_ops_3, var_ops_4, var_ops_5, var_ops_6, var_o
 
 struct VarData {
     int nq = 0, Q = 0, NA = 0;
-    double *d_S = nullptr, *d_M = nullptr, *d_w = nullptr, *d_pre = nullptr, *d_face = nullptr;
+    double *d_w = nullptr, *d_pre = nullptr, *d_face = nullptr;
     double *d_dS = nullptr;
     int2 *d_fx = nullptr;                        // packed integer matrices: S, M (, A^-1, M^-1)
     short *d_fxd = nullptr;                      // their row exponents
@@ -91,7 +91,7 @@ struct VarData {
     short2 *d_FMq = nullptr;
     int2 *d_Psx = nullptr;
     double *d_time = nullptr, *d_src = nullptr;  // point source: time, weights [NA]
-    double *d_Ainv = nullptr, *d_Minv = nullptr; // setup temporaries of the inverses, freed after it
+    double *d_work = nullptr;                    // setup: the element matrices (and inverses) in FP64, a part of the mesh at a time
     double *d_tab = nullptr, *d_nodes = nullptr;
     unsigned char *d_affine = nullptr;           // per element: a parallelogram
     double *d_state = nullptr, *d_tr = nullptr;
@@ -731,13 +731,14 @@ k_fdm_diag(const double *__restrict__ lam, double *pre, double *dS) {
 
 // --------------------------------------------------------- assembly -------
 
+// Sout, Mout: of the elements e0, e0 + 1, ..., a block each
 template <int N1>
 __global__ void __launch_bounds__(GEOM_THREADS)
-k_var_geom(VarParams P, const double *X, const double *Y, const double *C2, double *Sout, double *Mout,
+k_var_geom(VarParams P, int e0, const double *X, const double *Y, const double *C2, double *Sout, double *Mout,
            double *wout, double *pre, double *face) {
     constexpr int NA = N1 * N1;
     extern __shared__ __align__(16) double sm[];
-    const int Q = P.Q, e = blockIdx.x, t = threadIdx.x;
+    const int Q = P.Q, e = e0 + blockIdx.x, t = threadIdx.x;
     double *tb = sm;
     double *nx_ = tb + tab_len(Q, N1);
     double *ny_ = nx_ + NA, *nc = ny_ + NA;
@@ -827,7 +828,7 @@ k_var_geom(VarParams P, const double *X, const double *Y, const double *C2, doub
             }
             __syncthreads();
         }
-        double *out = (pass == 0 ? Mout : Sout) + (size_t)e * NA * NA;
+        double *out = (pass == 0 ? Mout : Sout) + (size_t)blockIdx.x * NA * NA;
 #pragma unroll
         for (int m = 0; m < PER; ++m) {
             const int o = t + m * GEOM_THREADS;
@@ -849,7 +850,7 @@ k_var_geom(VarParams P, const double *X, const double *Y, const double *C2, doub
     sGss = block_sum(sGss, red);
     sW = block_sum(sW, red);
     if (t < NA) {
-        const double *row = Mout + (size_t)e * NA * NA + (size_t)t * NA;
+        const double *row = Mout + (size_t)blockIdx.x * NA * NA + (size_t)t * NA;
         double s = 0.0;
         for (int k = 0; k < NA; ++k) s += row[k];
         wout[(size_t)e * NA + t] = s / sW;   // w = M_J 1 / |e|
@@ -1712,24 +1713,27 @@ __global__ void k_fx_pack(int ne, const double *__restrict__ src, int2 *__restri
         __syncthreads();
     }
 }
-// per-element V^T M V + U^T S U
+
+// per-element V^T M V + U^T S U, the products by the packed matrices (a squared FP64 copy of
+// both would hold as much memory as everything else)
 template <int N1>
 __global__ void __launch_bounds__(nthreads_for(N1 * N1), kVarMinBlocks)
-k_var_energy(VarParams P, const double *u, const double *v, double *part) {
+k_var_energy(const __grid_constant__ VarParams P, const double *u, const double *v, double *part) {
     constexpr int NA = N1 * N1;
-    __shared__ double U[NA], V[NA], red[32];
+    extern __shared__ __align__(16) double smraw[];
+    const StageSmem<N1, true> s(smraw);
     const int e = blockIdx.x, t = threadIdx.x;
-    if (t < NA) { U[t] = u[(size_t)e * NA + t]; V[t] = v[(size_t)e * NA + t]; }
+    const size_t at = (size_t)e * NA + (t < NA ? t : 0);
+    load_fx<N1>(s.A, P.Sx, e);
+    const double U = t < NA ? u[at] : 0.0, V = t < NA ? v[at] : 0.0;
+    fx_arrived();
+    const double SU = fx_matvec<NA>(s.system(P.Sx, e), U, 0);
     __syncthreads();
-    double s = 0.0;
-    if (t < NA) {
-        const double *Mr = P.M + ((size_t)e * NA + t) * NA, *Sr = P.S + ((size_t)e * NA + t) * NA;
-        double mv = 0.0, su = 0.0;
-        for (int k = 0; k < NA; ++k) { mv += Mr[k] * V[k]; su += Sr[k] * U[k]; }
-        s = V[t] * mv + U[t] * su;
-    }
-    s = block_sum(s, red);
-    if (t == 0) part[e] = s;
+    load_fx<N1>(s.A, P.Mx, e);
+    fx_arrived();
+    const double MV = fx_matvec<NA>(s.system(P.Mx, e), V, 0);
+    const double sum = block_sum(t < NA ? V * MV + U * SU : 0.0, s.red);
+    if (t == 0) part[e] = sum;
 }
 
 __global__ void k_var_sum(int n, const double *part, double *out) {
