@@ -896,10 +896,11 @@ __global__ void k_sum_partials(int n, const double *partial, double *out) {
 
 // ------------------------------------------------------------ 1-D --------
 
-// k = f(Y) of gdg_rhs (time steps run in k_run1)
-template <int N1>
+// One stage (or k = f(Y), M_RHS), an element a thread, with the traces of its
+// result: gdg_rhs, and the steps of meshes too large for k_run1's windows.
+template <int N1, int MODE>
 __global__ void __launch_bounds__(TPB1)
-k_stage1(const __grid_constant__ ModalParams mp, const StageBufs b) {
+k_stage1(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= mp.ne) return;
     const int nx = mp.nx;
@@ -921,14 +922,45 @@ k_stage1(const __grid_constant__ ModalParams mp, const StageBufs b) {
     } else { vo = -vi; dO = -di; }
     flux(vi, di, vo, dO, mp.beta, mp.tau, mp.c2, mp.alt, 1, en >= nx, gp, qp);
     const size_t row = (size_t)e * N1;
+    // whole rows at once, before the first store and after the last sum: a thread strides the others by N1, so
+    // the rest of a row's lines has to be used while they are in L1
+    double Ru[N1], Rv[N1], Nu[N1], Nv[N1];
 #pragma unroll
     for (int k = 0; k < N1; ++k) {
-        const double Yu = b.yU[row + k], Yv = b.yV[row + k];
+        Ru[k] = b.yU[row + k];
+        Rv[k] = b.yV[row + k];
+        if (MODE == M_S23) {   // (the output may be y_n itself)
+            Nu[k] = b.nU[row + k];
+            Nv[k] = b.nV[row + k];
+        }
+    }
+    double vL = 0, vR = 0, dL = 0, dR = 0;
+#pragma unroll
+    for (int k = 0; k < N1; ++k) {
+        const double Yu = Ru[k], Yv = Rv[k];
         const double ru = mp.d[0].gL[k] * gm + mp.d[0].gR[k] * gp;
         const double rv = mp.d[0].eL[k] * qm + mp.d[0].eR[k] * qp;
-        b.oU[row + k] = Yv + b.lam2[N1 + k] * ru;
-        b.oV[row + k] = b.lam2[k] * Yu + rv;
+        if (MODE == M_RHS) {
+            Ru[k] = Yv + b.lam2[N1 + k] * ru;
+            Rv[k] = b.lam2[k] * Yu + rv;
+            continue;
+        }
+        // lam2 carries sc
+        Ru[k] = fma(sc, Yv, fma(b.lam2[N1 + k], ru, MODE == M_S1 ? Yu : Nu[k]));
+        Rv[k] = fma(b.lam2[k], Yu, fma(sc, rv, MODE == M_S1 ? Yv : Nv[k]));
+        vL = fma(mp.d[0].eL[k], Rv[k], vL);
+        vR = fma(mp.d[0].eR[k], Rv[k], vR);
+        dL = fma(mp.d[0].gL[k], Ru[k], dL);
+        dR = fma(mp.d[0].gR[k], Ru[k], dR);
     }
+#pragma unroll
+    for (int k = 0; k < N1; ++k) {
+        b.oU[row + k] = Ru[k];
+        b.oV[row + k] = Rv[k];
+    }
+    if (MODE == M_RHS) return;
+    b.trout[tix1(e, 0, 0)] = vL; b.trout[tix1(e, 0, 1)] = dL;
+    b.trout[tix1(e, 1, 0)] = vR; b.trout[tix1(e, 1, 1)] = dR;
 }
 
 // Time steps of a 1-D mesh: a block holds a window of W elements in shared
@@ -1197,8 +1229,9 @@ void launch_stage2(int mode, const ModalParams &mp, const StageBufs &b, double s
 }
 
 template <int N1>
-void launch_stage1(const ModalParams &mp, const StageBufs &b, cudaStream_t s) {
-    k_stage1<N1><<<(mp.ne + TPB1 - 1) / TPB1, TPB1, 0, s>>>(mp, b);
+void launch_stage1(int mode, const ModalParams &mp, const StageBufs &b, double sc, cudaStream_t s) {
+    (mode == M_RHS ? k_stage1<N1, M_RHS> : mode == M_S1 ? k_stage1<N1, M_S1> : k_stage1<N1, M_S23>)
+        <<<(mp.ne + TPB1 - 1) / TPB1, TPB1, 0, s>>>(mp, b, sc);
 }
 
 void launch_stage_raw(const gdg_ctx *ctx, int mode, const StageBufs &b, double sc, cudaStream_t s) {
@@ -1215,7 +1248,7 @@ void launch_stage_raw(const gdg_ctx *ctx, int mode, const StageBufs &b, double s
         }
     } else {
         switch (n1) {
-#define X(n) case n: launch_stage1<n>(ctx->mp, b, s); break;
+#define X(n) case n: launch_stage1<n>(mode, ctx->mp, b, sc, s); break;
             GDG_N1_CASES(X)
 #undef X
         }
@@ -1667,6 +1700,21 @@ void enqueue_rk4_stage(gdg_ctx *ctx, int st, double dt, cudaStream_t s) {
 
 void enqueue_rk4_step(gdg_ctx *ctx, double dt, cudaStream_t s) {
     for (int st = 0; st < RK_STAGES; ++st) enqueue_rk4_stage(ctx, st, dt, s);
+}
+
+// Windows (k_run1) or stages (k_stage1) for a 1-D mesh.  A window takes a whole SM and
+// advances it in about the same time whatever N1 (350 us for 16 steps), so the windows cost
+// a unit a wave of the SMs; the stages, blocks of 128 elements, cost (N1/8)(0.4 + 0.7 w) of
+// it in w waves (fitted at N1 = 9, 12, 16; less, where it does not matter, below).  16 steps,
+// windows and stages in us: N1 = 9, 14000 elements 380 and 480, 30000 1125 and 757, 10^6
+// 25.1 and 16.7 ms; N1 = 16, 14000 736 and 792, 20000 1089 and 1300, 45000 2505 and 1884; N1 =
+// 3, 45000 482 and 525, 70000 1001 and 670.
+bool run1_takes(const gdg_ctx *ctx) {
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+    const long long ne = ctx->ne, own = RUN1_MAXT / ctx->n1 - 2 * RK_STAGES * RUN1_STEPS;
+    const long long windows = (ne + sms * own - 1) / (sms * own), stages = (ne + sms * TPB1 - 1) / (sms * TPB1);
+    return windows <= 1 || 80 * windows <= ctx->n1 * (4 + 7 * stages);
 }
 
 // nsteps of a 1-D mesh on the nodal (u, v) in place (k_run1)
@@ -2160,7 +2208,7 @@ int gdg_const_step(gdg_ctx *ctx, double *u, double *v, double dt, int nsteps, cu
     int st;
     if (ctx->pb.route == GDG_ROUTE_NODAL) return step_nodal(ctx, u, v, dt, nsteps, s);
     stage_tables(ctx, dt, s);
-    if (ctx->dim == 1) return step_1d(ctx, u, v, dt, nsteps, s);
+    if (ctx->dim == 1 && run1_takes(ctx)) return step_1d(ctx, u, v, dt, nsteps, s);
     launch_enter(ctx, u, v, buf(ctx, B_NU), buf(ctx, B_NV), ctx->d_tr, s);
     if ((st = gdg_cuda_check(ctx, cudaGetLastError(), "gdg_step prologue"))) return st;
     if (has_halo(ctx)) {   // partitioned mesh: stages launched one by one, exchanges between them
