@@ -897,7 +897,13 @@ __global__ void k_sum_partials(int n, const double *partial, double *out) {
 // ------------------------------------------------------------ 1-D --------
 
 // One stage (or k = f(Y), M_RHS), an element a thread, with the traces of its
-// result: gdg_rhs, and the steps of meshes too large for k_run1's windows.
+// result: gdg_rhs, and the steps of meshes too large for k_run1's windows.  A thread
+// strides the others by N1, so the lines of a row have to stay in L1 until it is through:
+// for long rows they are read and written whole, at the price of registers.  16 steps of
+// 10^6 elements, entry by entry and whole rows over the time of the stages before (with an accumulator):
+// N1 = 9 0.87 and 0.88, N1 = 14 1.13 and 0.80, N1 = 16 1.25 and 0.73; of 30000 elements
+// N1 = 9 0.80 and 0.88, N1 = 13 0.81 and 0.90, N1 = 16 0.74 and 0.78.
+constexpr int STAGE1_ROWS = 13;
 template <int N1, int MODE>
 __global__ void __launch_bounds__(TPB1)
 k_stage1(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) {
@@ -922,41 +928,49 @@ k_stage1(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) {
     } else { vo = -vi; dO = -di; }
     flux(vi, di, vo, dO, mp.beta, mp.tau, mp.c2, mp.alt, 1, en >= nx, gp, qp);
     const size_t row = (size_t)e * N1;
-    // whole rows at once, before the first store and after the last sum: a thread strides the others by N1, so
-    // the rest of a row's lines has to be used while they are in L1
+    constexpr bool ROWS = N1 > STAGE1_ROWS;
     double Ru[N1], Rv[N1], Nu[N1], Nv[N1];
-#pragma unroll
-    for (int k = 0; k < N1; ++k) {
+    auto load = [&](int k) {
         Ru[k] = b.yU[row + k];
         Rv[k] = b.yV[row + k];
         if (MODE == M_S23) {   // (the output may be y_n itself)
             Nu[k] = b.nU[row + k];
             Nv[k] = b.nV[row + k];
         }
+    };
+    auto store = [&](int k) {
+        b.oU[row + k] = Ru[k];
+        b.oV[row + k] = Rv[k];
+    };
+    if (ROWS) {
+#pragma unroll
+        for (int k = 0; k < N1; ++k) load(k);
     }
     double vL = 0, vR = 0, dL = 0, dR = 0;
 #pragma unroll
     for (int k = 0; k < N1; ++k) {
+        if (!ROWS) load(k);
         const double Yu = Ru[k], Yv = Rv[k];
         const double ru = mp.d[0].gL[k] * gm + mp.d[0].gR[k] * gp;
         const double rv = mp.d[0].eL[k] * qm + mp.d[0].eR[k] * qp;
         if (MODE == M_RHS) {
             Ru[k] = Yv + b.lam2[N1 + k] * ru;
             Rv[k] = b.lam2[k] * Yu + rv;
+            if (!ROWS) store(k);
             continue;
         }
         // lam2 carries sc
         Ru[k] = fma(sc, Yv, fma(b.lam2[N1 + k], ru, MODE == M_S1 ? Yu : Nu[k]));
         Rv[k] = fma(b.lam2[k], Yu, fma(sc, rv, MODE == M_S1 ? Yv : Nv[k]));
+        if (!ROWS) store(k);
         vL = fma(mp.d[0].eL[k], Rv[k], vL);
         vR = fma(mp.d[0].eR[k], Rv[k], vR);
         dL = fma(mp.d[0].gL[k], Ru[k], dL);
         dR = fma(mp.d[0].gR[k], Ru[k], dR);
     }
+    if (ROWS) {
 #pragma unroll
-    for (int k = 0; k < N1; ++k) {
-        b.oU[row + k] = Ru[k];
-        b.oV[row + k] = Rv[k];
+        for (int k = 0; k < N1; ++k) store(k);
     }
     if (MODE == M_RHS) return;
     b.trout[tix1(e, 0, 0)] = vL; b.trout[tix1(e, 0, 1)] = dL;
@@ -1707,7 +1721,7 @@ void enqueue_rk4_step(gdg_ctx *ctx, double dt, cudaStream_t s) {
 // a unit a wave of the SMs; the stages, blocks of 128 elements, cost (N1/8)(0.4 + 0.7 w) of
 // it in w waves (fitted at N1 = 9, 12, 16; less, where it does not matter, below).  16 steps,
 // windows and stages in us: N1 = 9, 14000 elements 380 and 480, 30000 1125 and 757, 10^6
-// 25.1 and 16.7 ms; N1 = 16, 14000 736 and 792, 20000 1089 and 1300, 45000 2505 and 1884; N1 =
+// 25.1 and 16.6 ms; N1 = 16, 14000 736 and 792, 20000 1089 and 1300, 45000 2505 and 1884; N1 =
 // 3, 45000 482 and 525, 70000 1001 and 670.
 bool run1_takes(const gdg_ctx *ctx) {
     int sms = 152;
