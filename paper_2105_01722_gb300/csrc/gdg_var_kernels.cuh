@@ -1558,7 +1558,7 @@ k_var_stage(const __grid_constant__ VarParams P, const __grid_constant__ VarBufs
 }
 
 // standalone element PCG (gdg_pcg): which = 0 M, 1 S (+ w w^T)
-template <int N1>
+template <int N1, int ROUTE>
 __global__ void __launch_bounds__(nthreads_for(N1 * N1), var_stage_min_blocks(N1, ROUTE_ANY))
 k_var_pcg(VarParams P, int which, const double *bvec, double *xvec, int *iters, double *rel, int *sweeps) {
     constexpr int NA = N1 * N1;
@@ -1578,7 +1578,7 @@ k_var_pcg(VarParams P, int which, const double *bvec, double *xvec, int *iters, 
     }
     load_psi<N1>(P, s);
     fx_arrived();
-    solve<N1, ROUTE_ANY>(P, s, T, e, which != 0, w, b, x, false, false, &it, &sw, &fell, &rr, true);
+    solve<N1, ROUTE>(P, s, T, e, which != 0, w, b, x, false, false, &it, &sw, &fell, &rr, true);
     if (on) xvec[at] = x;
     if (t == 0) {
         iters[e] = it;

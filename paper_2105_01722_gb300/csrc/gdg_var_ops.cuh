@@ -15,7 +15,8 @@ struct VarLaunch {
         cudaFuncSetAttribute(k_var_stage<N1, ROUTE_ANY>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_var_stage<N1, ROUTE_MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_var_stage<N1, ROUTE_INVERSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_var_pcg<N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_var_pcg<N1, ROUTE_ANY>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_var_pcg<N1, ROUTE_MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     }
     static void stage(const VarParams &P, size_t sm, int mode, const VarBufs &b, double cA, double cY, cudaStream_t s) {
         const dim3 grid(P.ne), block(nthreads_for(N1 * N1));   // one block per element
@@ -24,7 +25,7 @@ struct VarLaunch {
     }
     static void pcg(const VarParams &P, size_t sm, int which, const double *b, double *x, int *iters, double *rel,
                     int *sweeps, cudaStream_t s) {
-        k_var_pcg<N1><<<P.ne, nthreads_for(N1 * N1), sm, s>>>(P, which, b, x, iters, rel, sweeps);
+        (P.mixed ? k_var_pcg<N1, ROUTE_MIXED> : k_var_pcg<N1, ROUTE_ANY>)<<<P.ne, nthreads_for(N1 * N1), sm, s>>>(P, which, b, x, iters, rel, sweeps);
     }
 };
 
