@@ -259,7 +259,9 @@ int gdg_var_setup(gdg_ctx *ctx) {
     P.stats = D->d_stats;
     P.mixed = ctx->pb.precision == GDG_MIXED;
     P.inverse = ctx->pb.solver == GDG_SOLVE_INVERSE;
-    P.staged = P.inverse && !ctx->batched;
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+    P.staged = P.inverse && !ctx->batched && staged_lifts(n1, ctx->ne, sms);
     P.refine_max = ctx->pb.refine_max > 0 ? ctx->pb.refine_max : 8;
     P.refine_rtol = (float)(ctx->pb.refine_rtol > 0.0 ? ctx->pb.refine_rtol : 1e-5);
     D->smem_geom = geom_smem(n1, Q);

@@ -1544,6 +1544,20 @@ __device__ __forceinline__ void var_stage_body(const VarParams &P, const VarBufs
     face_lines<N1>(s.U, s.V, T, b.trout + lix<N1>(e, 0), t, blockDim.x);
 }
 
+// Where a problem's own steps with inverses stage their face operators: where the passes over the
+// 3 N1 rows of a face (ten rows a warp) fill the block better than the direct form's over the 12 N1
+// rows of all four (a row a pair of threads), N1 = 3, 6 and 9; and in blocks of one warp on
+// meshes beyond the 16 blocks an SM that the registers of the any-route kernel leave.
+// Eight steps, staged and direct, in ms.  100 x 100 elements: N1 = 9 9.2 and 10.6, 8 8.5 and 6.9, 7 7.0 and
+// 6.3, 6 5.56 and 5.45, 10 14.4 and 14.1, 5 2.8 and 3.5, 4 2.6 and 3.0; 40 x 41: 5 0.60 and 0.55, 4
+// 0.56 and 0.47, 3 0.42 and 0.44, 2 0.33 and 0.32.
+__host__ __device__ constexpr bool staged_lifts(int n1, int ne, int sms) {
+    const int bd = nthreads_for(n1 * n1), warps = bd / 32;
+    const int staged = (3 * n1 + 10 * warps - 1) / (10 * warps) * 10 * warps;   // places for 3 N1 rows
+    const int direct = (12 * n1 + bd / 2 - 1) / (bd / 2) * (bd / 2);            // ... for 12 N1
+    return 4 * staged < direct || (warps == 1 && ne > 16 * sms);
+}
+
 // Resident blocks promised to ptxas for the stage kernel: the 7 (inverse route 8)
 // that the shared memory of a block of at most 3 warps allows, 4 for larger elements.
 __host__ __device__ constexpr int var_stage_min_blocks(int n1, int route) {

@@ -33,3 +33,29 @@ def test_batched_steps_are_the_problems_own_to_the_last_bit(N, p, form):
         assert torch.equal(u, us[i]) and torch.equal(v, vs[i])
         ctx.close()
     batch.close()
+
+
+@pytest.mark.parametrize("N,p", [(3, 3), (4, 3), (8, 5)])
+def test_large_and_small_meshes_give_the_same_bits(N, p):
+    """Inverse route on 3000 elements and on 3 x 3 of them: N + 1 = 4 and 5 stage their face operators on
+    the large mesh only."""
+    import torch
+    X, Y = inputs.mapped_nodes((60, 50), N, 0.05)
+    C2, na = inputs.c2_sine(X, Y), (N + 1) ** 2
+    U, V = (inputs.random_state((50, 60, na), k) for k in (1, 2))
+
+    def rhs(rows, cols):
+        x, y, c2 = (np.ascontiguousarray(f[rows, cols]) for f in (X, Y, C2))
+        ctx = gdg.Context(gdg.make_problem(2, (x.shape[1], x.shape[0]), N, p, coef=gdg.COEF_NODAL, x_nodes=x, y_nodes=y,
+                                           c2_nodes=c2, solver=gdg.SOLVE_INVERSE))
+        u, v = (torch.tensor(np.ascontiguousarray(f[rows, cols]).ravel(), device="cuda") for f in (U, V))
+        out = torch.empty_like(u), torch.empty_like(u)
+        ctx.rhs(u, v, *out)
+        ctx.close()
+        return [f.view(x.shape[0], x.shape[1], na) for f in out]
+
+    whole = rhs(slice(0, 50), slice(0, 60))
+    for ey, ex in ((1, 1), (25, 31), (48, 58)):
+        part = rhs(slice(ey - 1, ey + 2), slice(ex - 1, ex + 2))
+        for a, b in zip(whole, part):
+            assert torch.equal(a[ey, ex], b[1, 1])
