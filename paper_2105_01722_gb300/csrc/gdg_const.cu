@@ -995,12 +995,12 @@ constexpr int RUN1_STEPS = 2;    // steps a launch: window overlap (8 elements a
 constexpr int RUN1_MAXT = 1024;
 
 __host__ __device__ constexpr size_t run1_doubles(int n1, int W) {
-    return (size_t)W * (2 * n1 + 8) + 2 * n1 * n1 + 4 * n1 + RK_STAGES * 3 * n1;
+    return (size_t)W * (2 * n1 + 8) + 2 * n1 * n1 + 2 * n1 + RK_STAGES * 3 * n1;
 }
 
-// PAR: modes even or odd, even ones first (as in the 2-D kernels): a face pair
+// The modes are even or odd, even ones first (as in the 2-D kernels): a face pair
 // lifts onto an entry with one product and a trace pair is one sum in two parts.
-template <int N1, bool PAR>
+template <int N1>
 __global__ void __launch_bounds__(RUN1_MAXT)
 k_run1(const __grid_constant__ ModalParams mp, const double *P, const double *Psi, const double *lams, const double *u,
        const double *v, double *ou, double *ov, double dt, int steps, int own, int halo, int first, int last) {
@@ -1012,13 +1012,11 @@ k_run1(const __grid_constant__ ModalParams mp, const double *P, const double *Ps
     const int lo = mp.per_x ? b0 - halo : max(0, b0 - halo);
     const int W = (mp.per_x ? b0 + nown + halo : min(nx, b0 + nown + halo)) - lo;
     double *wU = smem, *wV = wU + W * N1, *tr = wV + W * N1, *fl = tr + 4 * W;   // tr: vL, vR, dL, dR
-    double *sP = fl + 4 * W, *sPsi = sP + N1 * N1, *vec = sPsi + N1 * N1, *lam = vec + 4 * N1;
+    double *sP = fl + 4 * W, *sPsi = sP + N1 * N1, *vec = sPsi + N1 * N1, *lam = vec + 2 * N1;
     for (int i = t; i < N1 * N1; i += nt) { sP[i] = P[i]; sPsi[i] = Psi[i]; }
-    for (int i = t; i < N1; i += nt) {   // trace vectors: vL, vR, dL, dR
+    for (int i = t; i < N1; i += nt) {   // trace vectors: v, d
         vec[i] = mp.d[0].eL[i];
-        vec[N1 + i] = mp.d[0].eR[i];
-        vec[2 * N1 + i] = mp.d[0].gL[i];
-        vec[3 * N1 + i] = mp.d[0].gR[i];
+        vec[N1 + i] = mp.d[0].gL[i];
     }
     for (int i = t; i < RK_STAGES * 3 * N1; i += nt) lam[i] = lams[i];
     const int e = t / N1, k = t - e * N1;
@@ -1043,39 +1041,28 @@ k_run1(const __grid_constant__ ModalParams mp, const double *P, const double *Ps
         if (on) { wU[t] = Yu; wV[t] = Yv; }
         __syncthreads();
     }
-    const double gLk = vec[2 * N1 + k], gRk = vec[3 * N1 + k], eLk = vec[k], eRk = vec[N1 + k], ceL = mp.d[0].ceL[k];
+    const double ceL = mp.d[0].ceL[k];
     for (int step = 0; step < steps; ++step) {
         const double Nu = Yu, Nv = Yv;
         for (int st = 0; st < RK_STAGES; ++st) {
             const double sc = dt / (RK_STAGES - st);
-            // traces of the stage input, four sums an element (PAR: even and odd
-            // parts, swapped between neighbouring lanes)
+            // traces of the stage input, four sums an element (even and odd parts,
+            // swapped between neighbouring lanes)
             for (int i0 = warp0; i0 < 4 * W; i0 += nt) {   // (warps without a sum skip it)
                 const int i = i0 + lane, ee = min(i, 4 * W - 1) >> 2, f = (i >> 1) & 1, par = i & 1;   // f: 0 v, 1 u
-                const double *w = (f ? wU : wV) + ee * N1, *c = vec + (2 * f + (PAR ? 0 : par)) * N1;
+                const double *w = (f ? wU : wV) + ee * N1, *c = vec + f * N1;
+                const int m0 = par ? NE : 0, m1 = par ? N1 : NE;
                 double s = 0.0;
-                if (PAR) {
-                    const int m0 = par ? NE : 0, m1 = par ? N1 : NE;
 #pragma unroll
-                    for (int m = 0; m < NE; ++m)
-                        if (m0 + m < m1) s = fma(c[m0 + m], w[m0 + m], s);
-                    const double o = __shfl_xor_sync(0xffffffffu, s, 1);
-                    s = o + (par ? -s : s);
-                } else {
-                    double s1 = 0.0;
-#pragma unroll
-                    for (int m = 0; m + 1 < N1; m += 2) {
-                        s = fma(c[m], w[m], s);
-                        s1 = fma(c[m + 1], w[m + 1], s1);
-                    }
-                    if (N1 & 1) s = fma(c[N1 - 1], w[N1 - 1], s);
-                    s += s1;
-                }
+                for (int m = 0; m < NE; ++m)
+                    if (m0 + m < m1) s = fma(c[m0 + m], w[m0 + m], s);
+                const double o = __shfl_xor_sync(0xffffffffu, s, 1);
+                s = o + (par ? -s : s);
                 if (i < 4 * W) tr[i] = s;
             }
             __syncthreads();
-            // fluxes of the minus (0) and plus (1) face (PAR: doubled, their sums
-            // and differences, those of v times sc)
+            // fluxes of the minus (0) and plus (1) face, doubled: their sums and
+            // differences, those of v times sc
             for (int i0 = warp0; i0 < 2 * W; i0 += nt) {
                 const int i = i0 + lane, ee = min(i, 2 * W - 1) >> 1, side = i & 1;
                 const double vi = tr[4 * ee + side], di = tr[4 * ee + 2 + side];
@@ -1087,14 +1074,10 @@ k_run1(const __grid_constant__ ModalParams mp, const double *P, const double *Ps
                 }
                 const double vo = wall ? -vi : tr[4 * nb + 1 - side], dO = wall ? -di : tr[4 * nb + 3 - side];
                 double g, q;
-                if (PAR) {
-                    flux2(vi, di, vo, dO, mp.beta2, mp.tau2, mp.alt, side, wall, g, q);
-                    const double go = __shfl_xor_sync(0xffffffffu, g, 1), qo = __shfl_xor_sync(0xffffffffu, q, 1);
-                    g = go + (side ? -g : g);
-                    q = sc * (qo + (side ? -q : q));
-                } else {
-                    flux(vi, di, vo, dO, mp.beta, mp.tau, mp.c2, mp.alt, side, wall, g, q);
-                }
+                flux2(vi, di, vo, dO, mp.beta2, mp.tau2, mp.alt, side, wall, g, q);
+                const double go = __shfl_xor_sync(0xffffffffu, g, 1), qo = __shfl_xor_sync(0xffffffffu, q, 1);
+                g = go + (side ? -g : g);
+                q = sc * (qo + (side ? -q : q));
                 if (i < 2 * W) {
                     fl[4 * ee + side] = g;
                     fl[4 * ee + 2 + side] = q;
@@ -1103,16 +1086,9 @@ k_run1(const __grid_constant__ ModalParams mp, const double *P, const double *Ps
             __syncthreads();
             if (on) {
                 const double *f = fl + 4 * e, *L = lam + st * 3 * N1;
-                double nu;
-                if (PAR) {
-                    const int px = k < NE ? 0 : 1;
-                    nu = fma(sc, Yv, fma(L[2 * N1 + k], f[px], Nu));
-                    Yv = fma(L[k], Yu, fma(ceL, f[2 + px], Nv));
-                } else {
-                    const double ru = fma(gLk, f[0], gRk * f[1]), rv = fma(eLk, f[2], eRk * f[3]);
-                    nu = fma(sc, Yv, fma(L[N1 + k], ru, Nu));
-                    Yv = fma(L[k], Yu, fma(sc, rv, Nv));
-                }
+                const int px = k < NE ? 0 : 1;
+                const double nu = fma(sc, Yv, fma(L[2 * N1 + k], f[px], Nu));
+                Yv = fma(L[k], Yu, fma(ceL, f[2 + px], Nv));
                 Yu = nu;
                 wU[t] = Yu;
                 wV[t] = Yv;
@@ -1635,8 +1611,7 @@ int set_smem_limits() {
     GDG_N1_CASES(X)
 #undef X
 #define X(n)                                                                                    \
-    cudaFuncSetAttribute(k_run1<n, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);   \
-    cudaFuncSetAttribute(k_run1<n, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_run1<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     GDG_N1_CASES(X)
 #undef X
 #define X(n)                                                                                   \
@@ -1728,7 +1703,7 @@ bool run1_takes(const gdg_ctx *ctx) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
     const long long ne = ctx->ne, own = RUN1_MAXT / ctx->n1 - 2 * RK_STAGES * RUN1_STEPS;
     const long long windows = (ne + sms * own - 1) / (sms * own), stages = (ne + sms * TPB1 - 1) / (sms * TPB1);
-    return windows <= 1 || 80 * windows <= ctx->n1 * (4 + 7 * stages);
+    return ctx->mp.parity && (windows <= 1 || 80 * windows <= ctx->n1 * (4 + 7 * stages));
 }
 
 // nsteps of a 1-D mesh on the nodal (u, v) in place (k_run1)
@@ -1752,7 +1727,7 @@ void run1_n(gdg_ctx *ctx, double *u, double *v, double dt, int nsteps, cudaStrea
         const int out = iu == buf(ctx, B_XU) ? B_YU : B_XU;
         const bool nodal = last && (whole || !first);
         double *ou = nodal ? u : buf(ctx, out), *ov = nodal ? v : buf(ctx, out + 1);
-        GDG_PROF(ctx, GDG_K_STAGE, s, ((mp.parity ? k_run1<N1, true> : k_run1<N1, false>)<<<grid, threads, sm, s>>>(mp, P, Psi, ctx->d_lams, iu, iv, ou, ov, dt, k,
+        GDG_PROF(ctx, GDG_K_STAGE, s, (k_run1<N1><<<grid, threads, sm, s>>>(mp, P, Psi, ctx->d_lams, iu, iv, ou, ov, dt, k,
                                                                             own, halo, first, nodal)));
         iu = ou;
         iv = ov;
