@@ -1359,7 +1359,9 @@ void launch_fx2(const gdg_ctx *ctx, int kind, const double *in0, const double *i
         A.pe[d] = ctx->fx.pe[d][kind - 1];
     }
     // blocks of up to 128 threads, smaller where that leaves SMs without one
-    const int nf = in1 ? 2 : 1, sms = 152, epb = std::max(1, std::min(FX2_THREADS / (2 * N1), ctx->ne / (2 * sms)));
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+    const int nf = in1 ? 2 : 1, epb = std::max(1, std::min(FX2_THREADS / (2 * N1), ctx->ne / (2 * sms)));
     (kind == FX_TO_MODES ? k_fx2<N1, FX_TO_MODES> : k_fx2<N1, FX_TO_NODES>)<<<(ctx->ne + epb - 1) / epb, nf * epb * N1,
         (size_t)nf * epb * fx2_tile<N1>() * sizeof(double), s>>>(ctx->mp, A, in0, in1, out0, out1, tr, epb);
 }
