@@ -42,17 +42,30 @@ def dof(w=WORKLOAD):
 
 
 def executed_flops_per_stage_launch(w=WORKLOAD):
-    """FP64 flops the parity stage kernels execute per stage launch (FMA = 2,
-    averaged over the four RK stages).  With the modes ordered even first,
+    """FP64 flops a stage of the parity kernels takes with an RK accumulator
+    (FMA = 2, averaged over the four stages), the form this measure was set up
+    for; step2r_flops_per_stage counts what runs now.  With the modes ordered even first,
     gR = +-gL and eR = +-eL, so per element 2-D: fluxes 2 directions x n1
     lines x (2 faces x 7 + 4 sums/differences); per modal entry 23.5: k_u with
     the lifts folded into the solve 4, r_v 5, the RK update 6.5 (stage 1: 4,
     stages 2-3: 8, stage 4: 6), the traces' split dots 8; + 8 n1 trace
-    sums/differences.  (ncu on the persistent step: 2,339 per element and
-    stage from its DFMA / DADD / DMUL counts, this count 2,300.)"""
+    sums/differences."""
     n1 = w["N"] + 1
     nel = w["n"][0] * w["n"][1]
     return nel * (44 * n1 + 23.5 * n1 * n1)
+
+
+def step2r_flops_per_stage(w=WORKLOAD):
+    """FP64 flops a stage of the parity kernels executes (FMA = 2), RK4 in
+    nested form: fluxes 2 directions x n1 lines x (2 faces x 7 + 4 sums and
+    differences), 2 scalings a line, per modal entry 6 FMAs for both fields
+    and 4 for the traces, 8 n1 trace sums and differences, one scaled lift a
+    line.  (ncu on the persistent step: 2,179 per element and stage from its
+    DFMA / DADD / DMUL counts, this count 2,043; the rest is the quotient of
+    the stage's factor, in every thread.)"""
+    n1 = w["N"] + 1
+    nel = w["n"][0] * w["n"][1]
+    return nel * (47 * n1 + 20 * n1 * n1)
 
 
 # FP64 peak derived from unit counts and clock: 152 SMs x 2070 MHz x 4 FP64
@@ -114,9 +127,8 @@ def var_counts(n1, it_u, it_v, form, sweeps_u=0.0, sweeps_v=0.0):
     their FP32 copies plus the FP64 matrices once per sweep; inverse: the
     folded operators 189 NA * 8) plus the face operators (72 n1^2 * 8) and
     the state.
-    These are the counts of the forms in floating point, kept as the measure;
-    the kernels form most products on integers, read each matrix as a packed
-    triangle of 8-byte integers, and apply the inverses unfolded."""
+    The counts of the forms in floating point, a measure of the work a form
+    stands for: no rate of a unit of the GPU (element_work counts what runs)."""
     NA = n1 * n1
     face = 144 * n1 * n1 + 16 * NA
     it_cost = 2 * NA * NA + 8 * n1 ** 3 + 12 * NA
@@ -133,6 +145,55 @@ def var_counts(n1, it_u, it_v, form, sweeps_u=0.0, sweeps_v=0.0):
         cols = 12 * n1 + NA
         return 2 * cols * NA + face, 0.0, cols * NA * 8 + 72 * n1 * n1 * 8 + state
     raise ValueError(form)
+
+
+# 32 x 32 + 64-bit integer multiply-adds (IMAD.WIDE): one warp instruction per
+# 1.06 clocks of an SM, measured with instruction chains.
+IMAD_PEAK_T = 152 * 32 * 2.070e9 / 1.06 / 1e12
+
+
+def element_work(n1, it_u, it_v, form, sweeps_u=0.0, sweeps_v=0.0):
+    """What the element stage kernels do per element and RK stage, NA = n1^2
+    nodes: (integer multiply-adds, bytes).  A product of 58-bit integers is 4
+    multiply-adds an entry, one with the upper limbs alone (the inner products
+    of the mixed form) 1.
+      stiffness product 4 NA^2; face operators 4 faces x 3 n1 x 6 n1 entries;
+      PCG: per iteration a product and the preconditioner (four contractions
+        of n1 terms, 16 n1^3), which each solve also applies once first;
+      mixed: 1 NA^2 an inner iteration, a product per refinement sweep (its
+        preconditioner, vectors and scalars are FP32 and not counted);
+      inverse: two products;
+    bytes: the packed triangles of 8-byte integers (S and M, or S and both
+    inverses), the face operators (72 n1^2 * 8) and the state."""
+    NA = n1 * n1
+    tri = NA * (NA + 1) // 2 * 8
+    imad = 4 * NA * NA + 288 * n1 * n1
+    if form == "fp64":
+        imad += (it_u + it_v) * (4 * NA * NA + 16 * n1 ** 3) + 2 * 16 * n1 ** 3
+    elif form == "mixed":
+        imad += (it_u + it_v) * NA * NA + (sweeps_u + sweeps_v) * 4 * NA * NA
+    elif form == "inverse":
+        imad += 8 * NA * NA
+    else:
+        raise ValueError(form)
+    return imad, (3 if form == "inverse" else 2) * tri + 72 * n1 * n1 * 8 + 8 * NA * 8
+
+
+def element_roofline(imad, byt, seconds, f64, f32):
+    """Roofline block of the element forms: integer multiply-adds and bytes
+    (element_work) over the measured time; bound = the larger fraction (the
+    FP64 scalars and conversions are in neither).  `equivalent`: the work of
+    the form in floating point (var_counts) over the same time, no rate of a
+    unit."""
+    hbm, hbm_src = hbm_peak_gbs()
+    rate, gbs = imad / seconds / 1e12, byt / seconds / 1e9
+    alu = rate / IMAD_PEAK_T >= gbs / hbm
+    return {"bound": "alu" if alu else "hbm", "achieved": rate if alu else gbs,
+            "peak": IMAD_PEAK_T if alu else hbm, "unit": "T IMAD/s" if alu else "GB/s",
+            "frac": rate / IMAD_PEAK_T if alu else gbs / hbm, "resource": "imad" if alu else "hbm",
+            "imad_t": rate, "frac_imad": rate / IMAD_PEAK_T, "hbm_gbs": gbs, "frac_hbm": gbs / hbm,
+            "hbm_peak_source": hbm_src,
+            "equivalent": {"fp64_tflops": f64 / seconds / 1e12, "fp32_tflops": f32 / seconds / 1e12}}
 
 
 def alu_roofline(f64, f32, byt, seconds, probe):
@@ -156,17 +217,17 @@ def alu_roofline(f64, f32, byt, seconds, probe):
     return out
 
 # FP64 thread instructions (DFMA + DADD + DMUL) per element and RK stage of the
-# persistent step, from the ncu capture of the current kernel (16.04 M + 4.81 M
-# + 1.44 M per one-step launch of the 64x64 mesh): the FP64 pipe's share of a
+# persistent step, from the ncu capture of the current kernel (15.48 M + 4.15 M
+# + 0.59 M per one-step launch of the 64x64 mesh): the FP64 pipe's share of a
 # stage's time follows from it at 2 FP64 lanes per SM and clock.
-STEP2R_FP64_INST_PER_ELEMENT_STAGE = 22.28e6 / (4 * 4096)
+STEP2R_FP64_INST_PER_ELEMENT_STAGE = 20.22e6 / (4 * 4096)
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per RK stage of
 # this workload, from one ncu capture per stage kernel (None for a kernel
 # without a capture of its current code):
 #   k_stage2p: the mean over the four stage launches of one RK4 step
 #   k_step2r: one persistent launch of one RK4 step, over its 4 stages
-STAGE_TRAFFIC_BYTES = {0: None, 3: (7.772160e6 + 256) / 4}
+STAGE_TRAFFIC_BYTES = {0: None, 3: 7.724800e6 / 4}
 
 
 PROBE = {}   # in-process measured peaks (filled by run_gdg)
@@ -366,15 +427,17 @@ def forms_variable(steps=16):
             ms = _timed_ms(lambda: ctx.step(u, v, 0.0, dt, steps))
             su, sv = ctx.step_stats()
             states[name] = torch.cat([u, v]).cpu().numpy()
-            f64, f32, byt = var_counts(9, su["mean_iters"], sv["mean_iters"], name,
-                                       su["mean_sweeps"], sv["mean_sweeps"])
+            counts = (9, su["mean_iters"], sv["mean_iters"], name, su["mean_sweeps"], sv["mean_sweeps"])
+            f64, f32, _ = var_counts(*counts)
+            imad, byt = element_work(*counts)
             stages = 128 * 128 * 4 * steps
             out["p%d_%s" % (p, name)] = {
                 "dof_steps_per_s": 128 * 128 * 81 * steps / (ms / 1e3), "ms_per_step": ms / steps,
                 "pcg_u_mean_iters": su["mean_iters"], "pcg_v_mean_iters": sv["mean_iters"],
                 "refine_sweeps_u": su["mean_sweeps"], "refine_sweeps_v": sv["mean_sweeps"],
-                "roofline": alu_roofline(f64 * stages, f32 * stages, byt * stages, ms / 1e3, PROBE.get("fp64")),
-                "per_element_stage": {"fp64_flops": f64, "fp32_flops": f32, "bytes": byt}}
+                "roofline": element_roofline(imad * stages, byt * stages, ms / 1e3, f64 * stages, f32 * stages),
+                "per_element_stage": {"imad": imad, "bytes": byt, "equivalent_fp64_flops": f64,
+                                      "equivalent_fp32_flops": f32}}
             ctx.close()
         b = states["fp64"]
         for name in ("mixed", "inverse"):
@@ -489,9 +552,9 @@ def forms_routes(steps=64):
 def executed_flops_per_element_stage_3d(n1):
     """FP64 flops the 3-D parity stage kernel executes per element (FMA = 2):
     fluxes 3 directions x n1^2 x (2 faces x 7 + 4 sums/differences), per
-    modal entry 22 (lifts 5 + 7, diagonal solve 2, RK 8), traces one split
+    modal entry 8 FMAs for both fields (RK4 in nested form), traces one split
     dot per direction and field (12 per entry) + 12 n1^2 sums/differences."""
-    return 66 * n1 ** 2 + 34 * n1 ** 3
+    return 66 * n1 ** 2 + 28 * n1 ** 3
 
 
 def ocean_sound_speed(depth):
@@ -534,9 +597,10 @@ def forms_ocean(nx=500, ny=250, N=8, p=3, steps=16):
     E = ctx.energy(u, v)
     ctx.close()
     dof = nx * ny * (N + 1) ** 2
-    f64, _, byt = var_counts(N + 1, 0, 0, "inverse")
+    f64, _, _ = var_counts(N + 1, 0, 0, "inverse")
+    imad, byt = element_work(N + 1, 0, 0, "inverse")
     stages = nx * ny * 4 * steps
-    roof = alu_roofline(f64 * stages, 0.0, byt * stages, ms / 1e3, PROBE.get("fp64"))
+    roof = element_roofline(imad * stages, byt * stages, ms / 1e3, f64 * stages, 0.0)
     return {"roofline": roof,
             "workload": "ocean channel 4000 x 2000 m, c(depth), point source sin(400 pi t) at (1004 m, 300 m "
                         "deep), %d x %d elements of %d x %d cells, p=%d, element inverses" % (nx, ny, N, N, p),
@@ -569,7 +633,7 @@ def forms_three_d(n=32, N=8, p=5, steps=16):
             "dof": dof, "dof_steps_per_s": dof * steps / (ms / 1e3), "ms_per_step": ms / steps,
             "roofline": alu_roofline(f64, 0.0, 16.0 * dof * 4 * steps, ms / 1e3, PROBE.get("fp64")),
             "flops_note": "FP64 flops the 3-D parity stage kernel executes per element and stage "
-                          "(66 n1^2 + 34 n1^3, FMA = 2) over the whole step's time (entry and exit "
+                          "(66 n1^2 + 28 n1^3, FMA = 2) over the whole step's time (entry and exit "
                           "transforms included); bytes: one pass of the FP64 (u, v) state per stage",
             "energy_ratio_after_20_steps": E1 / E0}
 
@@ -611,21 +675,23 @@ def forms_batched(steps=8, nmin=16, nmax=128):
             if sp["variable"] and name != "inverse":
                 batch.stats(i)
         ms = _timed_ms(lambda: batch.step(us, vs, dts, steps))
-        f64 = f32 = byt = 0.0
+        f64 = f32 = imad = byt = 0.0
         for i, sp in enumerate(specs):
             stages = sp["n"] ** 2 * 4 * steps
             if sp["variable"]:
                 su, sv = batch.stats(i) if name != "inverse" else ({"mean_iters": 0, "mean_sweeps": 0},) * 2
-                a, b_, c = var_counts(9, su["mean_iters"], sv["mean_iters"], name, su["mean_sweeps"],
-                                      sv["mean_sweeps"])
+                counts = (9, su["mean_iters"], sv["mean_iters"], name, su["mean_sweeps"], sv["mean_sweeps"])
+                a, b_, _ = var_counts(*counts)
+                d, c = element_work(*counts)
             else:
-                a, b_, c = ALG_FLOPS_PER_DOF_STAGE * 81, 0.0, 16.0 * 81
+                a, b_, d, c = ALG_FLOPS_PER_DOF_STAGE * 81, 0.0, 0.0, 16.0 * 81
             f64 += a * stages
             f32 += b_ * stages
+            imad += d * stages
             byt += c * stages
         out["batched_" + name] = {"dof_steps_per_s": dof * steps / (ms / 1e3), "ms_per_step": ms / steps,
                                   "tuning": batch.tuning(),
-                                  "roofline": alu_roofline(f64, f32, byt, ms / 1e3, PROBE.get("fp64"))}
+                                  "roofline": element_roofline(imad, byt, ms / 1e3, f64, f32)}
         batch.close()
         ctxs = [gdg.Context(b[0]) for b in built]
         for c, u, v, d in zip(ctxs, us, vs, dts):
@@ -670,14 +736,16 @@ def forms_learned(rows=20000, epochs=30, steps=16):
             ctx.step_stats()
             ms = _timed_ms(lambda: ctx.step(u, v, 0.0, dt, steps))
             su, sv = ctx.step_stats()
-            f64, f32, byt = var_counts(9, su["mean_iters"], sv["mean_iters"], name, su["mean_sweeps"],
-                                       sv["mean_sweeps"])
+            counts = (9, su["mean_iters"], sv["mean_iters"], name, su["mean_sweeps"], sv["mean_sweeps"])
+            f64, f32, _ = var_counts(*counts)
+            imad, byt = element_work(*counts)
             stages = 128 * 128 * 4 * steps
-            if attach:   # one forward pass per u_t solve (FP32), plus the guess's FP64 residual product
+            if attach:   # one forward pass per u_t solve (FP32), plus the guess's residual product
                 f32 += 2.0 * (162 * 64 + 64 * 64 + 64 * 81)
                 f64 += 2.0 * 81 * 81
+                imad += 4.0 * 81 * 81
             out[name + ("_learned" if attach else "_plain")] = {
-                "roofline": alu_roofline(f64 * stages, f32 * stages, byt * stages, ms / 1e3, PROBE.get("fp64")),
+                "roofline": element_roofline(imad * stages, byt * stages, ms / 1e3, f64 * stages, f32 * stages),
                 "dof_steps_per_s": 128 * 128 * 81 * steps / (ms / 1e3), "ms_per_step": ms / steps,
                 "pcg_u_mean_iters": su["mean_iters"], "pcg_u_max_iters": su["max_iters"],
                 "guess_fallbacks": su["fell_back"], "guessed": su["guessed"]}
@@ -784,7 +852,7 @@ def run_gdg(args):
         # stage kernel's own duration is the one measured around each launch
         step_stage_ms, stage_ms = stage_ms, stage_ms_isolated
     achieved = ALG_FLOPS_PER_DOF_STAGE * dof() / (stage_ms / 1e3) / 1e12
-    achieved_x = executed_flops_per_stage_launch() / (stage_ms / 1e3) / 1e12
+    achieved_x = step2r_flops_per_stage() / (stage_ms / 1e3) / 1e12
 
     # end to end through the C ABI with host buffers (pinned), copies timed
     hu = torch.tensor(U0.ravel()).pin_memory()
@@ -863,7 +931,7 @@ def run_gdg(args):
                                              "launch (per-stage figures); _isolated: events around that launch "
                                              "in a separate pass, over its 4R stages"),
                          "flops_per_stage": ALG_FLOPS_PER_DOF_STAGE * dof(),
-                         "flops_per_stage_executed": executed_flops_per_stage_launch(),
+                         "flops_per_stage_executed": step2r_flops_per_stage(),
                          "achieved_executed": achieved_x,
                          "frac_executed": achieved_x / FP64_PEAK_TFLOPS,
                          "fp64_pipe_frac": (STEP2R_FP64_INST_PER_ELEMENT_STAGE * w["n"][0] * w["n"][1]
@@ -872,7 +940,7 @@ def run_gdg(args):
                                            if stage_variant == 3 else None,
                          "flops_note": "achieved: 40 algorithmic FP64 flops per DOF and stage (the modal "
                                        "route's per-DOF count) x DOF, per stage of the timed region; "
-                                       "_executed: the flops the parity stage body performs (28.4 per DOF, "
+                                       "_executed: the flops the parity stage body performs (25.2 per DOF, "
                                        "FMA = 2; the r -> 1-r symmetry halves the lifts and trace dots); "
                                        "fp64_pipe_frac: the persistent step's FP64 instructions per stage "
                                        "(ncu count) over the stage time at 2 lanes per SM and clock, the "
