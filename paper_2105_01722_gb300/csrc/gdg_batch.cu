@@ -72,8 +72,8 @@ void enqueue_steps(gdg_batch *b, int nsteps, cudaStream_t s) {
 }
 
 // best of two runs of stages 1, 2 and 3 of the current shape: they read y_n
-// and write the stage buffers and the accumulator, which the real step's
-// stage 1 rewrites, and (stage 2) the traces of y_n, which the caller
+// and write the stage buffers (and the element solves' accumulators), which the
+// real step's stage 1 rewrites, and (stage 2) the traces of y_n, which the caller
 // rebuilds after tuning; stage 4, the one that writes y_n, is not run
 float time_stages(gdg_batch *b, cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1) {
     float t = 1e30f;

@@ -3,18 +3,19 @@
 //
 // The kernel is compiled under three register budgets, one translation unit
 // each so that they compile in parallel; the tuner times them on the batch's
-// own data.  The element-solve bodies need about 60 registers; what a budget
-// buys is resident blocks where shared memory allows them:
-//   BATCH_HI  (gdg_batch.cu)      3 blocks of 96 threads per SM promised:
-//                                 up to 168 registers, nothing spills;
-//   BATCH_MID (gdg_batch_mid.cu)  480 threads per SM: <= 128 registers (the
-//                                 FP64 PCG's 40 KB allow 5 blocks);
-//   BATCH_LO  (gdg_batch_lo.cu)   960 threads per SM: <= 64 registers (the
-//                                 mixed solves' 27 KB allow 8 blocks, and the
-//                                 precomputed-inverse route streams its
-//                                 operators and wants every warp it can get);
-//                                 the modal body reads y_n where it
-//                                 uses it (LEAN).
+// own data.  Every element solve uses the same shared memory (StageSmem; with
+// the parameter slots 33 KB at N1 = 9) and 80 to 128 registers; what a budget
+// buys is resident blocks, and what it costs is spills:
+//   BATCH_HI  (gdg_batch.cu)      3 blocks promised: 240 registers at N1 = 8, 168 above;
+//                                 4, 4 and 3 blocks an SM at N1 = 8, 9 and 10;
+//   BATCH_MID (gdg_batch_mid.cu)  480 threads per SM: 128 registers (N1 = 10 168); 8, 5
+//                                 and 3 blocks;
+//   BATCH_LO  (gdg_batch_lo.cu)   960 threads per SM: 64 registers (N1 = 10 72); 10, 6
+//                                 and 4 blocks, where shared memory ends; the
+//                                 modal body reads y_n where it uses it (LEAN).
+// Picked on batches of 24 problems: MID at N1 = 9 in all forms (8 steps of mixed solves 256 ms,
+// LO 282); LO for inverses at N1 = 8 (66.8 ms for 8
+// steps, MID 70.3) and for PCG and inverses at N1 = 10; HI for mixed solves there.
 #pragma once
 
 #include "gdg_checks.cuh"

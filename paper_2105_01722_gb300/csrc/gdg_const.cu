@@ -19,9 +19,9 @@
 //
 // One RK4 stage is one kernel: read the traces of the stage input (own and
 // neighbours', written by the previous kernel), form fluxes, lifts and the
-// diagonal solves, update the RK accumulator and the next stage input, and
-// write the traces of that next input.  The grid-wide dependency between
-// traces and lifts is the kernel boundary.
+// diagonal solves, form the next stage input (RK4 in nested form, without an
+// accumulator: stage2p_body), and write the traces of that next input.  The
+// grid-wide dependency between traces and lifts is the kernel boundary.
 #include <cstdio>
 #include <algorithm>
 #include <cmath>
@@ -322,9 +322,9 @@ k_stage2f(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) 
 
 // ------------------------------------------------ persistent 2-D step --
 // All RK4 stages of nsteps steps in one cooperative launch (every CTA
-// resident).  Each thread keeps its line's stage input, y_n and RK
-// accumulator in registers from stage to stage; only the face traces go
-// through global memory, and a grid barrier separates the stages.  Every
+// resident).  Each thread keeps its line's stage input and y_n in registers
+// from stage to stage; only the face traces go through global memory, and
+// neighbouring blocks wait for each other between the stages.  Every
 // floating-point operation is the one stage2p_body performs, in the same
 // order, on the same values: bit-identical results to the per-stage kernels.
 
@@ -694,9 +694,9 @@ k_step2e(const __grid_constant__ ModalParams mp, const double *lams, double *nU,
 // Nodes to modes or modes to nodes on the integer pipe (gdg_fxline.cuh), a line
 // of one field of an element a thread: rows through the table of x, then
 // columns through that of y.  tr (modal output (U, V)): also its face traces.
-// 97 x 70 elements, N1 = 9, both fields: 18 us in with the traces and 15 us out,
+// 97 x 70 elements, N1 = 9, both fields: 19 us in with the traces and 15 us out,
 // where FP64 lines by node pairs took 39 and 29 (its pipe was the bound).  Now
-// latency between barriers (issue 30 to 36 %) and, for the traces, the FP64 pipe.
+// latency between barriers (issue 32 to 37 %) and, for the traces, the FP64 pipe.
 constexpr int FX2_THREADS = 128;
 template <int N1> __host__ __device__ constexpr int fx2_tile() { return N1 * (N1 | 1); }   // odd row stride: no bank conflicts
 
@@ -1170,7 +1170,7 @@ __global__ void k_sep1(int ne, const double *in0, const double *in1, double *out
 // ------------------------------------------------------ dispatch ---------
 
 #define GDG_N1_CASES(X) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15) X(16)
-// element sizes of the persistent step (its register state is 6 N1 doubles per thread)
+// element sizes of the persistent step (its register state is 4 N1 doubles per thread)
 #define GDG_N1_CASES_P(X) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10)
 
 size_t smem_stage2(int n1, int epb) { return (size_t)epb * (4 * n1 + 2 * n1 * (n1 + 1)) * sizeof(double); }
@@ -1639,7 +1639,8 @@ int choose_epb(int ne, int n1, int sms, int tpe) {
         int resident = 48 / warps;                          // 48 warps per SM
         const int by_smem = (int)((200.0 * 1024) / (double)sm);
         if (by_smem < resident) resident = by_smem;
-        const int by_regs = 65536 / (warps * 32 * 168);     // the stage kernels use up to ~168 registers
+        const int by_regs = 65536 / (warps * 32 * 168);     // 168 registers a thread: the choices were timed with this
+                                                            // bound (the one-line kernel needs 102)
         if (by_regs < resident) resident = by_regs;
         if (resident < 1) continue;
         const int blocks = (ne + epb - 1) / epb;

@@ -339,9 +339,9 @@ k_stage3p(const __grid_constant__ ModalParams mp, const StageBufs b, double sc) 
 
 // Nodes to modes or modes to nodes on the integer pipe (gdg_fxline.cuh), one
 // line of an element a thread and pass; tr (modal output (U, V)): also its face
-// traces.  32^3 elements, N1 = 9, both fields: 572 us in with the traces (FP64
-// pipe 66 %, those sums and the conversions to doubles; issue 40 %) and 483 us
-// out (issue 44 %), where FP64 lines by node pairs took 2115 and 1641.
+// traces.  32^3 elements, N1 = 9, both fields: 585 us in with the traces (FP64
+// pipe 65 %, those sums and the conversions to doubles; issue 41 %) and 507 us
+// out (issue 45 %), where FP64 lines by node pairs took 2115 and 1641.
 template <int N1, int KIND>
 __global__ void __launch_bounds__(MAXB3, 4)
 k_fx3(const __grid_constant__ ModalParams mp, const __grid_constant__ FxLines<N1, 3> A, const double *in0,
