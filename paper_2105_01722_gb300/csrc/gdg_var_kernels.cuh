@@ -201,12 +201,13 @@ __device__ __forceinline__ T block_sum(T v, double *red) {
 // one element's matrix and the block's scratch
 struct FxSystem {
     const int2 *A;   // packed integers (shared)
-    int d;           // exponent of the thread's row (FX_NAN: the matrix is not finite)
+    int d;           // exponent of the thread's row (FX_BAD: the matrix is not finite)
     int2 *X, *X2;    // limb vectors (shared, 16-byte aligned)
     int *slot;       // shared: two sets of 8 ints, used in turn
 };
 
 constexpr int FX_NAN = 1 << 20;   // block exponent of a vector with an Inf or NaN
+constexpr int FX_NOT = 1 << 14;   // exponents from here on (FX_NAN, FX_BAD): the result is NaN
 #define FX_QNAN __longlong_as_double(0x7ff8000000000000ll)
 
 // exponent of v 2^shift for the maximum of a vector (zero and subnormals: below every other)
@@ -229,7 +230,7 @@ __device__ __forceinline__ int fx_block_max(int k, int *slot, int set) {
 
 // T 2^q, or NaN where the vector behind T had an Inf or NaN
 __device__ __forceinline__ double fx_value(long long T, int q, int emax) {
-    return emax >= FX_NAN / 2 ? FX_QNAN : fx_scale(T, q);
+    return emax >= FX_NOT ? FX_QNAN : fx_scale(T, q);
 }
 
 // mad(entry (t, k), k) over row t of the packed matrix: the columns of earlier
@@ -1003,8 +1004,7 @@ struct StageSmem {
     }
     static constexpr size_t bytes() { return sizeof(double) * (size_t)LEN; }
     __device__ __forceinline__ FxSystem system(const FxMatrix &m, int e) const {
-        const int d = threadIdx.x < NA ? m.d[(size_t)e * NA + threadIdx.x] : 0;
-        return FxSystem{A, d == FX_BAD ? FX_NAN : d, X, X2, slot};
+        return FxSystem{A, threadIdx.x < NA ? m.d[(size_t)e * NA + threadIdx.x] : 0, X, X2, slot};
     }
     __device__ __forceinline__ SolveBufs bufs() const { return SolveBufs{r, z, p, Ap, red, w}; }
 };
@@ -1166,7 +1166,7 @@ k_fm_pack(double *FM, int slope_exp, int staged, short2 *FMq) {
 
 // a row's sum T as a line integral; q: the exponent of its columns
 __device__ __forceinline__ double fx_face_value(long long T, int q, int emax) {
-    return fx_value(T, fx_top_exp(emax) + q, q == FX_BAD ? FX_NAN : emax);
+    return fx_value(T, fx_top_exp(emax) + q, max(emax, q));
 }
 
 // line integrals L[f][m][j] of the element's four faces from its own face
