@@ -2220,8 +2220,11 @@ int gdg_const_step(gdg_ctx *ctx, double *u, double *v, double dt, int nsteps, cu
             return gdg_set_err(ctx, GDG_ETIMEOUT, "persistent step: a grid barrier gave up (wait limit)");
         return gdg_cuda_check(ctx, cudaGetLastError(), "gdg_step (persistent)");
     }
-    // graph of G steps, replayed; the remainder is launched directly
-    const int G = (nsteps >= 16 && !ctx->prof.on) ? 16 : 0;
+    // graph of G steps, replayed; the remainder is launched directly.  A caller's own capture takes the launches of a
+    // 1-D mesh, of any size, one by one (a graph can be launched into none)
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (ctx->dim == 1) cudaStreamIsCapturing(s, &cs);
+    const int G = (nsteps >= 16 && !ctx->prof.on && cs == cudaStreamCaptureStatusNone) ? 16 : 0;
     if (G) {
         GraphCache &gc = ctx->graph;
         if (!gc.exec || gc.dt != dt || gc.steps != G) {

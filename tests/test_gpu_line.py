@@ -52,3 +52,30 @@ def test_periodic_mesh_of_equal_pieces(N, p, n, flux):
     got = _run(n, N, p, np.tile(u, (n // 20, 1)), np.tile(v, (n // 20, 1)), 5, dt, flux=flux, bc=(gdg.BC_PERIODIC,))
     for a, b in zip(got, want):
         assert np.abs(a.reshape(n // 20, 20, N + 1) - b).max() <= 2e-13 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("n", [1000, 14745, 40001])
+@pytest.mark.parametrize("warm", [False, True])
+def test_captured_steps(n, warm):
+    """A call inside a caller's capture, also a context's first one and more steps than the library's own
+    graph has, replays to the bits of the call outside."""
+    import torch
+    problem = lambda: gdg.make_problem(1, (n,), 8, 5)  # noqa: E731
+    u0, v0 = (_gpu(inputs.random_state((n, 9), k)) for k in (1, 2))
+    ctx = gdg.Context(problem())
+    want = u0.clone(), v0.clone()
+    ctx.step(*want, 0.0, 1e-6, 18)
+    if not warm:
+        ctx.close()
+        ctx = gdg.Context(problem())
+    u, v = u0.clone(), v0.clone()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ctx.step(u, v, 0.0, 1e-6, 18)
+    u.copy_(u0)
+    v.copy_(v0)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(u, want[0]) and torch.equal(v, want[1])
+    ctx.close()
