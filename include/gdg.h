@@ -68,7 +68,9 @@ enum { GDG_COEF_CONST = 0, GDG_COEF_NODAL = 1 };
  * every stage then applies them instead of running PCG.  FP64 only
  * (GDG_EUNSUPPORTED with GDG_MIXED); gdg_pcg still runs PCG on such a context.
  * Products with the element matrices and inverses run on 58-bit integers with
- * exact sums in every form, as accurate as FP64 sums (gdg_fx.cuh). */
+ * exact sums in every form, on fields that the element resolves at least as
+ * accurate as FP64 sums on average (gdg_fx.cuh).  Right-hand sides, matrices and
+ * face operators that are not finite give NaN. */
 enum { GDG_SOLVE_DIAG = 0, GDG_SOLVE_PCG = 1, GDG_SOLVE_INVERSE = 2 };
 /* PCG preconditioner: frozen-coefficient diagonalisation, none (plain CG),
  * or the zero fill-in incomplete Cholesky factors of Section 7.1, which the
