@@ -949,7 +949,8 @@ def run_gdg(args):
                                         "152 SM x 2070 MHz x 4 flop/clk; peak_probe: gdg_probe_fp64 "
                                         "(independent FMA chains) timed in this process"},
             "kernels": {k: {"launches": n, "ms": t} for k, (n, t) in prof.items()},
-            "gpu_launches": ((4 * R if stage_variant != 3 else 1) * args.steps + 3 * args.steps
+            # the stages, the transform in (with its traces) and the one out
+            "gpu_launches": ((4 * R if stage_variant != 3 else 1) * args.steps + 2 * args.steps
                              + (2 * (4 * R) * args.steps if world > 1 else 0)),
             "e2e": {"value": e2e_val, "unit": "DOF-steps/s", "h2d_bytes_per_step": 2 * dof() * 8,
                     "d2h_bytes_per_step": 2 * dof() * 8},
